@@ -87,74 +87,6 @@ __global__ void __launch_bounds__(224) conv1_fwd(GradStepArgs a, WorkerTable wt,
   }
 }
 
-// ---- conv2 (16->32, 3x3, pad 1) + ReLU + 2x2 max pool.  A block handles up to CONV_SPB samples of
-// one worker; the filter bank stays in shared memory.  Thread = (pooled position, group of 8 output
-// channels): it accumulates the 2x2 pre-pool window of its 8 channels from a 4x4 input patch.
-__global__ void __launch_bounds__(256) conv2_fwd(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws) {
-  __shared__ float w[4608 + 32];
-  __shared__ float in[16][16][17];
-  const int s = blockIdx.y, tid = threadIdx.x;
-  const float* theta = group_theta(wt, gt, s);
-  for (int t = tid; t < 4640; t += 256) w[t] = theta[OFF_C2W + t];
-  for (int t = tid; t < 16 * 16 * 17; t += 256) (&in[0][0][0])[t] = 0.f;
-  const int i0 = blockIdx.x * CONV_SPB;
-  const int i1 = min(i0 + CONV_SPB, a.b);
-  for (int i = i0; i < i1; ++i) {
-    const int64_t row = (int64_t)s * a.b + i;
-    __syncthreads();
-    for (int t = tid; t < P1_ELEMS; t += 256) {
-      int ic = t / 196, pp = t % 196;
-      in[ic][pp / 14 + 1][pp % 14 + 1] = ws.p1[row * P1_ELEMS + t];
-    }
-    __syncthreads();
-    if (tid < 196) {
-      const int pos = tid % 49, og = tid / 49;
-      const int py = pos / 7, px = pos % 7;
-      float acc[8][4];
-#pragma unroll
-      for (int o = 0; o < 8; ++o) {
-        float bias = w[4608 + og * 8 + o];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[o][j] = bias;
-      }
-      for (int ic = 0; ic < 16; ++ic) {
-        float patch[4][4];
-#pragma unroll
-        for (int yy = 0; yy < 4; ++yy)
-#pragma unroll
-          for (int xx = 0; xx < 4; ++xx) patch[yy][xx] = in[ic][2 * py + yy][2 * px + xx];
-#pragma unroll
-        for (int o = 0; o < 8; ++o) {
-          const float* wk = &w[((og * 8 + o) * 16 + ic) * 9];
-#pragma unroll
-          for (int ky = 0; ky < 3; ++ky)
-#pragma unroll
-            for (int kx = 0; kx < 3; ++kx) {
-              float wv = wk[ky * 3 + kx];
-              acc[o][0] = fmaf(wv, patch[ky][kx], acc[o][0]);
-              acc[o][1] = fmaf(wv, patch[ky][kx + 1], acc[o][1]);
-              acc[o][2] = fmaf(wv, patch[ky + 1][kx], acc[o][2]);
-              acc[o][3] = fmaf(wv, patch[ky + 1][kx + 1], acc[o][3]);
-            }
-        }
-      }
-#pragma unroll
-      for (int o = 0; o < 8; ++o) {
-        float best = 0.f;
-        int bi = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          float r = fmaxf(acc[o][j], 0.f);
-          if (j == 0 || r > best) { best = r; bi = j; }
-        }
-        int idx = (og * 8 + o) * 49 + pos;
-        ws.p2[row * FLAT + idx] = best;
-        ws.code2[row * FLAT + idx] = best > 0.f ? (uint8_t)bi : (uint8_t)4;
-      }
-    }
-  }
-}
-
 // ---- 64x64x16 tiled FP32 product, 256 threads, 4x4 outputs per thread.
 // A(m,k) = A[m*lda + k] (A_KC) or A[k*lda + m]; B(k,n) = B[n*ldb + k] (B_KC) or B[k*ldb + n].
 // All leading dimensions and tile origins are multiples of 4, so float4 loads stay aligned.
@@ -495,88 +427,6 @@ __global__ void __launch_bounds__(256) fc1_dx(GradStepArgs a, GroupTable gt, Wor
   }
 }
 
-// ---- backward through pool2, ReLU and conv2 for up to CONV_SPB samples of one worker:
-// writes dp1 per sample and the block's partial filter / bias gradients.
-constexpr int C2B_SMEM_FLOATS = 4608 + 32 * 16 * 17 + 16 * 16 * 17;
-__global__ void __launch_bounds__(256) conv2_bwd(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws, int n_chunks) {
-  extern __shared__ float smem[];
-  float* w = smem;                                                        // [32][16][9]
-  float (*g2)[16][17] = reinterpret_cast<float (*)[16][17]>(smem + 4608); // [32] padded gradient at conv2 output
-  float (*in)[16][17] = reinterpret_cast<float (*)[16][17]>(smem + 4608 + 32 * 16 * 17);  // [16] padded p1
-  const int s = blockIdx.y, tid = threadIdx.x;
-  const float* theta = group_theta(wt, gt, s);
-  for (int t = tid; t < 4608; t += 256) w[t] = theta[OFF_C2W + t];
-  for (int t = tid; t < 16 * 16 * 17; t += 256) (&in[0][0][0])[t] = 0.f;
-  const int oc_w = tid >> 3, ic_w = (tid & 7) * 2;   // filter-gradient ownership: (oc, two input channels)
-  float gw[2][9], gb = 0.f;
-#pragma unroll
-  for (int h = 0; h < 2; ++h)
-#pragma unroll
-    for (int k = 0; k < 9; ++k) gw[h][k] = 0.f;
-  const int i0 = blockIdx.x * CONV_SPB;
-  const int i1 = min(i0 + CONV_SPB, a.b);
-  for (int i = i0; i < i1; ++i) {
-    const int64_t row = (int64_t)s * a.b + i;
-    __syncthreads();
-    for (int t = tid; t < 32 * 16 * 17; t += 256) (&g2[0][0][0])[t] = 0.f;
-    for (int t = tid; t < P1_ELEMS; t += 256) {
-      int ic = t / 196, pp = t % 196;
-      in[ic][pp / 14 + 1][pp % 14 + 1] = ws.p1[row * P1_ELEMS + t];
-    }
-    __syncthreads();
-    for (int t = tid; t < FLAT; t += 256) {
-      int code = ws.code2[row * FLAT + t];
-      if (code < 4) {
-        int oc = t / 49, pp = t % 49;
-        int y = 2 * (pp / 7) + (code >> 1), x = 2 * (pp % 7) + (code & 1);
-        g2[oc][y + 1][x + 1] = ws.dp2[row * FLAT + t];
-      }
-    }
-    __syncthreads();
-    // gradient with respect to the conv2 input (p1)
-    if (tid < 196) {
-      const int y = tid / 14, x = tid % 14;
-      float acc[16];
-#pragma unroll
-      for (int ic = 0; ic < 16; ++ic) acc[ic] = 0.f;
-      for (int oc = 0; oc < 32; ++oc) {
-#pragma unroll
-        for (int ky = 0; ky < 3; ++ky)
-#pragma unroll
-          for (int kx = 0; kx < 3; ++kx) {
-            float g = g2[oc][y - ky + 2][x - kx + 2];
-            if (g != 0.f) {
-#pragma unroll
-              for (int ic = 0; ic < 16; ++ic) acc[ic] = fmaf(g, w[(oc * 16 + ic) * 9 + ky * 3 + kx], acc[ic]);
-            }
-          }
-      }
-#pragma unroll
-      for (int ic = 0; ic < 16; ++ic) ws.dp1[row * P1_ELEMS + ic * 196 + tid] = acc[ic];
-    }
-    // filter and bias gradients
-    for (int y = 0; y < 14; ++y)
-      for (int x = 0; x < 14; ++x) {
-        float g = g2[oc_w][y + 1][x + 1];
-        if (g != 0.f) {
-          if ((tid & 7) == 0) gb += g;
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int ky = 0; ky < 3; ++ky)
-#pragma unroll
-              for (int kx = 0; kx < 3; ++kx) gw[h][ky * 3 + kx] = fmaf(g, in[ic_w + h][y + ky][x + kx], gw[h][ky * 3 + kx]);
-        }
-      }
-  }
-  float* part = ws.part2 + ((int64_t)s * n_chunks + blockIdx.x) * C2_GRAD;
-#pragma unroll
-  for (int h = 0; h < 2; ++h)
-#pragma unroll
-    for (int k = 0; k < 9; ++k) part[(oc_w * 16 + ic_w + h) * 9 + k] = gw[h][k];
-  if ((tid & 7) == 0) part[4608 + oc_w] = gb;
-}
-
 // ---- backward through pool1, ReLU and conv1 (filter / bias gradients only: the input needs none).
 // Thread (channel, lane of 16) owns 13 pooled positions of its channel.  The image, the pooling decisions
 // and the pooled gradients of the NEXT sample are fetched into registers while the current one is
@@ -805,17 +655,10 @@ int launch_dropout_mask(uint64_t seed, uint32_t worker, uint64_t step, int b, ui
   return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
-int configure_grad_kernels() {
-  cudaError_t e = cudaFuncSetAttribute(conv2_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(C2B_SMEM_FLOATS * sizeof(float)));
-  return e == cudaSuccess ? 0 : -1;
-}
-
 // Evaluation pass: the forward kernels of the grad step with the dropout switched off (the output-layer kernel also
 // produces backward quantities into the workspace; nothing reads them), then the per-worker loss and hit count.
 int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, int32_t* correct,
                 cudaStream_t st, Profiler* prof) {
-  const int n_chunks = (a.b + CONV_SPB - 1) / CONV_SPB;
   const int mt = group_tiles(gt, a.b, 64);
   int launches = 0;
   if (a.precision != 0) {
@@ -828,7 +671,7 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
   } else {
     const int n_chunks1 = (a.b + CONV1_SPB - 1) / CONV1_SPB;
     TIMED(K_CONV1_FWD, (conv1_fwd<<<dim3(n_chunks1, a.W), 224, 0, st>>>(a, wt, gt, ws)));
-    TIMED(K_CONV2_FWD, (conv2_fwd<<<dim3(n_chunks, a.W), 256, 0, st>>>(a, wt, gt, ws)));
+    launch_conv2_direct(true, a, gt, ws, st, prof);
     TIMED(K_FC1_FWD, (fc1_fwd<<<dim3(HID / 64, mt), 256, 0, st>>>(a, wt, gt, ws)));
     launches += 3;
   }
@@ -846,12 +689,11 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
 // first convolution's backward.  Everything joins before the final reduction.
 int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                      cudaStream_t st, const SideStreams& side, Profiler* prof, const SummedStep* sum) {
-  const int n_chunks = (a.b + CONV_SPB - 1) / CONV_SPB;
   const int mt = group_tiles(gt, a.b, 64);
   const bool tc = a.precision != 0;
   const int n_chunks1 = (a.b + CONV1_SPB - 1) / CONV1_SPB;
   const int n_chunks1b = (a.b + CONV1B_SPB - 1) / CONV1B_SPB;
-  int launches = 0, n_chunks2 = n_chunks, seg_len = 0;
+  int launches = 0, n_chunks2 = 0, seg_len = 0;
   // Summed step: the 512-unit layer's weight gradient is taken over groups of workers at once ("super-workers" of
   // W / n_super workers: their samples are consecutive rows, so the product only sees a longer batch) and written to
   // n_super partial vectors instead of one vector per worker.
@@ -900,17 +742,18 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     launches += 4;
   } else {
     TIMED(K_CONV1_FWD, (conv1_fwd<<<dim3(n_chunks1, a.W), 224, 0, st>>>(a, wt, gt, ws)));
-    TIMED(K_CONV2_FWD, (conv2_fwd<<<dim3(n_chunks, a.W), 256, 0, st>>>(a, wt, gt, ws)));
+    launch_conv2_direct(true, a, gt, ws, st, prof);
     TIMED(K_FC1_FWD, (fc1_fwd<<<dim3(HID / 64, mt), 256, 0, st>>>(a, wt, gt, ws)));
     TIMED(K_FC2_FWD_BWD, (fc2_fwd_bwd<<<dim3(a.W, FC2_SPLIT), FC2_THREADS, 0, st>>>(a, wt, gt, ws)));
     if (sum) TIMED(K_FC1_DW, (fc1_dw<<<dim3((FLAT + 63) / 64, HID / 64, a_dw.W), 256, 0, st>>>(a_dw, wt_dw, ws)));
     else TIMED(K_FC1_DW, (fc1_dw<<<dim3((FLAT + 63) / 64, HID / 64, a.W), 256, 0, st>>>(a, wt, ws)));
     TIMED(K_FC1_DX, (fc1_dx<<<dim3((FLAT + 63) / 64, mt), 256, 0, st>>>(a, gt, ws)));
-    TIMED(K_CONV2_BWD, (conv2_bwd<<<dim3(n_chunks, a.W), 256, C2B_SMEM_FLOATS * sizeof(float), st>>>(a, wt, gt, ws, n_chunks)));
+    n_chunks2 = launch_conv2_dw_direct(a, ws, st, prof, &seg_len);
+    launch_conv2_direct(false, a, gt, ws, st, prof);
     TIMED(K_CONV1_BWD, (conv1_bwd<<<dim3(n_chunks1b, a.W), 256, 0, st>>>(a, wt, ws, n_chunks1b)));
-    if (sum) TIMED(K_CONV_GRAD_REDUCE, (fused_finish<<<FUSED_W1_BLOCKS + FUSED_SMALL_BLOCKS, 256, 0, st>>>(a, wt, ws, sum->super_part, sum->n_super, sum->grad_sum, n_chunks1b, 0, n_chunks2, 0)));
-    else TIMED(K_CONV_GRAD_REDUCE, (conv_grad_reduce<<<dim3(a.W, RED_BLOCKS), 256, 0, st>>>(a, wt, ws, n_chunks1b, 0, n_chunks2, 0)));
-    launches = 9;
+    if (sum) TIMED(K_CONV_GRAD_REDUCE, (fused_finish<<<FUSED_W1_BLOCKS + FUSED_SMALL_BLOCKS, 256, 0, st>>>(a, wt, ws, sum->super_part, sum->n_super, sum->grad_sum, n_chunks1b, 0, n_chunks2, seg_len)));
+    else TIMED(K_CONV_GRAD_REDUCE, (conv_grad_reduce<<<dim3(a.W, RED_BLOCKS), 256, 0, st>>>(a, wt, ws, n_chunks1b, 0, n_chunks2, seg_len)));
+    launches = 10;
   }
   return cudaGetLastError() == cudaSuccess ? launches : -1;
 }

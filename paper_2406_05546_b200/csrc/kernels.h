@@ -24,7 +24,7 @@ constexpr int P1_PLANE_ELEMS = 2 * 256 * 4;   // 32-bit words of one sample's p1
 constexpr int FLAT = C2 * H2 * H2;       // 1568
 constexpr int HID = 512, NCLS = 10;
 constexpr int DZ_STRIDE = 16;            // logits gradient row, padded
-constexpr int CONV_SPB = 4;              // samples per block in the conv backward kernels
+constexpr int CONV_SPB = 4;              // samples per partial-sum slot of the convolutions' filter gradients
 constexpr int C2_GRAD = 4608 + 32, C1_GRAD = 144 + 16;
 constexpr int FC2_SPLIT = 1;             // blocks per worker in the output-layer kernel, each with its own partial sums (at 128 registers x 512 threads one block fills an SM, so more blocks only queue)
 constexpr int FC_PART = NCLS * HID + HID + NCLS + 2;   // fc2.w, fc1.b, fc2.b gradients, loss sum, padding
@@ -147,7 +147,9 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
                      cudaStream_t st, const SideStreams& side, Profiler* prof, const SummedStep* sum = nullptr);
 int launch_dropout_mask(uint64_t seed, uint32_t worker, uint64_t step, int b, uint32_t thresh,
                         uint8_t* keep, cudaStream_t st, Profiler* prof);
-int configure_grad_kernels();
+int configure_fp32_conv2_kernels();
+void launch_conv2_direct(bool fwd, const GradStepArgs& a, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
+int launch_conv2_dw_direct(const GradStepArgs& a, const Workspace& ws, cudaStream_t st, Profiler* prof, int* seg_len);
 extern int g_sm_count;   // SMs of the current device, set by configure_tc5_kernels
 int configure_tc5_kernels();
 int configure_conv5_kernels();

@@ -132,8 +132,8 @@ int32_t check_cfg(const ps_config* c) {
 // Lays the context's device and pinned buffers out over the two caller-owned blocks.
 void layout(ps_ctx* x, const ps_config& c, void* arena, void* pinned, uint64_t* arena_bytes, uint64_t* pinned_bytes) {
   const uint64_t rows = (uint64_t)c.max_workers * c.max_batch;
-  // partial-sum slots per worker: one per block of CONV_SPB samples, or four per range of the tensor-core
-  // filter-gradient kernel (at most (b - 1) / 16 + 2 ranges meet a worker)
+  // partial-sum slots per worker: one per block of samples or range of rows that meets the worker, of which the
+  // launch code makes at most this many
   const uint64_t chunks = ((uint64_t)c.max_batch + psk::CONV_SPB - 1) / psk::CONV_SPB + 8;
   Carver a(arena);
   for (int i = 0; i < c.ring_depth; ++i) { float* p = a.take<float>(VEC_BYTES); if (x) x->ring[i] = p; }
@@ -267,7 +267,7 @@ int32_t ps_create(const ps_config* cfg, const float* init_params_host, ps_ctx** 
   x->ckpt_version.assign(x->ckpt_buf.size(), 0);
   double t = std::floor((double)cfg->dropout_p * 4294967296.0);
   x->drop_thresh = t <= 0.0 ? 0u : (t >= 4294967295.0 ? 0xFFFFFFFFu : (uint32_t)t);
-  if (psk::configure_grad_kernels() != 0 || psk::configure_tc5_kernels() != 0 || psk::configure_conv5_kernels() != 0 || psk::configure_conv1_kernels() != 0 || psk::configure_dw5_kernels() != 0 || psk::configure_c1d5_kernels() != 0) { delete x; return fail(PS_ERR_CUDA, "kernel configuration failed: %s", cudaGetErrorString(cudaGetLastError())); }
+  if (psk::configure_fp32_conv2_kernels() != 0 || psk::configure_tc5_kernels() != 0 || psk::configure_conv5_kernels() != 0 || psk::configure_conv1_kernels() != 0 || psk::configure_dw5_kernels() != 0 || psk::configure_c1d5_kernels() != 0) { delete x; return fail(PS_ERR_CUDA, "kernel configuration failed: %s", cudaGetErrorString(cudaGetLastError())); }
   if (cfg->precision != PS_FP32) {
     // two side streams let independent branches of the backward pass overlap (they allocate no device memory)
     bool ok = cudaStreamCreateWithFlags(&x->side.s1, cudaStreamNonBlocking) == cudaSuccess &&

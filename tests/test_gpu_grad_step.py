@@ -21,7 +21,7 @@ def _setup(W, b, n_versions=1, drop_p=0.25, precision=0):
 
 
 def _run_and_compare(W, b, lags=None, n_versions=1, step=3, drop_p=0.25, worker_ids=None, in_slots=False,
-                     precision=0):
+                     precision=0, check=None):
     from oracle import cnn
     tol = TOL_TENSOR if precision else TOL_FP32
     torch, ps, srv, theta0 = _setup(W, b, n_versions, drop_p, precision)
@@ -54,6 +54,8 @@ def _run_and_compare(W, b, lags=None, n_versions=1, step=3, drop_p=0.25, worker_
     og, ol, oa, oz = cnn.workers_grad_step(thetas, ids, x, y, SEED, step, drop_p, precision=precision)
     for w in range(W):
         assert (grads[w, ps.P:] == 0).all()
+        if check is not None and w not in check:
+            continue
         if precision and W * b > 500:
             # several hundred thousand ReLU decisions: a hidden unit within rounding distance of zero may come out the
             # other way; the helper admits that, and only that (see its docstring), so the oracle's intermediates of
@@ -90,6 +92,17 @@ def test_batch_spanning_several_tiles_with_tail():
 def test_stale_snapshots_grouped_over_three_versions():
     # five workers over three distinct weight versions, interleaved so that grouping must reorder
     _run_and_compare(5, 6, lags=[2, 0, 1, 2, 0], n_versions=3)
+
+
+# 128 / 129 and 1,536 / 1,547 rows: the last and first sizes of the FP32 path's three forms of the second convolution;
+# batches that leave one sample over in blocks of five, ranges of rows that cross workers, two weight versions.  At the
+# larger sizes three workers spread over the blocks are compared: all 1,500 samples hold 5 million pooling windows, about
+# one of which has its two largest values within single-precision rounding (2 x 2^-24 x the sum of 10 terms) of a tie, and
+# a winner taken the other way moves the first filter's gradient by more than the tolerance.
+@pytest.mark.parametrize("W,b,kw", [(2, 64, {}), (3, 43, {"lags": [1, 0, 1], "n_versions": 2}), (16, 96, {"check": (0, 8, 15)}),
+                                     (17, 91, {"check": (0, 8, 16)})])
+def test_fp32_path_at_the_edges_of_its_kernel_choices(W, b, kw):
+    _run_and_compare(W, b, **kw)
 
 
 @pytest.mark.parametrize("W,b,kw", [(2, 8, {}), (3, 5, {"worker_ids": [11, 4, 200]}), (2, 150, {}),

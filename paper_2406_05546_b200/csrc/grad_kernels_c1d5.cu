@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(D1_THREADS, 1) conv1_dw_tc5(GradStepArgs a, Wo
 #define TIMED(id, launch) do { if (prof) prof->begin(id, st); launch; if (prof) prof->end(st); } while (0)
 
 int configure_c1d5_kernels() {
-  return cudaFuncSetAttribute(conv1_dw_tc5, cudaFuncAttributeMaxDynamicSharedMemorySize, D1_SMEM) == cudaSuccess ? 0 : -1;
+  return allow_smem((const void*)(conv1_dw_tc5), D1_SMEM) == cudaSuccess ? 0 : -1;
 }
 
 // Returns the number of partial-sum slots reserved per worker (the stride of part1: eight per range), or -1;

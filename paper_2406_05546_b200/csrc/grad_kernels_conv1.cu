@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(C1_THREADS, C1_BLOCKS_PER_SM) conv1_fwd_planes
 #define TIMED(id, launch) do { if (prof) prof->begin(id, st); launch; if (prof) prof->end(st); } while (0)
 
 int configure_conv1_kernels() {
-  return cudaFuncSetAttribute(conv1_fwd_planes, cudaFuncAttributeMaxDynamicSharedMemorySize, C1_SMEM) == cudaSuccess ? 0 : -1;
+  return allow_smem((const void*)(conv1_fwd_planes), C1_SMEM) == cudaSuccess ? 0 : -1;
 }
 
 // The caller's images [W*b][28][28] as a 3-d tensor; a.x must be 16-byte aligned.  Returns 1 (kernels launched) or -1.

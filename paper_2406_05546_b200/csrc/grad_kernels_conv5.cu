@@ -453,8 +453,8 @@ __global__ void __launch_bounds__(THREADS, 2) conv2_dx_tc5(GradStepArgs a, Group
 #define TIMED(id, launch) do { if (prof) prof->begin(id, st); launch; if (prof) prof->end(st); } while (0)
 
 int configure_conv5_kernels() {
-  cudaError_t e = cudaFuncSetAttribute(conv2_fwd_tc5, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(conv2_dx_tc5, cudaFuncAttributeMaxDynamicSharedMemorySize, X_SMEM);
+  cudaError_t e = allow_smem((const void*)(conv2_fwd_tc5), F_SMEM);
+  if (e == cudaSuccess) e = allow_smem((const void*)(conv2_dx_tc5), X_SMEM);
   return e == cudaSuccess ? 0 : -1;
 }
 

@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(W5_THREADS, 1) conv2_dw_tc5(GradStepArgs a, Wo
 #define TIMED(id, launch) do { if (prof) prof->begin(id, st); launch; if (prof) prof->end(st); } while (0)
 
 int configure_dw5_kernels() {
-  return cudaFuncSetAttribute(conv2_dw_tc5, cudaFuncAttributeMaxDynamicSharedMemorySize, W5_SMEM) == cudaSuccess ? 0 : -1;
+  return allow_smem((const void*)(conv2_dw_tc5), W5_SMEM) == cudaSuccess ? 0 : -1;
 }
 
 // Returns the number of partial-sum slots reserved per worker (the stride of part2) and, in *seg_len, the length

@@ -87,89 +87,6 @@ __global__ void __launch_bounds__(224) conv1_fwd(GradStepArgs a, WorkerTable wt,
   }
 }
 
-// ---- 64x64x16 tiled FP32 product, 256 threads, 4x4 outputs per thread.
-// A(m,k) = A[m*lda + k] (A_KC) or A[k*lda + m]; B(k,n) = B[n*ldb + k] (B_KC) or B[k*ldb + n].
-// All leading dimensions and tile origins are multiples of 4, so float4 loads stay aligned.
-template <bool A_KC, bool B_KC>
-__device__ __forceinline__ void gemm_tile_64(const float* __restrict__ A, int lda, const float* __restrict__ B,
-                                             int ldb, int M, int N, int K, int m0, int n0,
-                                             float (&acc)[4][4]) {
-  __shared__ __align__(16) float As[16][68];
-  __shared__ __align__(16) float Bs[16][68];
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    {
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (A_KC) {
-        int m = tid >> 2, k = (tid & 3) * 4;
-        if (m0 + m < M && k0 + k < K) v = *reinterpret_cast<const float4*>(A + (int64_t)(m0 + m) * lda + k0 + k);
-        As[k][m] = v.x; As[k + 1][m] = v.y; As[k + 2][m] = v.z; As[k + 3][m] = v.w;
-      } else {
-        int k = tid >> 4, m = (tid & 15) * 4;
-        if (k0 + k < K && m0 + m < M) v = *reinterpret_cast<const float4*>(A + (int64_t)(k0 + k) * lda + m0 + m);
-        *reinterpret_cast<float4*>(&As[k][m]) = v;
-      }
-    }
-    {
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (B_KC) {
-        int n = tid >> 2, k = (tid & 3) * 4;
-        if (n0 + n < N && k0 + k < K) v = *reinterpret_cast<const float4*>(B + (int64_t)(n0 + n) * ldb + k0 + k);
-        Bs[k][n] = v.x; Bs[k + 1][n] = v.y; Bs[k + 2][n] = v.z; Bs[k + 3][n] = v.w;
-      } else {
-        int k = tid >> 4, n = (tid & 15) * 4;
-        if (k0 + k < K && n0 + n < N) v = *reinterpret_cast<const float4*>(B + (int64_t)(k0 + k) * ldb + n0 + n);
-        *reinterpret_cast<float4*>(&Bs[k][n]) = v;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      float4 av = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-      float4 bv = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-      float ar[4] = {av.x, av.y, av.z, av.w}, br[4] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(ar[r], br[c], acc[r][c]);
-    }
-    __syncthreads();
-  }
-}
-
-// ---- fc1 forward: d = dropout(ReLU(p2 * W1^T + b1)), one product per weight group.
-__global__ void __launch_bounds__(256) fc1_fwd(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws) {
-  int g, m0, m_end;
-  if (!locate_group_tile<64>(gt, a.b, blockIdx.y, g, m0, m_end)) return;
-  const float* theta = gt.theta[g];
-  const int n0 = blockIdx.x * 64;
-  float acc[4][4];
-  gemm_tile_64<true, true>(ws.p2, FLAT, theta + OFF_F1W, FLAT, m_end, HID, FLAT, m0, n0, acc);
-  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-  const int n = n0 + tx * 4;
-  const float4 bias = *reinterpret_cast<const float4*>(theta + OFF_F1B + n);
-  const float scale = 1.0f / (1.0f - a.drop_p);
-  const uint2 key = make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32));
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    int m = m0 + ty * 4 + r;
-    if (m >= m_end) continue;
-    int s = m / a.b, i = m - s * a.b;
-    uint32_t q = (uint32_t)((i * HID + n) >> 2);
-    uint4 rnd = philox4x32_10(make_uint4(q, (uint32_t)wt.wid[s], (uint32_t)a.step, (uint32_t)(a.step >> 32)), key);
-    float4 o;
-    o.x = rnd.x >= a.drop_thresh ? fmaxf(acc[r][0] + bias.x, 0.f) * scale : 0.f;
-    o.y = rnd.y >= a.drop_thresh ? fmaxf(acc[r][1] + bias.y, 0.f) * scale : 0.f;
-    o.z = rnd.z >= a.drop_thresh ? fmaxf(acc[r][2] + bias.z, 0.f) * scale : 0.f;
-    o.w = rnd.w >= a.drop_thresh ? fmaxf(acc[r][3] + bias.w, 0.f) * scale : 0.f;
-    *reinterpret_cast<float4*>(ws.d + (int64_t)m * HID + n) = o;
-  }
-}
-
 // ---- fc2 forward, softmax cross-entropy, argmax, and the backward pass down to the gradient with
 // respect to fc1's pre-activation; then the worker's fc2 weight/bias and fc1 bias gradients.
 // FC2_SPLIT blocks of 16 warps per worker, each with its share of the worker's samples: first four samples per
@@ -389,42 +306,6 @@ __global__ void __launch_bounds__(FC2_THREADS, 1) fc2_fwd_bwd(GradStepArgs a, Wo
   for (int c = 0; c < NCLS; ++c) part[c * HID + j] = gw[c];
   part[NCLS * HID + j] = gb1;
   if (j < NCLS) part[NCLS * HID + HID + j] = gb2;
-}
-
-// ---- fc1 weight gradient of one worker: dW1 [512][1568] = da1^T [512 x b] * p2 [b x 1568].
-__global__ void __launch_bounds__(256) fc1_dw(GradStepArgs a, WorkerTable wt, Workspace ws) {
-  const int s = blockIdx.z, m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  const float* A = ws.da1 + (int64_t)s * a.b * HID;
-  const float* B = ws.p2 + (int64_t)s * a.b * FLAT;
-  float acc[4][4];
-  gemm_tile_64<false, false>(A, HID, B, FLAT, HID, FLAT, a.b, m0, n0, acc);
-  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-  const int n = n0 + tx * 4;
-  if (n >= FLAT) return;
-  float* out = wt.grad[s] + OFF_F1W;
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    int m = m0 + ty * 4 + r;
-    *reinterpret_cast<float4*>(out + (int64_t)m * FLAT + n) = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
-  }
-}
-
-// ---- gradient with respect to p2: dp2 [rows][1568] = da1 [rows][512] * W1 [512][1568], per group.
-__global__ void __launch_bounds__(256) fc1_dx(GradStepArgs a, GroupTable gt, Workspace ws) {
-  int g, m0, m_end;
-  if (!locate_group_tile<64>(gt, a.b, blockIdx.y, g, m0, m_end)) return;
-  const int n0 = blockIdx.x * 64;
-  float acc[4][4];
-  gemm_tile_64<true, false>(ws.da1, HID, gt.theta[g] + OFF_F1W, FLAT, m_end, FLAT, HID, m0, n0, acc);
-  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-  const int n = n0 + tx * 4;
-  if (n >= FLAT) return;
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    int m = m0 + ty * 4 + r;
-    if (m >= m_end) continue;
-    *reinterpret_cast<float4*>(ws.dp2 + (int64_t)m * FLAT + n) = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
-  }
 }
 
 // ---- backward through pool1, ReLU and conv1 (filter / bias gradients only: the input needs none).
@@ -659,7 +540,6 @@ int launch_dropout_mask(uint64_t seed, uint32_t worker, uint64_t step, int b, ui
 // produces backward quantities into the workspace; nothing reads them), then the per-worker loss and hit count.
 int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, int32_t* correct,
                 cudaStream_t st, Profiler* prof) {
-  const int mt = group_tiles(gt, a.b, 64);
   int launches = 0;
   if (a.precision != 0) {
     if (!a.skip_prep_w1) launches += launch_prep_w1(gt, ws, st, prof);
@@ -672,7 +552,7 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
     const int n_chunks1 = (a.b + CONV1_SPB - 1) / CONV1_SPB;
     TIMED(K_CONV1_FWD, (conv1_fwd<<<dim3(n_chunks1, a.W), 224, 0, st>>>(a, wt, gt, ws)));
     launch_conv2_direct(true, a, gt, ws, st, prof);
-    TIMED(K_FC1_FWD, (fc1_fwd<<<dim3(HID / 64, mt), 256, 0, st>>>(a, wt, gt, ws)));
+    launch_fc1_fwd_fp32(a, wt, gt, ws, st, prof);
     launches += 3;
   }
   TIMED(K_FC2_FWD_BWD, (fc2_fwd_bwd<<<dim3(a.W, FC2_SPLIT), FC2_THREADS, 0, st>>>(a, wt, gt, ws)));
@@ -689,7 +569,6 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
 // first convolution's backward.  Everything joins before the final reduction.
 int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                      cudaStream_t st, const SideStreams& side, Profiler* prof, const SummedStep* sum) {
-  const int mt = group_tiles(gt, a.b, 64);
   const bool tc = a.precision != 0;
   const int n_chunks1 = (a.b + CONV1_SPB - 1) / CONV1_SPB;
   const int n_chunks1b = (a.b + CONV1B_SPB - 1) / CONV1B_SPB;
@@ -743,11 +622,10 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
   } else {
     TIMED(K_CONV1_FWD, (conv1_fwd<<<dim3(n_chunks1, a.W), 224, 0, st>>>(a, wt, gt, ws)));
     launch_conv2_direct(true, a, gt, ws, st, prof);
-    TIMED(K_FC1_FWD, (fc1_fwd<<<dim3(HID / 64, mt), 256, 0, st>>>(a, wt, gt, ws)));
+    launch_fc1_fwd_fp32(a, wt, gt, ws, st, prof);
     TIMED(K_FC2_FWD_BWD, (fc2_fwd_bwd<<<dim3(a.W, FC2_SPLIT), FC2_THREADS, 0, st>>>(a, wt, gt, ws)));
-    if (sum) TIMED(K_FC1_DW, (fc1_dw<<<dim3((FLAT + 63) / 64, HID / 64, a_dw.W), 256, 0, st>>>(a_dw, wt_dw, ws)));
-    else TIMED(K_FC1_DW, (fc1_dw<<<dim3((FLAT + 63) / 64, HID / 64, a.W), 256, 0, st>>>(a, wt, ws)));
-    TIMED(K_FC1_DX, (fc1_dx<<<dim3((FLAT + 63) / 64, mt), 256, 0, st>>>(a, gt, ws)));
+    launch_fc1_dw_fp32(sum ? a_dw : a, sum ? wt_dw : wt, gt, ws, st, prof);
+    launch_fc1_dx_fp32(a, wt, gt, ws, st, prof);
     n_chunks2 = launch_conv2_dw_direct(a, ws, st, prof, &seg_len);
     launch_conv2_direct(false, a, gt, ws, st, prof);
     TIMED(K_CONV1_BWD, (conv1_bwd<<<dim3(n_chunks1b, a.W), 256, 0, st>>>(a, wt, ws, n_chunks1b)));

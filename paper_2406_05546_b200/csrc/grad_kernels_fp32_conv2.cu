@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(DW_THREADS, 2) conv2_dw_direct(GradStepArgs a,
 
 template <bool FWD, int NC, int SPB, int CH>
 bool set_smem() {
-  return cudaFuncSetAttribute(conv2_direct<FWD, NC, SPB, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, conv_smem_bytes<FWD, NC, SPB, CH>()) == cudaSuccess;
+  return allow_smem((const void*)(conv2_direct<FWD, NC, SPB, CH>), conv_smem_bytes<FWD, NC, SPB, CH>()) == cudaSuccess;
 }
 
 template <bool FWD, int NC, int SPB, int CH>
@@ -327,7 +327,7 @@ void run_conv(const GradStepArgs& a, const GroupTable& gt, const Workspace& ws, 
 int configure_fp32_conv2_kernels() {
   const bool ok = set_smem<true, 16, 5, 4>() && set_smem<true, 8, 5, 4>() && set_smem<true, 4, 1, 16>() && set_smem<false, 16, 5, 4>() &&
                   set_smem<false, 8, 5, 4>() && set_smem<false, 4, 1, 32>() &&
-                  cudaFuncSetAttribute(conv2_dw_direct, cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM) == cudaSuccess;
+                  allow_smem((const void*)(conv2_dw_direct), DW_SMEM) == cudaSuccess;
   return ok ? 0 : -1;
 }
 

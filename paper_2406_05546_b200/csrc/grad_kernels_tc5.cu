@@ -387,9 +387,9 @@ int configure_tc5_kernels() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || g_sm_count <= 0) return -1;
-  cudaError_t e = cudaFuncSetAttribute(tc5_gemm<EPI_FC1_FWD, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(256, MAX_STAGES, epi_warps(EPI_FC1_FWD)));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(tc5_gemm<EPI_STORE_BF16, 224>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(224, MAX_STAGES, epi_warps(EPI_STORE_BF16)));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(tc5_gemm<EPI_STORE, 224, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(224, MAX_STAGES, epi_warps(EPI_STORE)));
+  cudaError_t e = allow_smem((const void*)(tc5_gemm<EPI_FC1_FWD, 256>), gemm_smem_bytes(256, MAX_STAGES, epi_warps(EPI_FC1_FWD)));
+  if (e == cudaSuccess) e = allow_smem((const void*)(tc5_gemm<EPI_STORE_BF16, 224>), gemm_smem_bytes(224, MAX_STAGES, epi_warps(EPI_STORE_BF16)));
+  if (e == cudaSuccess) e = allow_smem((const void*)(tc5_gemm<EPI_STORE, 224, true>), gemm_smem_bytes(224, MAX_STAGES, epi_warps(EPI_STORE)));
   return e == cudaSuccess ? 0 : -1;
 }
 

@@ -142,6 +142,15 @@ struct SummedStep {
   int n_super;          // groups of W / n_super workers (a divisor of W, at most 16)
 };
 
+// Lets a kernel use `bytes` of dynamic shared memory.  Asked for by every ps_create, so what is already in force is left
+// alone: setting it again for the library's twenty kernels made a new server's first pass 0.1 ms longer.
+inline cudaError_t allow_smem(const void* kernel, int bytes) {
+  cudaFuncAttributes at;
+  const cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+  if (e != cudaSuccess || at.maxDynamicSharedSizeBytes >= bytes) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
 // Part A. Returns the number of kernels launched, or -1 on a launch error.  sum == nullptr: one gradient per worker.
 int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                      cudaStream_t st, const SideStreams& side, Profiler* prof, const SummedStep* sum = nullptr);
@@ -149,6 +158,10 @@ int launch_dropout_mask(uint64_t seed, uint32_t worker, uint64_t step, int b, ui
                         uint8_t* keep, cudaStream_t st, Profiler* prof);
 int configure_fp32_conv2_kernels();
 void launch_conv2_direct(bool fwd, const GradStepArgs& a, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
+int configure_fp32_gemm_kernels();
+void launch_fc1_fwd_fp32(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
+void launch_fc1_dx_fp32(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
+void launch_fc1_dw_fp32(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
 int launch_conv2_dw_direct(const GradStepArgs& a, const Workspace& ws, cudaStream_t st, Profiler* prof, int* seg_len);
 extern int g_sm_count;   // SMs of the current device, set by configure_tc5_kernels
 int configure_tc5_kernels();

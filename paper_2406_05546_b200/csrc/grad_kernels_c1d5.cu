@@ -55,10 +55,10 @@ constexpr int D1_RAW_G = P1_ELEMS * 2, D1_RAW_CODE = P1_ELEMS;
 constexpr int D1_RAW_BYTES = D1_RAW_X + D1_RAW_G + D1_RAW_CODE;                        // 12,544 copied per sample
 constexpr int D1_RAW_SLOT = (D1_RAW_ZERO + D1_RAW_BYTES + 127) / 128 * 128;            // 12,672
 constexpr int D1_NRAW = 5;                               // raw input slots: the q-th sample of the range -> slot q % 5
-constexpr int D1_SMEM = D1_NSTAGE * D1_STAGE_BYTES + D1_NRAW * D1_RAW_SLOT + 256 + 128;
+constexpr int D1_SUM_BYTES = 4 * C1_GRAD * 4;             // one set of sums per write-out warp, added up before they leave
+constexpr int D1_SMEM = D1_NSTAGE * D1_STAGE_BYTES + D1_NRAW * D1_RAW_SLOT + 256 + D1_SUM_BYTES + 128;
 constexpr int D1_TMEM_COLS = 64;                         // 48 accumulator columns
 constexpr int D1_KSTEPS = D1_CHUNKS / 2;                 // 13
-constexpr int D1_SUBSLOTS = 8;                           // partial sums per range: (sample of the pair, window element)
 static_assert(D1_SMEM <= 227 * 1024, "shared memory");
 static_assert(D1_GT == 256, "the item split below assumes 256 threads per group");
 
@@ -99,11 +99,12 @@ __device__ __forceinline__ bool d1_next_unit(D1Walk& w, int r1, int b, D1Unit& u
 }
 
 // Rows (sorted worker, sample) are split into gridDim.x contiguous ranges of seg_len.  Partial sums of worker s go
-// to part1[s][8 (range index - first range of s) + 4 (sample of the pair) + window element].
+// to part1[s][range index - first range of s].
 __global__ void __launch_bounds__(D1_THREADS, 1) conv1_dw_tc5(GradStepArgs a, WorkerTable wt, Workspace ws, int seg_len, int slots) {
   extern __shared__ __align__(1024) uint8_t sm[];
   uint8_t* raw = sm + D1_NSTAGE * D1_STAGE_BYTES;
   D1Bars* bars = reinterpret_cast<D1Bars*>(raw + D1_NRAW * D1_RAW_SLOT);
+  float* sums = reinterpret_cast<float*>(raw + D1_NRAW * D1_RAW_SLOT + 256);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int total = a.W * a.b;
   const int r0 = blockIdx.x * seg_len, r1 = min(r0 + seg_len, total);
@@ -283,9 +284,8 @@ __global__ void __launch_bounds__(D1_THREADS, 1) conv1_dw_tc5(GradStepArgs a, Wo
     }
   } else {
     // ---------------- write-out: warp q reads the accumulator lanes 32 q .. 32 q + 31 = rows (sample q / 2 of the pair,
-    // window elements 2 (q % 2) and 2 (q % 2) + 1, 16 channels each); a sample's sums are in its own 24 columns.  Every
-    // (sample, window element) writes its share of the 160 sums to a partial slot of its own (the final reduction adds
-    // them in a fixed order), so the warps exchange nothing.
+    // window elements 2 (q % 2) and 2 (q % 2) + 1, 16 channels each); a sample's sums are in its own 24 columns.  The two
+    // window elements are added by an exchange, the four warps' sums through shared memory, in a fixed order.
     const int quarter = warp & 3, half = quarter >> 1, my_w = 2 * (quarter & 1) + (lane >> 4), oc = lane & 15;
     int writes = 0;
     D1Walk walk = d1_begin(r0, a.b);
@@ -302,15 +302,27 @@ __global__ void __launch_bounds__(D1_THREADS, 1) conv1_dw_tc5(GradStepArgs a, Wo
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars->acc_empty);
       const int s = un.s;
-      float* part = ws.part1 + (((int64_t)s * slots + (blockIdx.x - (s * a.b) / seg_len)) * D1_SUBSLOTS + 4 * half + my_w) * C1_GRAD;
+      float v[10];                             // the nine taps of the lane's channel, and its bias
       // dW[oc][ky][kx] takes shift (wy + ky, wx + kx) of this window element
 #pragma unroll
       for (int w = 0; w < 4; ++w)
         if (w == my_w) {
 #pragma unroll
-          for (int tap = 0; tap < 9; ++tap) part[oc * 9 + tap] = __uint_as_float(v0[((w >> 1) + tap / 3) * 4 + (w & 1) + tap % 3]);
+          for (int tap = 0; tap < 9; ++tap) v[tap] = __uint_as_float(v0[((w >> 1) + tap / 3) * 4 + (w & 1) + tap % 3]);
         }
-      part[144 + oc] = __uint_as_float(v1[0]);
+      v[9] = __uint_as_float(v1[0]);
+#pragma unroll
+      for (int k = 0; k < 10; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], 16);
+      if (lane < 16) {
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) sums[quarter * C1_GRAD + oc * 9 + tap] = v[tap];
+        sums[quarter * C1_GRAD + 144 + oc] = v[9];
+      }
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      float* part = ws.part1 + ((int64_t)s * slots + (blockIdx.x - (s * a.b) / seg_len)) * C1_GRAD;
+      for (int o = quarter * 32 + lane; o < C1_GRAD; o += 128)
+        part[o] = (sums[o] + sums[C1_GRAD + o]) + (sums[2 * C1_GRAD + o] + sums[3 * C1_GRAD + o]);
+      asm volatile("bar.sync 1, 128;" ::: "memory");
       ++writes;
     }
   }
@@ -334,12 +346,14 @@ int configure_c1d5_kernels() {
   return allow_smem((const void*)(conv1_dw_tc5), D1_SMEM) == cudaSuccess ? 0 : -1;
 }
 
-// Returns the number of partial-sum slots reserved per worker (the stride of part1: eight per range), or -1;
-// *seg_len receives the length of a CTA's range of rows: worker s owns eight partial sums per range that meets its rows.
+// Returns the number of partial-sum slots reserved per worker (the stride of part1); *seg_len receives the length of a
+// CTA's range of rows: worker s owns one partial sum per range that meets its rows.
 int launch_conv1_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const Workspace& ws, cudaStream_t st, Profiler* prof,
                         int* seg_len) {
   const int total = a.W * a.b;
-  int grid = total / 16;                  // a range is at least 16 rows long (bounds the partial sums per worker)
+  // A range is at least four rows long (bounds the partial sums per worker).  With sixteen, and eight partial sums per range,
+  // the kernel took 18 us at 16 to 1,024 rows (conv2's likewise 21 - 25); now 12 - 15 (13 - 19).
+  int grid = total / MIN_RANGE;
   if (grid > g_sm_count) grid = g_sm_count;
   if (grid < 1) grid = 1;
   const int len = (total + grid - 1) / grid;
@@ -347,7 +361,7 @@ int launch_conv1_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const Work
   const int slots = (a.b - 1) / len + 2;
   TIMED(K_CONV1_BWD, (conv1_dw_tc5<<<grid, D1_THREADS, D1_SMEM, st>>>(a, wt, ws, len, slots)));
   *seg_len = len;
-  return D1_SUBSLOTS * slots;
+  return slots;
 }
 
 }  // namespace psk

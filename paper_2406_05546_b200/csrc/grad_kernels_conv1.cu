@@ -23,7 +23,7 @@ namespace {
 constexpr int C1_SPS = 1;                                // samples per step
 constexpr int C1_THREADS = 112 * C1_SPS;
 constexpr int C1_BLOCKS_PER_SM = 6 / C1_SPS;
-constexpr int C1_SPB = 4;                                // samples per block, taken C1_SPS at a time
+constexpr int C1_SPB = 4;                                // most samples per block, taken C1_SPS at a time
 constexpr int C1_BOX_W = 36, C1_BOX_H = 30;              // image box: columns -4..31 (a 16-byte aligned start), rows -1..28
 constexpr int C1_BOX_BYTES = C1_BOX_W * C1_BOX_H * 4;    // 4320
 constexpr int C1_IMG_SLOT = 4352;                        // box padded to a multiple of 128 bytes
@@ -40,13 +40,13 @@ constexpr int C1_SMEM = C1_STAGES * C1_IN_BYTES + 2 * C1_OUT_BYTES + 64 + 128;
 // multiply-add phases of all warps of a block, and with few large blocks the FMA pipe idles while all of them
 // pool and store.
 __global__ void __launch_bounds__(C1_THREADS, C1_BLOCKS_PER_SM) conv1_fwd_planes(const __grid_constant__ CUtensorMap xmap, GradStepArgs a,
-                                                                  WorkerTable wt, GroupTable gt, Workspace ws) {
+                                                                  WorkerTable wt, GroupTable gt, Workspace ws, int spb) {
   extern __shared__ __align__(128) uint8_t sm[];
   const float* in = reinterpret_cast<const float*>(sm);
   uint8_t* outb = sm + C1_STAGES * C1_IN_BYTES;
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + C1_STAGES * C1_IN_BYTES + 2 * C1_OUT_BYTES);
   const int s = blockIdx.y, tid = threadIdx.x, cg = tid & 3;
-  const int i0 = blockIdx.x * C1_SPB, i1 = min(i0 + C1_SPB, a.b);
+  const int i0 = blockIdx.x * spb, i1 = min(i0 + spb, a.b);
   const int n_steps = (i1 - i0 + C1_SPS - 1) / C1_SPS;
   const float* theta = group_theta(wt, gt, s);
   if (tid == 0) {
@@ -161,8 +161,13 @@ int launch_conv1_fwd_planes(const GradStepArgs& a, const WorkerTable& wt, const 
   const uint64_t strides[2] = {IMG * 4, IMG * IMG * 4};
   const uint32_t box[3] = {C1_BOX_W, C1_BOX_H, 1};
   if (!encode_tensor_map_f32(&xmap, a.x, 3, dims, strides, box)) return -1;
-  const int chunks = (a.b + C1_SPB - 1) / C1_SPB;
-  TIMED(K_CONV1_FWD, (conv1_fwd_planes<<<dim3(chunks, a.W), C1_THREADS, C1_SMEM, st>>>(xmap, a, wt, gt, ws)));
+  // A block's samples follow one another, so with fewer blocks than fit on the chip (six per SM) it takes fewer of them:
+  // 16.5 -> 9 / 10 / 12 us at 16 / 185 / 512 rows with one sample per block, 19 -> 17 us at 1,024 rows with two
+  // (~6 us of event overhead included)
+  const int slots = C1_BLOCKS_PER_SM * g_sm_count, rows = a.W * a.b;
+  const int spb = rows <= slots ? 1 : (rows <= 2 * slots ? 2 : C1_SPB);
+  const int chunks = (a.b + spb - 1) / spb;
+  TIMED(K_CONV1_FWD, (conv1_fwd_planes<<<dim3(chunks, a.W), C1_THREADS, C1_SMEM, st>>>(xmap, a, wt, gt, ws, spb)));
   return 1;
 }
 

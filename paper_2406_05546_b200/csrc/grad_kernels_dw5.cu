@@ -301,7 +301,7 @@ int configure_dw5_kernels() {
 int launch_conv2_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const Workspace& ws, cudaStream_t st, Profiler* prof,
                         int* seg_len) {
   const int total = a.W * a.b;
-  int grid = total / 16;                  // a range is at least 16 rows long (bounds the partial sums per worker)
+  int grid = total / MIN_RANGE;           // a range is at least four rows long (bounds the partial sums per worker)
   if (grid > g_sm_count) grid = g_sm_count;
   if (grid < 1) grid = 1;
   const int len = (total + grid - 1) / grid;

@@ -382,8 +382,8 @@ __global__ void __launch_bounds__(256) conv1_bwd(GradStepArgs a, WorkerTable wt,
 }
 
 // ---- sums the per-block partial gradients in block order, finishes the loss and zeroes the padding.
-// part2 holds n_chunks2 slots per worker; all of them are summed when seg_len == 0, otherwise one for every
-// range of seg_len rows that meets the worker's b rows (the tensor-core filter-gradient kernel's layout).
+// part1 and part2 hold n_chunks / n_chunks2 slots per worker; all of them are summed when seg_len == 0, otherwise one
+// for every range of seg_len rows that meets the worker's b rows.
 // A worker's outputs are numbered conv2 (4640), conv1 (160), output layer (5642), loss, padding; a block takes
 // RED_PER_BLOCK of them.
 constexpr int RED_PER_BLOCK = 1024;
@@ -394,8 +394,7 @@ __global__ void __launch_bounds__(256) conv_grad_reduce(GradStepArgs a, WorkerTa
   const int s = blockIdx.x, b = a.b;
   float* grad = wt.grad[s];
   const int used2 = seg_len > 0 ? (s * b + b - 1) / seg_len - (s * b) / seg_len + 1 : n_chunks2;
-  // part1 likewise: all n_chunks slots, or eight (sample of a pair x window element) for every range of seg_len1 rows
-  const int used1 = seg_len1 > 0 ? 8 * ((s * b + b - 1) / seg_len1 - (s * b) / seg_len1 + 1) : n_chunks;
+  const int used1 = seg_len1 > 0 ? (s * b + b - 1) / seg_len1 - (s * b) / seg_len1 + 1 : n_chunks;
   for (int v = blockIdx.y * RED_PER_BLOCK + threadIdx.x; v < min(RED_OUTPUTS, ((int)blockIdx.y + 1) * RED_PER_BLOCK); v += 256) {
     int o = v;
     if (o < C2_GRAD) {
@@ -473,7 +472,7 @@ __global__ void __launch_bounds__(256) fused_finish(GradStepArgs a, WorkerTable 
   } else if (o < C2_GRAD + C1_GRAD) {
     const int oo = o - C2_GRAD;
     for (int s = lane; s < a.W; s += 32) {
-      const int used1 = seg_len1 > 0 ? 8 * ((s * b + b - 1) / seg_len1 - (s * b) / seg_len1 + 1) : n_chunks;
+      const int used1 = seg_len1 > 0 ? (s * b + b - 1) / seg_len1 - (s * b) / seg_len1 + 1 : n_chunks;
       for (int c = 0; c < used1; ++c) t += ws.part1[((int64_t)s * n_chunks + c) * C1_GRAD + oo];
     }
     dst = grad_sum + OFF_C1W + oo;

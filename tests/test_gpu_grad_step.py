@@ -145,7 +145,10 @@ def test_fp32_path_at_the_edges_of_its_kernel_choices(W, b, kw):
                                      (2, 4, {"drop_p": 0.0}),
                                      # 777 rows over two weight versions: the persistent convolution kernels take
                                      # ranges of several rows that cross worker boundaries inside a version group
-                                     (7, 111, {"lags": [1, 0, 1, 1, 0, 0, 1], "n_versions": 2})])
+                                     (7, 111, {"lags": [1, 0, 1, 1, 0, 0, 1], "n_versions": 2}),
+                                     # 896 rows: the first convolution takes two samples per block; 6 rows: ranges of
+                                     # the filter gradients shorter than four rows
+                                     (8, 112, {}), (3, 2, {})])
 def test_tensor_core_path(W, b, kw):
     _run_and_compare(W, b, precision=2, **kw)
 

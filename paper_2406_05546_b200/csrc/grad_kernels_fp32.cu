@@ -87,227 +87,6 @@ __global__ void __launch_bounds__(224) conv1_fwd(GradStepArgs a, WorkerTable wt,
   }
 }
 
-// ---- fc2 forward, softmax cross-entropy, argmax, and the backward pass down to the gradient with
-// respect to fc1's pre-activation; then the worker's fc2 weight/bias and fc1 bias gradients.
-// FC2_SPLIT blocks of 16 warps per worker, each with its share of the worker's samples: first four samples per
-// warp at a time; then thread = hidden unit sums its outputs over the block's samples in sample order, many
-// loads in flight.  The block's sums (and its share of the loss) are partial results added later in block order.
-constexpr int FC2_THREADS = 512;
-constexpr int FC2_NS = 4;          // samples per warp and pass
-constexpr int DZ_CHUNK = 128;      // samples whose logits gradients are held in shared memory at a time
-constexpr int W2T_PITCH = 12;      // 48-byte rows: 16-byte loads of consecutive rows fall on distinct banks
-__global__ void __launch_bounds__(FC2_THREADS, 1) fc2_fwd_bwd(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws) {
-  __shared__ __align__(16) float w2t[HID][W2T_PITCH];     // w2t[j][c] = W2[c][j]; the two pad columns are zero
-  __shared__ __align__(16) float dzs[DZ_CHUNK][W2T_PITCH];   // logits gradients of a chunk of samples
-  __shared__ float b2[NCLS];
-  __shared__ float warp_loss[FC2_THREADS / 32];
-  const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float* theta = group_theta(wt, gt, s);
-  const int src = wt.src[s];
-  const int per = ((a.b + FC2_SPLIT - 1) / FC2_SPLIT + 1) & ~1;          // samples per block, even
-  const int i_lo = min(a.b, (int)blockIdx.y * per), i_hi = min(a.b, i_lo + per);
-  for (int t = tid; t < NCLS * HID; t += FC2_THREADS) w2t[t % HID][t / HID] = theta[OFF_F2W + t];
-  w2t[tid][NCLS] = w2t[tid][NCLS + 1] = 0.f;
-  if (tid < NCLS) b2[tid] = theta[OFF_F2B + tid];
-  __syncthreads();
-  const float scale = 1.0f / (1.0f - a.drop_p);
-  const float inv_b = 1.0f / (float)a.b;
-  float loss_acc = 0.f;
-  // Four samples per warp and pass, so that every weight read from shared memory is used four times.  A lane owns
-  // the 16 hidden units lane + 32 t.
-  const bool hi16 = lane & 16, hi8 = lane & 8, hi4 = lane & 4;
-  const int my_u = lane >> 3, sub = lane & 7;          // after the reduction a lane works for sample my_u of the pass
-  for (int i0 = i_lo + FC2_NS * warp; i0 < i_hi; i0 += FC2_NS * (FC2_THREADS / 32)) {
-    const int n_s = min(FC2_NS, i_hi - i0);              // warp-uniform
-    const bool mine = my_u < n_s;
-    // the weights are re-read from shared memory on every pass: 160 of them per lane would not fit in the
-    // registers of a 512-thread block, so their address is made to look pass-dependent
-    uint32_t opaque_zero;
-    asm volatile("mov.u32 %0, 0;" : "=r"(opaque_zero));
-    const float4* w2p = reinterpret_cast<const float4*>(&w2t[0][0] + opaque_zero);
-    const int64_t row0 = (int64_t)s * a.b + i0;
-    // the label is asked for now: by the time the softmax needs it, it has arrived
-    int label = a.y[(int64_t)src * a.b + i0 + (mine ? my_u : 0)];
-    // classes in pairs, one packed multiply-add per pair: zp[u][k] = logits 2k and 2k + 1 of sample u
-    u64 zp[FC2_NS][NCLS / 2];
-    uint32_t live[FC2_NS];                               // which of the lane's 16 units passed ReLU and dropout
-#pragma unroll
-    for (int u = 0; u < FC2_NS; ++u) {
-      live[u] = 0u;
-#pragma unroll
-      for (int k = 0; k < NCLS / 2; ++k) zp[u][k] = 0ull;
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {                        // the units in two halves, to bound the registers
-      float dv[FC2_NS][8];
-#pragma unroll
-      for (int u = 0; u < FC2_NS; ++u)
-#pragma unroll
-        for (int t = 0; t < 8; ++t) dv[u][t] = ws.d[(row0 + (u < n_s ? u : 0)) * HID + lane + 32 * (8 * h + t)];
-#pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        const float4* wr = w2p + (lane + 32 * (8 * h + t)) * (W2T_PITCH / 4);
-        const float4 q0 = wr[0], q1 = wr[1], q2 = wr[2];
-        const u64 wk[NCLS / 2] = {pack2(q0.x, q0.y), pack2(q0.z, q0.w), pack2(q1.x, q1.y), pack2(q1.z, q1.w), pack2(q2.x, q2.y)};
-#pragma unroll
-        for (int u = 0; u < FC2_NS; ++u) {
-          live[u] |= (dv[u][t] > 0.f ? 1u : 0u) << (8 * h + t);
-          const u64 du = pack2(dv[u][t], dv[u][t]);
-#pragma unroll
-          for (int k = 0; k < NCLS / 2; ++k) zp[u][k] = ffma2(wk[k], du, zp[u][k]);
-        }
-      }
-    }
-    // Sum over the lanes.  Each exchange halves what a lane goes on with: after the first two a lane holds the ten
-    // partial logits of sample lane / 8 only, after the third five of them; two plain exchanges finish the sums and a
-    // last one brings the two halves of the classes together.
-    float v[FC2_NS * NCLS];
-#pragma unroll
-    for (int u = 0; u < FC2_NS; ++u)
-#pragma unroll
-      for (int k = 0; k < NCLS / 2; ++k) unpack2(zp[u][k], v[u * NCLS + 2 * k], v[u * NCLS + 2 * k + 1]);
-    float w20[2 * NCLS], x10[NCLS], y5[NCLS / 2], z[NCLS];
-#pragma unroll
-    for (int k = 0; k < 2 * NCLS; ++k) {
-      const float keep = hi16 ? v[2 * NCLS + k] : v[k], send = hi16 ? v[k] : v[2 * NCLS + k];
-      w20[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-    }
-#pragma unroll
-    for (int k = 0; k < NCLS; ++k) {
-      const float keep = hi8 ? w20[NCLS + k] : w20[k], send = hi8 ? w20[k] : w20[NCLS + k];
-      x10[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-#pragma unroll
-    for (int k = 0; k < NCLS / 2; ++k) {
-      const float keep = hi4 ? x10[NCLS / 2 + k] : x10[k], send = hi4 ? x10[k] : x10[NCLS / 2 + k];
-      y5[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-      y5[k] += __shfl_xor_sync(0xffffffffu, y5[k], 2);
-      y5[k] += __shfl_xor_sync(0xffffffffu, y5[k], 1);
-    }
-#pragma unroll
-    for (int k = 0; k < NCLS / 2; ++k) {
-      const float other = __shfl_xor_sync(0xffffffffu, y5[k], 4);
-      z[k] = (hi4 ? other : y5[k]) + b2[k];
-      z[NCLS / 2 + k] = (hi4 ? y5[k] : other) + b2[NCLS / 2 + k];
-    }
-    // softmax, loss and logits gradient of the lane's sample (the eight lanes of a sample do the same work)
-    float dzl[NCLS];
-    {
-      float zmax = z[0];
-      int am = 0;
-#pragma unroll
-      for (int c = 1; c < NCLS; ++c)
-        if (z[c] > zmax) { zmax = z[c]; am = c; }
-      float ez[NCLS], se = 0.f;
-#pragma unroll
-      for (int c = 0; c < NCLS; ++c) { ez[c] = expf(z[c] - zmax); se += ez[c]; }
-      const float lse = zmax + logf(se), inv_se = 1.0f / se;
-      if (label < 0 || label >= NCLS) {
-        if (mine && sub == 0) atomicOr(ws.status, STATUS_BAD_LABEL);
-        label = 0;
-      }
-      float zy = 0.f;
-#pragma unroll
-      for (int c = 0; c < NCLS; ++c) {
-        if (c == label) zy = z[c];
-        const float g = (ez[c] * inv_se - (c == label ? 1.f : 0.f)) * inv_b;     // softmax from the exponentials already taken
-        dzl[c] = mine ? g : 0.f;
-      }
-      if (mine) {
-        loss_acc += lse - zy;
-        if (sub == 0) a.argmax[(int64_t)src * a.b + i0 + my_u] = am;
-        float e0 = 0.f, e1 = 0.f;                          // lane sub of a sample stores elements 2 sub and 2 sub + 1 of its padded row
-#pragma unroll
-        for (int m = 0; m < NCLS / 2; ++m)
-          if (sub == m) { e0 = dzl[2 * m]; e1 = dzl[2 * m + 1]; }
-        *reinterpret_cast<float2*>(ws.dz + (row0 + my_u) * DZ_STRIDE + 2 * sub) = make_float2(e0, e1);
-      }
-    }
-    // every lane needs the logits gradients of all four samples, as class pairs
-    u64 dzk[FC2_NS][NCLS / 2];
-#pragma unroll
-    for (int u = 0; u < FC2_NS; ++u)
-#pragma unroll
-      for (int k = 0; k < NCLS / 2; ++k)
-        dzk[u][k] = pack2(__shfl_sync(0xffffffffu, dzl[2 * k], 8 * u), __shfl_sync(0xffffffffu, dzl[2 * k + 1], 8 * u));
-    asm volatile("mov.u32 %0, 0;" : "=r"(opaque_zero));    // second read of the weights, as above
-    w2p = reinterpret_cast<const float4*>(&w2t[0][0] + opaque_zero);
-#pragma unroll 2
-    for (int t = 0; t < 16; ++t) {
-      const int j = lane + 32 * t;
-      const float4* wr = w2p + j * (W2T_PITCH / 4);
-      const float4 q0 = wr[0], q1 = wr[1], q2 = wr[2];
-      const u64 wk[NCLS / 2] = {pack2(q0.x, q0.y), pack2(q0.z, q0.w), pack2(q1.x, q1.y), pack2(q1.z, q1.w), pack2(q2.x, q2.y)};
-#pragma unroll
-      for (int u = 0; u < FC2_NS; ++u) {
-        // even classes accumulate in the low half, odd classes in the high half; the halves are added at the end
-        u64 e = 0ull;
-#pragma unroll
-        for (int k = 0; k < NCLS / 2; ++k) e = ffma2(wk[k], dzk[u][k], e);
-        float lo, hi;
-        unpack2(e, lo, hi);
-        float o = (live[u] >> t) & 1u ? (lo + hi) * scale : 0.f;
-        if (a.precision != 0) o = round_tf32(o);             // it feeds tensor-core products only
-        if (u < n_s) ws.da1[(row0 + u) * HID + j] = o;
-      }
-    }
-  }
-  {
-    // the eight lanes of a sample hold the same loss: one of each, in lane order
-    const float l0 = __shfl_sync(0xffffffffu, loss_acc, 0), l1 = __shfl_sync(0xffffffffu, loss_acc, 8);
-    const float l2 = __shfl_sync(0xffffffffu, loss_acc, 16), l3 = __shfl_sync(0xffffffffu, loss_acc, 24);
-    loss_acc = (l0 + l1) + (l2 + l3);
-  }
-  if (lane == 0) warp_loss[warp] = loss_acc;
-  __syncthreads();   // also makes this block's dz / da1 stores visible to all of its threads
-  float* part = ws.partf + ((int64_t)s * FC2_SPLIT + blockIdx.y) * FC_PART;
-  if (tid == 0) {
-    float t = 0.f;
-    for (int w = 0; w < FC2_THREADS / 32; ++w) t += warp_loss[w];
-    part[NCLS * HID + HID + NCLS] = t;
-  }
-  const int j = tid;                                  // hidden unit (FC2_THREADS == HID)
-  float gw[NCLS], gb1 = 0.f, gb2 = 0.f;
-#pragma unroll
-  for (int c = 0; c < NCLS; ++c) gw[c] = 0.f;
-  const float* dzp = ws.dz + (int64_t)s * a.b * DZ_STRIDE;
-  const float* dp = ws.d + (int64_t)s * a.b * HID + j;
-  const float* da1p = ws.da1 + (int64_t)s * a.b * HID + j;
-  u64 gwk[NCLS / 2];
-#pragma unroll
-  for (int k = 0; k < NCLS / 2; ++k) gwk[k] = 0ull;
-  // The logits gradients of DZ_CHUNK samples at a time are brought into shared memory, where every thread reads
-  // them as broadcasts; what is left per sample is two loads from global memory, many of them in flight.
-  for (int c0 = i_lo; c0 < i_hi; c0 += DZ_CHUNK) {
-    const int n = min(DZ_CHUNK, i_hi - c0);
-    __syncthreads();
-    for (int t = tid; t < n * (W2T_PITCH / 4); t += FC2_THREADS) {
-      const int i = t / (W2T_PITCH / 4), q = t - i * (W2T_PITCH / 4);
-      reinterpret_cast<float4*>(&dzs[i][0])[q] = *reinterpret_cast<const float4*>(dzp + (c0 + i) * DZ_STRIDE + 4 * q);
-    }
-    __syncthreads();
-#pragma unroll 16
-    for (int i = 0; i < n; ++i) {
-      const float dval = dp[(int64_t)(c0 + i) * HID];
-      const float4* zr = reinterpret_cast<const float4*>(&dzs[i][0]);
-      const float4 z0 = zr[0], z1 = zr[1], z2 = zr[2];
-      const u64 dzk[NCLS / 2] = {pack2(z0.x, z0.y), pack2(z0.z, z0.w), pack2(z1.x, z1.y), pack2(z1.z, z1.w), pack2(z2.x, z2.y)};
-      const u64 dd = pack2(dval, dval);
-#pragma unroll
-      for (int k = 0; k < NCLS / 2; ++k) gwk[k] = ffma2(dzk[k], dd, gwk[k]);
-      gb1 += da1p[(int64_t)(c0 + i) * HID];
-    }
-    if (j < NCLS)
-      for (int i = 0; i < n; ++i) gb2 += dzs[i][j];
-  }
-#pragma unroll
-  for (int k = 0; k < NCLS / 2; ++k) unpack2(gwk[k], gw[2 * k], gw[2 * k + 1]);
-#pragma unroll
-  for (int c = 0; c < NCLS; ++c) part[c * HID + j] = gw[c];
-  part[NCLS * HID + j] = gb1;
-  if (j < NCLS) part[NCLS * HID + HID + j] = gb2;
-}
-
 // ---- backward through pool1, ReLU and conv1 (filter / bias gradients only: the input needs none).
 // Thread (channel, lane of 16) owns 13 pooled positions of its channel.  The image, the pooling decisions
 // and the pooled gradients of the NEXT sample are fetched into registers while the current one is
@@ -385,36 +164,45 @@ __global__ void __launch_bounds__(256) conv1_bwd(GradStepArgs a, WorkerTable wt,
 // part1 and part2 hold n_chunks / n_chunks2 slots per worker; all of them are summed when seg_len == 0, otherwise one
 // for every range of seg_len rows that meets the worker's b rows.
 // A worker's outputs are numbered conv2 (4640), conv1 (160), output layer (5642), loss, padding; a block takes
-// RED_PER_BLOCK of them.
-constexpr int RED_PER_BLOCK = 1024;
+// `per_block` of them.  With few workers the time is a thread's chain of loads, so its terms are fetched eight at a time.
 constexpr int RED_OUTPUTS = C2_GRAD + C1_GRAD + (NCLS * HID + HID + NCLS) + 1 + (P_PAD - P);
-constexpr int RED_BLOCKS = (RED_OUTPUTS + RED_PER_BLOCK - 1) / RED_PER_BLOCK;
-__global__ void __launch_bounds__(256) conv_grad_reduce(GradStepArgs a, WorkerTable wt, Workspace ws, int n_chunks, int seg_len1,
+
+// p[0] + p[stride] + ... (n terms, in order), eight loads in flight
+__device__ __forceinline__ float sum_slots(const float* p, int n, int64_t stride) {
+  float t = 0.f;
+  for (int c = 0; c < n; c += 8) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = c + u < n ? p[(c + u) * stride] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) t += v[u];
+  }
+  return t;
+}
+// slots of worker s in use
+__device__ __forceinline__ int used_slots(int s, int b, int seg_len, int n_chunks) {
+  return seg_len > 0 ? (s * b + b - 1) / seg_len - (s * b) / seg_len + 1 : n_chunks;
+}
+
+__global__ void __launch_bounds__(256) conv_grad_reduce(GradStepArgs a, WorkerTable wt, Workspace ws, int per_block, int n_chunks, int seg_len1,
                                                         int n_chunks2, int seg_len) {
-  const int s = blockIdx.x, b = a.b;
+  const int s = blockIdx.x, b = a.b, split = fc2_split(a.W, b);
   float* grad = wt.grad[s];
-  const int used2 = seg_len > 0 ? (s * b + b - 1) / seg_len - (s * b) / seg_len + 1 : n_chunks2;
-  const int used1 = seg_len1 > 0 ? (s * b + b - 1) / seg_len1 - (s * b) / seg_len1 + 1 : n_chunks;
-  for (int v = blockIdx.y * RED_PER_BLOCK + threadIdx.x; v < min(RED_OUTPUTS, ((int)blockIdx.y + 1) * RED_PER_BLOCK); v += 256) {
+  const int used2 = used_slots(s, b, seg_len, n_chunks2), used1 = used_slots(s, b, seg_len1, n_chunks);
+  for (int v = blockIdx.y * per_block + threadIdx.x; v < min(RED_OUTPUTS, ((int)blockIdx.y + 1) * per_block); v += 256) {
     int o = v;
     if (o < C2_GRAD) {
-      float t = 0.f;
-      for (int c = 0; c < used2; ++c) t += ws.part2[((int64_t)s * n_chunks2 + c) * C2_GRAD + o];
-      grad[OFF_C2W + o] = t;
+      grad[OFF_C2W + o] = sum_slots(ws.part2 + (int64_t)s * n_chunks2 * C2_GRAD + o, used2, C2_GRAD);
       continue;
     }
     o -= C2_GRAD;
     if (o < C1_GRAD) {
-      float t = 0.f;
-      for (int c = 0; c < used1; ++c) t += ws.part1[((int64_t)s * n_chunks + c) * C1_GRAD + o];
-      grad[OFF_C1W + o] = t;
+      grad[OFF_C1W + o] = sum_slots(ws.part1 + (int64_t)s * n_chunks * C1_GRAD + o, used1, C1_GRAD);
       continue;
     }
     o -= C1_GRAD;
     if (o <= NCLS * HID + HID + NCLS) {
-      float t = 0.f;
-#pragma unroll
-      for (int c = 0; c < FC2_SPLIT; ++c) t += ws.partf[((int64_t)s * FC2_SPLIT + c) * FC_PART + o];
+      const float t = sum_slots(ws.partf + (int64_t)s * split * FC_PART + o, split, FC_PART);
       if (o < NCLS * HID) grad[OFF_F2W + o] = t;
       else if (o < NCLS * HID + HID) grad[OFF_F1B + o - NCLS * HID] = t;
       else if (o < NCLS * HID + HID + NCLS) grad[OFF_F2B + o - NCLS * HID - HID] = t;
@@ -429,72 +217,67 @@ __global__ void __launch_bounds__(256) conv_grad_reduce(GradStepArgs a, WorkerTa
 // ---- the summed step's final reduction: ONE gradient vector, the sum over all workers (who share one weight
 // snapshot).  The 512-unit layer's weight gradient arrives as n_super partial vectors (one per group of workers whose
 // samples went through one product), every other tensor as the per-worker, per-block partial sums the per-worker
-// reduction also reads; everything is added in a fixed order (group after group, worker after worker, block after
-// block).  Blocks 0 .. FUSED_W1_BLOCKS - 1 take the float4 columns of the big tensor, the rest the small outputs.
+// reduction also reads; everything is added in a fixed order.  Blocks 0 .. FUSED_W1_BLOCKS - 1 take the float4 columns of
+// the big tensor, the rest 32 small outputs each: warp w of eight adds the partial sums of workers w, w + 8, ... (lane =
+// output, so a warp's loads are consecutive), then the warps' sums are added in order.
 constexpr int FUSED_W1_VEC = HID * FLAT / 4;                                 // 200,704 float4
 constexpr int FUSED_W1_BLOCKS = (FUSED_W1_VEC + 255) / 256;                  // 784
 constexpr int FUSED_SMALL = C2_GRAD + C1_GRAD + (NCLS * HID + HID + NCLS) + (P_PAD - P);
-constexpr int FUSED_SMALL_BLOCKS = (FUSED_SMALL + 7) / 8;                    // one warp per small output
+constexpr int FUSED_SMALL_BLOCKS = (FUSED_SMALL + 31) / 32;
 __global__ void __launch_bounds__(256) fused_finish(GradStepArgs a, WorkerTable wt, Workspace ws, const float* __restrict__ super_part,
                                                     int n_super, float* __restrict__ grad_sum, int n_chunks, int seg_len1,
                                                     int n_chunks2, int seg_len) {
-  const int b = a.b;
+  __shared__ float warp_sum[8][32];
+  const int b = a.b, split = fc2_split(a.W, b);
   if (blockIdx.x < FUSED_W1_BLOCKS) {
     const int i = blockIdx.x * 256 + threadIdx.x;
     if (i >= FUSED_W1_VEC) return;
     float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int g = 0; g < n_super; ++g) {
-      const float4 v = reinterpret_cast<const float4*>(super_part + (int64_t)g * P_PAD + OFF_F1W)[i];
-      t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
+    for (int g0 = 0; g0 < n_super; g0 += 8) {
+      float4 v[8];
+#pragma unroll
+      for (int g = 0; g < 8; ++g)
+        v[g] = g0 + g < n_super ? reinterpret_cast<const float4*>(super_part + (int64_t)(g0 + g) * P_PAD + OFF_F1W)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int g = 0; g < 8; ++g) { t.x += v[g].x; t.y += v[g].y; t.z += v[g].z; t.w += v[g].w; }
     }
     reinterpret_cast<float4*>(grad_sum + OFF_F1W)[i] = t;
     return;
   }
-  // A small output is summed by one warp: lane l adds the partial sums of workers l, l + 32, ... in order, then the
-  // lanes are combined by a butterfly, which is the same sequence of additions on every run.
-  const int lane = threadIdx.x & 31;
-  int o = (blockIdx.x - FUSED_W1_BLOCKS) * 8 + (threadIdx.x >> 5);
-  if (blockIdx.x == FUSED_W1_BLOCKS && threadIdx.x < a.W) {      // the per-worker losses ride along (W <= 256)
-    float t = 0.f;
-#pragma unroll
-    for (int c = 0; c < FC2_SPLIT; ++c) t += ws.partf[((int64_t)threadIdx.x * FC2_SPLIT + c) * FC_PART + NCLS * HID + HID + NCLS];
-    a.loss[wt.src[threadIdx.x]] = t * (1.0f / (float)b);
-  }
-  if (o >= FUSED_SMALL) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int o = (blockIdx.x - FUSED_W1_BLOCKS) * 32 + lane;
+  if (blockIdx.x == FUSED_W1_BLOCKS && threadIdx.x < a.W)        // the per-worker losses ride along (W <= 256)
+    a.loss[wt.src[threadIdx.x]] = sum_slots(ws.partf + (int64_t)threadIdx.x * split * FC_PART + NCLS * HID + HID + NCLS, split, FC_PART) * (1.0f / (float)b);
   float t = 0.f;
-  float* dst;
+  float* dst = nullptr;
   if (o < C2_GRAD) {
-    for (int s = lane; s < a.W; s += 32) {
-      const int used2 = seg_len > 0 ? (s * b + b - 1) / seg_len - (s * b) / seg_len + 1 : n_chunks2;
-      for (int c = 0; c < used2; ++c) t += ws.part2[((int64_t)s * n_chunks2 + c) * C2_GRAD + o];
-    }
+    for (int s = warp; s < a.W; s += 8) t += sum_slots(ws.part2 + (int64_t)s * n_chunks2 * C2_GRAD + o, used_slots(s, b, seg_len, n_chunks2), C2_GRAD);
     dst = grad_sum + OFF_C2W + o;
   } else if (o < C2_GRAD + C1_GRAD) {
     const int oo = o - C2_GRAD;
-    for (int s = lane; s < a.W; s += 32) {
-      const int used1 = seg_len1 > 0 ? (s * b + b - 1) / seg_len1 - (s * b) / seg_len1 + 1 : n_chunks;
-      for (int c = 0; c < used1; ++c) t += ws.part1[((int64_t)s * n_chunks + c) * C1_GRAD + oo];
-    }
+    for (int s = warp; s < a.W; s += 8) t += sum_slots(ws.part1 + (int64_t)s * n_chunks * C1_GRAD + oo, used_slots(s, b, seg_len1, n_chunks), C1_GRAD);
     dst = grad_sum + OFF_C1W + oo;
   } else if (o < C2_GRAD + C1_GRAD + NCLS * HID + HID + NCLS) {
-    const int oo = o - C2_GRAD - C1_GRAD;
-    for (int s = lane; s < a.W; s += 32)
-#pragma unroll
-      for (int c = 0; c < FC2_SPLIT; ++c) t += ws.partf[((int64_t)s * FC2_SPLIT + c) * FC_PART + oo];
+    const int oo = o - C2_GRAD - C1_GRAD, n = a.W * split, per = (n + 7) / 8;      // all workers' slots lie end to end
+    const int c0 = min(n, warp * per), c1 = min(n, c0 + per);
+    t = sum_slots(ws.partf + (int64_t)c0 * FC_PART + oo, c1 - c0, FC_PART);
     dst = oo < NCLS * HID ? grad_sum + OFF_F2W + oo : (oo < NCLS * HID + HID ? grad_sum + OFF_F1B + oo - NCLS * HID : grad_sum + OFF_F2B + oo - NCLS * HID - HID);
-  } else {
+  } else if (o < FUSED_SMALL) {
     dst = grad_sum + P + (o - C2_GRAD - C1_GRAD - NCLS * HID - HID - NCLS);      // padding: zero
   }
+  warp_sum[warp][lane] = t;
+  __syncthreads();
+  if (warp != 0 || !dst) return;
 #pragma unroll
-  for (int sh = 16; sh > 0; sh >>= 1) t += __shfl_xor_sync(0xffffffffu, t, sh);
-  if (lane == 0) *dst = t;
+  for (int w = 1; w < 8; ++w) t += warp_sum[w][lane];
+  *dst = t;
 }
 
 // ---- evaluation: per worker, the mean loss from the output-layer kernel's partial sums and the number of samples
 // whose predicted label equals the given one (an integer count, summed in a fixed order).
 __global__ void __launch_bounds__(128) eval_finish(GradStepArgs a, WorkerTable wt, Workspace ws, int32_t* __restrict__ correct) {
   __shared__ int warp_hits[4];
-  const int s = blockIdx.x, src = wt.src[s];
+  const int s = blockIdx.x, src = wt.src[s], split = fc2_split(a.W, a.b);
   int hits = 0;
   for (int i = threadIdx.x; i < a.b; i += 128) {
     const int64_t r = (int64_t)src * a.b + i;
@@ -507,8 +290,7 @@ __global__ void __launch_bounds__(128) eval_finish(GradStepArgs a, WorkerTable w
   if (threadIdx.x == 0) {
     correct[src] = warp_hits[0] + warp_hits[1] + warp_hits[2] + warp_hits[3];
     float t = 0.f;
-#pragma unroll
-    for (int c = 0; c < FC2_SPLIT; ++c) t += ws.partf[((int64_t)s * FC2_SPLIT + c) * FC_PART + NCLS * HID + HID + NCLS];
+    for (int c = 0; c < split; ++c) t += ws.partf[((int64_t)s * split + c) * FC_PART + NCLS * HID + HID + NCLS];
     a.loss[src] = t * (1.0f / (float)a.b);
   }
 }
@@ -535,8 +317,8 @@ int launch_dropout_mask(uint64_t seed, uint32_t worker, uint64_t step, int b, ui
   return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
-// Evaluation pass: the forward kernels of the grad step with the dropout switched off (the output-layer kernel also
-// produces backward quantities into the workspace; nothing reads them), then the per-worker loss and hit count.
+// Evaluation pass: the forward kernels of the grad step with the dropout switched off, then the per-worker loss and hit
+// count.
 int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, int32_t* correct,
                 cudaStream_t st, Profiler* prof) {
   int launches = 0;
@@ -554,7 +336,7 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
     launch_fc1_fwd_fp32(a, wt, gt, ws, st, prof);
     launches += 3;
   }
-  TIMED(K_FC2_FWD_BWD, (fc2_fwd_bwd<<<dim3(a.W, FC2_SPLIT), FC2_THREADS, 0, st>>>(a, wt, gt, ws)));
+  launch_output_layer(true, a, wt, gt, ws, st, prof);
   TIMED(K_EVAL_FINISH, (eval_finish<<<a.W, 128, 0, st>>>(a, wt, ws, correct)));
   launches += 2;
   return cudaGetLastError() == cudaSuccess ? launches : -1;
@@ -569,6 +351,9 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
 int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                      cudaStream_t st, const SideStreams& side, Profiler* prof, const SummedStep* sum) {
   const bool tc = a.precision != 0;
+  // one output of the final reduction per thread while the blocks are few: 8.6 against 10.7 us at 8 and 16 workers; four from
+  // 64 workers on: 12.7 against 14.1 us at 128
+  const int red_per_block = a.W >= 64 ? 1024 : 256;
   const int n_chunks1 = (a.b + CONV1_SPB - 1) / CONV1_SPB;
   const int n_chunks1b = (a.b + CONV1B_SPB - 1) / CONV1B_SPB;
   int launches = 0, n_chunks2 = 0, seg_len = 0;
@@ -596,7 +381,7 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     int n = launch_fc1_fwd_tc5(a, wt, gt, ws, st, prof);
     if (n < 0) return -1;
     launches += 2 + n;
-    TIMED(K_FC2_FWD_BWD, (fc2_fwd_bwd<<<dim3(a.W, FC2_SPLIT), FC2_THREADS, 0, st>>>(a, wt, gt, ws)));
+    launch_output_layer(false, a, wt, gt, ws, st, prof);
     launches += 1;
     if (side.s1) { cudaEventRecord(side.fork1, st); cudaStreamWaitEvent(s1, side.fork1, 0); }
     n = sum ? launch_fc1_dw_tc5(a_dw, wt_dw, gt, ws, s1, prof) : launch_fc1_dw_tc5(a, wt, gt, ws, s1, prof);
@@ -616,20 +401,20 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     if (side.s1) cudaStreamWaitEvent(st, side.join1, 0);
     if (side.s2) cudaStreamWaitEvent(st, side.join2, 0);
     if (sum) TIMED(K_CONV_GRAD_REDUCE, (fused_finish<<<FUSED_W1_BLOCKS + FUSED_SMALL_BLOCKS, 256, 0, st>>>(a, wt, ws, sum->super_part, sum->n_super, sum->grad_sum, n_chunks1t, seg_len1, n_chunks2, seg_len)));
-    else TIMED(K_CONV_GRAD_REDUCE, (conv_grad_reduce<<<dim3(a.W, RED_BLOCKS), 256, 0, st>>>(a, wt, ws, n_chunks1t, seg_len1, n_chunks2, seg_len)));
+    else TIMED(K_CONV_GRAD_REDUCE, (conv_grad_reduce<<<dim3(a.W, (RED_OUTPUTS + red_per_block - 1) / red_per_block), 256, 0, st>>>(a, wt, ws, red_per_block, n_chunks1t, seg_len1, n_chunks2, seg_len)));
     launches += 4;
   } else {
     TIMED(K_CONV1_FWD, (conv1_fwd<<<dim3(n_chunks1, a.W), 224, 0, st>>>(a, wt, gt, ws)));
     launch_conv2_direct(true, a, gt, ws, st, prof);
     launch_fc1_fwd_fp32(a, wt, gt, ws, st, prof);
-    TIMED(K_FC2_FWD_BWD, (fc2_fwd_bwd<<<dim3(a.W, FC2_SPLIT), FC2_THREADS, 0, st>>>(a, wt, gt, ws)));
+    launch_output_layer(false, a, wt, gt, ws, st, prof);
     launch_fc1_dw_fp32(sum ? a_dw : a, sum ? wt_dw : wt, gt, ws, st, prof);
     launch_fc1_dx_fp32(a, wt, gt, ws, st, prof);
     n_chunks2 = launch_conv2_dw_direct(a, ws, st, prof, &seg_len);
     launch_conv2_direct(false, a, gt, ws, st, prof);
     TIMED(K_CONV1_BWD, (conv1_bwd<<<dim3(n_chunks1b, a.W), 256, 0, st>>>(a, wt, ws, n_chunks1b)));
     if (sum) TIMED(K_CONV_GRAD_REDUCE, (fused_finish<<<FUSED_W1_BLOCKS + FUSED_SMALL_BLOCKS, 256, 0, st>>>(a, wt, ws, sum->super_part, sum->n_super, sum->grad_sum, n_chunks1b, 0, n_chunks2, seg_len)));
-    else TIMED(K_CONV_GRAD_REDUCE, (conv_grad_reduce<<<dim3(a.W, RED_BLOCKS), 256, 0, st>>>(a, wt, ws, n_chunks1b, 0, n_chunks2, seg_len)));
+    else TIMED(K_CONV_GRAD_REDUCE, (conv_grad_reduce<<<dim3(a.W, (RED_OUTPUTS + red_per_block - 1) / red_per_block), 256, 0, st>>>(a, wt, ws, red_per_block, n_chunks1b, 0, n_chunks2, seg_len)));
     launches = 10;
   }
   return cudaGetLastError() == cudaSuccess ? launches : -1;

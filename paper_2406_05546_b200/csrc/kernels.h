@@ -23,12 +23,19 @@ constexpr int P1_ELEMS = C1 * H1 * H1;   // 3136
 constexpr int P1_PLANE_ELEMS = 2 * 256 * 4;   // 32-bit words of one sample's p1 in the tensor-core plane layout (8 KB of BF16)
 constexpr int FLAT = C2 * H2 * H2;       // 1568
 constexpr int HID = 512, NCLS = 10;
-constexpr int DZ_STRIDE = 16;            // logits gradient row, padded
 constexpr int CONV_SPB = 4;              // samples per partial-sum slot of the convolutions' filter gradients
 constexpr int MIN_RANGE = CONV_SPB;       // shortest range of rows of a filter-gradient block (tensor-core path)
 constexpr int C2_GRAD = 4608 + 32, C1_GRAD = 144 + 16;
-constexpr int FC2_SPLIT = 1;             // blocks per worker in the output-layer kernel, each with its own partial sums (at 128 registers x 512 threads one block fills an SM, so more blocks only queue)
 constexpr int FC_PART = NCLS * HID + HID + NCLS + 2;   // fc2.w, fc1.b, fc2.b gradients, loss sum, padding
+// Blocks per worker in the output layer's kernel, each with its own partial sums: at least eight samples to a block, about
+// two blocks per SM in all (W * fc2_split(W, b) <= max(W, FC2_BLOCKS)).
+constexpr int FC2_BLOCKS = 296, FC2_MAX_SPLIT = 8;
+__host__ __device__ inline int fc2_split(int W, int b) {
+  int s = FC2_BLOCKS / W;
+  s = s < 1 ? 1 : (s > FC2_MAX_SPLIT ? FC2_MAX_SPLIT : s);
+  const int most = (b + 7) / 8;
+  return s < most ? s : most;
+}
 
 constexpr uint32_t STATUS_BAD_LABEL = 1u;
 constexpr uint32_t STATUS_WAIT_TIMEOUT = 2u;   // a bounded barrier wait in a tensor-core kernel gave up
@@ -104,12 +111,11 @@ struct Workspace {
   uint8_t* code2;  // [rows][1568]
   float* d;        // [rows][512]         fc1 -> ReLU -> dropout (scaled)
   float* da1;      // [rows][512]         gradient w.r.t. fc1 pre-activation
-  float* dz;       // [rows][16]          gradient w.r.t. logits (10 used)
   float* dp2;      // [rows][1568]        gradient w.r.t. p2 (tensor-core path: BF16 in the first half of each row)
   float* dp1;      // [rows][3136]        gradient w.r.t. p1; [16][196] fp32 (FP32 path) or [4 channel quads][196][4] BF16 in the first half of the row (tensor-core path)
   float* part2;    // [W][chunks][4640]   per-block partial conv2 weight/bias gradients
   float* part1;    // [W][chunks][160]    per-block partial conv1 weight/bias gradients
-  float* partf;    // [W][FC2_SPLIT][FC_PART] per-block partial output-layer gradients and loss sums
+  float* partf;    // [W][fc2_split][FC_PART] per-block partial output-layer gradients and loss sums
   float* w1r;      // [groups][512][1568] TF32-rounded fc1 weights of each weight group of the call
   float* w1tr;     // [groups][1568][512] and their transpose
   uint32_t* status;
@@ -170,6 +176,7 @@ int configure_conv5_kernels();
 int configure_conv1_kernels();
 int configure_dw5_kernels();
 int configure_c1d5_kernels();
+void launch_output_layer(bool eval, const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
 int launch_conv1_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const Workspace& ws, cudaStream_t st, Profiler* prof,
                         int* seg_len);
 int launch_conv2_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const Workspace& ws, cudaStream_t st, Profiler* prof,

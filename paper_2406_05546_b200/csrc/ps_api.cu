@@ -150,12 +150,11 @@ void layout(ps_ctx* x, const ps_config& c, void* arena, void* pinned, uint64_t* 
   ws.code2 = a.take<uint8_t>(rows * psk::FLAT);
   ws.d = a.take<float>(rows * psk::HID * 4);
   ws.da1 = a.take<float>(rows * psk::HID * 4);
-  ws.dz = a.take<float>(rows * psk::DZ_STRIDE * 4);
   ws.dp2 = a.take<float>(rows * psk::FLAT * 4);
   ws.dp1 = a.take<float>(rows * psk::P1_ELEMS * 4);
   ws.part2 = a.take<float>((uint64_t)c.max_workers * chunks * psk::C2_GRAD * 4);
   ws.part1 = a.take<float>((uint64_t)c.max_workers * chunks * psk::C1_GRAD * 4);
-  ws.partf = a.take<float>((uint64_t)c.max_workers * psk::FC2_SPLIT * psk::FC_PART * 4);
+  ws.partf = a.take<float>((uint64_t)std::min(c.max_workers * psk::FC2_MAX_SPLIT, std::max<int>(c.max_workers, psk::FC2_BLOCKS)) * psk::FC_PART * 4);
   ws.status = a.take<uint32_t>(ALIGN);
   ws.w1r = ws.w1tr = nullptr;
   if (c.precision != PS_FP32) {

@@ -135,7 +135,9 @@ def test_stale_snapshots_grouped_over_three_versions():
                                      # change form; groups of rows that leave remainders in every tile
                                      (4, 8, {"lags": [0, 1, 1, 0], "n_versions": 2}), (3, 11, {}), (12, 85, {"check": (0, 6, 11)}),
                                      (41, 25, {"check": (0, 20, 40), "lags": [w % 2 for w in range(41)], "n_versions": 2}),
-                                     (40, 103, {"check": (0, 39)}), (50, 60, {"check": (0, 49)})])
+                                     (40, 103, {"check": (0, 39)}), (50, 60, {"check": (0, 49)}),
+                                     # 130 samples to a block of the output layer: two chunks
+                                     (2, 1040, {"check": (0, 1)})])
 def test_fp32_path_at_the_edges_of_its_kernel_choices(W, b, kw):
     _run_and_compare(W, b, **kw)
 

@@ -82,6 +82,18 @@ __device__ __forceinline__ const float* group_theta(const WorkerTable& wt, const
 }
 
 
+// bias + ReLU + dropout of four consecutive units n..n+3 of row m
+__device__ __forceinline__ float4 fc1_activation(float4 v, int m, int n, const float* theta, const GradStepArgs& a, const WorkerTable& wt) {
+  const float4 bias = *reinterpret_cast<const float4*>(theta + OFF_F1B + n);
+  const float scale = 1.0f / (1.0f - a.drop_p);
+  const int s = m / a.b, i = m - s * a.b;
+  const uint4 rnd = philox4x32_10(make_uint4((uint32_t)((i * HID + n) >> 2), (uint32_t)wt.wid[s], (uint32_t)a.step, (uint32_t)(a.step >> 32)),
+                                  make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32)));
+  return make_float4(rnd.x >= a.drop_thresh ? fmaxf(v.x + bias.x, 0.f) * scale : 0.f, rnd.y >= a.drop_thresh ? fmaxf(v.y + bias.y, 0.f) * scale : 0.f,
+                     rnd.z >= a.drop_thresh ? fmaxf(v.z + bias.z, 0.f) * scale : 0.f, rnd.w >= a.drop_thresh ? fmaxf(v.w + bias.w, 0.f) * scale : 0.f);
+}
+
+
 // Maps a tile index to (group, first row of the tile, end row of the group) for TM-row tiles laid
 // out group after group.
 template <int TM>
@@ -132,6 +144,24 @@ inline int group_tiles(const GroupTable& gt, int b, int tm) {
   int t = 0;
   for (int g = 0; g < gt.n_groups; ++g) t += ((gt.first[g + 1] - gt.first[g]) * b + tm - 1) / tm;
   return t;
+}
+
+// Host: launches a kernel in clusters of cluster_z blocks along z.
+template <typename F, typename... Args>
+inline void launch_cluster(F* fn, dim3 grid, int threads, int smem, int cluster_z, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 1;
+  at.val.clusterDim.y = 1;
+  at.val.clusterDim.z = (unsigned)cluster_z;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, fn, args...);
 }
 
 }  // namespace psk

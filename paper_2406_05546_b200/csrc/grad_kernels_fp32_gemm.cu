@@ -39,17 +39,6 @@ template <int OP> struct GemmShape {
   static constexpr int LDA = OP == G_FWD ? FLAT : HID, LDB = FLAT, LDC = N;
 };
 
-// bias + ReLU + dropout of four consecutive units n..n+3 of row m
-__device__ __forceinline__ float4 fc1_activation(float4 v, int m, int n, const float* theta, const GradStepArgs& a, const WorkerTable& wt) {
-  const float4 bias = *reinterpret_cast<const float4*>(theta + OFF_F1B + n);
-  const float scale = 1.0f / (1.0f - a.drop_p);
-  const int s = m / a.b, i = m - s * a.b;
-  const uint4 rnd = philox4x32_10(make_uint4((uint32_t)((i * HID + n) >> 2), (uint32_t)wt.wid[s], (uint32_t)a.step, (uint32_t)(a.step >> 32)),
-                                  make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32)));
-  return make_float4(rnd.x >= a.drop_thresh ? fmaxf(v.x + bias.x, 0.f) * scale : 0.f, rnd.y >= a.drop_thresh ? fmaxf(v.y + bias.y, 0.f) * scale : 0.f,
-                     rnd.z >= a.drop_thresh ? fmaxf(v.z + bias.z, 0.f) * scale : 0.f, rnd.w >= a.drop_thresh ? fmaxf(v.w + bias.w, 0.f) * scale : 0.f);
-}
-
 // Operands and destination of the block's tile: rows m0 .. m_end - 1 (all of them < m_end are valid)
 struct TileIo { const float *A, *B, *theta; float* C; int m0, m_end, K; };
 template <int OP, int BM>
@@ -327,23 +316,6 @@ __global__ void __launch_bounds__(256) sgemm_skinny(GradStepArgs a, WorkerTable 
     }
   }
   cl.sync();
-}
-
-template <typename F, typename... Args>
-void launch_cluster(F* fn, dim3 grid, int threads, int smem, int cluster_z, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = 1;
-  at.val.clusterDim.y = 1;
-  at.val.clusterDim.z = (unsigned)cluster_z;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, fn, args...);
 }
 
 // Which form a grouped product takes, by its number of rows.  us for forward / input gradient, with ~6 us of event overhead:

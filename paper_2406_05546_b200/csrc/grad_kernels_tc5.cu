@@ -14,6 +14,7 @@
 //
 // Every wait on an mbarrier is bounded: when a bound is exceeded the kernel raises a status flag,
 // stops issuing work, frees its tensor memory and returns.
+#include <cooperative_groups.h>
 #include <cuda.h>
 
 #include "device_common.cuh"
@@ -23,6 +24,8 @@
 namespace psk {
 
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int BM = 128, BK = 32;                    // CTA tile rows; BK floats = one 128-byte swizzle row
 constexpr int A_BYTES = BM * BK * 4;
@@ -71,8 +74,7 @@ __host__ __device__ constexpr uint32_t instr_desc_tf32(int m, int n, bool mn_maj
 
 // Tensor maps of one launch, passed by value in the kernel's parameter space.
 struct GemmMaps {
-  CUtensorMap a;
-  CUtensorMap b[MAX_GROUPS];
+  CUtensorMap a, b;         // b: one slab per weight group (or worker)
 };
 
 enum { EPI_FC1_FWD = 0, EPI_STORE = 1, EPI_STORE_BF16 = 2 };   // the last: the output rounded to BF16 (its readers multiply in BF16)
@@ -174,7 +176,8 @@ __global__ void __launch_bounds__(gemm_threads(EPI), 1) tc5_gemm(const __grid_co
         TileCoord c;
         if (!decode_tile<BN>(tw, ga, gt, a.b, c)) continue;
         const CUtensorMap* map_a = &maps.a;
-        const CUtensorMap* map_b = &maps.b[c.grp];
+        const CUtensorMap* map_b = &maps.b;
+        const int slab_b = ga.per_worker ? c.z : c.grp;
         for (int kb = 0; kb < n_k; ++kb, ++it) {
           const int s = it % STAGES;
           if (it >= STAGES && !mbar_wait(&empty[s], ((it / STAGES) - 1) & 1)) { *abort_flag = 1; ok = false; break; }
@@ -182,10 +185,10 @@ __global__ void __launch_bounds__(gemm_threads(EPI), 1) tc5_gemm(const __grid_co
           mbar_expect_tx(&full[s], STAGE_BYTES);
           if (MN) {      // boxes of {32 columns, BK samples, BM/32 or BN/32 column blocks} of worker z
             tma_load_4d(tiles + s * STAGE_BYTES, map_a, &full[s], 0, kb * BK, c.m0 / 32, c.z);
-            tma_load_4d(tiles + s * STAGE_BYTES + A_BYTES, map_b, &full[s], 0, kb * BK, c.n0 / 32, c.z);
+            tma_load_4d(tiles + s * STAGE_BYTES + A_BYTES, map_b, &full[s], 0, kb * BK, c.n0 / 32, slab_b);
           } else {
             tma_load_3d(tiles + s * STAGE_BYTES, map_a, &full[s], kb * BK, c.m0, c.z);
-            tma_load_3d(tiles + s * STAGE_BYTES + A_BYTES, map_b, &full[s], kb * BK, c.n0, c.z);
+            tma_load_3d(tiles + s * STAGE_BYTES + A_BYTES, map_b, &full[s], kb * BK, c.n0, slab_b);
           }
         }
       }
@@ -306,6 +309,218 @@ __global__ void __launch_bounds__(gemm_threads(EPI), 1) tc5_gemm(const __grid_co
   }
 }
 
+// Forward product, few rows: 128 x 256 tiles would be a handful of serial chains of 49 k-blocks (23 us) on a chip mostly
+// idle.  An MMA of M = 64, N = 32 takes 52 clocks where one of 128 x 256 takes 130, so tiles of 64 x 32 shorten the chain
+// and make thirty-two times as many of them; the sums are the same bits, as every accumulator still takes its products in
+// the same order (a split of k would not: a unit whose sum lies within rounding distance of zero then flips).
+// A stage holds two k-blocks: waits, commits and the issuing loop's overhead come once per eight MMAs.
+constexpr int NR_BM = 64, NR_BN = 32, NR_STAGES = 4, NR_A = NR_BM * BK * 4, NR_HALF = NR_A + NR_BN * BK * 4, NR_STAGE = 2 * NR_HALF;
+constexpr int NR_SMEM = NR_STAGES * NR_STAGE + 1024 /* alignment slack */ + 256 /* barriers */ + NR_BM * EPI_ROW_FLOATS * 4;
+static_assert(2 * NR_SMEM <= 227 * 1024, "two CTAs per SM");
+
+// Warps: 0 = TMA producer, 1 = tensor-memory owner and MMA issuer, 2..5 = epilogue.  One tile per CTA.
+__global__ void __launch_bounds__(192, 2) tc5_fwd_narrow(const __grid_constant__ GemmMaps maps, GemmArgs ga, GradStepArgs a, WorkerTable wt,
+                                                         GroupTable gt, Workspace ws) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* tiles = smem_raw + (base - smem_u32(smem_raw));
+  uint64_t* full = reinterpret_cast<uint64_t*>(tiles + NR_STAGES * NR_STAGE);
+  uint64_t* empty = full + NR_STAGES;
+  uint64_t* acc_full = empty + NR_STAGES;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
+  volatile uint32_t* abort_flag = tmem_slot + 1;
+  float* stage_out = reinterpret_cast<float*>(tiles + NR_STAGES * NR_STAGE + 256);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, n0 = blockIdx.x * NR_BN;
+  int grp = 0, m0 = 0, m_end = 0;
+  if (!locate_group_tile<NR_BM>(gt, a.b, blockIdx.y, grp, m0, m_end)) return;
+  const int n_k = (ga.K + 2 * BK - 1) / (2 * BK);      // what lies beyond K arrives as zeros
+  if (tid == 0) {
+    for (int s = 0; s < NR_STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+    mbar_init(acc_full, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(32) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  if (warp == 0) {
+    if (lane == 0) {
+      uint32_t parity = 1;                     // the first round of stages is free
+      for (int kb = 0, s = 0; kb < n_k; ++kb) {
+        if (kb >= NR_STAGES && (!mbar_wait(&empty[s], parity) || *abort_flag)) { *abort_flag = 1; break; }
+        mbar_expect_tx(&full[s], NR_STAGE);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          tma_load_3d(tiles + s * NR_STAGE + h * NR_HALF, &maps.a, &full[s], (2 * kb + h) * BK, m0, 0);
+          tma_load_3d(tiles + s * NR_STAGE + h * NR_HALF + NR_A, &maps.b, &full[s], (2 * kb + h) * BK, n0, grp);
+        }
+        if (++s == NR_STAGES) { s = 0; parity ^= 1; }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      constexpr uint32_t idesc = instr_desc_tf32(NR_BM, NR_BN);
+      const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0) >> 32);
+      const uint32_t a_lo0 = (uint32_t)smem_desc_sw128(base), b_lo0 = (uint32_t)smem_desc_sw128(base + NR_A);
+      const uint32_t full0 = smem_u32(full), empty0 = smem_u32(empty);
+      bool go_on = true;
+      uint32_t parity = 0;
+      for (int kb = 0; go_on && kb < n_k; parity ^= 1) {
+#pragma unroll
+        for (int s = 0; s < NR_STAGES; ++s, ++kb) {
+          if (kb >= n_k) { go_on = false; break; }
+          if (!mbar_wait_addr(full0 + 8 * s, parity) || *abort_flag) { *abort_flag = 1; go_on = false; break; }
+          tc_fence_after();
+#pragma unroll
+          for (int k = 0; k < 2 * BK / 8; ++k) {
+            const uint32_t off = s * (NR_STAGE / 16) + (k / 4) * (NR_HALF / 16) + 2 * (k % 4);
+            umma_tf32_split(tmem, a_lo0 + off, desc_hi, b_lo0 + off, desc_hi, idesc, (s | k) ? 1u : (kb ? 1u : 0u));
+          }
+          umma_commit_addr(empty0 + 8 * s);
+        }
+      }
+      umma_commit(acc_full);
+    }
+  } else {
+    if (mbar_wait(acc_full, 0)) {
+      tc_fence_after();
+      const int quarter = warp & 3;            // an accumulator of 64 rows keeps rows 16 q .. 16 q + 15 in the first sixteen lanes of quarter q
+      uint32_t r[32];
+      tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16), r);
+      if (lane < 16) {
+        uint4* d = reinterpret_cast<uint4*>(stage_out + (quarter * 16 + lane) * EPI_ROW_FLOATS);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) d[q] = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+      }
+      tc_fence_before();
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int e = (tid - 64) + 128 * i, row = e >> 3, q = e & 7, m = m0 + row, n = n0 + 4 * q;
+        if (m < m_end)
+          *reinterpret_cast<float4*>(ga.c + (int64_t)m * ga.ldc + n) =
+              fc1_activation(*reinterpret_cast<const float4*>(stage_out + row * EPI_ROW_FLOATS + 4 * q), m, n, gt.theta[grp], a, wt);
+      }
+    } else {
+      *abort_flag = 1;                         // all four warps give up together: the barrier is theirs alone
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(32) : "memory");
+  }
+  if (tid == 0 && *abort_flag) {
+    atomicOr(ws.status, STATUS_WAIT_TIMEOUT);
+    for (int i = 0; i < 1000; ++i) __nanosleep(1000);      // let copies already issued land before the CTA ends
+  }
+}
+
+// Input gradient, few rows: a tile's products would be one SM's serial chain of 16 k-blocks while most of the chip is idle.
+// So a cluster of SPLITS CTAs shares a tile: each takes KB of the k-blocks, has all of them in flight at
+// once (its shared memory holds them all, so no stage is waited for twice), and the partial tiles are added through
+// distributed shared memory in a fixed order, every CTA finishing its share of the tile's quads.
+template <int BN_, int KB_, int SPLITS_> struct SplitShape {
+  static constexpr int BN = BN_, KB = KB_, SPLITS = SPLITS_, STAGE_BYTES = A_BYTES + BN * BK * 4, PITCH = BN + 4;
+  static constexpr int SMEM = KB * STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */, TMEM = BN <= 128 ? 128 : 256;
+  static_assert(BM * PITCH * 4 <= KB * STAGE_BYTES, "the partial tile takes the operands' place");
+  static_assert(STAGE_BYTES % 1024 == 0 && BN % 32 == 0 && SMEM <= 227 * 1024, "tile shape");
+};
+using DxSplit = SplitShape<224, 4, 4>;       // 16 k-blocks, 7 column tiles
+
+template <typename S>
+__global__ void __launch_bounds__(256, 1) tc5_dx_split(const __grid_constant__ GemmMaps maps, GemmArgs ga, GradStepArgs a, GroupTable gt, Workspace ws) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* tiles = smem_raw + (base - smem_u32(smem_raw));
+  uint64_t* full = reinterpret_cast<uint64_t*>(tiles + S::KB * S::STAGE_BYTES);      // [KB], then "all products done"
+  uint64_t* acc_full = full + S::KB;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
+  volatile uint32_t* abort_flag = tmem_slot + 1;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rank = blockIdx.z, n0 = blockIdx.x * S::BN;
+  int grp = 0, m0 = 0, m_end = 0;
+  if (!locate_group_tile<BM>(gt, a.b, blockIdx.y, grp, m0, m_end)) return;           // the same for all CTAs of a cluster
+  if (tid == 0) {
+    for (int i = 0; i <= S::KB; ++i) mbar_init(&full[i], 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int i = 0; i < S::KB; ++i) {
+      mbar_expect_tx(&full[i], S::STAGE_BYTES);
+      tma_load_3d(tiles + i * S::STAGE_BYTES, &maps.a, &full[i], (rank * S::KB + i) * BK, m0, 0);
+      tma_load_3d(tiles + i * S::STAGE_BYTES + A_BYTES, &maps.b, &full[i], (rank * S::KB + i) * BK, n0, grp);
+    }
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(S::TMEM) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  if (warp == 1 && lane == 0) {
+    constexpr uint32_t idesc = instr_desc_tf32(BM, S::BN);
+    const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0) >> 32);
+    for (int i = 0; i < S::KB; ++i) {
+      if (!mbar_wait(&full[i], 0)) { *abort_flag = 1; break; }
+      tc_fence_after();
+      const uint32_t a_lo = (uint32_t)smem_desc_sw128(base + i * S::STAGE_BYTES), b_lo = (uint32_t)smem_desc_sw128(base + i * S::STAGE_BYTES + A_BYTES);
+#pragma unroll
+      for (int k = 0; k < BK / 8; ++k) umma_tf32_split(tmem, a_lo + 2 * k, desc_hi, b_lo + 2 * k, desc_hi, idesc, (i | k) ? 1u : 0u);
+    }
+    umma_commit(acc_full);
+  }
+  __syncwarp();
+  float* part = reinterpret_cast<float*>(tiles);
+  if (mbar_wait(acc_full, 0)) {
+    tc_fence_after();
+    const int quarter = warp & 3;
+    for (int ch = warp >> 2; ch < S::BN / 32; ch += 2) {
+      uint32_t r[32];
+      tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ch * 32), r);
+      uint4* d = reinterpret_cast<uint4*>(part + (quarter * 32 + lane) * S::PITCH + ch * 32);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) d[q] = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+    }
+    tc_fence_before();
+  } else {
+    *abort_flag = 1;
+  }
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(S::TMEM) : "memory");
+  }
+  const float* parts[S::SPLITS];
+#pragma unroll
+  for (int r = 0; r < S::SPLITS; ++r) parts[r] = cl.map_shared_rank(part, r);
+  constexpr int QUADS = S::BN / 4;
+  const int n_quads = min(BM, m_end - m0) * QUADS;
+  for (int e = rank * 256 + tid; e < n_quads; e += S::SPLITS * 256) {
+    const int r = e / QUADS, q = e - r * QUADS, m = m0 + r, n = n0 + 4 * q;
+    float4 u[S::SPLITS];
+#pragma unroll
+    for (int k = 0; k < S::SPLITS; ++k) u[k] = *reinterpret_cast<const float4*>(parts[k] + r * S::PITCH + 4 * q);
+    float4 v = u[0];
+#pragma unroll
+    for (int k = 1; k < S::SPLITS; ++k) { v.x += u[k].x; v.y += u[k].y; v.z += u[k].z; v.w += u[k].w; }
+    // ga.ldc counts BF16 elements here
+    *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(ga.c) + (int64_t)m * ga.ldc + n) = make_uint2(bf16_pair(v.x, v.y), bf16_pair(v.z, v.w));
+  }
+  cl.sync();                                   // a CTA's shared memory outlives its readers
+  if (tid == 0 && *abort_flag) {
+    atomicOr(ws.status, STATUS_WAIT_TIMEOUT);
+    for (int i = 0; i < 1000; ++i) __nanosleep(1000);      // let copies already issued land before the CTA ends
+  }
+}
+
 // ---- operand preparation ----------------------------------------------------------------------
 __device__ __forceinline__ float rna_tf32(float x) { return round_tf32(x); }
 
@@ -388,10 +603,28 @@ int configure_tc5_kernels() {
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || g_sm_count <= 0) return -1;
   cudaError_t e = allow_smem((const void*)(tc5_gemm<EPI_FC1_FWD, 256>), gemm_smem_bytes(256, MAX_STAGES, epi_warps(EPI_FC1_FWD)));
+  if (e == cudaSuccess) e = allow_smem((const void*)tc5_fwd_narrow, NR_SMEM);
+  if (e == cudaSuccess) e = allow_smem((const void*)tc5_dx_split<DxSplit>, DxSplit::SMEM);
   if (e == cudaSuccess) e = allow_smem((const void*)(tc5_gemm<EPI_STORE_BF16, 224>), gemm_smem_bytes(224, MAX_STAGES, epi_warps(EPI_STORE_BF16)));
   if (e == cudaSuccess) e = allow_smem((const void*)(tc5_gemm<EPI_STORE, 224, true>), gemm_smem_bytes(224, MAX_STAGES, epi_warps(EPI_STORE)));
   return e == cudaSuccess ? 0 : -1;
 }
+
+namespace {
+
+// Which form the grouped products take.  us, ~6 us of event overhead included:
+//   rows                           16   185   384   512   768   1024   1536   2048
+//   forward, 128 x 256             29    29    29    29    29     29     29     29
+//            64 x 32               16    17    17    17    17     18     28     29
+//            64 x 32, one k-block per stage and no unrolled stages: 21 - 23;  128 x 128 with k split over clusters of
+//            seven CTAs: 11 - 19 up to 768 rows, 27 at 1024 (other bits, see above)
+//   input gradient, 128 x 224      13    15    15    15    15     17     17     17
+//                   split over 4   11    13    14    15    21     23     31     38
+// The narrow tiles fit on the chip at once (two per SM) up to 18 x 64 rows.
+bool fwd_is_narrow(int mt64) { return mt64 * (HID / NR_BN) <= 2 * g_sm_count; }
+bool dx_splits(int mt) { return mt <= 3; }
+
+}  // namespace
 
 // Rounded / transposed copies of W1 for every weight group of this call.
 int launch_prep_w1(const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof) {
@@ -404,10 +637,15 @@ int launch_fc1_fwd_tc5(const GradStepArgs& a, const WorkerTable& wt, const Group
                        cudaStream_t st, Profiler* prof) {
   GemmMaps maps;
   const uint64_t rows = (uint64_t)a.W * a.b;
-  if (!make_map(&maps.a, ws.p2, FLAT, rows, 1, FLAT, rows * FLAT, BM)) return -1;
-  for (int g = 0; g < gt.n_groups; ++g)
-    if (!make_map(&maps.b[g], ws.w1r + (int64_t)g * HID * FLAT, FLAT, HID, 1, FLAT, (uint64_t)HID * FLAT, 256)) return -1;
-  const int mt = group_tiles(gt, a.b, BM);
+  const int mt = group_tiles(gt, a.b, BM), mt_narrow = group_tiles(gt, a.b, NR_BM);
+  const bool narrow = fwd_is_narrow(mt_narrow);
+  if (!make_map(&maps.a, ws.p2, FLAT, rows, 1, FLAT, rows * FLAT, narrow ? NR_BM : BM)) return -1;
+  if (!make_map(&maps.b, ws.w1r, FLAT, HID, (uint64_t)gt.n_groups, FLAT, (uint64_t)HID * FLAT, narrow ? NR_BN : 256)) return -1;
+  if (narrow) {
+    GemmArgs ga{FLAT, HID, HID, 0, ws.d, HID / NR_BN, 0};
+    TIMED(K_FC1_FWD, (tc5_fwd_narrow<<<dim3(HID / NR_BN, mt_narrow), 192, NR_SMEM, st>>>(maps, ga, a, wt, gt, ws)));
+    return 1;
+  }
   GemmArgs ga{FLAT, HID, HID, 0, ws.d, HID / 256, (HID / 256) * mt};
   const int grid = ga.n_tiles < g_sm_count ? ga.n_tiles : g_sm_count;
   TIMED(K_FC1_FWD, (tc5_gemm<EPI_FC1_FWD, 256><<<grid, gemm_threads(EPI_FC1_FWD), gemm_smem_bytes(256, MAX_STAGES, epi_warps(EPI_FC1_FWD)), st>>>(maps, ga, a, wt, gt, ws)));
@@ -419,12 +657,15 @@ int launch_fc1_dx_tc5(const GradStepArgs& a, const WorkerTable& wt, const GroupT
   GemmMaps maps;
   const uint64_t rows = (uint64_t)a.W * a.b;
   if (!make_map(&maps.a, ws.da1, HID, rows, 1, HID, rows * HID, BM)) return -1;
-  for (int g = 0; g < gt.n_groups; ++g)
-    if (!make_map(&maps.b[g], ws.w1tr + (int64_t)g * HID * FLAT, HID, FLAT, 1, HID, (uint64_t)HID * FLAT, 224)) return -1;
+  if (!make_map(&maps.b, ws.w1tr, HID, FLAT, (uint64_t)gt.n_groups, HID, (uint64_t)HID * FLAT, 224)) return -1;
   const int mt = group_tiles(gt, a.b, BM);
   // dp2 leaves as BF16, in the first half of each row of the fp32-sized buffer (row pitch 2 FLAT half-words): the
   // convolution's two backward kernels multiply it in BF16, so rounding it here once changes no result
   GemmArgs ga{HID, FLAT, 2 * FLAT, 0, ws.dp2, FLAT / 224, (FLAT / 224) * mt};
+  if (dx_splits(mt)) {
+    TIMED(K_FC1_DX, launch_cluster(tc5_dx_split<DxSplit>, dim3(FLAT / DxSplit::BN, mt, DxSplit::SPLITS), 256, DxSplit::SMEM, DxSplit::SPLITS, st, maps, ga, a, gt, ws));
+    return 1;
+  }
   const int grid = ga.n_tiles < g_sm_count ? ga.n_tiles : g_sm_count;
   TIMED(K_FC1_DX, (tc5_gemm<EPI_STORE_BF16, 224><<<grid, gemm_threads(EPI_STORE_BF16), gemm_smem_bytes(224, MAX_STAGES, epi_warps(EPI_STORE_BF16)), st>>>(maps, ga, a, wt, gt, ws)));
   return 1;
@@ -434,7 +675,7 @@ int launch_fc1_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const GroupT
                       cudaStream_t st, Profiler* prof) {
   GemmMaps maps;
   if (!make_map_mn(&maps.a, ws.da1, HID, a.b, a.W, BM / 32)) return -1;
-  if (!make_map_mn(&maps.b[0], ws.p2, FLAT, a.b, a.W, 224 / 32)) return -1;
+  if (!make_map_mn(&maps.b, ws.p2, FLAT, a.b, a.W, 224 / 32)) return -1;
   GemmArgs ga{a.b, FLAT, FLAT, 1, nullptr, FLAT / 224, (FLAT / 224) * (HID / BM) * a.W};
   const int grid = ga.n_tiles < g_sm_count ? ga.n_tiles : g_sm_count;
   TIMED(K_FC1_DW, (tc5_gemm<EPI_STORE, 224, true><<<grid, gemm_threads(EPI_STORE), gemm_smem_bytes(224, MAX_STAGES, epi_warps(EPI_STORE)), st>>>(maps, ga, a, wt, gt, ws)));

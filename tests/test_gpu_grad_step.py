@@ -169,7 +169,10 @@ def test_output_layer_split_over_blocks(b):
                                      (7, 111, {"lags": [1, 0, 1, 1, 0, 0, 1], "n_versions": 2}),
                                      # 896 rows: the first convolution takes two samples per block; 6 rows: ranges of
                                      # the filter gradients shorter than four rows
-                                     (8, 112, {}), (3, 2, {})])
+                                     (8, 112, {}), (3, 2, {}),
+                                     # three and four 128-row tiles, eighteen and nineteen 64-row tiles: where the dense
+                                     # layer's products change form; ragged last tiles, two weight versions (tiles never cross them)
+                                     (3, 100, {}), (5, 101, {"lags": [1, 0, 0, 1, 0], "n_versions": 2}), (9, 128, {}), (9, 130, {})])
 def test_tensor_core_path(W, b, kw):
     _run_and_compare(W, b, precision=2, **kw)
 

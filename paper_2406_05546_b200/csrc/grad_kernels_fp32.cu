@@ -18,8 +18,8 @@ namespace {
 // worker.  Thread = pooled position: it reads the 4x4 input patch under its 2x2 window once and
 // evaluates all 16 channels from registers (576 multiply-adds per 8 + 48 shared-memory loads).
 // (FP32 path; the tensor-core path has its own kernel, which writes the layout its convolutions copy from.)
-constexpr int CONV1_SPB = 8;
-__global__ void __launch_bounds__(224) conv1_fwd(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws) {
+constexpr int CONV1_SPB = 8;      // most samples per block
+__global__ void __launch_bounds__(224) conv1_fwd(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws, int spb) {
   __shared__ __align__(16) float xs[2][30][32];
   __shared__ __align__(16) float w[16][12];   // 9 taps + bias + padding
   const int s = blockIdx.y, tid = threadIdx.x;
@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(224) conv1_fwd(GradStepArgs a, WorkerTable wt,
     else w[tid - 144][9] = theta[OFF_C1B + tid - 144];
   }
   for (int t = tid; t < 2 * 30 * 32; t += 224) (&xs[0][0][0])[t] = 0.f;
-  const int i0 = blockIdx.x * CONV1_SPB, i1 = min(i0 + CONV1_SPB, a.b);
+  const int i0 = blockIdx.x * spb, i1 = min(i0 + spb, a.b);
   const int py = tid / 14, px = tid - py * 14;
   const bool active = tid < 196;
   __syncthreads();
@@ -91,8 +91,8 @@ __global__ void __launch_bounds__(224) conv1_fwd(GradStepArgs a, WorkerTable wt,
 // Thread (channel, lane of 16) owns 13 pooled positions of its channel.  The image, the pooling decisions
 // and the pooled gradients of the NEXT sample are fetched into registers while the current one is
 // accumulated, so that no global-memory latency sits between the multiply-adds.
-constexpr int CONV1B_SPB = 16;
-__global__ void __launch_bounds__(256) conv1_bwd(GradStepArgs a, WorkerTable wt, Workspace ws, int n_chunks) {
+constexpr int CONV1B_SPB = 16;            // most samples per block
+__global__ void __launch_bounds__(256) conv1_bwd(GradStepArgs a, WorkerTable wt, Workspace ws, int spb, int n_chunks) {
   __shared__ float xs[30][31];
   constexpr int PER = 13;                   // ceil(196 / 16)
   const int s = blockIdx.y, tid = threadIdx.x;
@@ -101,8 +101,8 @@ __global__ void __launch_bounds__(256) conv1_bwd(GradStepArgs a, WorkerTable wt,
 #pragma unroll
   for (int k = 0; k < 9; ++k) gw[k] = 0.f;
   for (int t = tid; t < 30 * 31; t += 256) (&xs[0][0])[t] = 0.f;
-  const int i0 = blockIdx.x * CONV1B_SPB;
-  const int i1 = min(i0 + CONV1B_SPB, a.b);
+  const int i0 = blockIdx.x * spb;
+  const int i1 = min(i0 + spb, a.b);
   float xr[4], gr[PER];
   int cr[PER];
   auto prefetch = [&](int i) {
@@ -317,6 +317,19 @@ int launch_dropout_mask(uint64_t seed, uint32_t worker, uint64_t step, int b, ui
   return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
+// Samples of a block follow one another, so blocks take fewer of them while all blocks fit on the chip (eight per SM):
+// at 2 x 8 the forward kernel went from 22 to 10 us and the filter-gradient kernel from 19 to 13, at 16 x 64 from 26 to
+// 19 and from 33 to 19 (~6 us of event overhead included).
+static int samples_per_block(int rows, int least, int most) {
+  int spb = least;
+  while (spb < most && (rows + spb - 1) / spb > 8 * g_sm_count) spb *= 2;
+  return spb;
+}
+static void launch_conv1_fwd(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof) {
+  const int spb = samples_per_block(a.W * a.b, 1, CONV1_SPB);
+  TIMED(K_CONV1_FWD, (conv1_fwd<<<dim3((a.b + spb - 1) / spb, a.W), 224, 0, st>>>(a, wt, gt, ws, spb)));
+}
+
 // Evaluation pass: the forward kernels of the grad step with the dropout switched off, then the per-worker loss and hit
 // count.
 int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, int32_t* correct,
@@ -330,8 +343,7 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
     if (n < 0) return -1;
     launches += 2 + n;
   } else {
-    const int n_chunks1 = (a.b + CONV1_SPB - 1) / CONV1_SPB;
-    TIMED(K_CONV1_FWD, (conv1_fwd<<<dim3(n_chunks1, a.W), 224, 0, st>>>(a, wt, gt, ws)));
+      launch_conv1_fwd(a, wt, gt, ws, st, prof);
     launch_conv2_direct(true, a, gt, ws, st, prof);
     launch_fc1_fwd_fp32(a, wt, gt, ws, st, prof);
     launches += 3;
@@ -343,7 +355,8 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
 }
 
 // Launch order of one grad step.  On the tensor-core path the copies of the dense layer's weights are made on a
-// side stream while the convolutions run, and the backward pass forks: once the output
+// side stream while the convolutions run; on both paths the backward pass forks (FP32 path: 402 -> 350 us at 16 x 64,
+// 109 -> 85 at 2 x 8, most of it from the branches filling each other's last waves): once the output
 // layer's backward has produced da1, the dense layer's per-worker weight gradient (bound by its 3.2 MB
 // per worker of writes) runs on a side stream next to the input-gradient chain, and once dp2 exists the
 // second convolution's filter gradient runs on another side stream next to its input gradient and the
@@ -354,8 +367,8 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
   // one output of the final reduction per thread while the blocks are few: 8.6 against 10.7 us at 8 and 16 workers; four from
   // 64 workers on: 12.7 against 14.1 us at 128
   const int red_per_block = a.W >= 64 ? 1024 : 256;
-  const int n_chunks1 = (a.b + CONV1_SPB - 1) / CONV1_SPB;
-  const int n_chunks1b = (a.b + CONV1B_SPB - 1) / CONV1B_SPB;
+  const int spb1b = samples_per_block(a.W * a.b, CONV_SPB, CONV1B_SPB);      // at least as many as the partial-sum slots allow
+  const int n_chunks1b = (a.b + spb1b - 1) / spb1b;
   int launches = 0, n_chunks2 = 0, seg_len = 0;
   // Summed step: the 512-unit layer's weight gradient is taken over groups of workers at once ("super-workers" of
   // W / n_super workers: their samples are consecutive rows, so the product only sees a longer batch) and written to
@@ -404,15 +417,22 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     else TIMED(K_CONV_GRAD_REDUCE, (conv_grad_reduce<<<dim3(a.W, (RED_OUTPUTS + red_per_block - 1) / red_per_block), 256, 0, st>>>(a, wt, ws, red_per_block, n_chunks1t, seg_len1, n_chunks2, seg_len)));
     launches += 4;
   } else {
-    TIMED(K_CONV1_FWD, (conv1_fwd<<<dim3(n_chunks1, a.W), 224, 0, st>>>(a, wt, gt, ws)));
+    cudaStream_t s1 = side.s1 ? side.s1 : st, s2 = side.s2 ? side.s2 : st;
+    launch_conv1_fwd(a, wt, gt, ws, st, prof);
     launch_conv2_direct(true, a, gt, ws, st, prof);
     launch_fc1_fwd_fp32(a, wt, gt, ws, st, prof);
     launch_output_layer(false, a, wt, gt, ws, st, prof);
-    launch_fc1_dw_fp32(sum ? a_dw : a, sum ? wt_dw : wt, gt, ws, st, prof);
+    if (side.s1) { cudaEventRecord(side.fork1, st); cudaStreamWaitEvent(s1, side.fork1, 0); }
+    launch_fc1_dw_fp32(sum ? a_dw : a, sum ? wt_dw : wt, gt, ws, s1, prof);
+    if (side.s1) cudaEventRecord(side.join1, s1);
     launch_fc1_dx_fp32(a, wt, gt, ws, st, prof);
-    n_chunks2 = launch_conv2_dw_direct(a, ws, st, prof, &seg_len);
+    if (side.s2) { cudaEventRecord(side.fork2, st); cudaStreamWaitEvent(s2, side.fork2, 0); }
+    n_chunks2 = launch_conv2_dw_direct(a, ws, s2, prof, &seg_len);
+    if (side.s2) cudaEventRecord(side.join2, s2);
     launch_conv2_direct(false, a, gt, ws, st, prof);
-    TIMED(K_CONV1_BWD, (conv1_bwd<<<dim3(n_chunks1b, a.W), 256, 0, st>>>(a, wt, ws, n_chunks1b)));
+    TIMED(K_CONV1_BWD, (conv1_bwd<<<dim3(n_chunks1b, a.W), 256, 0, st>>>(a, wt, ws, spb1b, n_chunks1b)));
+    if (side.s1) cudaStreamWaitEvent(st, side.join1, 0);
+    if (side.s2) cudaStreamWaitEvent(st, side.join2, 0);
     if (sum) TIMED(K_CONV_GRAD_REDUCE, (fused_finish<<<FUSED_W1_BLOCKS + FUSED_SMALL_BLOCKS, 256, 0, st>>>(a, wt, ws, sum->super_part, sum->n_super, sum->grad_sum, n_chunks1b, 0, n_chunks2, seg_len)));
     else TIMED(K_CONV_GRAD_REDUCE, (conv_grad_reduce<<<dim3(a.W, (RED_OUTPUTS + red_per_block - 1) / red_per_block), 256, 0, st>>>(a, wt, ws, red_per_block, n_chunks1b, 0, n_chunks2, seg_len)));
     launches = 10;

@@ -131,8 +131,11 @@ def test_stale_snapshots_grouped_over_three_versions():
 # what pooling decisions within single-precision rounding of a tie can move it by (there are millions of them).
 @pytest.mark.parametrize("W,b,kw", [(2, 64, {}), (3, 43, {"lags": [1, 0, 1], "n_versions": 2}), (16, 96, {"check": (0, 8, 15)}),
                                      (17, 91, {"check": (0, 8, 16)}),
-                                     # 32 / 33, 1,020 / 1,025 rows and two sizes beyond, where the dense layer's products
-                                     # change form; groups of rows that leave remainders in every tile
+                                     # 32 / 33, 64 / 65, 448 / 450, 1,020 / 1,025, 1,280 / 1,290 rows and two sizes beyond,
+                                     # where the dense layer's products and the blocks of the first convolution change
+                                     # form; groups of rows that leave remainders in every tile
+                                     (4, 16, {}), (5, 13, {"lags": [0, 1, 1, 0, 1], "n_versions": 2}), (4, 112, {}), (9, 50, {"check": (0, 4, 8)}),
+                                     (10, 128, {"check": (0, 9)}), (10, 129, {"check": (0, 9)}),
                                      (4, 8, {"lags": [0, 1, 1, 0], "n_versions": 2}), (3, 11, {}), (12, 85, {"check": (0, 6, 11)}),
                                      (41, 25, {"check": (0, 20, 40), "lags": [w % 2 for w in range(41)], "n_versions": 2}),
                                      (40, 103, {"check": (0, 39)}), (50, 60, {"check": (0, 49)})])

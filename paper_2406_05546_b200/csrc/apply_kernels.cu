@@ -7,6 +7,8 @@
 // and store is a coalesced 16-byte access; the K loop is unrolled to keep many independent loads
 // in flight per thread.
 #include "kernels.h"
+#include "tc5_common.cuh"
+#include "device_common.cuh"
 
 namespace psk {
 
@@ -186,6 +188,179 @@ __global__ void __launch_bounds__(TPB) clip_coef_finish(const float* __restrict_
   coef_k[k] *= fminf(1.0f, clip / sqrtf(n2));      // a zero gradient keeps its factor (clip / 0 = inf)
 }
 
+// ---- clipping by global norm, summed and applied in one pass over a long queue ------------------------------------
+// A gradient's factor needs its whole norm, so summing clipped gradients takes two reads of the queue, unless a gradient
+// stays on the chip in between.  It does here: one CTA per SM owns a fixed range of float4 columns, every gradient's share
+// of it (22 KB) arrives by a bulk copy in a ring of ten shared-memory slots, is squared, and stays in its slot until the
+// CTAs have exchanged their partial sums of squares through global memory; then it is added with its factor.  HBM sees
+// every gradient once: the kernel's bound is one read of the queue.
+// Warps: one group squares, one adds (each thread keeps the sums of its four columns in registers): a warp's step per
+// gradient is a chain of latencies, which two groups halve.  One warp issues the copies, one publishes the CTA's partial
+// sums, CS_GATHER gather the other CTAs' in turn.  A word of the exchange carries its gradient's number beside the sum, so
+// it needs no flag, and the words of CS_RING gradients are used in turn; every CTA writes its word CS_COPIES times and a
+// CTA polls one of the copies only: the polls of all CTAs on one copy slow the stores down.
+// Measured (B200), us for clipping by norm, summing and applying K gradients, two passes over the queue (norms, factors,
+// weighted sum) -> this kernel: K = 1: 27 -> 12, 16: 39 -> 19, 128: 159 -> 86, 1600: 1466 -> 793 (6.6 TB/s), 6400: 5700 -> 3131.
+// At 1600 also: three gathering warps 902, four 1028 (more polls); 16 copies 812; squaring and adding by the same warps,
+// four gradients held in registers behind the ring, 887; a copy polled word by word by everybody 1124.
+// The CTAs wait for one another, so the launch is cooperative; every wait is bounded, and a warp gives up as a whole.
+constexpr int CS_ADD = 11, CS_ADD_PER = 4, CS_SQ = 8, CS_SQ_PER = 6, CS_GATHER = 2;      // warps, columns per thread
+constexpr int CS_THREADS = 32 * (CS_ADD + CS_SQ + 2 + CS_GATHER);
+constexpr int CS_MAX_COLS = 32 * CS_ADD * CS_ADD_PER;
+static_assert(CS_MAX_COLS <= 32 * CS_SQ * CS_SQ_PER, "both groups cover the columns");
+constexpr int CS_DEPTH = 16;                       // gradients whose sums / factors are kept in shared memory (>= slots)
+constexpr int CS_MAX_SLOTS = 16, CS_MISC = 2048, CS_SMEM = 227 * 1024;
+struct ClipShared {
+  uint64_t full[CS_MAX_SLOTS], empty[CS_MAX_SLOTS], norm_ready[CS_DEPTH], coef_ready[CS_DEPTH];
+  float warp_sum[CS_DEPTH][CS_SQ];
+  float coef[CS_DEPTH];
+  volatile uint32_t abort_flag;
+};
+static_assert(sizeof(ClipShared) <= CS_MISC, "shared memory");
+
+__global__ void __launch_bounds__(CS_THREADS, 1) clip_sum_apply(const float4* __restrict__ queue, int K, int cols, int slots, float clip,
+                                                                const float* __restrict__ coef_k, u64* words, const float4* theta_in,
+                                                                float4* theta_out, float4* __restrict__ replica, uint32_t* status) {
+  extern __shared__ __align__(128) uint8_t sm[];
+  ClipShared* sh = reinterpret_cast<ClipShared*>(sm);
+  float4* ring = reinterpret_cast<float4*>(sm + CS_MISC);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_cta = gridDim.x;
+  const int col0 = blockIdx.x * cols, n = min(cols, P_VEC4 - col0);      // n > 0 for every block
+  if (tid == 0) {
+    for (int i = 0; i < slots; ++i) { mbar_init(&sh->full[i], 1); mbar_init(&sh->empty[i], CS_ADD); }
+    for (int i = 0; i < CS_DEPTH; ++i) { mbar_init(&sh->norm_ready[i], CS_SQ); mbar_init(&sh->coef_ready[i], 1); }
+    sh->abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  // true for the whole warp or for none of it
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    if (__all_sync(0xffffffffu, mbar_try(smem_u32(bar), parity))) return true;
+    const bool done = mbar_wait(bar, parity) && !sh->abort_flag;
+    if (__all_sync(0xffffffffu, done)) return true;
+    sh->abort_flag = 1;
+    return false;
+  };
+  bool ok = true;
+  if (warp < CS_ADD) {
+    // ---------------- sums
+    float4 acc[CS_ADD_PER];
+#pragma unroll
+    for (int j = 0; j < CS_ADD_PER; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    int slot = 0;
+    for (int k = 0; k < K; ++k) {
+      if (!(ok = wait(&sh->coef_ready[k % CS_DEPTH], (k / CS_DEPTH) & 1))) break;
+      const float c = sh->coef[k % CS_DEPTH];
+      const float4* g = ring + slot * cols;
+      float4 v[CS_ADD_PER];
+#pragma unroll
+      for (int j = 0; j < CS_ADD_PER; ++j) {
+        const int i = tid + 32 * CS_ADD * j;
+        v[j] = i < n ? g[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sh->empty[slot]);
+#pragma unroll
+      for (int j = 0; j < CS_ADD_PER; ++j) fma4(c, v[j], acc[j]);
+      if (++slot == slots) slot = 0;
+    }
+    if (ok) {
+#pragma unroll
+      for (int j = 0; j < CS_ADD_PER; ++j) {
+        const int i = tid + 32 * CS_ADD * j;
+        if (i < n) {
+          float4 t = theta_in[col0 + i];
+          t.x -= acc[j].x; t.y -= acc[j].y; t.z -= acc[j].z; t.w -= acc[j].w;
+          theta_out[col0 + i] = t;
+          if (replica) replica[col0 + i] = t;
+        }
+      }
+    }
+  } else if (warp < CS_ADD + CS_SQ) {
+    // ---------------- sums of squares
+    const int id = tid - 32 * CS_ADD;
+    int slot = 0;
+    uint32_t phase = 0;
+    for (int k = 0; k < K; ++k) {
+      if (!(ok = wait(&sh->full[slot], phase))) break;
+      const float4* g = ring + slot * cols;
+      float s[CS_SQ_PER];
+#pragma unroll
+      for (int j = 0; j < CS_SQ_PER; ++j) {
+        const int i = id + 32 * CS_SQ * j;
+        const float4 v = i < n ? g[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        s[j] = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, v.w * v.w)));
+      }
+      float t = ((s[0] + s[1]) + (s[2] + s[3])) + (s[4] + s[5]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) { sh->warp_sum[k % CS_DEPTH][warp - CS_ADD] = t; mbar_arrive(&sh->norm_ready[k % CS_DEPTH]); }
+      if (++slot == slots) { slot = 0; phase ^= 1; }
+    }
+  } else if (warp == CS_ADD + CS_SQ) {
+    // ---------------- copies
+    int slot = 0;
+    uint32_t phase = 1;                              // flips to 0 when the first slot is used again
+    for (int k = 0; k < K; ++k) {
+      if (k >= slots && !(ok = wait(&sh->empty[slot], phase))) break;
+      if (lane == 0) {
+        mbar_expect_tx(&sh->full[slot], n * 16);
+        bulk_load(ring + slot * cols, queue + k * (int64_t)P_VEC4 + col0, n * 16, &sh->full[slot]);
+      }
+      if (++slot == slots) { slot = 0; phase ^= 1; }
+    }
+  } else if (warp == CS_ADD + CS_SQ + 1) {
+    // ---------------- this CTA's partial sums out
+    for (int k = 0; k < K; ++k) {
+      if (!(ok = wait(&sh->norm_ready[k % CS_DEPTH], (k / CS_DEPTH) & 1))) break;
+      if (lane < CS_COPIES) {
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < CS_SQ; ++w) t += sh->warp_sum[k % CS_DEPTH][w];
+        const u64 word = ((u64)(uint32_t)(k + 1) << 32) | __float_as_uint(t);
+        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(words + ((k % CS_RING) * CS_COPIES + lane) * NORM_WORDS + blockIdx.x), "l"(word) : "memory");
+      }
+    }
+  } else {
+    // ---------------- all CTAs' partial sums in, and the factor
+    for (int k = warp - (CS_ADD + CS_SQ + 2); k < K; k += CS_GATHER) {
+      const u64* w = words + ((k % CS_RING) * CS_COPIES + blockIdx.x % CS_COPIES) * NORM_WORDS;
+      // a lane's words are asked for together, the missing ones again and again until all have arrived
+      constexpr int PER_LANE = (NORM_WORDS + 31) / 32;
+      u64 v[PER_LANE];
+#pragma unroll
+      for (int i = 0; i < PER_LANE; ++i) v[i] = lane + 32 * i < n_cta ? 0ull : (u64)(uint32_t)(k + 1) << 32;
+      const long long t0 = clock64();
+      for (;;) {
+        bool all = true;
+#pragma unroll
+        for (int i = 0; i < PER_LANE; ++i)
+          if ((uint32_t)(v[i] >> 32) != (uint32_t)(k + 1)) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v[i]) : "l"(w + lane + 32 * i) : "memory");
+#pragma unroll
+        for (int i = 0; i < PER_LANE; ++i) all = all && (uint32_t)(v[i] >> 32) == (uint32_t)(k + 1);
+        if (__all_sync(0xffffffffu, all)) break;
+        if (__any_sync(0xffffffffu, clock64() - t0 > WAIT_LIMIT_CYCLES || sh->abort_flag)) { ok = false; break; }
+        __nanosleep(20);
+      }
+      float t = 0.f;
+#pragma unroll
+      for (int i = 0; i < PER_LANE; ++i) t += __uint_as_float((uint32_t)v[i]);
+      if (!__all_sync(0xffffffffu, ok)) { sh->abort_flag = 1; break; }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) {
+        sh->coef[k % CS_DEPTH] = coef_k[k] * fminf(1.0f, clip / sqrtf(t));      // a zero gradient keeps its factor (clip / 0 = inf)
+        mbar_arrive(&sh->coef_ready[k % CS_DEPTH]);
+      }
+    }
+  }
+  __syncthreads();
+  if (tid == 0 && sh->abort_flag) {
+    atomicOr(status, STATUS_WAIT_TIMEOUT);
+    for (int i = 0; i < 1000; ++i) __nanosleep(1000);      // let copies already issued land before the CTA ends
+  }
+}
+
 }  // namespace
 
 #define TIMED(id, launch) do { if (prof) prof->begin(id, st); launch; if (prof) prof->end(st); } while (0)
@@ -194,7 +369,7 @@ const char* kernel_name(int id) {
   static const char* names[K_COUNT] = {
       "conv1_fwd", "conv2_fwd", "fc1_fwd", "fc2_fwd_bwd", "fc1_dw", "fc1_dx", "conv2_bwd", "conv1_bwd",
       "conv_grad_reduce", "sum_apply_direct", "sum_partial", "sum_finish", "async_apply", "copy_rows",
-      "dropout_mask", "conv2_dw", "prep_w1", "sq_norm_partial", "clip_coef_finish", "eval_finish"};
+      "dropout_mask", "conv2_dw", "prep_w1", "sq_norm_partial", "clip_coef_finish", "eval_finish", "clip_sum_apply"};
   return id >= 0 && id < K_COUNT ? names[id] : "?";
 }
 
@@ -229,6 +404,33 @@ int launch_clip_factors(const float* queue, int64_t K, float clip, float* coef_k
   TIMED(K_SQ_NORM, (sq_norm_partial<<<dim3(NORM_CHUNKS, (unsigned)K), TPB, 0, st>>>(reinterpret_cast<const float4*>(queue), norm_part)));
   TIMED(K_COEF_FINISH, (clip_coef_finish<<<(unsigned)((K + TPB - 1) / TPB), TPB, 0, st>>>(norm_part, K, clip, coef_k)));
   return cudaGetLastError() == cudaSuccess ? 2 : -1;
+}
+
+int configure_apply_kernels() {
+  return allow_smem((const void*)clip_sum_apply, CS_SMEM) == cudaSuccess ? 0 : -1;
+}
+
+int launch_clip_sum_apply(const SumApplyArgs& a, float clip, uint64_t* words, uint32_t* status, cudaStream_t st, Profiler* prof) {
+  const int grid = g_sm_count < NORM_WORDS ? g_sm_count : NORM_WORDS;
+  const int cols = (P_VEC4 + grid - 1) / grid;
+  int slots = (CS_SMEM - CS_MISC) / (cols * 16);
+  if (slots > CS_MAX_SLOTS) slots = CS_MAX_SLOTS;
+  if (cols > CS_MAX_COLS || slots < 3 || (int64_t)(grid - 1) * cols >= P_VEC4) return -1;
+  if (cudaMemsetAsync(words, 0, CLIP_EXCHANGE_BYTES, st) != cudaSuccess) return -1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(CS_THREADS);
+  cfg.dynamicSmemBytes = (size_t)(CS_MISC + slots * cols * 16);
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeCooperative;
+  at.val.cooperative = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  TIMED(K_CLIP_SUM, cudaLaunchKernelEx(&cfg, clip_sum_apply, reinterpret_cast<const float4*>(a.queue), (int)a.K, cols, slots, clip, a.coef_k,
+                                       reinterpret_cast<u64*>(words), reinterpret_cast<const float4*>(a.theta_in),
+                                       reinterpret_cast<float4*>(a.theta_out), reinterpret_cast<float4*>(a.replica), status));
+  return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
 int launch_async_apply(const AsyncApplyArgs& a, const AsyncOrder& ord, cudaStream_t st, Profiler* prof) {

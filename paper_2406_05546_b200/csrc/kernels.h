@@ -45,7 +45,7 @@ constexpr uint32_t STATUS_WAIT_TIMEOUT = 2u;   // a bounded barrier wait in a te
 enum KernelId {
   K_CONV1_FWD = 0, K_CONV2_FWD, K_FC1_FWD, K_FC2_FWD_BWD, K_FC1_DW, K_FC1_DX, K_CONV2_BWD, K_CONV1_BWD,
   K_CONV_GRAD_REDUCE, K_SUM_APPLY_DIRECT, K_SUM_PARTIAL, K_SUM_FINISH, K_ASYNC_APPLY, K_COPY_ROWS,
-  K_DROPOUT_MASK, K_CONV2_DW, K_PREP_W1, K_SQ_NORM, K_COEF_FINISH, K_EVAL_FINISH, K_COUNT
+  K_DROPOUT_MASK, K_CONV2_DW, K_PREP_W1, K_SQ_NORM, K_COEF_FINISH, K_EVAL_FINISH, K_CLIP_SUM, K_COUNT
 };
 const char* kernel_name(int id);
 
@@ -231,6 +231,12 @@ int launch_copy_rows(float* dst, const float* src, int64_t rows, cudaStream_t st
 
 // Clipping by global norm: coef_k[k] *= min(1, clip / ||queue[k]||_2) for k < K.  norm_part: [K][NORM_CHUNKS] scratch.
 constexpr int NORM_CHUNKS = 8;
+// Clipping, summing and applying in one pass (sync and replay steps).  words: CLIP_EXCHANGE_BYTES of scratch, where the
+// CTAs exchange their partial sums of squares.
+constexpr int NORM_WORDS = 160, CS_RING = 64, CS_COPIES = 8;      // words per copy (one per CTA, at most), gradients, copies
+constexpr int CLIP_EXCHANGE_BYTES = NORM_WORDS * CS_RING * CS_COPIES * 8;
+int configure_apply_kernels();
+int launch_clip_sum_apply(const SumApplyArgs& a, float clip, uint64_t* words, uint32_t* status, cudaStream_t st, Profiler* prof);
 int launch_clip_factors(const float* queue, int64_t K, float clip, float* coef_k, float* norm_part, cudaStream_t st, Profiler* prof);
 
 // Evaluation pass: forward only, no dropout; loss [W] mean cross-entropy, argmax [W][b], correct [W] = samples whose

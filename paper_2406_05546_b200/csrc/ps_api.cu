@@ -58,6 +58,7 @@ struct ps_ctx {
   float* queue;
   float* coef_dev;                      // [queue_slots] per-gradient factors of a treated apply
   float* norm_part;                     // [queue_slots][NORM_CHUNKS] partial sums of squares
+  uint64_t* clip_words;                 // where the CTAs of the one-pass clipped apply exchange theirs
   cudaEvent_t coef_uploaded = nullptr;  // the staged factors have left coef_host
   psk::Workspace ws;
   float* x_stage[2]; int32_t* y_stage[2]; float* loss_stage[2]; int32_t* argmax_stage[2];   // two sets: two ticks may be in flight
@@ -142,6 +143,7 @@ void layout(ps_ctx* x, const ps_config& c, void* arena, void* pinned, uint64_t* 
   float* queue = a.take<float>(VEC_BYTES * (uint64_t)c.queue_slots);
   float* coef_dev = a.take<float>((uint64_t)c.queue_slots * 4);
   float* norm_part = a.take<float>((uint64_t)c.queue_slots * psk::NORM_CHUNKS * 4);
+  uint64_t* clip_words = a.take<uint64_t>(psk::CLIP_EXCHANGE_BYTES);
   psk::Workspace ws;
   const uint64_t p1_elems = c.precision != PS_FP32 ? psk::P1_PLANE_ELEMS : psk::P1_ELEMS;
   ws.p1 = a.take<float>(rows * p1_elems * 4);
@@ -176,7 +178,7 @@ void layout(ps_ctx* x, const ps_config& c, void* arena, void* pinned, uint64_t* 
   uint32_t* status_host = h.take<uint32_t>(ALIGN);
   if (x) {
     x->partial = partial; x->queue = queue; x->ws = ws; x->status_dev = ws.status;
-    x->coef_dev = coef_dev; x->norm_part = norm_part; x->coef_host = coef_host;
+    x->coef_dev = coef_dev; x->norm_part = norm_part; x->clip_words = clip_words; x->coef_host = coef_host;
     for (int k = 0; k < 2; ++k) { x->x_stage[k] = x_stage[k]; x->y_stage[k] = y_stage[k]; x->loss_stage[k] = loss_stage[k]; x->argmax_stage[k] = argmax_stage[k]; }
     x->io_stage = io_stage; x->status_host = status_host;
   }
@@ -266,7 +268,7 @@ int32_t ps_create(const ps_config* cfg, const float* init_params_host, ps_ctx** 
   x->ckpt_version.assign(x->ckpt_buf.size(), 0);
   double t = std::floor((double)cfg->dropout_p * 4294967296.0);
   x->drop_thresh = t <= 0.0 ? 0u : (t >= 4294967295.0 ? 0xFFFFFFFFu : (uint32_t)t);
-  if (psk::configure_fp32_conv2_kernels() != 0 || psk::configure_fp32_gemm_kernels() != 0 || psk::configure_tc5_kernels() != 0 || psk::configure_conv5_kernels() != 0 || psk::configure_conv1_kernels() != 0 || psk::configure_dw5_kernels() != 0 || psk::configure_c1d5_kernels() != 0) { delete x; return fail(PS_ERR_CUDA, "kernel configuration failed: %s", cudaGetErrorString(cudaGetLastError())); }
+  if (psk::configure_apply_kernels() != 0 || psk::configure_fp32_conv2_kernels() != 0 || psk::configure_fp32_gemm_kernels() != 0 || psk::configure_tc5_kernels() != 0 || psk::configure_conv5_kernels() != 0 || psk::configure_conv1_kernels() != 0 || psk::configure_dw5_kernels() != 0 || psk::configure_c1d5_kernels() != 0) { delete x; return fail(PS_ERR_CUDA, "kernel configuration failed: %s", cudaGetErrorString(cudaGetLastError())); }
   {
     // two side streams let independent branches of the backward pass overlap (they allocate no device memory)
     bool ok = cudaStreamCreateWithFlags(&x->side.s1, cudaStreamNonBlocking) == cudaSuccess &&
@@ -574,6 +576,7 @@ static int32_t apply_impl(ps_ctx* x, ps_mode mode, float lr, float scale, const 
     }
   }
   const bool treated = clip_norm > 0.f || staleness_alpha > 0.f;
+  const bool one_pass = clip_norm > 0.f && mode != PS_ASYNC;      // the ordered apply reads the norms' factors instead
   if (treated) {
     // factor of the gradient in queue slot k: the step size of its mode times 1 / (1 + alpha * staleness), where the
     // staleness is the version the update is applied to minus the version the worker had read
@@ -592,7 +595,7 @@ static int32_t apply_impl(ps_ctx* x, ps_mode mode, float lr, float scale, const 
     }
     CUDA_TRY(cudaMemcpyAsync(x->coef_dev, x->coef_host, (size_t)K * sizeof(float), cudaMemcpyHostToDevice, x->st));
     CUDA_TRY(cudaEventRecord(x->coef_uploaded, x->st));
-    if (clip_norm > 0.f) {
+    if (clip_norm > 0.f && !one_pass) {
       int n = psk::launch_clip_factors(x->queue, K, clip_norm, x->coef_dev, x->norm_part, x->st, &x->prof);
       if (n < 0) return cuda_fail(cudaGetLastError(), "clipping launch");
       x->launches += n;
@@ -612,7 +615,8 @@ static int32_t apply_impl(ps_ctx* x, ps_mode mode, float lr, float scale, const 
     a.coef = lr * scale / (float)(mode == PS_SYNC ? K : (int64_t)x->w_tick);
     a.partial = x->partial; a.max_split = MAX_SPLIT;
     a.coef_k = treated ? x->coef_dev : nullptr;
-    int n = psk::launch_sum_apply(a, x->st, &x->prof);
+    int n = one_pass ? psk::launch_clip_sum_apply(a, clip_norm, x->clip_words, x->status_dev, x->st, &x->prof)
+                     : psk::launch_sum_apply(a, x->st, &x->prof);
     if (n < 0) return cuda_fail(cudaGetLastError(), "apply launch");
     x->launches += n;
     x->version += 1;

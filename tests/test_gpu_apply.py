@@ -415,7 +415,8 @@ def _known_norm_grads(norms, seed):
     return g
 
 
-@pytest.mark.parametrize("mode_name,K", [("SYNC", 6), ("REPLAY", 300), ("ASYNC", 9)])
+# 1, 10 and 11: one gradient, as many as the one-pass kernel's ring has slots, and one more; 300: its exchange words wrap
+@pytest.mark.parametrize("mode_name,K", [("SYNC", 1), ("SYNC", 6), ("SYNC", 10), ("REPLAY", 11), ("REPLAY", 300), ("ASYNC", 9)])
 def test_clipping_by_global_norm(mode_name, K):
     ops, ps, o, g = _pair(queue_slots=max(K, 8), ring_depth=3, external_store=(mode_name == "REPLAY"), max_workers=64)
     norms = np.random.default_rng(K).uniform(0.2, 5.0, size=K)

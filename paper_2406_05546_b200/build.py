@@ -1,12 +1,15 @@
-"""Compile the CUDA library in-tree: paper_2406_05546_b200/libps_b200.so (sm_100a only)."""
+"""Compile the CUDA library in-tree: paper_2406_05546_b200/libps_b200.so (sm_100a only), and the binding's argument
+marshalling, _marshal.so."""
 import glob
 import os
 import subprocess
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libps_b200.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 
@@ -35,6 +38,14 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def build_marshal(force: bool = False) -> str:
+    src, header = os.path.join(CSRC, "marshal.c"), os.path.join(ROOT, "include", "ps.h")
+    if force or not os.path.exists(MARSHAL) or any(os.path.getmtime(d) > os.path.getmtime(MARSHAL) for d in (src, header)):
+        subprocess.run(["gcc", "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"),
+                        "-o", MARSHAL, src], check=True)
+    return MARSHAL
+
+
 if __name__ == "__main__":
     import sys
-    print(build(force=True, verbose="-v" in sys.argv))
+    print(build(force=True, verbose="-v" in sys.argv), build_marshal(force=True))

@@ -60,11 +60,12 @@ class Stats(C.Structure):
 
 
 _lib = None
+_marshal = None      # the extension that passes the arguments of the per-tick calls
 
 
 def load(path=None):
     """Loads the shared library (building it if its sources are newer) and declares the ABI."""
-    global _lib
+    global _lib, _marshal
     if _lib is not None and path is None:
         return _lib
     L = C.CDLL(path or _build.build())
@@ -110,7 +111,12 @@ def load(path=None):
     L.ps_last_error.argtypes = [vp]
     L.ps_last_error.restype = C.c_char_p
     if path is None:
-        _lib = L
+        _build.build_marshal()
+        from . import _marshal as m
+        m.bind({n: C.cast(getattr(L, n), C.c_void_p).value for n in
+                ("ps_pull_snapshot", "ps_queue_reserve", "workers_grad_step", "workers_grad_step_summed", "workers_eval",
+                 "ps_enqueue", "ps_apply", "ps_apply_summed", "ps_last_error")}, Snapshot, PSError)
+        _lib, _marshal = L, m
     return L
 
 
@@ -133,7 +139,7 @@ def ps_replay_sum_static(queue_dev, theta_in_dev, theta_out_dev, coef, stream=No
 
 
 def _np_ptr(a):
-    return a.ctypes.data_as(C.c_void_p) if a is not None else None
+    return a.ctypes.data if a is not None else None
 
 
 class ParameterServer:
@@ -168,6 +174,7 @@ class ParameterServer:
         ctx = C.c_void_p()
         self._check(self.lib.ps_create(C.byref(cfg), _np_ptr(init), C.byref(ctx)))
         self.ctx = ctx
+        self._addr = ctx.value
 
     def _check(self, rc):
         if rc != 0:
@@ -176,7 +183,7 @@ class ParameterServer:
     def close(self):
         if getattr(self, "ctx", None):
             self.lib.ps_destroy(self.ctx)
-            self.ctx = None
+            self.ctx = self._addr = None
 
     def __del__(self):
         try:
@@ -186,13 +193,11 @@ class ParameterServer:
 
     # -- worker side ---------------------------------------------------------
     def ps_pull_snapshot(self, worker, lag=0):
-        s = Snapshot()
-        self._check(self.lib.ps_pull_snapshot(self.ctx, int(worker), int(lag), C.byref(s)))
-        return s
+        return _marshal.pull(self._addr, worker, lag)
 
     def ps_queue_reserve(self, n):
-        ids = np.zeros(n, dtype=np.int64)
-        self._check(self.lib.ps_queue_reserve(self.ctx, int(n), _np_ptr(ids)))
+        ids = np.empty(n, dtype=np.int64)
+        _marshal.reserve(self._addr, ids)
         return ids
 
     def ps_slot_ptr(self, slot):
@@ -207,7 +212,6 @@ class ParameterServer:
         W, b = int(y_dev.shape[0]), int(y_dev.shape[1])
         assert x_dev.is_cuda and x_dev.dtype == torch.float32 and x_dev.is_contiguous() and x_dev.numel() == W * b * 784
         assert y_dev.is_cuda and y_dev.dtype == torch.int32 and y_dev.is_contiguous()
-        arr = (Snapshot * W)(*snaps)
         wid = np.ascontiguousarray(worker_ids, dtype=np.int32)
         assert wid.shape == (W,)
         if loss_dev is None:
@@ -217,10 +221,8 @@ class ParameterServer:
         sid = None if slot_ids is None else np.ascontiguousarray(slot_ids, dtype=np.int64)
         if grads_dev is not None:
             assert grads_dev.is_cuda and grads_dev.dtype == torch.float32 and grads_dev.shape == (W, P_PAD) and grads_dev.is_contiguous()
-        self._check(self.lib.workers_grad_step(
-            self.ctx, W, b, C.cast(arr, C.c_void_p), _np_ptr(wid), x_dev.data_ptr(), y_dev.data_ptr(),
-            int(seed), int(step), _np_ptr(sid), grads_dev.data_ptr() if grads_dev is not None else None,
-            loss_dev.data_ptr(), argmax_dev.data_ptr()))
+        _marshal.grad_step(self._addr, W, b, snaps, wid, x_dev.data_ptr(), y_dev.data_ptr(), seed, step, sid,
+                           grads_dev.data_ptr() if grads_dev is not None else None, loss_dev.data_ptr(), argmax_dev.data_ptr())
         return loss_dev, argmax_dev
 
     def workers_grad_step_summed(self, snaps, worker_ids, x_dev, y_dev, seed, step, grad_sum_dev=None, loss_dev=None,
@@ -230,7 +232,6 @@ class ParameterServer:
         W, b = int(y_dev.shape[0]), int(y_dev.shape[1])
         assert x_dev.is_cuda and x_dev.dtype == torch.float32 and x_dev.is_contiguous() and x_dev.numel() == W * b * 784
         assert y_dev.is_cuda and y_dev.dtype == torch.int32 and y_dev.is_contiguous()
-        arr = (Snapshot * W)(*snaps)
         wid = np.ascontiguousarray(worker_ids, dtype=np.int32)
         if grad_sum_dev is None:
             grad_sum_dev = torch.empty(P_PAD, dtype=torch.float32, device="cuda")
@@ -238,16 +239,12 @@ class ParameterServer:
             loss_dev = torch.empty(W, dtype=torch.float32, device="cuda")
         if argmax_dev is None:
             argmax_dev = torch.empty((W, b), dtype=torch.int32, device="cuda")
-        self._check(self.lib.workers_grad_step_summed(
-            self.ctx, W, b, C.cast(arr, C.c_void_p), _np_ptr(wid), x_dev.data_ptr(), y_dev.data_ptr(), int(seed), int(step),
-            grad_sum_dev.data_ptr(), loss_dev.data_ptr(), argmax_dev.data_ptr()))
+        _marshal.grad_step_summed(self._addr, W, b, snaps, wid, x_dev.data_ptr(), y_dev.data_ptr(), seed, step,
+                                  grad_sum_dev.data_ptr(), loss_dev.data_ptr(), argmax_dev.data_ptr())
         return grad_sum_dev, loss_dev, argmax_dev
 
     def ps_apply_summed(self, grad_sum_dev, n_workers, lr, scale=1.0):
-        res = ApplyResult()
-        self._check(self.lib.ps_apply_summed(self.ctx, grad_sum_dev.data_ptr(), int(n_workers), float(lr), float(scale), C.byref(res)))
-        return {"applied": res.applied, "new_version": res.new_version, "checkpointed": res.checkpointed,
-                "replicated": res.replicated}
+        return _marshal.apply_summed(self._addr, grad_sum_dev.data_ptr(), n_workers, lr, scale)
 
     def workers_eval(self, snaps, x_dev, y_dev):
         """Forward pass without dropout.  Returns (loss_dev [W], argmax_dev [W,b], correct_dev [W])."""
@@ -255,12 +252,10 @@ class ParameterServer:
         W, b = int(y_dev.shape[0]), int(y_dev.shape[1])
         assert x_dev.is_cuda and x_dev.dtype == torch.float32 and x_dev.is_contiguous() and x_dev.numel() == W * b * 784
         assert y_dev.is_cuda and y_dev.dtype == torch.int32 and y_dev.is_contiguous()
-        arr = (Snapshot * W)(*snaps)
         loss = torch.empty(W, dtype=torch.float32, device="cuda")
         am = torch.empty((W, b), dtype=torch.int32, device="cuda")
         correct = torch.empty(W, dtype=torch.int32, device="cuda")
-        self._check(self.lib.workers_eval(self.ctx, W, b, C.cast(arr, C.c_void_p), x_dev.data_ptr(), y_dev.data_ptr(),
-                                          loss.data_ptr(), am.data_ptr(), correct.data_ptr()))
+        _marshal.eval(self._addr, W, b, snaps, x_dev.data_ptr(), y_dev.data_ptr(), loss.data_ptr(), am.data_ptr(), correct.data_ptr())
         return loss, am, correct
 
     def ps_dropout_mask(self, seed, worker_id, step, b):
@@ -275,17 +270,12 @@ class ParameterServer:
         sid = None if slot_ids is None else np.ascontiguousarray(slot_ids, dtype=np.int64)
         if grads_dev is not None:
             assert grads_dev.is_cuda and grads_dev.dtype == self._torch.float32 and grads_dev.shape == (n, P_PAD) and grads_dev.is_contiguous()
-        self._check(self.lib.ps_enqueue(self.ctx, n, _np_ptr(sid),
-                                        grads_dev.data_ptr() if grads_dev is not None else None,
-                                        _np_ptr(wid), _np_ptr(bv), int(step)))
+        _marshal.enqueue(self._addr, n, sid, grads_dev.data_ptr() if grads_dev is not None else None, wid, bv, step)
 
     # -- server side -----------------------------------------------------------
     def ps_apply(self, mode, lr, scale=1.0, order=None):
-        res = ApplyResult()
         o = None if order is None else np.ascontiguousarray(order, dtype=np.int32)
-        self._check(self.lib.ps_apply(self.ctx, int(mode), float(lr), float(scale), _np_ptr(o), C.byref(res)))
-        return {"applied": res.applied, "new_version": res.new_version, "checkpointed": res.checkpointed,
-                "replicated": res.replicated}
+        return _marshal.apply(self._addr, mode, lr, scale, o)
 
     def ps_apply_stale(self, mode, lr, scale=1.0, order=None, clip_norm=0.0, staleness_alpha=0.0):
         res = ApplyResult()

@@ -12,6 +12,11 @@
 //     pooling decisions leave the same way, one byte per element (1 << winner, 0 = no gradient) as
 //     [channel quad][position][4 channels].
 // Every wait on an mbarrier is bounded.
+//
+// Measured at 128 x 128 (3.7 GFLOP, 58 us at the packed multiply-add's rate): 119.5 -> 110 us with the pooling's maximum by
+// three-input instructions, ReLU folded into it, and the winner by comparing for equality from the last element back.  The
+// integer and comparison instructions of the pooling and the operand moves take as long as the multiply-adds.  Pairs over
+// window columns instead of channels (weights duplicated instead of pixels) took 128 us, unpacked multiply-adds 121 - 125.
 #include "device_common.cuh"
 #include "kernels.h"
 #include "tc5_common.cuh"
@@ -19,6 +24,12 @@
 namespace psk {
 
 namespace {
+
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
 
 constexpr int C1_SPS = 1;                                // samples per step
 constexpr int C1_THREADS = 112 * C1_SPS;
@@ -115,16 +126,20 @@ __global__ void __launch_bounds__(C1_THREADS, C1_BLOCKS_PER_SM) conv1_fwd_planes
 #pragma unroll
         for (int j = 0; j < 4; ++j) unpack2(acc[cp][j], v[2 * cp][j], v[2 * cp + 1][j]);
       // ReLU then max = max then ReLU; the winner is the first window element that reaches the maximum (stored as the
-      // byte 1 << winner), and an element whose maximum is not positive passes no gradient (byte 0)
+      // byte 1 << winner), and an element whose maximum is not positive passes no gradient (byte 0).  The maximum is taken
+      // against the smallest positive number: no element of a dead window equals it, and it rounds to zero.
       float best[4];
-      uint32_t codes = 0;
+      uint32_t code[4];
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        const float m = fmaxf(fmaxf(v[c][0], v[c][1]), fmaxf(v[c][2], v[c][3]));
-        const uint32_t bi = v[c][0] == m ? 0u : (v[c][1] == m ? 1u : (v[c][2] == m ? 2u : 3u));
-        best[c] = fmaxf(m, 0.f);
-        codes |= (m > 0.f ? (1u << bi) : 0u) << (8 * c);      // one bit per window element: the filter-gradient kernel shifts it into a mask
+        const float m = max3(max3(v[c][0], v[c][1], v[c][2]), v[c][3], __int_as_float(1));
+        best[c] = m;
+        uint32_t e = v[c][3] == m ? 8u << (8 * c) : 0u;
+        e = v[c][2] == m ? 4u << (8 * c) : e;
+        e = v[c][1] == m ? 2u << (8 * c) : e;
+        code[c] = v[c][0] == m ? 1u << (8 * c) : e;
       }
+      const uint32_t codes = code[0] | code[1] | code[2] | code[3];
       const int row = (py + 1) * 16 + col_row, pos = py * 14 + px;
       *reinterpret_cast<uint2*>(ob + sp * C1_PLANES_BYTES + (cg >> 1) * (C1_PLANES_BYTES / 2) + row * 16 + (cg & 1) * 8) =
           make_uint2(bf16_pair(best[0], best[1]), bf16_pair(best[2], best[3]));

@@ -874,7 +874,12 @@ int32_t ps_tick_host_submit(ps_ctx* x, int32_t W, int32_t b, const int32_t* lags
   // copies of this tick behind the previous tick's work.  This staging set was last read by the tick before the
   // previous one; the copy stream waits for that tick's grad step.
   if (x->ticks_submitted >= 2) CUDA_TRY(cudaStreamWaitEvent(x->copy_st, x->stage_free[set], 0));
-  const int n_chunks = W >= 8 ? 4 : 1, per = (W + n_chunks - 1) / n_chunks;
+  // A chunk has to be worth a grad step of its own: it costs the host a dozen launches and the device a chain of short
+  // kernels.  us for a tick in 1 / 2 / 4 chunks, tensor-core path: 512 rows 216 / 268 / 394, 2,048 351 / 395 / 596,
+  // 4,096 562 / 584 / 702, 8,192 914 / 796 / 891, 16,384 1,694 / 1,417 / 1,312; FP32 path: 512 354 / 405 / 508,
+  // 1,024 607 / 591 / 704, 2,048 885 / 812 / 916, 8,192 2,548 / 2,410 / 2,459.
+  const bool two = rows >= (x->cfg.precision != PS_FP32 ? 6144u : 1024u);
+  const int n_chunks = std::min(W, rows >= 12288 ? 4 : (two ? 2 : 1)), per = (W + n_chunks - 1) / n_chunks;
   for (int c = 0; c < n_chunks; ++c) {
     const int w0 = c * per, w1 = std::min(W, w0 + per);
     if (w0 >= w1) break;

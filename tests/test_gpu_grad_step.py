@@ -318,9 +318,10 @@ def test_argument_errors():
     srv.close()
 
 
-@pytest.mark.parametrize("precision,W,b", [(0, 3, 4), (0, 9, 5), (2, 9, 5), (2, 8, 16)])
+# 1,026 rows: two chunks on the FP32 path; 12,480 rows: four, the last of one worker
+@pytest.mark.parametrize("precision,W,b", [(0, 3, 4), (0, 9, 5), (2, 9, 5), (2, 8, 16), (0, 9, 114), (2, 13, 960)])
 def test_tick_from_host_buffers_matches_the_oracle(precision, W, b):
-    """ps_tick_host: inputs copied in by worker chunks (four when there are eight workers or more), snapshots
+    """ps_tick_host: inputs copied in by worker chunks (several from a thousand rows on), snapshots
     with lags, grad step into reserved slots, enqueue, sync apply, losses and labels copied out."""
     from oracle import cnn, ps as ops
     import torch

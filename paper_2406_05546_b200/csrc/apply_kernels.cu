@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(TPB) sum_apply_direct(const float4* __restrict
   // writes it, and the two pointers carry no no-alias promise
   int col = blockIdx.x * TPB + threadIdx.x;
   if (col >= P_VEC4) return;
+  pdl_enter();
   float4 s = column_sum<WEIGHTED>(queue + col, 0, K, coef_k);
   float4 t = theta_in[col];
   t.x = fmaf(-coef, s.x, t.x); t.y = fmaf(-coef, s.y, t.y);
@@ -82,6 +83,7 @@ __global__ void __launch_bounds__(TPB) sum_partial(const float4* __restrict__ qu
                                                    int n_split, float4* __restrict__ partial, const float* __restrict__ coef_k) {
   int col = blockIdx.x * TPB + threadIdx.x;
   if (col >= P_VEC4) return;
+  pdl_enter();
   int s = blockIdx.y;
   int64_t per = (K + n_split - 1) / n_split;
   int64_t k0 = s * per, k1 = k0 + per < K ? k0 + per : K;
@@ -95,6 +97,7 @@ __global__ void __launch_bounds__(TPB) sum_finish(const float4* __restrict__ par
                                                   float4* __restrict__ replica, float coef) {
   int col = blockIdx.x * TPB + threadIdx.x;
   if (col >= P_VEC4) return;
+  pdl_enter();
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int i = 0; i < n_split; ++i) add4(s, partial[(int64_t)i * P_VEC4 + col]);
   float4 t = theta_in[col];
@@ -110,6 +113,7 @@ __global__ void __launch_bounds__(TPB) sum_finish(const float4* __restrict__ par
 __global__ void __launch_bounds__(TPB) async_apply(AsyncApplyArgs a, AsyncOrder ord) {
   int col = blockIdx.x * TPB + threadIdx.x;
   if (col >= P_VEC4) return;
+  pdl_enter();
   const float4* q = reinterpret_cast<const float4*>(a.queue) + col;
   float4 t = reinterpret_cast<const float4*>(a.theta_in)[col];
   constexpr int U = 8;
@@ -388,13 +392,13 @@ int launch_sum_apply(const SumApplyArgs& a, cudaStream_t st, Profiler* prof) {
   const float coef = ck ? 1.0f : a.coef;      // the per-gradient factors already carry the learning rate
   if (n_split <= 1) {
     if (ck) TIMED(K_SUM_APPLY_DIRECT, (sum_apply_direct<true><<<COL_BLOCKS, TPB, 0, st>>>(q, a.K, tin, tout, rep, coef, ck)));
-    else TIMED(K_SUM_APPLY_DIRECT, (sum_apply_direct<false><<<COL_BLOCKS, TPB, 0, st>>>(q, a.K, tin, tout, rep, coef, nullptr)));
+    else TIMED(K_SUM_APPLY_DIRECT, launch_pdl(sum_apply_direct<false>, dim3(COL_BLOCKS), TPB, 0, st, q, a.K, tin, tout, rep, coef, nullptr));
     launches = 1;
   } else {
     float4* part = reinterpret_cast<float4*>(a.partial);
     if (ck) TIMED(K_SUM_PARTIAL, (sum_partial<true><<<dim3(COL_BLOCKS, n_split), TPB, 0, st>>>(q, a.K, n_split, part, ck)));
-    else TIMED(K_SUM_PARTIAL, (sum_partial<false><<<dim3(COL_BLOCKS, n_split), TPB, 0, st>>>(q, a.K, n_split, part, nullptr)));
-    TIMED(K_SUM_FINISH, (sum_finish<<<COL_BLOCKS, TPB, 0, st>>>(part, n_split, tin, tout, rep, coef)));
+    else TIMED(K_SUM_PARTIAL, launch_pdl(sum_partial<false>, dim3(COL_BLOCKS, n_split), TPB, 0, st, q, a.K, n_split, part, nullptr));
+    TIMED(K_SUM_FINISH, launch_pdl(sum_finish, dim3(COL_BLOCKS), TPB, 0, st, part, n_split, tin, tout, rep, coef));
     launches = 2;
   }
   return cudaGetLastError() == cudaSuccess ? launches : -1;
@@ -434,7 +438,7 @@ int launch_clip_sum_apply(const SumApplyArgs& a, float clip, uint64_t* words, ui
 }
 
 int launch_async_apply(const AsyncApplyArgs& a, const AsyncOrder& ord, cudaStream_t st, Profiler* prof) {
-  TIMED(K_ASYNC_APPLY, (async_apply<<<COL_BLOCKS, TPB, 0, st>>>(a, ord)));
+  TIMED(K_ASYNC_APPLY, launch_pdl(async_apply, dim3(COL_BLOCKS), TPB, 0, st, a, ord));
   return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 

@@ -129,6 +129,7 @@ __global__ void __launch_bounds__(D1_THREADS, 1) conv1_dw_tc5(GradStepArgs a, Wo
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
+  pdl_enter();
 
   if (warp == 0) {
     // ---------------- MMA issue
@@ -359,7 +360,7 @@ int launch_conv1_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const Work
   const int len = (total + grid - 1) / grid;
   grid = (total + len - 1) / len;
   const int slots = (a.b - 1) / len + 2;
-  TIMED(K_CONV1_BWD, (conv1_dw_tc5<<<grid, D1_THREADS, D1_SMEM, st>>>(a, wt, ws, len, slots)));
+  TIMED(K_CONV1_BWD, launch_pdl(conv1_dw_tc5, dim3(grid), D1_THREADS, D1_SMEM, st, a, wt, ws, len, slots));
   *seg_len = len;
   return slots;
 }

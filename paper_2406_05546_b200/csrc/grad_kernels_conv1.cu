@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(C1_THREADS, C1_BLOCKS_PER_SM) conv1_fwd_planes
   }
   // the border rows of the planes are never written below: cleared once, they leave as zeros with every sample
   for (int t = tid; t < 2 * C1_OUT_BYTES / 16; t += C1_THREADS) reinterpret_cast<uint4*>(outb)[t] = make_uint4(0u, 0u, 0u, 0u);
+  pdl_enter();       // the weights may come from the apply just before
   u64 wp[2][10];     // wp[cp][k] = tap k of channels 4 cg + 2 cp and + 1; k = 9 is the bias
 #pragma unroll
   for (int cp = 0; cp < 2; ++cp) {
@@ -182,7 +183,7 @@ int launch_conv1_fwd_planes(const GradStepArgs& a, const WorkerTable& wt, const 
   const int slots = C1_BLOCKS_PER_SM * g_sm_count, rows = a.W * a.b;
   const int spb = rows <= slots ? 1 : (rows <= 2 * slots ? 2 : C1_SPB);
   const int chunks = (a.b + spb - 1) / spb;
-  TIMED(K_CONV1_FWD, (conv1_fwd_planes<<<dim3(chunks, a.W), C1_THREADS, C1_SMEM, st>>>(xmap, a, wt, gt, ws, spb)));
+  TIMED(K_CONV1_FWD, launch_pdl(conv1_fwd_planes, dim3(chunks, a.W), C1_THREADS, C1_SMEM, st, xmap, a, wt, gt, ws, spb));
   return 1;
 }
 

@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(F_THREADS, 2) conv2_fwd_tc5(GradStepArgs a, Gr
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = pipe->tmem_base;
+  pdl_enter();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -304,6 +305,7 @@ __global__ void __launch_bounds__(THREADS, 2) conv2_dx_tc5(GradStepArgs a, Group
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = pipe->tmem_base;
+  pdl_enter();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -463,14 +465,14 @@ void launch_conv2_fwd_tc5(const GradStepArgs& a, const WorkerTable& wt, const Gr
   static const FoldTable fold = make_fold_table();
   int len;
   const int n = plan_row_ranges(gt, a.b, 2 * g_sm_count, 2, &len);      // two CTAs per SM, tiles of two samples
-  TIMED(K_CONV2_FWD, (conv2_fwd_tc5<<<n, F_THREADS, F_SMEM, st>>>(a, gt, ws, len, fold)));
+  TIMED(K_CONV2_FWD, launch_pdl(conv2_fwd_tc5, dim3(n), F_THREADS, F_SMEM, st, a, gt, ws, len, fold));
 }
 
 void launch_conv2_dx_tc5(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                          cudaStream_t st, Profiler* prof) {
   int len;
   const int n = plan_row_ranges(gt, a.b, 2 * g_sm_count, 1, &len);
-  TIMED(K_CONV2_BWD, (conv2_dx_tc5<<<n, THREADS, X_SMEM, st>>>(a, gt, ws, len)));
+  TIMED(K_CONV2_BWD, launch_pdl(conv2_dx_tc5, dim3(n), THREADS, X_SMEM, st, a, gt, ws, len));
 }
 
 }  // namespace psk

@@ -114,6 +114,7 @@ __global__ void __launch_bounds__(W5_THREADS, 1) conv2_dw_tc5(GradStepArgs a, Wo
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
+  pdl_enter();
 
   if (warp == 0) {
     // ---------------- MMA issue

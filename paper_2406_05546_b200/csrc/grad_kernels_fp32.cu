@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(224) conv1_fwd(GradStepArgs a, WorkerTable wt,
   __shared__ __align__(16) float w[16][12];   // 9 taps + bias + padding
   const int s = blockIdx.y, tid = threadIdx.x;
   const float* theta = group_theta(wt, gt, s);
+  pdl_enter();       // the weights may come from the apply just before
   if (tid < 160) {
     if (tid < 144) w[tid / 9][tid % 9] = theta[OFF_C1W + tid];
     else w[tid - 144][9] = theta[OFF_C1B + tid - 144];
@@ -117,6 +118,7 @@ __global__ void __launch_bounds__(256) conv1_bwd(GradStepArgs a, WorkerTable wt,
       gr[k] = pp < 196 ? ws.dp1[row * P1_ELEMS + oc * 196 + pp] : 0.f;
     }
   };
+  pdl_enter();
   prefetch(i0);
   for (int i = i0; i < i1; ++i) {
     __syncthreads();                        // the previous sample's image is no longer read
@@ -188,6 +190,7 @@ __global__ void __launch_bounds__(256) conv_grad_reduce(GradStepArgs a, WorkerTa
                                                         int n_chunks2, int seg_len) {
   const int s = blockIdx.x, b = a.b, split = fc2_split(a.W, b);
   float* grad = wt.grad[s];
+  pdl_enter();
   const int used2 = used_slots(s, b, seg_len, n_chunks2), used1 = used_slots(s, b, seg_len1, n_chunks);
   for (int v = blockIdx.y * per_block + threadIdx.x; v < min(RED_OUTPUTS, ((int)blockIdx.y + 1) * per_block); v += 256) {
     int o = v;
@@ -228,6 +231,7 @@ __global__ void __launch_bounds__(256) fused_finish(GradStepArgs a, WorkerTable 
                                                     int n_super, float* __restrict__ grad_sum, int n_chunks, int seg_len1,
                                                     int n_chunks2, int seg_len) {
   __shared__ float warp_sum[8][32];
+  pdl_enter();
   const int b = a.b, split = fc2_split(a.W, b);
   if (blockIdx.x < FUSED_W1_BLOCKS) {
     const int i = blockIdx.x * 256 + threadIdx.x;
@@ -279,6 +283,7 @@ __global__ void __launch_bounds__(128) eval_finish(GradStepArgs a, WorkerTable w
   __shared__ int warp_hits[4];
   const int s = blockIdx.x, src = wt.src[s], split = fc2_split(a.W, a.b);
   int hits = 0;
+  pdl_enter();
   for (int i = threadIdx.x; i < a.b; i += 128) {
     const int64_t r = (int64_t)src * a.b + i;
     hits += a.argmax[r] == a.y[r] ? 1 : 0;
@@ -327,7 +332,7 @@ static int samples_per_block(int rows, int least, int most) {
 }
 static void launch_conv1_fwd(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof) {
   const int spb = samples_per_block(a.W * a.b, 1, CONV1_SPB);
-  TIMED(K_CONV1_FWD, (conv1_fwd<<<dim3((a.b + spb - 1) / spb, a.W), 224, 0, st>>>(a, wt, gt, ws, spb)));
+  TIMED(K_CONV1_FWD, launch_pdl(conv1_fwd, dim3((a.b + spb - 1) / spb, a.W), 224, 0, st, a, wt, gt, ws, spb));
 }
 
 // Evaluation pass: the forward kernels of the grad step with the dropout switched off, then the per-worker loss and hit
@@ -349,7 +354,7 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
     launches += 3;
   }
   launch_output_layer(true, a, wt, gt, ws, st, prof);
-  TIMED(K_EVAL_FINISH, (eval_finish<<<a.W, 128, 0, st>>>(a, wt, ws, correct)));
+  TIMED(K_EVAL_FINISH, launch_pdl(eval_finish, dim3(a.W), 128, 0, st, a, wt, ws, correct));
   launches += 2;
   return cudaGetLastError() == cudaSuccess ? launches : -1;
 }
@@ -391,7 +396,7 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     if (launch_conv1_fwd_planes(a, wt, gt, ws, st, prof) < 0) return -1;
     launch_conv2_fwd_tc5(a, wt, gt, ws, st, prof);
     if (!a.skip_prep_w1 && side.s1) cudaStreamWaitEvent(st, side.join1, 0);
-    int n = launch_fc1_fwd_tc5(a, wt, gt, ws, st, prof);
+    int n = launch_fc1_fwd_tc5(a, wt, gt, ws, st, prof, side.s1 && !a.skip_prep_w1);
     if (n < 0) return -1;
     launches += 2 + n;
     launch_output_layer(false, a, wt, gt, ws, st, prof);
@@ -413,7 +418,7 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     if (n_chunks1t < 0) return -1;
     if (side.s1) cudaStreamWaitEvent(st, side.join1, 0);
     if (side.s2) cudaStreamWaitEvent(st, side.join2, 0);
-    if (sum) TIMED(K_CONV_GRAD_REDUCE, (fused_finish<<<FUSED_W1_BLOCKS + FUSED_SMALL_BLOCKS, 256, 0, st>>>(a, wt, ws, sum->super_part, sum->n_super, sum->grad_sum, n_chunks1t, seg_len1, n_chunks2, seg_len)));
+    if (sum) TIMED(K_CONV_GRAD_REDUCE, (fused_finish<<<dim3(FUSED_W1_BLOCKS + FUSED_SMALL_BLOCKS), 256, 0, st>>>(a, wt, ws, sum->super_part, sum->n_super, sum->grad_sum, n_chunks1t, seg_len1, n_chunks2, seg_len)));
     else TIMED(K_CONV_GRAD_REDUCE, (conv_grad_reduce<<<dim3(a.W, (RED_OUTPUTS + red_per_block - 1) / red_per_block), 256, 0, st>>>(a, wt, ws, red_per_block, n_chunks1t, seg_len1, n_chunks2, seg_len)));
     launches += 4;
   } else {
@@ -430,10 +435,10 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     n_chunks2 = launch_conv2_dw_direct(a, ws, s2, prof, &seg_len);
     if (side.s2) cudaEventRecord(side.join2, s2);
     launch_conv2_direct(false, a, gt, ws, st, prof);
-    TIMED(K_CONV1_BWD, (conv1_bwd<<<dim3(n_chunks1b, a.W), 256, 0, st>>>(a, wt, ws, spb1b, n_chunks1b)));
+    TIMED(K_CONV1_BWD, launch_pdl(conv1_bwd, dim3(n_chunks1b, a.W), 256, 0, st, a, wt, ws, spb1b, n_chunks1b));
     if (side.s1) cudaStreamWaitEvent(st, side.join1, 0);
     if (side.s2) cudaStreamWaitEvent(st, side.join2, 0);
-    if (sum) TIMED(K_CONV_GRAD_REDUCE, (fused_finish<<<FUSED_W1_BLOCKS + FUSED_SMALL_BLOCKS, 256, 0, st>>>(a, wt, ws, sum->super_part, sum->n_super, sum->grad_sum, n_chunks1b, 0, n_chunks2, seg_len)));
+    if (sum) TIMED(K_CONV_GRAD_REDUCE, (fused_finish<<<dim3(FUSED_W1_BLOCKS + FUSED_SMALL_BLOCKS), 256, 0, st>>>(a, wt, ws, sum->super_part, sum->n_super, sum->grad_sum, n_chunks1b, 0, n_chunks2, seg_len)));
     else TIMED(K_CONV_GRAD_REDUCE, (conv_grad_reduce<<<dim3(a.W, (RED_OUTPUTS + red_per_block - 1) / red_per_block), 256, 0, st>>>(a, wt, ws, red_per_block, n_chunks1b, 0, n_chunks2, seg_len)));
     launches = 10;
   }

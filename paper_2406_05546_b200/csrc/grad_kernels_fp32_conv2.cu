@@ -100,6 +100,7 @@ __global__ void __launch_bounds__(conv_threads<SPB>(), SPB > 1 ? 2 : 1) conv2_di
     w[t] = FWD ? theta[OFF_C2W + ((n0 + n) * C1 + k) * 9 + tap] : theta[OFF_C2W + (k * C1 + n0 + n) * 9 + 8 - tap];
   }
   __syncthreads();                                 // the borders are in place before copies land beside them
+  pdl_enter();
   fetch(0, 0);
   place(0);
   const int sp = tid / 49, pos = tid - sp * 49, py = pos / 7, px = pos - py * 7;
@@ -316,8 +317,8 @@ bool set_smem() {
 
 template <bool FWD, int NC, int SPB, int CH>
 void run_conv(const GradStepArgs& a, const GroupTable& gt, const Workspace& ws, cudaStream_t st) {
-  conv2_direct<FWD, NC, SPB, CH><<<dim3(group_tiles(gt, a.b, SPB), ConvShape<FWD>::NOUT / NC), conv_threads<SPB>(),
-                                   conv_smem_bytes<FWD, NC, SPB, CH>(), st>>>(a, gt, ws);
+  launch_pdl(conv2_direct<FWD, NC, SPB, CH>, dim3(group_tiles(gt, a.b, SPB), ConvShape<FWD>::NOUT / NC), conv_threads<SPB>(),
+             conv_smem_bytes<FWD, NC, SPB, CH>(), st, a, gt, ws);
 }
 
 }  // namespace

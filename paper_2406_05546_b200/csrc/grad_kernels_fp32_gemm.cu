@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(256, 2) sgemm_tile(GradStepArgs a, WorkerTable
   const int ty = (warp >> 1) * 4 + (lane >> 3), tx = (warp & 1) * 8 + (lane & 7);     // a warp covers 4 x 8 threads of the 16 x 16
   TileIo io;
   if (!locate_tile<OP, BM>(a, wt, gt, ws, io)) return;
+  pdl_enter();
   const int n0 = blockIdx.x * BN;
   int kt0 = 0, kt1 = (io.K + GK - 1) / GK;
   if (SPLIT) {
@@ -253,6 +254,7 @@ __global__ void __launch_bounds__(128) sgemm_fwd_seq(GradStepArgs a, WorkerTable
   const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX, n0 = blockIdx.x * TN;
   TileIo io;
   if (!locate_tile<G_FWD, TM>(a, wt, gt, ws, io)) return;
+  pdl_enter();
   auto issue = [&](int step, int buf) {
     if (step < STEPS) {
       float* dst = sm + buf * STAGE;
@@ -337,6 +339,7 @@ __global__ void __launch_bounds__(128) sgemm_fwd_rows(GradStepArgs a, WorkerTabl
   const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3, n0 = blockIdx.x * 16;
   TileIo io;
   if (!locate_tile<G_FWD, 16>(a, wt, gt, ws, io)) return;
+  pdl_enter();
   for (int c = 0; c < RW_CHUNKS; ++c) {
 #pragma unroll
     for (int i = 0; i < 32 * RW_K / 4 / 128; ++i) {
@@ -403,6 +406,7 @@ __global__ void __launch_bounds__(256) sgemm_dx_skinny(GradStepArgs a, WorkerTab
   const int tid = threadIdx.x, n0 = blockIdx.x * 32, rank = blockIdx.z, k0 = rank * DXS_SLICE;
   TileIo io;
   if (!locate_tile<G_DX, 16>(a, wt, gt, ws, io)) return;    // the same for all CTAs of a cluster
+  pdl_enter();
   for (int e = tid; e < 16 * (DXS_SLICE / 4); e += 256) {
     const int m = e / (DXS_SLICE / 4), kq = (e % (DXS_SLICE / 4)) * 4;
     cp_async16(As + m * DXS_PITCH + kq, io.A + (int64_t)min(io.m0 + m, io.m_end - 1) * HID + k0 + kq, true);
@@ -470,9 +474,9 @@ void run_grouped(const GradStepArgs& a, const WorkerTable& wt, const GroupTable&
   const int rows = a.W * a.b;
   if constexpr (OP == G_FWD) {
     if (rows <= 1280) {
-      if (rows <= 64) sgemm_fwd_rows<<<dim3(HID / 16, group_tiles(gt, a.b, 16)), 128, RW_SMEM, st>>>(a, wt, gt, ws);
-      else if (rows <= 448) sgemm_fwd_seq<32, 16, 2, 2><<<dim3(HID / 16, group_tiles(gt, a.b, 32)), 128, 0, st>>>(a, wt, gt, ws);
-      else sgemm_fwd_seq<64, 16, 4, 2><<<dim3(HID / 16, group_tiles(gt, a.b, 64)), 128, 0, st>>>(a, wt, gt, ws);
+      if (rows <= 64) launch_pdl(sgemm_fwd_rows, dim3(HID / 16, group_tiles(gt, a.b, 16)), 128, RW_SMEM, st, a, wt, gt, ws);
+      else if (rows <= 448) launch_pdl(sgemm_fwd_seq<32, 16, 2, 2>, dim3(HID / 16, group_tiles(gt, a.b, 32)), 128, 0, st, a, wt, gt, ws);
+      else launch_pdl(sgemm_fwd_seq<64, 16, 4, 2>, dim3(HID / 16, group_tiles(gt, a.b, 64)), 128, 0, st, a, wt, gt, ws);
       return;
     }
   } else {
@@ -493,8 +497,8 @@ void run_grouped(const GradStepArgs& a, const WorkerTable& wt, const GroupTable&
     const int n = (int)((grid.x * grid.y + g_sm_count - 1) / g_sm_count);
     return (n / 2) * two + (n & 1) * one;
   };
-  if (cost(wide, 1.f, 1.73f) < cost(narrow, 0.605f, 1.1f)) sgemm_tile<OP, 7, 8, false><<<wide, 256, Tile<OP, 7, 8>::SMEM, st>>>(a, wt, gt, ws);
-  else sgemm_tile<OP, 8, 4, false><<<narrow, 256, Tile<OP, 8, 4>::SMEM, st>>>(a, wt, gt, ws);
+  if (cost(wide, 1.f, 1.73f) < cost(narrow, 0.605f, 1.1f)) launch_pdl(sgemm_tile<OP, 7, 8, false>, wide, 256, Tile<OP, 7, 8>::SMEM, st, a, wt, gt, ws);
+  else launch_pdl(sgemm_tile<OP, 8, 4, false>, narrow, 256, Tile<OP, 8, 4>::SMEM, st, a, wt, gt, ws);
 }
 
 }  // namespace

@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(FC2_THREADS, 1) output_layer(GradStepArgs a, W
   w2t[tid][NCLS] = w2t[tid][NCLS + 1] = 0.f;
   if (tid < NCLS) b2[tid] = theta[OFF_F2B + tid];
   __syncthreads();
+  pdl_enter();
   const float scale = 1.0f / (1.0f - a.drop_p);
   const float inv_b = 1.0f / (float)a.b;
   const bool hi16 = lane & 16, hi8 = lane & 8, hi4 = lane & 4;
@@ -217,8 +218,8 @@ __global__ void __launch_bounds__(FC2_THREADS, 1) output_layer(GradStepArgs a, W
 
 void launch_output_layer(bool eval, const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof) {
   const dim3 grid(a.W, fc2_split(a.W, a.b));
-  if (eval) TIMED(K_FC2_FWD_BWD, (output_layer<true><<<grid, FC2_THREADS, 0, st>>>(a, wt, gt, ws)));
-  else TIMED(K_FC2_FWD_BWD, (output_layer<false><<<grid, FC2_THREADS, 0, st>>>(a, wt, gt, ws)));
+  if (eval) TIMED(K_FC2_FWD_BWD, launch_pdl(output_layer<true>, dim3(grid), FC2_THREADS, 0, st, a, wt, gt, ws));
+  else TIMED(K_FC2_FWD_BWD, launch_pdl(output_layer<false>, dim3(grid), FC2_THREADS, 0, st, a, wt, gt, ws));
 }
 
 }  // namespace psk

@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(gemm_threads(EPI), 1) tc5_gemm(const __grid_co
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_acc = *tmem_slot;
+  pdl_enter();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -348,6 +349,7 @@ __global__ void __launch_bounds__(192, 2) tc5_fwd_narrow(const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_enter();
   if (warp == 0) {
     if (lane == 0) {
       uint32_t parity = 1;                     // the first round of stages is free
@@ -450,6 +452,7 @@ __global__ void __launch_bounds__(256, 1) tc5_dx_split(const __grid_constant__ G
     for (int i = 0; i <= S::KB; ++i) mbar_init(&full[i], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    pdl_enter();
     for (int i = 0; i < S::KB; ++i) {
       mbar_expect_tx(&full[i], S::STAGE_BYTES);
       tma_load_3d(tiles + i * S::STAGE_BYTES, &maps.a, &full[i], (rank * S::KB + i) * BK, m0, 0);
@@ -464,6 +467,7 @@ __global__ void __launch_bounds__(256, 1) tc5_dx_split(const __grid_constant__ G
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_enter();
   if (warp == 1 && lane == 0) {
     constexpr uint32_t idesc = instr_desc_tf32(BM, S::BN);
     const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0) >> 32);
@@ -634,7 +638,7 @@ int launch_prep_w1(const GroupTable& gt, const Workspace& ws, cudaStream_t st, P
 
 // The forward product; the copies of W1 must be in place.
 int launch_fc1_fwd_tc5(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
-                       cudaStream_t st, Profiler* prof) {
+                       cudaStream_t st, Profiler* prof, bool after_join) {
   GemmMaps maps;
   const uint64_t rows = (uint64_t)a.W * a.b;
   const int mt = group_tiles(gt, a.b, BM), mt_narrow = group_tiles(gt, a.b, NR_BM);
@@ -643,12 +647,12 @@ int launch_fc1_fwd_tc5(const GradStepArgs& a, const WorkerTable& wt, const Group
   if (!make_map(&maps.b, ws.w1r, FLAT, HID, (uint64_t)gt.n_groups, FLAT, (uint64_t)HID * FLAT, narrow ? NR_BN : 256)) return -1;
   if (narrow) {
     GemmArgs ga{FLAT, HID, HID, 0, ws.d, HID / NR_BN, 0};
-    TIMED(K_FC1_FWD, (tc5_fwd_narrow<<<dim3(HID / NR_BN, mt_narrow), 192, NR_SMEM, st>>>(maps, ga, a, wt, gt, ws)));
+    TIMED(K_FC1_FWD, launch_pdl_if(!after_join, tc5_fwd_narrow, dim3(HID / NR_BN, mt_narrow), 192, NR_SMEM, st, maps, ga, a, wt, gt, ws));
     return 1;
   }
   GemmArgs ga{FLAT, HID, HID, 0, ws.d, HID / 256, (HID / 256) * mt};
   const int grid = ga.n_tiles < g_sm_count ? ga.n_tiles : g_sm_count;
-  TIMED(K_FC1_FWD, (tc5_gemm<EPI_FC1_FWD, 256><<<grid, gemm_threads(EPI_FC1_FWD), gemm_smem_bytes(256, MAX_STAGES, epi_warps(EPI_FC1_FWD)), st>>>(maps, ga, a, wt, gt, ws)));
+  TIMED(K_FC1_FWD, launch_pdl_if(!after_join, tc5_gemm<EPI_FC1_FWD, 256>, dim3(grid), gemm_threads(EPI_FC1_FWD), gemm_smem_bytes(256, MAX_STAGES, epi_warps(EPI_FC1_FWD)), st, maps, ga, a, wt, gt, ws));
   return 1;
 }
 
@@ -667,7 +671,7 @@ int launch_fc1_dx_tc5(const GradStepArgs& a, const WorkerTable& wt, const GroupT
     return 1;
   }
   const int grid = ga.n_tiles < g_sm_count ? ga.n_tiles : g_sm_count;
-  TIMED(K_FC1_DX, (tc5_gemm<EPI_STORE_BF16, 224><<<grid, gemm_threads(EPI_STORE_BF16), gemm_smem_bytes(224, MAX_STAGES, epi_warps(EPI_STORE_BF16)), st>>>(maps, ga, a, wt, gt, ws)));
+  TIMED(K_FC1_DX, launch_pdl(tc5_gemm<EPI_STORE_BF16, 224>, dim3(grid), gemm_threads(EPI_STORE_BF16), gemm_smem_bytes(224, MAX_STAGES, epi_warps(EPI_STORE_BF16)), st, maps, ga, a, wt, gt, ws));
   return 1;
 }
 

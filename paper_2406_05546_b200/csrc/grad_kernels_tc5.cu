@@ -608,6 +608,7 @@ int configure_tc5_kernels() {
       cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || g_sm_count <= 0) return -1;
   cudaError_t e = allow_smem((const void*)(tc5_gemm<EPI_FC1_FWD, 256>), gemm_smem_bytes(256, MAX_STAGES, epi_warps(EPI_FC1_FWD)));
   if (e == cudaSuccess) e = allow_smem((const void*)tc5_fwd_narrow, NR_SMEM);
+  if (e == cudaSuccess) e = allow_smem((const void*)tc5_gemm<EPI_FC1_FWD, 128>, gemm_smem_bytes(128, MAX_STAGES, epi_warps(EPI_FC1_FWD)));
   if (e == cudaSuccess) e = allow_smem((const void*)tc5_dx_split<DxSplit>, DxSplit::SMEM);
   if (e == cudaSuccess) e = allow_smem((const void*)(tc5_gemm<EPI_STORE_BF16, 224>), gemm_smem_bytes(224, MAX_STAGES, epi_warps(EPI_STORE_BF16)));
   if (e == cudaSuccess) e = allow_smem((const void*)(tc5_gemm<EPI_STORE, 224, true>), gemm_smem_bytes(224, MAX_STAGES, epi_warps(EPI_STORE)));
@@ -625,6 +626,11 @@ namespace {
 //   input gradient, 128 x 224      13    15    15    15    15     17     17     17
 //                   split over 4   11    13    14    15    21     23     31     38
 // The narrow tiles fit on the chip at once (two per SM) up to 18 x 64 rows.
+// Between that and 128 x 256, tiles of 128 x 128 while one round of them covers the chip (four column tiles, so up to 37 row
+// tiles): 25 - 27 against 29 - 32 us from 1,280 to 3,840 rows, 29 against 35 for 2,048 rows in nine weight groups.  With a
+// second round they lose (43 against 33 at 5,120 rows): a k-block then costs 0.4 instead of 0.47 us for half the columns, as
+// L2 has to deliver 32 instead of 48 KB per SM.
+bool fwd_is_half(int mt) { return mt * (HID / 128) <= g_sm_count; }
 bool fwd_is_narrow(int mt64) { return mt64 * (HID / NR_BN) <= 2 * g_sm_count; }
 bool dx_splits(int mt) { return mt <= 3; }
 
@@ -642,12 +648,18 @@ int launch_fc1_fwd_tc5(const GradStepArgs& a, const WorkerTable& wt, const Group
   GemmMaps maps;
   const uint64_t rows = (uint64_t)a.W * a.b;
   const int mt = group_tiles(gt, a.b, BM), mt_narrow = group_tiles(gt, a.b, NR_BM);
-  const bool narrow = fwd_is_narrow(mt_narrow);
+  const bool narrow = fwd_is_narrow(mt_narrow), half = !narrow && fwd_is_half(mt);
   if (!make_map(&maps.a, ws.p2, FLAT, rows, 1, FLAT, rows * FLAT, narrow ? NR_BM : BM)) return -1;
-  if (!make_map(&maps.b, ws.w1r, FLAT, HID, (uint64_t)gt.n_groups, FLAT, (uint64_t)HID * FLAT, narrow ? NR_BN : 256)) return -1;
+  if (!make_map(&maps.b, ws.w1r, FLAT, HID, (uint64_t)gt.n_groups, FLAT, (uint64_t)HID * FLAT, narrow ? NR_BN : (half ? 128 : 256))) return -1;
   if (narrow) {
     GemmArgs ga{FLAT, HID, HID, 0, ws.d, HID / NR_BN, 0};
     TIMED(K_FC1_FWD, launch_pdl_if(!after_join, tc5_fwd_narrow, dim3(HID / NR_BN, mt_narrow), 192, NR_SMEM, st, maps, ga, a, wt, gt, ws));
+    return 1;
+  }
+  if (half) {
+    GemmArgs ga{FLAT, HID, HID, 0, ws.d, HID / 128, (HID / 128) * mt};
+    const int grid = ga.n_tiles < g_sm_count ? ga.n_tiles : g_sm_count;
+    TIMED(K_FC1_FWD, launch_pdl_if(!after_join, tc5_gemm<EPI_FC1_FWD, 128>, dim3(grid), gemm_threads(EPI_FC1_FWD), gemm_smem_bytes(128, MAX_STAGES, epi_warps(EPI_FC1_FWD)), st, maps, ga, a, wt, gt, ws));
     return 1;
   }
   GemmArgs ga{FLAT, HID, HID, 0, ws.d, HID / 256, (HID / 256) * mt};

@@ -173,9 +173,9 @@ def test_output_layer_split_over_blocks(b):
                                      # 896 rows: the first convolution takes two samples per block; 6 rows: ranges of
                                      # the filter gradients shorter than four rows
                                      (8, 112, {}), (3, 2, {}),
-                                     # three and four 128-row tiles, eighteen and nineteen 64-row tiles: where the dense
+                                     # three and four, 37 and 38 128-row tiles, eighteen and nineteen 64-row tiles: where the dense
                                      # layer's products change form; ragged last tiles, two weight versions (tiles never cross them)
-                                     (3, 100, {}), (5, 101, {"lags": [1, 0, 0, 1, 0], "n_versions": 2}), (9, 128, {}), (9, 130, {})])
+                                     (3, 100, {}), (5, 101, {"lags": [1, 0, 0, 1, 0], "n_versions": 2}), (9, 128, {}), (9, 130, {}), (37, 128, {}), (38, 128, {})])
 def test_tensor_core_path(W, b, kw):
     _run_and_compare(W, b, precision=2, **kw)
 

@@ -44,6 +44,25 @@ constexpr int C1_OUT_BYTES = C1_SPS * (C1_PLANES_BYTES + P1_ELEMS);   // a step'
 constexpr int C1_STAGES = 2;
 constexpr int C1_SMEM = C1_STAGES * C1_IN_BYTES + 2 * C1_OUT_BYTES + 64 + 128;
 
+// The second convolution's filters of weight group g in the layouts its kernels read, 16 bytes per thread.  Blocks of this
+// kernel beyond its workers do it, so that the next kernel finds them without a launch or a fork of their own.
+constexpr int BANK2_UNITS = (BANK2_BYTES / 16 + C1_THREADS - 1) / C1_THREADS;     // blocks per weight group
+__device__ __forceinline__ void build_bank2(const float* __restrict__ theta, uint8_t* __restrict__ bank, int piece, const Bank2Taps& taps) {
+  if (piece >= BANK2_BYTES / 16) return;
+  float v[8];
+  if (piece < 2 * BANK2_FWD_ROWS) {      // forward: [octet of input channels][row = block, output channel]
+    const int oct = piece / BANK2_FWD_ROWS, row = piece - oct * BANK2_FWD_ROWS, oc = row & 31;
+    const uint32_t tap = taps.tap[row >> 5];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = tap == BANK2_ZERO_BLOCK ? 0.f : theta[OFF_C2W + (oc * 16 + oct * 8 + i) * 9 + tap];
+  } else {                               // input gradient: [filter row ky][octet of output channels][column = kx, input channel]
+    const int e = piece - 2 * BANK2_FWD_ROWS, ko = e / 48, col = e - ko * 48, ky = ko >> 2, o8 = ko & 3, kx = col >> 4, ic = col & 15;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = theta[OFF_C2W + ((o8 * 8 + i) * 16 + ic) * 9 + ky * 3 + kx];
+  }
+  reinterpret_cast<uint4*>(bank)[piece] = make_uint4(bf16_pair(v[0], v[1]), bf16_pair(v[2], v[3]), bf16_pair(v[4], v[5]), bf16_pair(v[6], v[7]));
+}
+
 // Work items of a step = (sample, pooled position, group of four channels): C1_SPS * 196 * 4 = 7 per thread.
 // Thread tid takes channel group tid & 3 and the pooled positions (tid >> 2) + 28 C1_SPS k of the step's samples
 // laid end to end; 28 = two rows of 14, so its column is fixed and its row advances by 2 C1_SPS.  Small blocks
@@ -51,8 +70,14 @@ constexpr int C1_SMEM = C1_STAGES * C1_IN_BYTES + 2 * C1_OUT_BYTES + 64 + 128;
 // multiply-add phases of all warps of a block, and with few large blocks the FMA pipe idles while all of them
 // pool and store.
 __global__ void __launch_bounds__(C1_THREADS, C1_BLOCKS_PER_SM) conv1_fwd_planes(const __grid_constant__ CUtensorMap xmap, GradStepArgs a,
-                                                                  WorkerTable wt, GroupTable gt, Workspace ws, int spb) {
+                                                                  WorkerTable wt, GroupTable gt, Workspace ws, int spb, const __grid_constant__ Bank2Taps taps) {
   extern __shared__ __align__(128) uint8_t sm[];
+  if (blockIdx.y >= a.W) {
+    const int u = (blockIdx.y - a.W) * gridDim.x + blockIdx.x, g = u / BANK2_UNITS;
+    pdl_enter();
+    if (g < gt.n_groups) build_bank2(gt.theta[g], ws.bank2 + (int64_t)g * BANK2_BYTES, (u - g * BANK2_UNITS) * C1_THREADS + threadIdx.x, taps);
+    return;
+  }
   const float* in = reinterpret_cast<const float*>(sm);
   uint8_t* outb = sm + C1_STAGES * C1_IN_BYTES;
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + C1_STAGES * C1_IN_BYTES + 2 * C1_OUT_BYTES);
@@ -183,7 +208,7 @@ int launch_conv1_fwd_planes(const GradStepArgs& a, const WorkerTable& wt, const 
   const int slots = C1_BLOCKS_PER_SM * g_sm_count, rows = a.W * a.b;
   const int spb = rows <= slots ? 1 : (rows <= 2 * slots ? 2 : C1_SPB);
   const int chunks = (a.b + spb - 1) / spb;
-  TIMED(K_CONV1_FWD, launch_pdl(conv1_fwd_planes, dim3(chunks, a.W), C1_THREADS, C1_SMEM, st, xmap, a, wt, gt, ws, spb));
+  TIMED(K_CONV1_FWD, launch_pdl(conv1_fwd_planes, dim3(chunks, a.W + (gt.n_groups * BANK2_UNITS + chunks - 1) / chunks), C1_THREADS, C1_SMEM, st, xmap, a, wt, gt, ws, spb, conv2_fwd_taps()));
   return 1;
 }
 

@@ -13,6 +13,10 @@
 // and pools without exchanging data.  For that the planes keep even and odd columns apart
 // (position (Y, X) at row Y*16 + (X&1)*8 + X/2): consecutive pooled columns are then consecutive rows.
 //
+// The filters arrive by one bulk copy as the operands they are (the first convolution's kernel lays them out once per weight
+// group): laid out by every CTA for itself they took 3 to 5 us before its first tile.  Forward 17 -> 11.6 us at 8 x 64 and 66 ->
+// 62 at 128 x 128, input gradient 14.8 -> 10.7 and 78 -> 72 (~6 us of event overhead included).
+//
 // The stages of each kernel (staging, MMA issue, epilogue) run in different warps and overlap through
 // mbarriers; every wait is bounded.
 #include "device_common.cuh"
@@ -33,7 +37,7 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {     // fp32 ac
 constexpr int RAW_SLOTS = 8;          // raw input slots of the input-gradient kernel
 constexpr int F_NBUF = 4;             // shared-memory tile buffers of the forward kernel (copies run four tiles ahead)
 struct Pipe {
-  uint64_t a_full[F_NBUF], a_empty[F_NBUF], acc_full[2], acc_empty[2], raw_full[RAW_SLOTS], raw_empty[RAW_SLOTS];
+  uint64_t w_full, a_full[F_NBUF], a_empty[F_NBUF], acc_full[2], acc_empty[2], raw_full[RAW_SLOTS], raw_empty[RAW_SLOTS];
   uint32_t tmem_base;
   volatile uint32_t abort_flag;
 };
@@ -51,6 +55,7 @@ __device__ __forceinline__ void pipe_init(Pipe* p, int a_full_arrivals, int acc_
     mbar_init(&p->raw_full[i], 1);
     mbar_init(&p->raw_empty[i], LOADERS / 64);
   }
+  mbar_init(&p->w_full, 1);
   p->abort_flag = 0;
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
@@ -76,23 +81,19 @@ constexpr int F_BUF_BYTES = 2 * F_PLANE_BYTES;             // two planes of eigh
 // 36 of N = 32: the tensor core spends about as long on an MMA of M = 128, K = 16 with N = 32 as with N = 96.  The
 // host lists the MMAs (FoldTable).
 constexpr int F_OPS = 16;
-constexpr int F_W_BLOCKS = 40;                             // 32-row blocks of the stacked weight operand (1,280 rows)
-constexpr int F_W_ROWS = 32 * F_W_BLOCKS;
-constexpr int F_W_BYTES = 2 * F_W_ROWS * 16;               // [channel octet][row][8 bf16]
+constexpr int F_W_ROWS = BANK2_FWD_ROWS;                   // rows of the stacked weight operand
+constexpr int F_W_BYTES = BANK2_FWD_BYTES;                 // [channel octet][row][8 bf16]
 constexpr int F_SMEM = F_NBUF * F_BUF_BYTES + F_W_BYTES + 32 * 4 + sizeof(Pipe) + 128;
 static_assert(2 * F_SMEM <= 227 * 1024, "two CTAs per SM");
 
-constexpr uint8_t F_ZERO_BLOCK = 255;
 struct FoldTable {
   int32_t a_off[F_OPS];        // start of the shifted plane, in 16-byte rows
   int32_t d_col[F_OPS];        // first accumulator column
   int32_t b_row[F_OPS];        // first row of the op's block of the weight operand
   uint32_t idesc[F_OPS];       // instruction descriptor (M = 128, the op's N)
-  uint8_t tap_of_block[F_W_BLOCKS];   // filter tap ky * 3 + kx whose 32 filters fill a 32-row block; F_ZERO_BLOCK: 32 rows of zeros
 };
 
-FoldTable make_fold_table() {
-  FoldTable t;
+void make_fold_table(FoldTable& t, Bank2Taps& taps) {
   int n_ops = 0, row = 0;
   // one op: the plane shifted by (sy, sx) against the filters of the column blocks [first, first + n_blocks); block c
   // belongs to window element c = 2 jy + jx, whose tap for this shift is (sy - jy, sx - jx), or is a block of zeros
@@ -102,7 +103,7 @@ FoldTable make_fold_table() {
     t.b_row[n_ops] = row;
     t.idesc[n_ops] = idesc_bf16(128, 32 * n_blocks);
     for (int c = first; c < first + n_blocks; ++c, row += 32)
-      t.tap_of_block[row / 32] = (used >> c) & 1u ? (uint8_t)((sy - (c >> 1)) * 3 + (sx - (c & 1))) : F_ZERO_BLOCK;
+      taps.tap[row / 32] = (used >> c) & 1u ? (uint8_t)((sy - (c >> 1)) * 3 + (sx - (c & 1))) : BANK2_ZERO_BLOCK;
     ++n_ops;
   };
   for (int pass = 0; pass < 2; ++pass)          // the op that covers all 128 columns comes first: it starts the sums
@@ -120,7 +121,17 @@ FoldTable make_fold_table() {
         const int first = 2 * jy0 + jx0, last = 2 * (jy0 + ny - 1) + (jx0 + nx - 1);
         add(sy, sx, first, last - first + 1, used);
       }
-  return t;      // n_ops == F_OPS and row == F_W_ROWS by construction
+  // n_ops == F_OPS and row == F_W_ROWS by construction
+}
+
+struct FoldTables {
+  FoldTable fold;
+  Bank2Taps taps;
+  FoldTables() { make_fold_table(fold, taps); }
+};
+const FoldTables& fold_tables() {
+  static const FoldTables t;
+  return t;
 }
 
 __global__ void __launch_bounds__(F_THREADS, 2) conv2_fwd_tc5(GradStepArgs a, GroupTable gt, Workspace ws, int range_len, const __grid_constant__ FoldTable fold) {
@@ -135,19 +146,7 @@ __global__ void __launch_bounds__(F_THREADS, 2) conv2_fwd_tc5(GradStepArgs a, Gr
   const float* theta = gt.theta[grp];
   const int n_tiles = (r_end - r_begin + 1) / 2;
 
-  // the filter bank comes in once with coalesced 16-byte loads (into the tile buffers, which are cleared afterwards) ...
-  float* wtmp = reinterpret_cast<float*>(smem);
-  for (int idx = tid; idx < 4608 / 4; idx += F_THREADS) reinterpret_cast<float4*>(wtmp)[idx] = reinterpret_cast<const float4*>(theta + OFF_C2W)[idx];
   if (tid < 32) bias[tid] = theta[OFF_C2B + tid];
-  __syncthreads();
-  // ... and is laid out as the stacked weight operand: block rb holds the 32 filters of tap fold.tap_of_block[rb], one
-  // row per output channel
-  for (int idx = tid; idx < F_W_BLOCKS * 512; idx += F_THREADS) {
-    const int rb = idx >> 9, oc = (idx >> 4) & 31, ic = idx & 15;
-    const uint32_t tap = fold.tap_of_block[rb];
-    Wk[((ic >> 3) * F_W_ROWS + rb * 32 + oc) * 8 + (ic & 7)] = tap == F_ZERO_BLOCK ? (uint16_t)0 : bf16_bits(wtmp[(oc * 16 + ic) * 9 + tap]);
-  }
-  __syncthreads();
   // rows never written by a copy (the overrun of the padding rows, a missing second sample) only feed
   // results that are dropped; they are cleared once so that those results stay finite
   for (int idx = tid; idx < F_NBUF * F_BUF_BYTES / 16; idx += F_THREADS) reinterpret_cast<float4*>(smem)[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -156,7 +155,7 @@ __global__ void __launch_bounds__(F_THREADS, 2) conv2_fwd_tc5(GradStepArgs a, Gr
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&pipe->tmem_base)), "r"(256) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  fence_proxy_async_smem();      // the filter bank and the cleared rows are read by the tensor core
+  fence_proxy_async_smem();      // the cleared rows are read by the tensor core
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -170,7 +169,8 @@ __global__ void __launch_bounds__(F_THREADS, 2) conv2_fwd_tc5(GradStepArgs a, Gr
       // the accumulator's barrier are constants of each copy of the body, and the backward branch comes once per four tiles)
       static_assert(F_NBUF == 4, "the accumulator parities below assume four tile buffers");
       const uint32_t a_lo0 = plain_desc_lo(smem_u32(smem), F_PLANE_BYTES);
-      bool go_on = true;
+      bool go_on = mbar_wait(&pipe->w_full, 0);
+      if (!go_on) pipe->abort_flag = 1;
       uint32_t parity = 0;
       for (int t = 0; go_on && t < n_tiles; parity ^= 1) {
 #pragma unroll
@@ -196,6 +196,8 @@ __global__ void __launch_bounds__(F_THREADS, 2) conv2_fwd_tc5(GradStepArgs a, Gr
     }
   } else if (warp == 1) {
     if (lane == 0) {
+      mbar_expect_tx(&pipe->w_full, F_W_BYTES);
+      bulk_load(Wk, ws.bank2 + (int64_t)grp * BANK2_BYTES, F_W_BYTES, &pipe->w_full);
       for (int t = 0; t < n_tiles; ++t) {
         const int buf = t % F_NBUF;
         if (t >= F_NBUF && !mbar_wait(&pipe->a_empty[buf], ((t / F_NBUF) - 1) & 1)) { pipe->abort_flag = 1; break; }
@@ -273,7 +275,7 @@ __global__ void __launch_bounds__(F_THREADS, 2) conv2_fwd_tc5(GradStepArgs a, Gr
 constexpr int X_PLANE_ROWS = 256 + 51;                     // 34 rows of tap overrun (+ 17: a plane pitch of 3 rows mod 8 spreads the
 constexpr int X_PLANE_BYTES = X_PLANE_ROWS * 16;           // staging stores of the four planes over all shared-memory banks)
 constexpr int X_BUF_BYTES = 4 * X_PLANE_BYTES;             // four planes of eight output channels
-constexpr int X_W_BYTES = 12 * 48 * 16;                    // [filter row ky][k chunk oc/8][column = kx*16 + ic][8 bf16]
+constexpr int X_W_BYTES = BANK2_DX_BYTES;                  // [filter row ky][k chunk oc/8][column = kx*16 + ic][8 bf16]
 constexpr int X_RAW_BYTES = FLAT * 2 + FLAT;                // one sample's pooled gradients (BF16) and pooling decisions (bytes)
 constexpr int X_RAW_SLOTS = RAW_SLOTS;
 constexpr int X_SMEM = 2 * X_BUF_BYTES + X_W_BYTES + X_RAW_SLOTS * X_RAW_BYTES + sizeof(Pipe) + 128;
@@ -287,13 +289,8 @@ __global__ void __launch_bounds__(THREADS, 2) conv2_dx_tc5(GradStepArgs a, Group
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int grp, r_begin, r_end;
   if (!locate_row_range(gt, a.b, range_len, blockIdx.x, grp, r_begin, r_end)) return;
-  const float* theta = gt.theta[grp];
   const int n_tiles = r_end - r_begin;
 
-  for (int idx = tid; idx < 4608; idx += THREADS) {
-    int oc = idx / 144, rem = idx - oc * 144, ic = rem / 9, tap = rem - ic * 9;
-    Wk[(((tap / 3) * 4 + (oc >> 3)) * 48 + (tap % 3) * 16 + ic) * 8 + (oc & 7)] = bf16_bits(theta[OFF_C2W + idx]);
-  }
   for (int idx = tid; idx < 2 * X_BUF_BYTES / 16; idx += THREADS) reinterpret_cast<float4*>(smem)[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
   if (tid == 0) pipe_init(pipe, LOADERS / 64, 4);
   if (warp == 0) {
@@ -314,7 +311,8 @@ __global__ void __launch_bounds__(THREADS, 2) conv2_dx_tc5(GradStepArgs a, Group
       // one pass of the outer loop takes the two plane buffers in turn (unrolled: the buffer's addresses are constants
       // of its copy of the body, and the backward branch comes once per two tiles)
       const uint32_t a_lo0 = plain_desc_lo(smem_u32(smem), X_PLANE_BYTES);
-      bool go_on = true;
+      bool go_on = mbar_wait(&pipe->w_full, 0);
+      if (!go_on) pipe->abort_flag = 1;
       uint32_t parity = 0;
       for (int t = 0; go_on && t < n_tiles; parity ^= 1) {
 #pragma unroll
@@ -390,7 +388,9 @@ __global__ void __launch_bounds__(THREADS, 2) conv2_dx_tc5(GradStepArgs a, Group
   } else if (warp == THREADS / 32 - 1) {
     // ---------------- copies: one thread brings every sample's pooled gradients (BF16) and decisions into the raw slots
     // in turn, up to eight samples ahead; a slot is refilled once the four warps that staged its last sample have read it
-    if (lane == 0)
+    if (lane == 0) {
+      mbar_expect_tx(&pipe->w_full, X_W_BYTES);
+      bulk_load(Wk, ws.bank2 + (int64_t)grp * BANK2_BYTES + BANK2_FWD_BYTES, X_W_BYTES, &pipe->w_full);
       for (int t = 0; t < n_tiles; ++t) {
         const int slot_i = t & (X_RAW_SLOTS - 1);
         if (t >= X_RAW_SLOTS && (!mbar_wait(&pipe->raw_empty[slot_i], ((t >> 3) - 1) & 1) || pipe->abort_flag)) { pipe->abort_flag = 1; break; }
@@ -400,6 +400,7 @@ __global__ void __launch_bounds__(THREADS, 2) conv2_dx_tc5(GradStepArgs a, Group
         bulk_load(slot, ws.dp2 + row * FLAT, FLAT * 2, &pipe->raw_full[slot_i]);      // BF16 in the first half of the row
         bulk_load(slot + FLAT * 2, ws.code2 + row * FLAT, FLAT, &pipe->raw_full[slot_i]);
       }
+    }
   } else {
     const int quarter = warp & 3;
     for (int t = 0; t < n_tiles; ++t) {
@@ -460,9 +461,11 @@ int configure_conv5_kernels() {
   return e == cudaSuccess ? 0 : -1;
 }
 
+const Bank2Taps& conv2_fwd_taps() { return fold_tables().taps; }
+
 void launch_conv2_fwd_tc5(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                           cudaStream_t st, Profiler* prof) {
-  static const FoldTable fold = make_fold_table();
+  const FoldTable& fold = fold_tables().fold;
   int len;
   const int n = plan_row_ranges(gt, a.b, 2 * g_sm_count, 2, &len);      // two CTAs per SM, tiles of two samples
   TIMED(K_CONV2_FWD, launch_pdl(conv2_fwd_tc5, dim3(n), F_THREADS, F_SMEM, st, a, gt, ws, len, fold));

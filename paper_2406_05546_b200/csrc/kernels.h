@@ -37,6 +37,13 @@ __host__ __device__ inline int fc2_split(int W, int b) {
   return s < most ? s : most;
 }
 
+// The second convolution's filters as tensor-core operands, per weight group: BANK2_BLOCKS blocks of 32 rows of the forward
+// kernel (two planes of eight input channels), and the input gradient's 12 x 48 rows; a row is eight BF16 values.
+constexpr int BANK2_BLOCKS = 40, BANK2_FWD_ROWS = 32 * BANK2_BLOCKS, BANK2_FWD_BYTES = 2 * BANK2_FWD_ROWS * 16;
+constexpr int BANK2_DX_ROWS = 12 * 48, BANK2_DX_BYTES = BANK2_DX_ROWS * 16, BANK2_BYTES = BANK2_FWD_BYTES + BANK2_DX_BYTES;
+constexpr uint8_t BANK2_ZERO_BLOCK = 255;
+struct Bank2Taps { uint8_t tap[BANK2_BLOCKS]; };      // filter tap ky * 3 + kx of a block's 32 filters; BANK2_ZERO_BLOCK: zeros
+
 constexpr uint32_t STATUS_BAD_LABEL = 1u;
 constexpr uint32_t STATUS_WAIT_TIMEOUT = 2u;   // a bounded barrier wait in a tensor-core kernel gave up
 
@@ -118,6 +125,7 @@ struct Workspace {
   float* partf;    // [W][fc2_split][FC_PART] per-block partial output-layer gradients and loss sums
   float* w1r;      // [groups][512][1568] TF32-rounded fc1 weights of each weight group of the call
   float* w1tr;     // [groups][1568][512] and their transpose
+  uint8_t* bank2;  // [groups][BANK2_BYTES] conv2's filters as its kernels' tensor-core operands (forward, then input gradient)
   uint32_t* status;
 };
 
@@ -183,6 +191,7 @@ int launch_conv2_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const Work
                         int* seg_len);
 int launch_conv1_fwd_planes(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                             cudaStream_t st, Profiler* prof);
+const Bank2Taps& conv2_fwd_taps();
 void launch_conv2_fwd_tc5(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                           cudaStream_t st, Profiler* prof);
 void launch_conv2_dx_tc5(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,

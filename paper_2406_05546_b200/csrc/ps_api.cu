@@ -159,10 +159,12 @@ void layout(ps_ctx* x, const ps_config& c, void* arena, void* pinned, uint64_t* 
   ws.partf = a.take<float>((uint64_t)std::min(c.max_workers * psk::FC2_MAX_SPLIT, std::max<int>(c.max_workers, psk::FC2_BLOCKS)) * psk::FC_PART * 4);
   ws.status = a.take<uint32_t>(ALIGN);
   ws.w1r = ws.w1tr = nullptr;
+  ws.bank2 = nullptr;
   if (c.precision != PS_FP32) {
     const uint64_t groups = std::min<uint64_t>(psk::MAX_GROUPS, std::min<uint64_t>(c.max_workers, c.ring_depth));
     ws.w1r = a.take<float>(groups * psk::HID * psk::FLAT * 4);
     ws.w1tr = a.take<float>(groups * psk::HID * psk::FLAT * 4);
+    ws.bank2 = a.take<uint8_t>(groups * psk::BANK2_BYTES);
   }
   float* x_stage[2]; int32_t* y_stage[2]; float* loss_stage[2]; int32_t* argmax_stage[2];
   for (int k = 0; k < 2; ++k) {

@@ -298,9 +298,10 @@ int configure_dw5_kernels() {
 }
 
 // Returns the number of partial-sum slots reserved per worker (the stride of part2) and, in *seg_len, the length
-// of a CTA's range of rows: worker s owns one partial sum per range that meets its rows.
+// of a CTA's range of rows: worker s owns one partial sum per range that meets its rows.  in_line: the stream holds the kernel
+// before it in the chain, not a wait for it.
 int launch_conv2_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const Workspace& ws, cudaStream_t st, Profiler* prof,
-                        int* seg_len) {
+                        int* seg_len, bool in_line) {
   const int total = a.W * a.b;
   int grid = total / MIN_RANGE;           // a range is at least four rows long (bounds the partial sums per worker)
   if (grid > g_sm_count) grid = g_sm_count;
@@ -308,7 +309,7 @@ int launch_conv2_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const Work
   const int len = (total + grid - 1) / grid;
   grid = (total + len - 1) / len;
   const int slots = (a.b - 1) / len + 2;
-  TIMED(K_CONV2_DW, (conv2_dw_tc5<<<grid, W5_THREADS, W5_SMEM, st>>>(a, wt, ws, len, slots)));
+  TIMED(K_CONV2_DW, launch_pdl_if(in_line, conv2_dw_tc5, dim3(grid), W5_THREADS, W5_SMEM, st, a, wt, ws, len, slots));
   *seg_len = len;
   return slots;
 }

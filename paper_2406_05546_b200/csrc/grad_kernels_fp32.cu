@@ -386,7 +386,12 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     for (int g = 0; g < sum->n_super; ++g) wt_dw.grad[g] = sum->super_part + (int64_t)g * P_PAD;
   }
   if (tc) {
-    cudaStream_t s1 = side.s1 ? side.s1 : st, s2 = side.s2 ? side.s2 : st;
+    // The second convolution's filter gradient has a stream of its own only while its blocks are few but its chain of samples
+    // counts; from 512 rows on it and the input gradient fill the chip one after the other and the fork and join only cost, at
+    // up to 64 rows the host's event calls cost more than the overlap gives.  us per tick, side stream / in line: 2 x 8 60 / 56,
+    // 4 x 32 61 / 62, 5 x 37 80 / 82, 8 x 64 83.2 / 82.3, 16 x 64 107 / 105, 32 x 64 171 / 168, 64 x 32 241 / 239, 128 x 128 687 / 681.
+    const bool own_stream = side.s2 && a.W * a.b > 64 && a.W * a.b < 512;
+    cudaStream_t s1 = side.s1 ? side.s1 : st, s2 = own_stream ? side.s2 : st;
     // the copies of W1 are not needed before the dense layer: they are made next to the convolutions
     if (!a.skip_prep_w1) {
       if (side.s1) { cudaEventRecord(side.fork1, st); cudaStreamWaitEvent(s1, side.fork1, 0); }
@@ -409,15 +414,15 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     n = launch_fc1_dx_tc5(a, wt, gt, ws, st, prof);
     if (n < 0) return -1;
     launches += n;
-    if (side.s2) { cudaEventRecord(side.fork2, st); cudaStreamWaitEvent(s2, side.fork2, 0); }
-    n_chunks2 = launch_conv2_dw_tc5(a, wt, ws, s2, prof, &seg_len);
-    if (side.s2) cudaEventRecord(side.join2, s2);
+    if (own_stream) { cudaEventRecord(side.fork2, st); cudaStreamWaitEvent(s2, side.fork2, 0); }
+    n_chunks2 = launch_conv2_dw_tc5(a, wt, ws, s2, prof, &seg_len, !own_stream);
+    if (own_stream) cudaEventRecord(side.join2, s2);
     launch_conv2_dx_tc5(a, wt, gt, ws, st, prof);
     int seg_len1 = 0;
     const int n_chunks1t = launch_conv1_dw_tc5(a, wt, ws, st, prof, &seg_len1);
     if (n_chunks1t < 0) return -1;
     if (side.s1) cudaStreamWaitEvent(st, side.join1, 0);
-    if (side.s2) cudaStreamWaitEvent(st, side.join2, 0);
+    if (own_stream) cudaStreamWaitEvent(st, side.join2, 0);
     if (sum) TIMED(K_CONV_GRAD_REDUCE, (fused_finish<<<dim3(FUSED_W1_BLOCKS + FUSED_SMALL_BLOCKS), 256, 0, st>>>(a, wt, ws, sum->super_part, sum->n_super, sum->grad_sum, n_chunks1t, seg_len1, n_chunks2, seg_len)));
     else TIMED(K_CONV_GRAD_REDUCE, (conv_grad_reduce<<<dim3(a.W, (RED_OUTPUTS + red_per_block - 1) / red_per_block), 256, 0, st>>>(a, wt, ws, red_per_block, n_chunks1t, seg_len1, n_chunks2, seg_len)));
     launches += 4;

@@ -188,7 +188,7 @@ void launch_output_layer(bool eval, const GradStepArgs& a, const WorkerTable& wt
 int launch_conv1_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const Workspace& ws, cudaStream_t st, Profiler* prof,
                         int* seg_len);
 int launch_conv2_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const Workspace& ws, cudaStream_t st, Profiler* prof,
-                        int* seg_len);
+                        int* seg_len, bool in_line);
 int launch_conv1_fwd_planes(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                             cudaStream_t st, Profiler* prof);
 const Bank2Taps& conv2_fwd_taps();

@@ -193,6 +193,24 @@ def test_tensor_core_path_repeatable_bit_for_bit():
     assert (a == b).all()
 
 
+@pytest.mark.parametrize("W,b", [(2, 32), (5, 13), (7, 73), (8, 64)])
+def test_filter_gradient_in_line_and_on_its_own_stream(W, b):
+    """64, 65, 511 and 512 rows: the choice changes where the kernel runs, never a bit of what it gives.  The profiled
+    call runs the same kernels one at a time in one stream."""
+    torch, ps, srv, _ = _setup(W, b, precision=2)
+    rng = np.random.default_rng(W)
+    x = torch.from_numpy(rng.random((W, b, 28, 28), dtype=np.float32)).cuda()
+    y = torch.from_numpy(rng.integers(0, 10, (W, b), dtype=np.int32)).cuda()
+    snaps = [srv.ps_pull_snapshot(w) for w in range(W)]
+    grads = torch.zeros((4, W, ps.P_PAD), device="cuda")
+    for k in range(4):
+        srv.ps_profile(1 if k == 3 else 0)
+        srv.workers_grad_step(snaps, range(W), x, y, SEED, 1, grads_dev=grads[k])
+    srv.ps_profile(0)
+    assert (grads[0] != 0).any() and all(torch.equal(grads[0], g) for g in grads[1:])
+    srv.close()
+
+
 @pytest.mark.parametrize("W,b", [(2, 8), (3, 40)])
 def test_tensor_core_path_against_the_plain_definition(W, b):
     """The tensor-core path against the oracle with EVERY decision taken on exact values (precision 0): what the

@@ -1,7 +1,9 @@
 /* Argument marshalling of the calls a training loop makes every tick, as a CPython extension: snapshots in and out of their
  * ctypes structures, numpy arrays by the buffer protocol, the results as Python objects.  Through ctypes alone these calls
  * cost the host more than the library's own work (measured per call, ctypes -> here: pull 0.9 -> 0.3 us, reserve 3.6 -> 0.9,
- * enqueue 9 -> 2, apply 5 -> 1.5, the grad step's arguments 20 -> 8).  No step of the method happens here. */
+ * enqueue 9 -> 2, apply 5 -> 1.5, the grad step's arguments 20 -> 8).  Arrays that already have their type and layout are read
+ * where they lie, and a list of versions is read element by element: only the rest goes through numpy.  No step of the method
+ * happens here. */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>
@@ -17,9 +19,10 @@ static int32_t (*f_summed)(ps_ctx*, int32_t, int32_t, const ps_snapshot*, const 
 static int32_t (*f_eval)(ps_ctx*, int32_t, int32_t, const ps_snapshot*, const float*, const int32_t*, float*, int32_t*, int32_t*);
 static int32_t (*f_enqueue)(ps_ctx*, int32_t, const int64_t*, const float*, const int32_t*, const uint64_t*, uint64_t);
 static int32_t (*f_apply)(ps_ctx*, ps_mode, float, float, const int32_t*, ps_apply_result*);
+static int32_t (*f_apply_stale)(ps_ctx*, ps_mode, float, float, const int32_t*, float, float, ps_apply_result*);
 static int32_t (*f_apply_summed)(ps_ctx*, const float*, int32_t, float, float, ps_apply_result*);
 static const char* (*f_error)(ps_ctx*);
-static PyObject *snapshot_type, *error_type;
+static PyObject *snapshot_type, *error_type, *as_array;   /* as_array(object, kind): numpy's conversion to a contiguous array */
 static PyObject *k_applied, *k_version, *k_checkpointed, *k_replicated;
 
 static PyObject* raise(int32_t rc) {
@@ -60,13 +63,33 @@ static int i32(PyObject* o, int32_t* v) {
   return 0;
 }
 
-/* A contiguous array of n items of the given size, or None; the caller has brought it to its type. */
-static int array(PyObject* o, Py_buffer* b, Py_ssize_t n, Py_ssize_t item) {
+/* The types of the library's integer arrays. */
+enum { I32, I64, U64 };
+
+/* A contiguous one-dimensional array of the given type, or None.  The buffer keeps whatever holds the items alive. */
+static int array(PyObject* o, Py_buffer* b, int kind) {
   b->obj = NULL;
   b->buf = NULL;
+  b->len = 0;
   if (o == Py_None) return 0;
-  if (PyObject_GetBuffer(o, b, PyBUF_SIMPLE)) return -1;
-  if (b->len < n * item) { PyBuffer_Release(b); PyErr_SetString(PyExc_ValueError, "array is too short"); return -1; }
+  if (PyObject_CheckBuffer(o)) {
+    if (PyObject_GetBuffer(o, b, PyBUF_C_CONTIGUOUS | PyBUF_FORMAT) == 0) {
+      const char f = b->ndim == 1 && b->format && b->format[0] && !b->format[1] ? b->format[0] : 0;
+      if (b->itemsize == (kind == I32 ? 4 : 8) && (kind == U64 ? f == 'L' || f == 'Q' : f == 'i' || f == 'l' || f == 'q')) return 0;
+      PyBuffer_Release(b);
+    } else PyErr_Clear();
+  }
+  PyObject* c = PyObject_CallFunction(as_array, "Oi", o, kind);
+  if (!c) { b->obj = NULL; return -1; }
+  const int rc = PyObject_GetBuffer(c, b, PyBUF_C_CONTIGUOUS);
+  Py_DECREF(c);
+  return rc;
+}
+static void done(Py_buffer* b) { if (b->obj) PyBuffer_Release(b); }
+
+static int long_enough(const Py_buffer* b, Py_ssize_t n, Py_ssize_t item) {
+  if (!b->obj || b->len >= n * item) return 1;
+  PyErr_SetString(PyExc_ValueError, "array is too short");
   return 0;
 }
 
@@ -104,11 +127,11 @@ static PyObject* result(const ps_apply_result* r) {
 #define WANT(n) if (nargs != (n)) { PyErr_SetString(PyExc_TypeError, "wrong number of arguments"); return NULL; }
 
 static PyObject* bind(PyObject* m, PyObject* const* a, Py_ssize_t nargs) {
-  WANT(3)
+  WANT(4)
   static const struct { const char* name; void** f; } table[] = {
       {"ps_pull_snapshot", (void**)&f_pull}, {"ps_queue_reserve", (void**)&f_reserve}, {"workers_grad_step", (void**)&f_grad},
       {"workers_grad_step_summed", (void**)&f_summed}, {"workers_eval", (void**)&f_eval}, {"ps_enqueue", (void**)&f_enqueue},
-      {"ps_apply", (void**)&f_apply}, {"ps_apply_summed", (void**)&f_apply_summed}, {"ps_last_error", (void**)&f_error}};
+      {"ps_apply", (void**)&f_apply}, {"ps_apply_stale", (void**)&f_apply_stale}, {"ps_apply_summed", (void**)&f_apply_summed}, {"ps_last_error", (void**)&f_error}};
   for (size_t i = 0; i < sizeof(table) / sizeof(table[0]); ++i) {
     PyObject* addr = PyDict_GetItemString(a[0], table[i].name);
     if (!addr) { PyErr_SetString(PyExc_KeyError, table[i].name); return NULL; }
@@ -119,6 +142,8 @@ static PyObject* bind(PyObject* m, PyObject* const* a, Py_ssize_t nargs) {
   Py_XSETREF(snapshot_type, a[1]);
   Py_INCREF(a[2]);
   Py_XSETREF(error_type, a[2]);
+  Py_INCREF(a[3]);
+  Py_XSETREF(as_array, a[3]);
   Py_RETURN_NONE;
 }
 
@@ -163,13 +188,16 @@ static PyObject* grad_step(PyObject* m, PyObject* const* a, Py_ssize_t nargs) {
     return NULL;
   if (W > PS_MAX_WORKERS) W = PS_MAX_WORKERS + 1;          /* the library refuses it */
   else if (snapshots(a[3], W, snaps)) return NULL;
-  if (array(a[4], &ids, W, 4)) return NULL;
-  if (array(a[9], &slots, W, 8)) { if (ids.obj) PyBuffer_Release(&ids); return NULL; }
+  if (array(a[4], &ids, I32)) return NULL;
+  if (array(a[9], &slots, I64)) { done(&ids); return NULL; }
+  if (!ids.obj || ids.ndim != 1 || ids.len != (Py_ssize_t)W * 4) PyErr_SetString(PyExc_AssertionError, "one worker id per worker is wanted");
+  else long_enough(&slots, W, 8);
+  if (PyErr_Occurred()) { done(&ids); done(&slots); return NULL; }
   int32_t rc;
   CALL(f_grad((ps_ctx*)ctx, W, b, snaps, (const int32_t*)ids.buf, (const float*)x, (const int32_t*)y, seed, step,
                             (const int64_t*)slots.buf, (float*)grads, (float*)loss, (int32_t*)argmax))
-  if (ids.obj) PyBuffer_Release(&ids);
-  if (slots.obj) PyBuffer_Release(&slots);
+  done(&ids);
+  done(&slots);
   if (rc) return raise(rc);
   Py_RETURN_NONE;
 }
@@ -187,11 +215,12 @@ static PyObject* grad_step_summed(PyObject* m, PyObject* const* a, Py_ssize_t na
     return NULL;
   if (W > PS_MAX_WORKERS) W = PS_MAX_WORKERS + 1;
   else if (snapshots(a[3], W, snaps)) return NULL;
-  if (array(a[4], &ids, W, 4)) return NULL;
+  if (array(a[4], &ids, I32)) return NULL;
+  if (!long_enough(&ids, W, 4)) { done(&ids); return NULL; }
   int32_t rc;
   CALL(f_summed((ps_ctx*)ctx, W, b, snaps, (const int32_t*)ids.buf, (const float*)x, (const int32_t*)y, seed, step,
                               (float*)sum, (float*)loss, (int32_t*)argmax))
-  if (ids.obj) PyBuffer_Release(&ids);
+  done(&ids);
   if (rc) return raise(rc);
   Py_RETURN_NONE;
 }
@@ -213,23 +242,42 @@ static PyObject* eval(PyObject* m, PyObject* const* a, Py_ssize_t nargs) {
   Py_RETURN_NONE;
 }
 
-/* (ctx, n, slot_ids int64[n] | None, grads | None, worker_ids int32[n], base_versions uint64[n], step) */
+/* A list of versions, read without an array in between; NULL without an error if it is anything else. */
+static uint64_t* version_list(PyObject* o, Py_ssize_t n) {
+  if (!PyList_CheckExact(o) || PyList_GET_SIZE(o) < n) return NULL;
+  uint64_t* v = PyMem_Malloc((size_t)(n ? n : 1) * sizeof(uint64_t));
+  for (Py_ssize_t i = 0; v && i < n; ++i) {
+    PyObject* e = PyList_GET_ITEM(o, i);
+    v[i] = PyLong_CheckExact(e) ? PyLong_AsUnsignedLongLong(e) : (uint64_t)-1;
+    if (v[i] == (uint64_t)-1) { PyErr_Clear(); PyMem_Free(v); return NULL; }
+  }
+  return v;
+}
+
+/* (ctx, slot_ids int64[n] | None, grads | None, worker_ids int32[n], base_versions uint64[n], step) */
 static PyObject* enqueue(PyObject* m, PyObject* const* a, Py_ssize_t nargs) {
-  WANT(7)
+  WANT(6)
   void *ctx, *grads;
-  int32_t n;
   uint64_t step;
-  Py_buffer slots, ids, base;
-  if (as_ptr(a[0], &ctx) || i32(a[1], &n) || as_ptr(a[3], &grads) || as_u64(a[6], &step) || array(a[2], &slots, n, 8)) return NULL;
-  if (array(a[4], &ids, n, 4)) { if (slots.obj) PyBuffer_Release(&slots); return NULL; }
-  if (array(a[5], &base, n, 8)) { if (slots.obj) PyBuffer_Release(&slots); if (ids.obj) PyBuffer_Release(&ids); return NULL; }
+  Py_buffer slots = {0}, ids = {0}, base = {0};
+  uint64_t* list = NULL;
+  PyObject* ret = NULL;
+  if (as_ptr(a[0], &ctx) || as_ptr(a[2], &grads) || as_u64(a[5], &step)) return NULL;
+  if (a[3] == Py_None || a[4] == Py_None) { PyErr_SetString(PyExc_TypeError, "worker_ids and base_versions are wanted"); return NULL; }
+  if (array(a[3], &ids, I32) || array(a[1], &slots, I64)) goto end;
+  const Py_ssize_t n = ids.shape[0];
+  if (!(list = version_list(a[4], n)) && array(a[4], &base, U64)) goto end;
+  if (!long_enough(&slots, n, 8) || !long_enough(&base, n, 8)) goto end;
   int32_t rc;
-  CALL(f_enqueue((ps_ctx*)ctx, n, (const int64_t*)slots.buf, (const float*)grads, (const int32_t*)ids.buf, (const uint64_t*)base.buf, step))
-  if (slots.obj) PyBuffer_Release(&slots);
-  if (ids.obj) PyBuffer_Release(&ids);
-  if (base.obj) PyBuffer_Release(&base);
-  if (rc) return raise(rc);
-  Py_RETURN_NONE;
+  CALL(f_enqueue((ps_ctx*)ctx, (int32_t)n, (const int64_t*)slots.buf, (const float*)grads, (const int32_t*)ids.buf,
+                 list ? list : (const uint64_t*)base.buf, step))
+  ret = rc ? raise(rc) : Py_NewRef(Py_None);
+end:
+  PyMem_Free(list);
+  done(&slots);
+  done(&ids);
+  done(&base);
+  return ret;
 }
 
 /* (ctx, mode, lr, scale, order int32[K] | None) -> dict */
@@ -240,10 +288,27 @@ static PyObject* apply(PyObject* m, PyObject* const* a, Py_ssize_t nargs) {
   float lr, scale;
   Py_buffer order;
   ps_apply_result r = {0, 0, 0, 0};
-  if (as_ptr(a[0], &ctx) || i32(a[1], &mode) || as_float(a[2], &lr) || as_float(a[3], &scale) || array(a[4], &order, 0, 4)) return NULL;
+  if (as_ptr(a[0], &ctx) || i32(a[1], &mode) || as_float(a[2], &lr) || as_float(a[3], &scale) || array(a[4], &order, I32)) return NULL;
   int32_t rc;
   CALL(f_apply((ps_ctx*)ctx, (ps_mode)mode, lr, scale, (const int32_t*)order.buf, &r))
-  if (order.obj) PyBuffer_Release(&order);
+  done(&order);
+  return rc ? raise(rc) : result(&r);
+}
+
+/* (ctx, mode, lr, scale, order int32[K] | None, clip_norm, staleness_alpha) -> dict */
+static PyObject* apply_stale(PyObject* m, PyObject* const* a, Py_ssize_t nargs) {
+  WANT(7)
+  void* ctx;
+  int32_t mode;
+  float lr, scale, clip, alpha;
+  Py_buffer order;
+  ps_apply_result r = {0, 0, 0, 0};
+  if (as_ptr(a[0], &ctx) || i32(a[1], &mode) || as_float(a[2], &lr) || as_float(a[3], &scale) || as_float(a[5], &clip) ||
+      as_float(a[6], &alpha) || array(a[4], &order, I32))
+    return NULL;
+  int32_t rc;
+  CALL(f_apply_stale((ps_ctx*)ctx, (ps_mode)mode, lr, scale, (const int32_t*)order.buf, clip, alpha, &r))
+  done(&order);
   return rc ? raise(rc) : result(&r);
 }
 
@@ -262,7 +327,7 @@ static PyObject* apply_summed(PyObject* m, PyObject* const* a, Py_ssize_t nargs)
 
 #define FAST(f) {#f, (PyCFunction)(void (*)(void))f, METH_FASTCALL, NULL}
 static PyMethodDef methods[] = {FAST(bind), FAST(pull), FAST(reserve), FAST(grad_step), FAST(grad_step_summed), FAST(eval),
-                                FAST(enqueue), FAST(apply), FAST(apply_summed), {NULL, NULL, 0, NULL}};
+                                FAST(enqueue), FAST(apply), FAST(apply_stale), FAST(apply_summed), {NULL, NULL, 0, NULL}};
 static struct PyModuleDef def = {PyModuleDef_HEAD_INIT, "_marshal", NULL, -1, methods, NULL, NULL, NULL, NULL};
 
 PyMODINIT_FUNC PyInit__marshal(void) {

@@ -115,7 +115,8 @@ def load(path=None):
         from . import _marshal as m
         m.bind({n: C.cast(getattr(L, n), C.c_void_p).value for n in
                 ("ps_pull_snapshot", "ps_queue_reserve", "workers_grad_step", "workers_grad_step_summed", "workers_eval",
-                 "ps_enqueue", "ps_apply", "ps_apply_summed", "ps_last_error")}, Snapshot, PSError)
+                 "ps_enqueue", "ps_apply", "ps_apply_stale", "ps_apply_summed", "ps_last_error")}, Snapshot, PSError,
+               lambda o, kind: np.ascontiguousarray(o, dtype=(np.int32, np.int64, np.uint64)[kind]))
         _lib, _marshal = L, m
     return L
 
@@ -212,16 +213,13 @@ class ParameterServer:
         W, b = int(y_dev.shape[0]), int(y_dev.shape[1])
         assert x_dev.is_cuda and x_dev.dtype == torch.float32 and x_dev.is_contiguous() and x_dev.numel() == W * b * 784
         assert y_dev.is_cuda and y_dev.dtype == torch.int32 and y_dev.is_contiguous()
-        wid = np.ascontiguousarray(worker_ids, dtype=np.int32)
-        assert wid.shape == (W,)
         if loss_dev is None:
             loss_dev = torch.empty(W, dtype=torch.float32, device="cuda")
         if argmax_dev is None:
             argmax_dev = torch.empty((W, b), dtype=torch.int32, device="cuda")
-        sid = None if slot_ids is None else np.ascontiguousarray(slot_ids, dtype=np.int64)
         if grads_dev is not None:
             assert grads_dev.is_cuda and grads_dev.dtype == torch.float32 and grads_dev.shape == (W, P_PAD) and grads_dev.is_contiguous()
-        _marshal.grad_step(self._addr, W, b, snaps, wid, x_dev.data_ptr(), y_dev.data_ptr(), seed, step, sid,
+        _marshal.grad_step(self._addr, W, b, snaps, worker_ids, x_dev.data_ptr(), y_dev.data_ptr(), seed, step, slot_ids,
                            grads_dev.data_ptr() if grads_dev is not None else None, loss_dev.data_ptr(), argmax_dev.data_ptr())
         return loss_dev, argmax_dev
 
@@ -232,14 +230,13 @@ class ParameterServer:
         W, b = int(y_dev.shape[0]), int(y_dev.shape[1])
         assert x_dev.is_cuda and x_dev.dtype == torch.float32 and x_dev.is_contiguous() and x_dev.numel() == W * b * 784
         assert y_dev.is_cuda and y_dev.dtype == torch.int32 and y_dev.is_contiguous()
-        wid = np.ascontiguousarray(worker_ids, dtype=np.int32)
         if grad_sum_dev is None:
             grad_sum_dev = torch.empty(P_PAD, dtype=torch.float32, device="cuda")
         if loss_dev is None:
             loss_dev = torch.empty(W, dtype=torch.float32, device="cuda")
         if argmax_dev is None:
             argmax_dev = torch.empty((W, b), dtype=torch.int32, device="cuda")
-        _marshal.grad_step_summed(self._addr, W, b, snaps, wid, x_dev.data_ptr(), y_dev.data_ptr(), seed, step,
+        _marshal.grad_step_summed(self._addr, W, b, snaps, worker_ids, x_dev.data_ptr(), y_dev.data_ptr(), seed, step,
                                   grad_sum_dev.data_ptr(), loss_dev.data_ptr(), argmax_dev.data_ptr())
         return grad_sum_dev, loss_dev, argmax_dev
 
@@ -264,26 +261,17 @@ class ParameterServer:
         return keep
 
     def ps_enqueue(self, worker_ids, base_versions, step, slot_ids=None, grads_dev=None):
-        wid = np.ascontiguousarray(worker_ids, dtype=np.int32)
-        bv = np.ascontiguousarray(base_versions, dtype=np.uint64)
-        n = wid.shape[0]
-        sid = None if slot_ids is None else np.ascontiguousarray(slot_ids, dtype=np.int64)
         if grads_dev is not None:
+            n = len(worker_ids)
             assert grads_dev.is_cuda and grads_dev.dtype == self._torch.float32 and grads_dev.shape == (n, P_PAD) and grads_dev.is_contiguous()
-        _marshal.enqueue(self._addr, n, sid, grads_dev.data_ptr() if grads_dev is not None else None, wid, bv, step)
+        _marshal.enqueue(self._addr, slot_ids, grads_dev.data_ptr() if grads_dev is not None else None, worker_ids, base_versions, step)
 
     # -- server side -----------------------------------------------------------
     def ps_apply(self, mode, lr, scale=1.0, order=None):
-        o = None if order is None else np.ascontiguousarray(order, dtype=np.int32)
-        return _marshal.apply(self._addr, mode, lr, scale, o)
+        return _marshal.apply(self._addr, mode, lr, scale, order)
 
     def ps_apply_stale(self, mode, lr, scale=1.0, order=None, clip_norm=0.0, staleness_alpha=0.0):
-        res = ApplyResult()
-        o = None if order is None else np.ascontiguousarray(order, dtype=np.int32)
-        self._check(self.lib.ps_apply_stale(self.ctx, int(mode), float(lr), float(scale), _np_ptr(o), float(clip_norm),
-                                            float(staleness_alpha), C.byref(res)))
-        return {"applied": res.applied, "new_version": res.new_version, "checkpointed": res.checkpointed,
-                "replicated": res.replicated}
+        return _marshal.apply_stale(self._addr, mode, lr, scale, order, clip_norm, staleness_alpha)
 
     def _version_call(self, fn):
         v = C.c_uint64()

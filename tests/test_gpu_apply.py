@@ -503,3 +503,34 @@ def test_two_failures_in_one_run():
     assert g.ps_stats()["version"] == o.version == 5 and g.ps_stats()["live_replicas"] == 0
     assert_params_close(g.ps_export_params()[0], o.head(), 1e-5, "after two failovers")
     g.close()
+
+
+@pytest.mark.parametrize("form", [list, tuple, lambda v: np.asarray(v, dtype=np.int16), lambda v: np.asarray(v, dtype=np.uint64),
+                                  lambda v: np.repeat(np.asarray(v, dtype=np.uint64), 2)[::2], lambda v: [np.int64(i) for i in v]])
+def test_the_binding_reads_integers_in_every_form(form):
+    """Lists, tuples, arrays of other types and with gaps give the update that plain arrays give."""
+    _, ps, _, _ = _pair(queue_slots=8)
+    theta, grads, got = synth.init_params(seed=1), synth.random_gradients(5, seed=3), []
+    for f in (form, lambda v: np.asarray(v, dtype=np.uint64)):
+        srv = ps.ParameterServer(theta, max_batch=1, max_workers=8, queue_slots=8)
+        for v in range(4):
+            srv.ps_enqueue([0], [v], v, grads_dev=_pad(grads[:1]))
+            srv.ps_apply(ps.SYNC, 0.01)
+        slots = srv.ps_queue_reserve(5)
+        for k in range(5):
+            srv.slot_tensor(slots[k]).copy_(_pad(grads[k:k + 1])[0])
+        srv.ps_enqueue(f([3, 1, 0, 2, 4]), f([4, 0, 2, 3, 1]), 9, slot_ids=f([int(s) for s in slots]))
+        srv.ps_apply_stale(ps.ASYNC, 0.01, order=f([2, 0, 4, 1, 3]), clip_norm=0.5, staleness_alpha=0.5)
+        got.append(srv.ps_export_params()[0])
+        srv.close()
+    assert (got[0] == got[1]).all() and (got[0] != theta).any()
+
+
+def test_the_binding_refuses_what_is_no_integer_array():
+    _, ps, _, srv = _pair(queue_slots=8)
+    g = _pad(synth.random_gradients(2, seed=3))
+    for ids, base in (([0, 1], [0]), ([0, 1], None), (None, [0, 0]), ([0, 1], ["a", 0]), ([0, 1], [-1, 0])):
+        with pytest.raises((TypeError, ValueError, OverflowError)):
+            srv.ps_enqueue(ids, base, 0, grads_dev=g)
+    assert srv.ps_apply(ps.SYNC, 0.01)["applied"] == 0
+    srv.close()

@@ -601,7 +601,7 @@ def kernel_roofline(name, ms_per_launch, W, b, peaks, precision, sustained=False
     flops = {
         "conv1_fwd": 2 * 112_896 * n, "conv2_fwd": 2 * 903_168 * n, "fc1_fwd": 2 * 802_816 * n,
         "fc1_dw": 2 * 802_816 * n, "fc1_dx": 2 * 802_816 * n,
-        "conv2_bwd": 2 * (2 if precision == "fp32" else 1) * 903_168 * n, "conv2_dw": 2 * 903_168 * n,
+        "conv2_bwd": 2 * 903_168 * n, "conv2_dw": 2 * 903_168 * n,
         "conv1_bwd": 2 * 112_896 * n, "fc2_fwd_bwd": 2 * 3 * 5_120 * n,
     }
     tf32_kernels = {"fc1_fwd", "fc1_dw", "fc1_dx"}                               # tcgen05 kind::tf32

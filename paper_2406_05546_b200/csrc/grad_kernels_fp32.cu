@@ -365,7 +365,7 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
 // layer's backward has produced da1, the dense layer's per-worker weight gradient (bound by its 3.2 MB
 // per worker of writes) runs on a side stream next to the input-gradient chain, and once dp2 exists the
 // second convolution's filter gradient runs on another side stream next to its input gradient and the
-// first convolution's backward.  Everything joins before the final reduction.
+// first convolution's backward (tensor-core path: at some numbers of rows only, by the rule below).  Everything joins before the final reduction.
 int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                      cudaStream_t st, const SideStreams& side, Profiler* prof, const SummedStep* sum) {
   const bool tc = a.precision != 0;

@@ -37,8 +37,8 @@ REPLAY_TRAFFIC_PER_GRADIENT = 2.654663e9 / 816
 # dram bytes (read + written) per sample of the grad-step kernels, from one ncu capture of a reduced case
 # (W=128, b=64: 8,192 samples; traffic grows in proportion to the samples, except for fc1_dw, whose 3.2 MB of output per
 # worker do not depend on the batch: its figure holds at b = 64 only); None = not captured since the kernel changed
-KERNEL_TRAFFIC_PER_SAMPLE = {"conv2_dw": 13406, "conv1_fwd": 7393, "conv2_bwd": 5515, "fc1_dw": 51641, "conv2_fwd": 10064,
-                             "fc1_dx": 2452, "fc1_fwd": 6745, "fc2_fwd_bwd": 2061, "conv1_bwd": 12972}
+KERNEL_TRAFFIC_PER_SAMPLE = {"conv2_dw": None, "conv1_fwd": None, "conv2_bwd": None, "fc1_dw": 51641, "conv2_fwd": None,
+                             "fc1_dx": 2452, "fc1_fwd": 6745, "fc2_fwd_bwd": None, "conv1_bwd": None}
 
 
 # Algorithmic HBM bytes of the tensor-core path's grad-step kernels at (W, b): what each must read and write once
@@ -227,7 +227,7 @@ def run_small_case(args):
 
 
 GRAD_KERNELS_EXCLUDED = ("sum_apply_direct", "sum_partial", "sum_finish", "async_apply", "copy_rows", "dropout_mask",
-                         "sq_norm_partial", "clip_coef_finish", "eval_finish")      # server-side and auxiliary kernels
+                         "sq_norm_partial", "clip_coef_finish", "clip_sum_apply", "eval_finish")      # server-side and auxiliary kernels
 
 
 def measure_config(n, precision, pool_x, pool_y, ticks=10, warmup=3):
@@ -471,7 +471,7 @@ def main():
                                # (2.654663 GB over 816 gradients), scaled to this launch
                                "traffic": K_replay * REPLAY_TRAFFIC_PER_GRADIENT, "peak_source": peaks["source"]},
                   "all_ms": reps}
-    # ---- the same replay with clipping by global norm: one pass that takes the norms, one that sums
+    # ---- the same replay with clipping by global norm, in one pass over the queue
     replay_clipped = None
     if do_replay:
         srv.ps_kill()
@@ -491,10 +491,9 @@ def main():
         srv.ps_profile(False)
         pass_bytes = K_replay * GRAD_BYTES
         replay_clipped = {"queue_gradients": K_replay, "ms": ms, "clip_norm": 1.0,
-                          "norm_pass_ms": prof_c["sq_norm_partial"][0], "norm_pass_gb_per_s": pass_bytes / (prof_c["sq_norm_partial"][0] * 1e-3) / 1e9,
-                          "sum_pass_ms": prof_c["sum_partial"][0], "sum_pass_gb_per_s": pass_bytes / (prof_c["sum_partial"][0] * 1e-3) / 1e9,
-                          "frac_of_hbm_peak_per_pass": [pass_bytes / (prof_c["sq_norm_partial"][0] * 1e-3) / 1e9 / peaks["hbm_gbs"],
-                                                        pass_bytes / (prof_c["sum_partial"][0] * 1e-3) / 1e9 / peaks["hbm_gbs"]]}
+                          "kernel_ms": prof_c["clip_sum_apply"][0],
+                          "kernel_gb_per_s": pass_bytes / (prof_c["clip_sum_apply"][0] * 1e-3) / 1e9,
+                          "frac_of_hbm_peak": pass_bytes / (prof_c["clip_sum_apply"][0] * 1e-3) / 1e9 / peaks["hbm_gbs"]}
     stats = srv.ps_stats()
 
     if rank == 0:

@@ -293,7 +293,9 @@ __global__ void __launch_bounds__(D1_THREADS, 1) conv1_dw_tc5(GradStepArgs a, Wo
     D1Unit un;
     while (d1_next_unit(walk, r1, a.b, un)) {
       if (!un.flush) continue;
-      if (!mbar_wait(&bars->acc_full, writes & 1) || bars->abort_flag) { bars->abort_flag = 1; break; }
+      // all four warps go on or none does: they meet at a barrier below.  This also is where the previous sums have been read.
+      const bool ok = mbar_wait(&bars->acc_full, writes & 1) && !bars->abort_flag;
+      if (!warps_agree<1, 128>(ok)) { bars->abort_flag = 1; break; }
       tc_fence_after();
       uint32_t v0[16], v1[16];
       tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(24 * half), v0);
@@ -323,7 +325,6 @@ __global__ void __launch_bounds__(D1_THREADS, 1) conv1_dw_tc5(GradStepArgs a, Wo
       float* part = ws.part1 + ((int64_t)s * slots + (blockIdx.x - (s * a.b) / seg_len)) * C1_GRAD;
       for (int o = quarter * 32 + lane; o < C1_GRAD; o += 128)
         part[o] = (sums[o] + sums[C1_GRAD + o]) + (sums[2 * C1_GRAD + o] + sums[3 * C1_GRAD + o]);
-      asm volatile("bar.sync 1, 128;" ::: "memory");
       ++writes;
     }
   }

@@ -39,6 +39,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
   return mbar_wait_addr(smem_u32(bar), parity, limit_cycles);
 }
 
+// What several warps do next: true in all of their THREADS threads if `ok` holds in every one of them, false in all otherwise.
+// Every wait runs out on its own thread's clock, so threads that go on to exchange data behind a barrier of theirs settle
+// first, here, whether all of them do: a warp that had given up alone would leave the others at that barrier for good.
+template <int BARRIER, int THREADS>
+__device__ __forceinline__ bool warps_agree(bool ok) {
+  uint32_t all;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %3, 0;\n\t"
+      "barrier.cta.red.and.pred q, %1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(all) : "n"(BARRIER), "n"(THREADS), "r"((uint32_t)ok) : "memory");
+  return all != 0;
+}
+
 __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1, int c2) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"

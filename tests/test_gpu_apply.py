@@ -405,6 +405,16 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_nothing_hangs():
     torch.cuda.synchronize()
 
 
+@pytest.mark.parametrize("limit_cycles", [1, 2000, 200000])
+def test_warps_that_wait_apart_give_up_together(limit_cycles):
+    """One of four warps waits on a barrier nobody arrives at, the others on a complete one: the status word is set only if
+    every thread of the four has learned that one of them gave up."""
+    _, ps, _, g = _pair(queue_slots=4)
+    g.ps_selftest_wait_timeout(limit_cycles)
+    assert g.ps_stats(check=False)["device_status"] == 2
+    g.close()
+
+
 # ---- treatments of stale gradients ------------------------------------------------------------------------------------
 
 def _known_norm_grads(norms, seed):

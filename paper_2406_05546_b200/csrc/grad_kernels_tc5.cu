@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(192, 2) tc5_fwd_narrow(const __grid_constant__
       umma_commit(acc_full);
     }
   } else {
-    if (mbar_wait(acc_full, 0)) {
+    if (warps_agree<1, 128>(mbar_wait(acc_full, 0))) {      // the four warps meet at a barrier below: all of them or none
       tc_fence_after();
       const int quarter = warp & 3;            // an accumulator of 64 rows keeps rows 16 q .. 16 q + 15 in the first sixteen lanes of quarter q
       uint32_t r[32];
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(192, 2) tc5_fwd_narrow(const __grid_constant__
               fc1_activation(*reinterpret_cast<const float4*>(stage_out + row * EPI_ROW_FLOATS + 4 * q), m, n, gt.theta[grp], a, wt);
       }
     } else {
-      *abort_flag = 1;                         // all four warps give up together: the barrier is theirs alone
+      *abort_flag = 1;
     }
   }
   tc_fence_before();

@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(256, 1) tc5_dx_split(const __grid_constant__ G
   }
   __syncwarp();
   float* part = reinterpret_cast<float*>(tiles);
-  if (mbar_wait(acc_full, 0)) {
+  if (__syncthreads_and(mbar_wait(acc_full, 0))) {          // tensor memory is read by whole warps: all threads or none
     tc_fence_after();
     const int quarter = warp & 3;
     for (int ch = warp >> 2; ch < S::BN / 32; ch += 2) {

@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(D1_THREADS, 1) conv1_dw_tc5(GradStepArgs a, Wo
       bool ok = true;
       if (mine) ok = mbar_wait(&bars->raw_full[slot], use & 1);
       if (ok && u >= 2) ok = mbar_wait(&bars->op_empty[st], ((u >> 1) - 1) & 1);      // the MMAs of unit u - 2 have read the stage
-      if (!__all_sync(0xffffffffu, ok) || bars->abort_flag) { bars->abort_flag = 1; break; }
+      if (!__all_sync(0xffffffffu, ok && !bars->abort_flag)) { bars->abort_flag = 1; break; }
       const uint8_t* rslot = raw + slot * D1_RAW_SLOT;
       const float* img = reinterpret_cast<const float*>(rslot);
       const uint8_t* rg = rslot + D1_RAW_ZERO + D1_RAW_X;

@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(F_THREADS, 2) conv2_fwd_tc5(GradStepArgs a, Gr
     const int r = quarter * 32 + lane, g = r >> 3, px = r & 7, sp = g >> 3, py = g & 7;
     for (int t = 0; t < n_tiles; ++t) {
       const int buf = t & 1;
-      if (!mbar_wait(&pipe->acc_full[buf], (t >> 1) & 1) || pipe->abort_flag) { pipe->abort_flag = 1; break; }
+      if (!warp_wait(&pipe->acc_full[buf], (t >> 1) & 1, &pipe->abort_flag)) { pipe->abort_flag = 1; break; }
       tc_fence_after();
       const int64_t row = r_begin + 2 * t + sp;
       const bool valid = py < 7 && px < 7 && row < r_end;
@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(THREADS, 2) conv2_dx_tc5(GradStepArgs a, Group
       // every staging warp waits and reports on its own (no block-level barrier among them)
       bool ok = mbar_wait(&pipe->raw_full[slot_i], (t >> 3) & 1);
       if (ok && t >= 2) ok = mbar_wait(&pipe->a_empty[buf], ((t >> 1) - 1) & 1);
-      if (!__all_sync(0xffffffffu, ok) || pipe->abort_flag) { pipe->abort_flag = 1; break; }
+      if (!__all_sync(0xffffffffu, ok && !pipe->abort_flag)) { pipe->abort_flag = 1; break; }
       uint16_t* dst = bufs + buf * (X_BUF_BYTES / 2);
       const uint2* rg = reinterpret_cast<const uint2*>(raw + slot_i * X_RAW_BYTES);      // four BF16 channels of a position
       const uint8_t* rc = raw + slot_i * X_RAW_BYTES + FLAT * 2;
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(THREADS, 2) conv2_dx_tc5(GradStepArgs a, Group
     const int quarter = warp & 3;
     for (int t = 0; t < n_tiles; ++t) {
       const int buf = t & 1;
-      if (!mbar_wait(&pipe->acc_full[buf], (t >> 1) & 1) || pipe->abort_flag) { pipe->abort_flag = 1; break; }
+      if (!warp_wait(&pipe->acc_full[buf], (t >> 1) & 1, &pipe->abort_flag)) { pipe->abort_flag = 1; break; }
       tc_fence_after();
       const int64_t row = r_begin + t;
 #pragma unroll

@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(W5_THREADS, 1) conv2_dw_tc5(GradStepArgs a, Wo
     for (int n = grp; n < n_samples; n += 2) {
       bool ok = mbar_wait(&bars->raw_full[slot], slot_use & 1);
       if (ok && st_use > 0) ok = mbar_wait(&bars->op_empty[st], (st_use - 1) & 1);      // the MMAs of sample n - 3 have read the stage
-      if (!__all_sync(0xffffffffu, ok) || bars->abort_flag) { bars->abort_flag = 1; break; }
+      if (!__all_sync(0xffffffffu, ok && !bars->abort_flag)) { bars->abort_flag = 1; break; }
       const uint8_t* rp1 = raw + slot * W5_RAW_SLOT;
       const uint16_t* rdp2h = reinterpret_cast<const uint16_t*>(rp1 + W5_RAW_P1);
       const uint8_t* rcode8 = rp1 + W5_RAW_P1 + W5_RAW_DP2;
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(W5_THREADS, 1) conv2_dw_tc5(GradStepArgs a, Wo
     int s = r0 / a.b;                                    // sorted worker of the rows being summed
     // the rows after which the sum is written out: the last of every worker in the range, and the range's last
     for (int row = min(r1, (s + 1) * a.b) - 1; row < r1; row = (row + 1 == r1) ? r1 : min(row + a.b, r1 - 1), ++s) {
-      if (!mbar_wait(&bars->acc_full, writes & 1) || bars->abort_flag) { bars->abort_flag = 1; break; }
+      if (!warp_wait(&bars->acc_full, writes & 1, &bars->abort_flag)) { bars->abort_flag = 1; break; }
       tc_fence_after();
       float* part = ws.part2 + ((int64_t)s * slots + (blockIdx.x - (s * a.b) / seg_len)) * C2_GRAD;
       const int rr = lane < 16 ? quarter * 16 + lane : 64;   // accumulator row: (kx, ic) for rr < 48, the ones row at 48

@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(gemm_threads(EPI), 1) tc5_gemm(const __grid_co
       TileCoord c;
       if (!decode_tile<BN>(tw, ga, gt, a.b, c)) continue;
       const int ab = tile_i & 1;
-      if (!mbar_wait(&acc_full[ab], (tile_i >> 1) & 1) || *abort_flag) {
+      if (!warp_wait(&acc_full[ab], (tile_i >> 1) & 1, abort_flag)) {
         if (lane == 0) { *abort_flag = 1; atomicOr(ws.status, STATUS_WAIT_TIMEOUT); }
         break;
       }

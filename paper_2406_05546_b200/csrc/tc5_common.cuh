@@ -39,6 +39,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
   return mbar_wait_addr(smem_u32(bar), parity, limit_cycles);
 }
 
+// A bounded wait of a whole warp that another role's abort ends too: the same answer in every lane, for the warp-wide
+// tensor-memory reads behind it.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, const volatile uint32_t* abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity) && !*abort_flag);
+}
+
 // What several warps do next: true in all of their THREADS threads if `ok` holds in every one of them, false in all otherwise.
 // Every wait runs out on its own thread's clock, so threads that go on to exchange data behind a barrier of theirs settle
 // first, here, whether all of them do: a warp that had given up alone would leave the others at that barrier for good.

@@ -27,6 +27,24 @@ __device__ __forceinline__ void fma4(float c, const float4& v, float4& a) {
   a.x = fmaf(c, v.x, a.x); a.y = fmaf(c, v.y, a.y); a.z = fmaf(c, v.z, a.z); a.w = fmaf(c, v.w, a.w);
 }
 
+// Adds p to a running sum and what the addition rounds away to another, for two columns at once.  (Exact while |acc| >= |p|;
+// otherwise off by a rounding of p, which is small then.)
+__device__ __forceinline__ void add_compensated(u64 p, u64& acc, u64& err) {
+  u64 t, d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(acc), "l"(p));
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(t), "l"(acc));
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(p), "l"(d));
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(err) : "l"(err), "l"(d));
+  acc = t;
+}
+// The two together; a sum that is not finite stays what it is (its second part is no number then).
+__device__ __forceinline__ float2 compensated(u64 acc, u64 err) {
+  float a0, a1, e0, e1;
+  unpack2(acc, a0, a1);
+  unpack2(err, e0, e1);
+  return make_float2(isfinite(e0) ? a0 + e0 : a0, isfinite(e1) ? a1 + e1 : a1);
+}
+
 // Sum of slots [k0, k1) of one float4 column, in a fixed order: eight interleaved running sums
 // (slot k goes to sum k mod 8 relative to k0), combined pairwise at the end.  With WEIGHTED every slot is
 // multiplied by its own factor coef_k[k] (the stale-gradient treatments) as it is added.
@@ -203,6 +221,11 @@ __global__ void __launch_bounds__(TPB) clip_coef_finish(const float* __restrict_
 // sums, CS_GATHER gather the other CTAs' in turn.  A word of the exchange carries its gradient's number beside the sum, so
 // it needs no flag, and the words of CS_RING gradients are used in turn; every CTA writes its word CS_COPIES times and a
 // CTA polls one of the copies only: the polls of all CTAs on one copy slow the stores down.
+// Precision: a thread adds `fold` gradients in single precision, and that to a sum kept in two parts, whose error does not
+// grow with its terms.  Relative error (2-norm) of the sum of gradients N(0.02, 0.01^2) with one running sum / so / in two
+// passes (eight running sums, from 160 gradients on in up to sixteen ranges): K = 16: 6.6e-8 / 3.1e-8 / 4.1e-8, 300: 2.6e-7 /
+// 2.8e-8 / 5.5e-8, 12,800: 1.5e-6 / 1.9e-8 / 5.6e-8.  It costs 1 % at K = 1600 (872 -> 880 us for the whole call); a sum in
+// two parts at every gradient, every second and every fourth cost 4.2, 4.1 and 2.3 %.
 // Measured (B200), us for clipping by norm, summing and applying K gradients, two passes over the queue (norms, factors,
 // weighted sum) -> this kernel: K = 1: 27 -> 12, 16: 39 -> 19, 128: 159 -> 86, 1600: 1466 -> 793 (6.6 TB/s), 6400: 5700 -> 3131.
 // At 1600 also: three gathering warps 902, four 1028 (more polls); 16 copies 812; squaring and adding by the same warps,
@@ -222,7 +245,10 @@ struct ClipShared {
 };
 static_assert(sizeof(ClipShared) <= CS_MISC, "shared memory");
 
-__global__ void __launch_bounds__(CS_THREADS, 1) clip_sum_apply(const float4* __restrict__ queue, int K, int cols, int slots, float clip,
+// Sixteen or more runs, so that what their own roundings add stays below the last one's; longer ones than 32 save no time.
+inline int clip_fold(int64_t K) { return (int)(K / 16 < 1 ? 1 : (K / 16 > 32 ? 32 : K / 16)); }
+
+__global__ void __launch_bounds__(CS_THREADS, 1) clip_sum_apply(const float4* __restrict__ queue, int K, int cols, int slots, int fold, float clip,
                                                                 const float* __restrict__ coef_k, u64* words, const float4* theta_in,
                                                                 float4* theta_out, float4* __restrict__ replica, uint32_t* status) {
   extern __shared__ __align__(128) uint8_t sm[];
@@ -248,13 +274,14 @@ __global__ void __launch_bounds__(CS_THREADS, 1) clip_sum_apply(const float4* __
   bool ok = true;
   if (warp < CS_ADD) {
     // ---------------- sums
-    float4 acc[CS_ADD_PER];
+    u64 part[2 * CS_ADD_PER], acc[2 * CS_ADD_PER], err[2 * CS_ADD_PER];
 #pragma unroll
-    for (int j = 0; j < CS_ADD_PER; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-    int slot = 0;
+    for (int j = 0; j < 2 * CS_ADD_PER; ++j) part[j] = acc[j] = err[j] = 0ull;
+    int slot = 0, run = 0;
     for (int k = 0; k < K; ++k) {
       if (!(ok = wait(&sh->coef_ready[k % CS_DEPTH], (k / CS_DEPTH) & 1))) break;
-      const float c = sh->coef[k % CS_DEPTH];
+      const float ck = sh->coef[k % CS_DEPTH];
+      const u64 c = pack2(ck, ck);
       const float4* g = ring + slot * cols;
       float4 v[CS_ADD_PER];
 #pragma unroll
@@ -265,7 +292,18 @@ __global__ void __launch_bounds__(CS_THREADS, 1) clip_sum_apply(const float4* __
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh->empty[slot]);
 #pragma unroll
-      for (int j = 0; j < CS_ADD_PER; ++j) fma4(c, v[j], acc[j]);
+      for (int j = 0; j < CS_ADD_PER; ++j) {
+        part[2 * j] = ffma2(c, pack2(v[j].x, v[j].y), part[2 * j]);
+        part[2 * j + 1] = ffma2(c, pack2(v[j].z, v[j].w), part[2 * j + 1]);
+      }
+      if (++run == fold || k == K - 1) {
+        run = 0;
+#pragma unroll
+        for (int j = 0; j < 2 * CS_ADD_PER; ++j) {
+          add_compensated(part[j], acc[j], err[j]);
+          part[j] = 0ull;
+        }
+      }
       if (++slot == slots) slot = 0;
     }
     if (ok) {
@@ -274,7 +312,8 @@ __global__ void __launch_bounds__(CS_THREADS, 1) clip_sum_apply(const float4* __
         const int i = tid + 32 * CS_ADD * j;
         if (i < n) {
           float4 t = theta_in[col0 + i];
-          t.x -= acc[j].x; t.y -= acc[j].y; t.z -= acc[j].z; t.w -= acc[j].w;
+          const float2 lo = compensated(acc[2 * j], err[2 * j]), hi = compensated(acc[2 * j + 1], err[2 * j + 1]);
+          t.x -= lo.x; t.y -= lo.y; t.z -= hi.x; t.w -= hi.y;
           theta_out[col0 + i] = t;
           if (replica) replica[col0 + i] = t;
         }
@@ -431,7 +470,7 @@ int launch_clip_sum_apply(const SumApplyArgs& a, float clip, uint64_t* words, ui
   at.val.cooperative = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  TIMED(K_CLIP_SUM, cudaLaunchKernelEx(&cfg, clip_sum_apply, reinterpret_cast<const float4*>(a.queue), (int)a.K, cols, slots, clip, a.coef_k,
+  TIMED(K_CLIP_SUM, cudaLaunchKernelEx(&cfg, clip_sum_apply, reinterpret_cast<const float4*>(a.queue), (int)a.K, cols, slots, clip_fold(a.K), clip, a.coef_k,
                                        reinterpret_cast<u64*>(words), reinterpret_cast<const float4*>(a.theta_in),
                                        reinterpret_cast<float4*>(a.theta_out), reinterpret_cast<float4*>(a.replica), status));
   return cudaGetLastError() == cudaSuccess ? 1 : -1;

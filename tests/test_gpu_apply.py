@@ -450,6 +450,36 @@ def test_clipping_by_global_norm(mode_name, K):
     _g2.close(); g.close()
 
 
+@pytest.mark.parametrize("K", [1, 16, 300, 4096])
+def test_clipped_sum_of_a_long_backlog_with_a_common_direction(K):
+    """A bound no gradient reaches leaves every factor at exactly 1 and weights of zero make the new weights the sum itself,
+    so that the sum's own error is all there is.  It may be about one rounding of the result at any number of gradients:
+    2^-24 of the value at most, 2^-24 / sqrt(3) in the mean square, and the runs of gradients that are added in single
+    precision before add a third of that at most (sixteen runs or more, whose errors are independent).  The values share a
+    mean: their sum grows with every one of them."""
+    import torch
+    from paper_2406_05546_b200 import ps
+    W = min(K, 128)
+    srv = ps.ParameterServer(np.zeros(ps.P, dtype=np.float32), max_workers=W, max_batch=1, queue_slots=K, external_store=True)
+    start = srv.ps_slot_ptr(0) - srv.arena.data_ptr()
+    queue = srv.arena[start:start + K * ps.P_PAD * 4].view(torch.float32).view(K, ps.P_PAD)
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    exact = torch.zeros(ps.P_PAD, dtype=torch.float64, device="cuda")
+    for rows in queue.split(256):
+        rows.uniform_(0.5, 1.5, generator=gen)
+        rows[:, ps.P:] = 0
+        exact += rows.double().sum(0)
+    n = W if K % W == 0 else K // 3      # gradients per enqueue
+    for t in range(K // n):
+        srv.ps_enqueue(range(n), [0] * n, t, slot_ids=srv.ps_queue_reserve(n))
+    assert srv.ps_apply_stale(ps.REPLAY, 1.0, float(n), clip_norm=1e9)["applied"] == K
+    got, want = -srv.ps_export_params()[0].astype(np.float64), exact[:ps.P].cpu().numpy()
+    error = np.sqrt(np.mean(((got - want) / want) ** 2))
+    assert error <= 2.0 ** -24, error
+    assert srv.ps_stats()["device_status"] == 0
+    srv.close()
+
+
 @pytest.mark.parametrize("mode_name", ["SYNC", "REPLAY", "ASYNC"])
 def test_staleness_scaled_learning_rate(mode_name):
     ops, ps, o, g = _pair(queue_slots=16, ring_depth=9, external_store=(mode_name == "REPLAY"), max_workers=16)

@@ -6,6 +6,8 @@
 // chain-replication mirror).  Threads own float4 columns of the parameter vector, so every load
 // and store is a coalesced 16-byte access; the K loop is unrolled to keep many independent loads
 // in flight per thread.
+#include <algorithm>
+
 #include "kernels.h"
 #include "tc5_common.cuh"
 #include "device_common.cuh"
@@ -453,26 +455,43 @@ int configure_apply_kernels() {
   return allow_smem((const void*)clip_sum_apply, CS_SMEM) == cudaSuccess ? 0 : -1;
 }
 
+// The one-pass kernel's shape on a device of `sms` SMs: a CTA per SM, its columns, its ring of gradients.  A CTA's threads cover
+// CS_MAX_COLS columns, so it takes 145 SMs or more.
+struct ClipShape { int grid, cols, slots; };
+static ClipShape clip_shape(int sms) {
+  ClipShape c;
+  c.grid = std::min(std::max(sms, 1), NORM_WORDS);
+  c.cols = (P_VEC4 + c.grid - 1) / c.grid;
+  c.slots = std::min(CS_MAX_SLOTS, (CS_SMEM - CS_MISC) / (c.cols * 16));
+  return c;
+}
+bool clip_sum_fits(int sms) {
+  const ClipShape c = clip_shape(sms);
+  return c.cols <= CS_MAX_COLS && c.slots >= 3 && (int64_t)(c.grid - 1) * c.cols < P_VEC4;
+}
+
 int launch_clip_sum_apply(const SumApplyArgs& a, float clip, uint64_t* words, uint32_t* status, cudaStream_t st, Profiler* prof) {
-  const int grid = g_sm_count < NORM_WORDS ? g_sm_count : NORM_WORDS;
-  const int cols = (P_VEC4 + grid - 1) / grid;
-  int slots = (CS_SMEM - CS_MISC) / (cols * 16);
-  if (slots > CS_MAX_SLOTS) slots = CS_MAX_SLOTS;
-  if (cols > CS_MAX_COLS || slots < 3 || (int64_t)(grid - 1) * cols >= P_VEC4) return -1;
+  if (!clip_sum_fits(g_sm_count)) return 0;
+  const ClipShape c = clip_shape(g_sm_count);
   if (cudaMemsetAsync(words, 0, CLIP_EXCHANGE_BYTES, st) != cudaSuccess) return -1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = dim3(c.grid);
   cfg.blockDim = dim3(CS_THREADS);
-  cfg.dynamicSmemBytes = (size_t)(CS_MISC + slots * cols * 16);
+  cfg.dynamicSmemBytes = (size_t)(CS_MISC + c.slots * c.cols * 16);
   cfg.stream = st;
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeCooperative;
   at.val.cooperative = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  TIMED(K_CLIP_SUM, cudaLaunchKernelEx(&cfg, clip_sum_apply, reinterpret_cast<const float4*>(a.queue), (int)a.K, cols, slots, clip_fold(a.K), clip, a.coef_k,
-                                       reinterpret_cast<u64*>(words), reinterpret_cast<const float4*>(a.theta_in),
-                                       reinterpret_cast<float4*>(a.theta_out), reinterpret_cast<float4*>(a.replica), status));
+  cudaError_t e = cudaSuccess;
+  TIMED(K_CLIP_SUM, e = cudaLaunchKernelEx(&cfg, clip_sum_apply, reinterpret_cast<const float4*>(a.queue), (int)a.K, c.cols, c.slots, clip_fold(a.K),
+                                           clip, a.coef_k, reinterpret_cast<u64*>(words), reinterpret_cast<const float4*>(a.theta_in),
+                                           reinterpret_cast<float4*>(a.theta_out), reinterpret_cast<float4*>(a.replica), status));
+  if (e == cudaErrorCooperativeLaunchTooLarge) {      // a stream that may use part of the device only
+    cudaGetLastError();
+    return 0;
+  }
   return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 

@@ -241,10 +241,12 @@ int launch_copy_rows(float* dst, const float* src, int64_t rows, cudaStream_t st
 // Clipping by global norm: coef_k[k] *= min(1, clip / ||queue[k]||_2) for k < K.  norm_part: [K][NORM_CHUNKS] scratch.
 constexpr int NORM_CHUNKS = 8;
 // Clipping, summing and applying in one pass (sync and replay steps).  words: CLIP_EXCHANGE_BYTES of scratch, where the
-// CTAs exchange their partial sums of squares.
+// CTAs exchange their partial sums of squares.  Returns 0, with nothing launched, where the kernel does not fit: on a device
+// with too few SMs (clip_sum_fits), or in a stream confined to a part of it.
 constexpr int NORM_WORDS = 160, CS_RING = 64, CS_COPIES = 8;      // words per copy (one per CTA, at most), gradients, copies
 constexpr int CLIP_EXCHANGE_BYTES = NORM_WORDS * CS_RING * CS_COPIES * 8;
 int configure_apply_kernels();
+bool clip_sum_fits(int sms);
 int launch_clip_sum_apply(const SumApplyArgs& a, float clip, uint64_t* words, uint32_t* status, cudaStream_t st, Profiler* prof);
 int launch_clip_factors(const float* queue, int64_t K, float clip, float* coef_k, float* norm_part, cudaStream_t st, Profiler* prof);
 

@@ -559,8 +559,9 @@ int32_t ps_replicate(ps_ctx* x, uint64_t* version_out) {
 }
 
 // One server step.  clip_norm > 0 and / or staleness_alpha > 0 switch the stale-gradient treatments on: every queued
-// gradient then gets a factor of its own (learning rate included), staged on the host, uploaded, and, for clipping,
-// multiplied on the device by min(1, clip_norm / ||g||) after one pass over the queue that takes the norms.
+// gradient then gets a factor of its own (learning rate included), staged on the host and uploaded.  For clipping it is
+// multiplied on the device by min(1, clip_norm / ||g||): by the kernel that also sums and applies (sync and replay), or,
+// in the ordered mode and where that kernel does not fit, after a pass over the queue that takes the norms.
 static int32_t apply_impl(ps_ctx* x, ps_mode mode, float lr, float scale, const int32_t* order, float clip_norm,
                           float staleness_alpha, ps_apply_result* out) {
   if (!x) return fail(PS_ERR_BAD_ARG, "ctx is NULL");
@@ -578,7 +579,12 @@ static int32_t apply_impl(ps_ctx* x, ps_mode mode, float lr, float scale, const 
     }
   }
   const bool treated = clip_norm > 0.f || staleness_alpha > 0.f;
-  const bool one_pass = clip_norm > 0.f && mode != PS_ASYNC;      // the ordered apply reads the norms' factors instead
+  auto clip_factors = [&]() -> int32_t {
+    int n = psk::launch_clip_factors(x->queue, K, clip_norm, x->coef_dev, x->norm_part, x->st, &x->prof);
+    if (n < 0) return cuda_fail(cudaGetLastError(), "clipping launch");
+    x->launches += n;
+    return PS_OK;
+  };
   if (treated) {
     // factor of the gradient in queue slot k: the step size of its mode times 1 / (1 + alpha * staleness), where the
     // staleness is the version the update is applied to minus the version the worker had read
@@ -597,10 +603,8 @@ static int32_t apply_impl(ps_ctx* x, ps_mode mode, float lr, float scale, const 
     }
     CUDA_TRY(cudaMemcpyAsync(x->coef_dev, x->coef_host, (size_t)K * sizeof(float), cudaMemcpyHostToDevice, x->st));
     CUDA_TRY(cudaEventRecord(x->coef_uploaded, x->st));
-    if (clip_norm > 0.f && !one_pass) {
-      int n = psk::launch_clip_factors(x->queue, K, clip_norm, x->coef_dev, x->norm_part, x->st, &x->prof);
-      if (n < 0) return cuda_fail(cudaGetLastError(), "clipping launch");
-      x->launches += n;
+    if (clip_norm > 0.f && mode == PS_ASYNC) {      // the ordered apply reads the factors
+      int32_t rc = clip_factors(); if (rc != PS_OK) return rc;
     }
   }
   const uint64_t depth = (uint64_t)x->cfg.ring_depth;
@@ -617,8 +621,11 @@ static int32_t apply_impl(ps_ctx* x, ps_mode mode, float lr, float scale, const 
     a.coef = lr * scale / (float)(mode == PS_SYNC ? K : (int64_t)x->w_tick);
     a.partial = x->partial; a.max_split = MAX_SPLIT;
     a.coef_k = treated ? x->coef_dev : nullptr;
-    int n = one_pass ? psk::launch_clip_sum_apply(a, clip_norm, x->clip_words, x->status_dev, x->st, &x->prof)
-                     : psk::launch_sum_apply(a, x->st, &x->prof);
+    int n = clip_norm > 0.f ? psk::launch_clip_sum_apply(a, clip_norm, x->clip_words, x->status_dev, x->st, &x->prof) : 0;
+    if (n == 0) {      // nothing to clip, or no room for the kernel that clips and sums in one pass
+      if (clip_norm > 0.f) { int32_t rc = clip_factors(); if (rc != PS_OK) return rc; }
+      n = psk::launch_sum_apply(a, x->st, &x->prof);
+    }
     if (n < 0) return cuda_fail(cudaGetLastError(), "apply launch");
     x->launches += n;
     x->version += 1;

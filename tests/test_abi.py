@@ -45,6 +45,13 @@ def test_struct_sizes_match_header_layout():
     assert ps.P_PAD % 64 == 0 and ps.P_PAD >= ps.P
 
 
+def test_one_pass_clipping_is_chosen_where_it_fits_only():
+    """A CTA of the one-pass kernel covers up to 1,408 of the 203,328 float4 columns: 145 SMs cover them all, 144 do not."""
+    fits = ps.load()["_ZN3psk13clip_sum_fitsEi"]
+    fits.argtypes, fits.restype = [C.c_int], C.c_bool
+    assert [n for n in range(0, 400) if fits(n)] == list(range(145, 400))
+
+
 def test_no_cpu_fallback():
     import pytest
     import torch

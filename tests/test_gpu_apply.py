@@ -450,6 +450,23 @@ def test_clipping_by_global_norm(mode_name, K):
     _g2.close(); g.close()
 
 
+@pytest.mark.parametrize("mode_name,K", [("SYNC", 6), ("REPLAY", 300)])
+def test_clipping_on_a_device_with_few_sms_takes_two_passes(mode_name, K):
+    import ctypes
+    ops, ps, o, g = _pair(queue_slots=K, ring_depth=3, external_store=(mode_name == "REPLAY"), max_workers=64)
+    grads = _known_norm_grads(np.random.default_rng(K).uniform(0.2, 5.0, size=K), seed=K)
+    _both_enqueue(o, g, grads)
+    ro = o.apply(getattr(ops, mode_name), 0.01, clip_norm=1.0)
+    sms = ctypes.c_int.in_dll(ps.load(), "_ZN3psk10g_sm_countE")
+    before, sms.value = sms.value, 132
+    try:
+        assert ro == g.ps_apply_stale(getattr(ps, mode_name), 0.01, clip_norm=1.0)
+    finally:
+        sms.value = before
+    assert_params_close(g.ps_export_params()[0], o.head(), TOL_APPLY, f"clipped {mode_name}, two passes")
+    g.close()
+
+
 @pytest.mark.parametrize("K", [1, 16, 300, 4096])
 def test_clipped_sum_of_a_long_backlog_with_a_common_direction(K):
     """A bound no gradient reaches leaves every factor at exactly 1 and weights of zero make the new weights the sum itself,

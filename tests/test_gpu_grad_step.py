@@ -143,6 +143,39 @@ def test_fp32_path_at_the_edges_of_its_kernel_choices(W, b, kw):
     _run_and_compare(W, b, **kw)
 
 
+def _float64_gradient(theta, x, y, keep, drop_p=0.25):
+    """One worker's gradient in float64 on the device: {tensor name: flat gradient}."""
+    import torch
+    import torch.nn.functional as F
+    p = {n: torch.from_numpy(theta[o:o + int(np.prod(s))].astype(np.float64).reshape(s)).cuda().requires_grad_(True) for n, o, s in synth.layout()}
+    h = F.max_pool2d(F.relu(F.conv2d(x.double()[:, None], p["conv1.w"], p["conv1.b"], padding=1)), 2)
+    h = F.max_pool2d(F.relu(F.conv2d(h, p["conv2.w"], p["conv2.b"], padding=1)), 2).flatten(1)
+    h = F.relu(F.linear(h, p["fc1.w"], p["fc1.b"])) * keep.double() / (1 - drop_p)
+    F.cross_entropy(F.linear(h, p["fc2.w"], p["fc2.b"]), y.long()).backward()
+    return {n: v.grad.flatten() for n, v in p.items()}
+
+
+def test_fp32_filter_gradient_is_as_precise_in_a_large_call_as_in_a_small_one():
+    """Rows of a call are summed in ranges that grow with the call, and what single precision loses grows as the root of a
+    sum's length.  At 16 x 128 rows a thread of conv2's filter gradient adds the 49 / 4 winners of its positions over 7
+    samples, and 20 such sums make a worker's gradient; at 128 x 128 it is 14 samples and 11 sums.  The errors of the first
+    sixteen workers may differ by sqrt((14 * 12.25 + 11) / (7 * 12.25 + 20)) = 1.32 then (median: a worker in which a pooling
+    decision fell the other way counts no more than another)."""
+    torch, ps, srv, theta = _setup(128, 128)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.rand((128, 128, 28, 28), generator=gen, device="cuda")
+    y = torch.randint(0, 10, (128, 128), generator=gen, device="cuda", dtype=torch.int32)
+    off, n = next((o, int(np.prod(s))) for name, o, s in synth.layout() if name == "conv2.w")
+    exact = [_float64_gradient(theta, x[w], y[w], srv.ps_dropout_mask(SEED, w, 1, 128))["conv2.w"] for w in range(16)]
+    median = {}
+    for W in (16, 128):
+        grads = torch.zeros((W, ps.P_PAD), device="cuda")
+        srv.workers_grad_step([srv.ps_pull_snapshot(w) for w in range(W)], range(W), x[:W], y[:W], SEED, 1, grads_dev=grads)
+        median[W] = float(np.median([float((grads[w, off:off + n].double() - e).norm() / e.norm()) for w, e in enumerate(exact)]))
+    srv.close()
+    assert median[128] <= 1.32 * median[16], median
+
+
 @pytest.mark.parametrize("b", [64, 65, 1040])
 def test_output_layer_split_over_blocks(b):
     # eight blocks per worker with eight samples each, with nine and a short last one, and with 130 each (two chunks of

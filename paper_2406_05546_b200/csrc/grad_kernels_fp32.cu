@@ -169,15 +169,15 @@ __global__ void __launch_bounds__(256) conv1_bwd(GradStepArgs a, WorkerTable wt,
 // `per_block` of them.  With few workers the time is a thread's chain of loads, so its terms are fetched eight at a time.
 constexpr int RED_OUTPUTS = C2_GRAD + C1_GRAD + (NCLS * HID + HID + NCLS) + 1 + (P_PAD - P);
 
-// p[0] + p[stride] + ... (n terms, in order), eight loads in flight
+// p[0] + p[stride] + ... (n terms), eight loads in flight.  Eight terms are added in pairs before they join the sum: it rounds
+// an eighth as often, and the error of a few hundred terms stays near a single rounding.
 __device__ __forceinline__ float sum_slots(const float* p, int n, int64_t stride) {
   float t = 0.f;
   for (int c = 0; c < n; c += 8) {
     float v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) v[u] = c + u < n ? p[(c + u) * stride] : 0.f;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) t += v[u];
+    t += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
   }
   return t;
 }
@@ -221,8 +221,9 @@ __global__ void __launch_bounds__(256) conv_grad_reduce(GradStepArgs a, WorkerTa
 // snapshot).  The 512-unit layer's weight gradient arrives as n_super partial vectors (one per group of workers whose
 // samples went through one product), every other tensor as the per-worker, per-block partial sums the per-worker
 // reduction also reads; everything is added in a fixed order.  Blocks 0 .. FUSED_W1_BLOCKS - 1 take the float4 columns of
-// the big tensor, the rest 32 small outputs each: warp w of eight adds the partial sums of workers w, w + 8, ... (lane =
-// output, so a warp's loads are consecutive), then the warps' sums are added in order.
+// the big tensor, the rest 32 small outputs each: warp w of eight adds the partial sums of workers w, w + 8, ... in four sums
+// taken in turn (lane = output, so a warp's loads are consecutive), then the four and the warps' sums are added in pairs: no
+// sum is longer than those of one lane in 32 were when a warp shared an output.
 constexpr int FUSED_W1_VEC = HID * FLAT / 4;                                 // 200,704 float4
 constexpr int FUSED_W1_BLOCKS = (FUSED_W1_VEC + 255) / 256;                  // 784
 constexpr int FUSED_SMALL = C2_GRAD + C1_GRAD + (NCLS * HID + HID + NCLS) + (P_PAD - P);
@@ -252,14 +253,23 @@ __global__ void __launch_bounds__(256) fused_finish(GradStepArgs a, WorkerTable 
   const int o = (blockIdx.x - FUSED_W1_BLOCKS) * 32 + lane;
   if (blockIdx.x == FUSED_W1_BLOCKS && threadIdx.x < a.W)        // the per-worker losses ride along (W <= 256)
     a.loss[wt.src[threadIdx.x]] = sum_slots(ws.partf + (int64_t)threadIdx.x * split * FC_PART + NCLS * HID + HID + NCLS, split, FC_PART) * (1.0f / (float)b);
+  auto sum_workers = [&](auto worker_sum) {
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int s = warp; s < a.W; s += 32) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (s + 8 * u < a.W) v[u] += worker_sum(s + 8 * u);
+    }
+    return (v[0] + v[1]) + (v[2] + v[3]);
+  };
   float t = 0.f;
   float* dst = nullptr;
   if (o < C2_GRAD) {
-    for (int s = warp; s < a.W; s += 8) t += sum_slots(ws.part2 + (int64_t)s * n_chunks2 * C2_GRAD + o, used_slots(s, b, seg_len, n_chunks2), C2_GRAD);
+    t = sum_workers([&](int s) { return sum_slots(ws.part2 + (int64_t)s * n_chunks2 * C2_GRAD + o, used_slots(s, b, seg_len, n_chunks2), C2_GRAD); });
     dst = grad_sum + OFF_C2W + o;
   } else if (o < C2_GRAD + C1_GRAD) {
     const int oo = o - C2_GRAD;
-    for (int s = warp; s < a.W; s += 8) t += sum_slots(ws.part1 + (int64_t)s * n_chunks * C1_GRAD + oo, used_slots(s, b, seg_len1, n_chunks), C1_GRAD);
+    t = sum_workers([&](int s) { return sum_slots(ws.part1 + (int64_t)s * n_chunks * C1_GRAD + oo, used_slots(s, b, seg_len1, n_chunks), C1_GRAD); });
     dst = grad_sum + OFF_C1W + oo;
   } else if (o < C2_GRAD + C1_GRAD + NCLS * HID + HID + NCLS) {
     const int oo = o - C2_GRAD - C1_GRAD, n = a.W * split, per = (n + 7) / 8;      // all workers' slots lie end to end
@@ -272,9 +282,8 @@ __global__ void __launch_bounds__(256) fused_finish(GradStepArgs a, WorkerTable 
   warp_sum[warp][lane] = t;
   __syncthreads();
   if (warp != 0 || !dst) return;
-#pragma unroll
-  for (int w = 1; w < 8; ++w) t += warp_sum[w][lane];
-  *dst = t;
+  *dst = ((warp_sum[0][lane] + warp_sum[1][lane]) + (warp_sum[2][lane] + warp_sum[3][lane])) +
+         ((warp_sum[4][lane] + warp_sum[5][lane]) + (warp_sum[6][lane] + warp_sum[7][lane]));
 }
 
 // ---- evaluation: per worker, the mean loss from the output-layer kernel's partial sums and the number of samples

@@ -529,6 +529,29 @@ def test_summed_step_equals_the_sum_of_the_workers_gradients_and_the_sync_update
     srv.close()
 
 
+@pytest.mark.parametrize("precision", [0, 2])
+def test_summed_step_adds_the_workers_in_pairs(precision):
+    """128 workers' gradients of the output layer are added up within the root of 1 + 1/2 + 1/4 + ... < 2 of one rounding's
+    root mean square, 2^-24 / sqrt(3), as sums in pairs are: the last rounding counts in full, those of the two halves by
+    half each, and so on."""
+    W = b = 128
+    torch, ps, srv, _ = _setup(W, b, precision=precision)
+    gen = torch.Generator(device="cuda").manual_seed(W * b)
+    x = torch.rand((W, b, 28, 28), generator=gen, device="cuda")
+    y = torch.randint(0, 10, (W, b), generator=gen, device="cuda", dtype=torch.int32)
+    snaps = [srv.ps_pull_snapshot(w) for w in range(W)]
+    grads = torch.zeros((W, ps.P_PAD), device="cuda")
+    srv.workers_grad_step(snaps, range(W), x, y, SEED, 1, grads_dev=grads)
+    got = srv.workers_grad_step_summed(snaps, range(W), x, y, SEED, 1)[0].double()
+    want = grads.double().sum(0)
+    for name, o, shape in synth.layout():
+        if name in ("fc1.b", "fc2.w"):
+            part = slice(o, o + int(np.prod(shape)))
+            error = float((got[part] - want[part]).norm() / want[part].norm())
+            assert error <= 2.0 ** -24 * (2 / 3) ** 0.5, (name, error)
+    srv.close()
+
+
 def test_summed_step_refuses_mixed_snapshots():
     torch, ps, srv, theta0 = _setup(2, 4, 2, 0.25, 0)
     g = np.zeros((1, ps.P_PAD), dtype=np.float32)

@@ -157,8 +157,11 @@ inline int group_tiles(const GroupTable& gt, int b, int tm) {
   return t;
 }
 
-// Host: launches a kernel that may start before the one before it in the stream has ended (see pdl_enter).  Not where the
-// stream has just been made to wait for another one: `overlap` false is a plain launch.
+// Host: launches a kernel that may start before the one before it in the stream has ended (see pdl_enter).  The attribute lifts
+// the dependence on that kernel only: a wait for another stream's event holds back all work behind it, this launch included.
+// Where the launch code has put such a wait just before the kernel there is nothing to overlap, and `overlap` false makes it a
+// plain launch; where the caller has, out of this code's sight, the kernel starts when the wait is over and finds the kernel
+// before it ended or waits for it.
 template <typename... P, typename... A>
 inline void launch_pdl_if(bool overlap, void (*fn)(P...), dim3 grid, int threads, int smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};

@@ -208,7 +208,7 @@ int launch_conv1_fwd_planes(const GradStepArgs& a, const WorkerTable& wt, const 
   const int slots = C1_BLOCKS_PER_SM * g_sm_count, rows = a.W * a.b;
   const int spb = rows <= slots ? 1 : (rows <= 2 * slots ? 2 : C1_SPB);
   const int chunks = (a.b + spb - 1) / spb;
-  TIMED(K_CONV1_FWD, launch_pdl(conv1_fwd_planes, dim3(chunks, a.W + (gt.n_groups * BANK2_UNITS + chunks - 1) / chunks), C1_THREADS, C1_SMEM, st, xmap, a, wt, gt, ws, spb, conv2_fwd_taps()));
+  TIMED(K_CONV1_FWD, launch_pdl_if(!a.after_wait, conv1_fwd_planes, dim3(chunks, a.W + (gt.n_groups * BANK2_UNITS + chunks - 1) / chunks), C1_THREADS, C1_SMEM, st, xmap, a, wt, gt, ws, spb, conv2_fwd_taps()));
   return 1;
 }
 

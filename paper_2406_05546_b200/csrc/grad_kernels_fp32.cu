@@ -341,7 +341,7 @@ static int samples_per_block(int rows, int least, int most) {
 }
 static void launch_conv1_fwd(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof) {
   const int spb = samples_per_block(a.W * a.b, 1, CONV1_SPB);
-  TIMED(K_CONV1_FWD, launch_pdl(conv1_fwd, dim3((a.b + spb - 1) / spb, a.W), 224, 0, st, a, wt, gt, ws, spb));
+  TIMED(K_CONV1_FWD, launch_pdl_if(!a.after_wait, conv1_fwd, dim3((a.b + spb - 1) / spb, a.W), 224, 0, st, a, wt, gt, ws, spb));
 }
 
 // Evaluation pass: the forward kernels of the grad step with the dropout switched off, then the per-worker loss and hit

@@ -396,9 +396,9 @@ static void prep_done(ps_ctx* x, const psk::GroupTable& gt) {
   for (int g = 0; g < gt.n_groups; ++g) x->prep_theta[g] = gt.theta[g];
 }
 
-int32_t workers_grad_step(ps_ctx* x, int32_t W, int32_t b, const ps_snapshot* snaps, const int32_t* worker_ids,
-                          const float* x_dev, const int32_t* y_dev, uint64_t seed, uint64_t step,
-                          const int64_t* slot_ids, float* grads_dev, float* loss_dev, int32_t* argmax_dev) {
+static int32_t grad_step(ps_ctx* x, int32_t W, int32_t b, const ps_snapshot* snaps, const int32_t* worker_ids,
+                         const float* x_dev, const int32_t* y_dev, uint64_t seed, uint64_t step,
+                         const int64_t* slot_ids, float* grads_dev, float* loss_dev, int32_t* argmax_dev, bool after_wait) {
   if (!x || !snaps || !worker_ids || !x_dev || !y_dev || !loss_dev || !argmax_dev) return fail(PS_ERR_BAD_ARG, "NULL argument");
   if (W < 1 || W > x->cfg.max_workers || b < 1 || b > x->cfg.max_batch) return fail(PS_ERR_BAD_ARG, "W=%d, b=%d outside 1..%d, 1..%d", W, b, x->cfg.max_workers, x->cfg.max_batch);
   if (!slot_ids && !grads_dev) return fail(PS_ERR_BAD_ARG, "neither slot_ids nor grads_dev given");
@@ -410,6 +410,7 @@ int32_t workers_grad_step(ps_ctx* x, int32_t W, int32_t b, const ps_snapshot* sn
   a.W = W; a.b = b; a.x = x_dev; a.y = y_dev; a.loss = loss_dev; a.argmax = argmax_dev;
   a.seed = seed; a.step = step; a.drop_p = x->cfg.dropout_p; a.drop_thresh = x->drop_thresh;
   a.precision = x->cfg.precision;
+  a.after_wait = after_wait;
   if (a.precision != PS_FP32 && ((uintptr_t)x_dev & 15) != 0) return fail(PS_ERR_BAD_ARG, "x_dev must be 16-byte aligned on the tensor-core path");
   a.skip_prep_w1 = prep_is_current(x, gt);
   int n = psk::launch_grad_step(a, wt, gt, x->ws, x->st, x->prof.on ? psk::SideStreams() : x->side, &x->prof);
@@ -417,6 +418,12 @@ int32_t workers_grad_step(ps_ctx* x, int32_t W, int32_t b, const ps_snapshot* sn
   if (n < 0) return cuda_fail(cudaGetLastError(), "grad step launch");
   x->launches += n;
   return PS_OK;
+}
+
+int32_t workers_grad_step(ps_ctx* x, int32_t W, int32_t b, const ps_snapshot* snaps, const int32_t* worker_ids,
+                          const float* x_dev, const int32_t* y_dev, uint64_t seed, uint64_t step,
+                          const int64_t* slot_ids, float* grads_dev, float* loss_dev, int32_t* argmax_dev) {
+  return grad_step(x, W, b, snaps, worker_ids, x_dev, y_dev, seed, step, slot_ids, grads_dev, loss_dev, argmax_dev, false);
 }
 
 int32_t workers_grad_step_summed(ps_ctx* x, int32_t W, int32_t b, const ps_snapshot* snaps, const int32_t* worker_ids,
@@ -902,8 +909,8 @@ int32_t ps_tick_host_submit(ps_ctx* x, int32_t W, int32_t b, const int32_t* lags
     if (w0 >= w1) break;
     const size_t r0 = (size_t)w0 * b;
     CUDA_TRY(cudaStreamWaitEvent(x->st, x->copy_ev[4 * set + c], 0));
-    rc = workers_grad_step(x, w1 - w0, b, snaps + w0, ids + w0, xs + r0 * PS_IMAGE_PIXELS, ys + r0, seed, step,
-                           slots + w0, nullptr, x->loss_stage[set] + w0, x->argmax_stage[set] + r0);
+    rc = grad_step(x, w1 - w0, b, snaps + w0, ids + w0, xs + r0 * PS_IMAGE_PIXELS, ys + r0, seed, step,
+                   slots + w0, nullptr, x->loss_stage[set] + w0, x->argmax_stage[set] + r0, true);
     if (rc != PS_OK) { cudaStreamSynchronize(x->copy_st); return rc; }
   }
   CUDA_TRY(cudaEventRecord(x->stage_free[set], x->st));

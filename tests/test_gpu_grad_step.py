@@ -450,6 +450,70 @@ def test_pipelined_ticks_equal_sequential_ticks(precision):
     assert (a[0] == p[0]).all() and (a[2] == p[2]).all() and (a[3] == p[3]).all()
 
 
+@pytest.mark.parametrize("precision,W,b", [(0, 9, 114), (2, 13, 960)])
+def test_pipelined_ticks_in_several_chunks_equal_resident_ones(precision, W, b):
+    """Two and four chunks, two ticks in flight: copies run beside the kernels of the chunk, and of the tick, before.  Every
+    chunk is a grad step of its own, so the resident ticks take the same workers in the same calls."""
+    import torch
+    from paper_2406_05546_b200 import ps
+    theta0, T = synth.init_params(seed=1, bias_scale=0.05), 3
+    gen = torch.Generator().manual_seed(3)
+    xs = [torch.rand((W, b, 28, 28), generator=gen).pin_memory() for _ in range(T)]
+    ys = [torch.randint(0, 10, (W, b), generator=gen, dtype=torch.int32).pin_memory() for _ in range(T)]
+    per = -(-W // (4 if W * b >= 12288 else 2))
+    out = []
+    for host in (True, False):
+        srv = ps.ParameterServer(theta0, max_workers=W, max_batch=b, queue_slots=W, precision=precision)
+        loss, am = torch.zeros((T, W)).pin_memory(), torch.zeros((T, W, b), dtype=torch.int32).pin_memory()
+        if host:
+            for t in range(T):
+                if t >= 2:
+                    srv.ps_tick_host_wait()
+                srv.ps_tick_host_submit(xs[t], ys[t], SEED, t, ps.SYNC, 0.01, loss_host=loss[t], argmax_host=am[t])
+            srv.ps_tick_host_wait(); srv.ps_tick_host_wait()
+        else:
+            for t in range(T):
+                x, y, snap, slots = xs[t].cuda(), ys[t].cuda(), srv.ps_pull_snapshot(0), srv.ps_queue_reserve(W)
+                for w0 in range(0, W, per):
+                    part = slice(w0, min(W, w0 + per))
+                    l, a = srv.workers_grad_step([snap] * len(range(W)[part]), range(W)[part], x[part], y[part], SEED, t, slot_ids=slots[part])
+                    loss[t, part], am[t, part] = l.cpu(), a.cpu()
+                srv.ps_enqueue(range(W), [snap.version] * W, t, slot_ids=slots)
+                srv.ps_apply(ps.SYNC, 0.01)
+        out.append((srv.ps_export_params()[0], loss.numpy().copy(), am.numpy().copy()))
+        srv.ps_stats()
+        srv.close()
+    for h, r in zip(*out):
+        assert (h == r).all()
+
+
+@pytest.mark.parametrize("precision", [0, 2])
+def test_a_grad_step_behind_a_wait_for_another_stream_reads_what_that_stream_wrote(precision):
+    """The images are still on their way, on another stream, when the grad step is enqueued right behind an update: the
+    stream's wait for them holds its first kernel back too, which is launched to overlap the kernel before it."""
+    import torch
+    W, b = 4, 32
+    _, ps, srv, _ = _setup(W, b, precision=precision)
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    y = torch.randint(0, 10, (W, b), generator=gen, device="cuda", dtype=torch.int32)
+    new = torch.rand((W, b, 28, 28), generator=gen, device="cuda")
+    x, other = torch.zeros_like(new), torch.cuda.Stream()
+    update = torch.zeros((1, ps.P_PAD), device="cuda")
+    grads = torch.zeros((2, W, ps.P_PAD), device="cuda")
+    torch.cuda.synchronize()
+    for late in (1, 0):
+        srv.ps_enqueue([0], [0], 0, grads_dev=update)
+        if late:
+            with torch.cuda.stream(other):
+                torch.cuda._sleep(20_000_000)      # about ten milliseconds
+                x.copy_(new)
+        srv.ps_apply(ps.SYNC, 0.01)
+        torch.cuda.current_stream().wait_stream(other)
+        srv.workers_grad_step([srv.ps_pull_snapshot(w) for w in range(W)], range(W), x, y, SEED, 1, grads_dev=grads[late])
+    assert (grads[0] != 0).any() and torch.equal(grads[0], grads[1])
+    srv.close()
+
+
 @pytest.mark.parametrize("precision,W,b,lags", [(0, 3, 17, None), (2, 3, 17, None), (2, 4, 150, [1, 0, 0, 1]), (0, 1, 1, None)])
 def test_evaluation_pass_matches_the_oracle(precision, W, b, lags):
     """workers_eval: forward only, no dropout; loss, labels and the count of correct labels per group."""

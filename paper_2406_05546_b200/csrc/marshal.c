@@ -186,8 +186,7 @@ static PyObject* grad_step(PyObject* m, PyObject* const* a, Py_ssize_t nargs) {
   if (as_ptr(a[0], &ctx) || i32(a[1], &W) || i32(a[2], &b) || as_ptr(a[5], &x) || as_ptr(a[6], &y) || as_u64(a[7], &seed) ||
       as_u64(a[8], &step) || as_ptr(a[10], &grads) || as_ptr(a[11], &loss) || as_ptr(a[12], &argmax))
     return NULL;
-  if (W > PS_MAX_WORKERS) W = PS_MAX_WORKERS + 1;          /* the library refuses it */
-  else if (snapshots(a[3], W, snaps)) return NULL;
+  if (W <= PS_MAX_WORKERS && snapshots(a[3], W, snaps)) return NULL;      /* of more workers the library reads nothing: it refuses the call */
   if (array(a[4], &ids, I32)) return NULL;
   if (array(a[9], &slots, I64)) { done(&ids); return NULL; }
   if (!ids.obj || ids.ndim != 1 || ids.len != (Py_ssize_t)W * 4) PyErr_SetString(PyExc_AssertionError, "one worker id per worker is wanted");
@@ -213,8 +212,7 @@ static PyObject* grad_step_summed(PyObject* m, PyObject* const* a, Py_ssize_t na
   if (as_ptr(a[0], &ctx) || i32(a[1], &W) || i32(a[2], &b) || as_ptr(a[5], &x) || as_ptr(a[6], &y) || as_u64(a[7], &seed) ||
       as_u64(a[8], &step) || as_ptr(a[9], &sum) || as_ptr(a[10], &loss) || as_ptr(a[11], &argmax))
     return NULL;
-  if (W > PS_MAX_WORKERS) W = PS_MAX_WORKERS + 1;
-  else if (snapshots(a[3], W, snaps)) return NULL;
+  if (W <= PS_MAX_WORKERS && snapshots(a[3], W, snaps)) return NULL;
   if (array(a[4], &ids, I32)) return NULL;
   if (!long_enough(&ids, W, 4)) { done(&ids); return NULL; }
   int32_t rc;
@@ -234,8 +232,7 @@ static PyObject* eval(PyObject* m, PyObject* const* a, Py_ssize_t nargs) {
   if (as_ptr(a[0], &ctx) || i32(a[1], &W) || i32(a[2], &b) || as_ptr(a[4], &x) || as_ptr(a[5], &y) || as_ptr(a[6], &loss) ||
       as_ptr(a[7], &argmax) || as_ptr(a[8], &correct))
     return NULL;
-  if (W > PS_MAX_WORKERS) W = PS_MAX_WORKERS + 1;
-  else if (snapshots(a[3], W, snaps)) return NULL;
+  if (W <= PS_MAX_WORKERS && snapshots(a[3], W, snaps)) return NULL;
   int32_t rc;
   CALL(f_eval((ps_ctx*)ctx, W, b, snaps, (const float*)x, (const int32_t*)y, (float*)loss, (int32_t*)argmax, (int32_t*)correct))
   if (rc) return raise(rc);

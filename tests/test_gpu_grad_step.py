@@ -369,6 +369,19 @@ def test_argument_errors():
     srv.close()
 
 
+@pytest.mark.parametrize("W", [257, 300])
+def test_more_workers_than_any_server_takes_are_refused_by_the_library(W):
+    torch, ps, srv, _ = _setup(2, 1)
+    x, y = torch.zeros((W, 1, 28, 28), device="cuda"), torch.zeros((W, 1), dtype=torch.int32, device="cuda")
+    snaps = [srv.ps_pull_snapshot(0)] * W
+    for call in (lambda: srv.workers_grad_step(snaps, list(range(W)), x, y, SEED, 0, grads_dev=torch.zeros((W, ps.P_PAD), device="cuda")),
+                 lambda: srv.workers_grad_step_summed(snaps, list(range(W)), x, y, SEED, 0), lambda: srv.workers_eval(snaps, x, y)):
+        with pytest.raises(ps.PSError) as e:
+            call()
+        assert e.value.name == "PS_ERR_BAD_ARG" and "outside" in str(e.value)
+    srv.close()
+
+
 # 1,026 rows: two chunks on the FP32 path; 12,480 rows: four, the last of one worker
 @pytest.mark.parametrize("precision,W,b", [(0, 3, 4), (0, 9, 5), (2, 9, 5), (2, 8, 16), (0, 9, 114), (2, 13, 960)])
 def test_tick_from_host_buffers_matches_the_oracle(precision, W, b):

@@ -7,6 +7,7 @@
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "ps.h"
 
@@ -22,7 +23,9 @@ static int32_t (*f_apply)(ps_ctx*, ps_mode, float, float, const int32_t*, ps_app
 static int32_t (*f_apply_stale)(ps_ctx*, ps_mode, float, float, const int32_t*, float, float, ps_apply_result*);
 static int32_t (*f_apply_summed)(ps_ctx*, const float*, int32_t, float, float, ps_apply_result*);
 static const char* (*f_error)(ps_ctx*);
-static PyObject *snapshot_type, *error_type, *as_array;   /* as_array(object, kind): numpy's conversion to a contiguous array */
+static PyObject *snapshot_type, *error_type;
+static PyObject *as_array;       /* as_array(object, kind): numpy's conversion to a contiguous array */
+static PyObject *as_snapshots;   /* as_snapshots(sequence, n): ctypes' conversion to an array of n structures */
 static PyObject *k_applied, *k_version, *k_checkpointed, *k_replicated;
 
 static PyObject* raise(int32_t rc) {
@@ -93,19 +96,28 @@ static int long_enough(const Py_buffer* b, Py_ssize_t n, Py_ssize_t item) {
   return 0;
 }
 
-/* The snapshots of a call, out of their structures. */
+/* The snapshots of a call, out of their structures.  Anything but a list or tuple of n Snapshots goes through ctypes, which
+ * converts or refuses it. */
 static int snapshots(PyObject* seq, Py_ssize_t n, ps_snapshot* out) {
-  PyObject* fast = PySequence_Fast(seq, "snaps must be a sequence");
-  if (!fast) return -1;
-  if (PySequence_Fast_GET_SIZE(fast) != n) { Py_DECREF(fast); PyErr_SetString(PyExc_ValueError, "one snapshot per worker is wanted"); return -1; }
-  for (Py_ssize_t i = 0; i < n; ++i) {
-    Py_buffer b;
-    if (PyObject_GetBuffer(PySequence_Fast_GET_ITEM(fast, i), &b, PyBUF_SIMPLE)) { Py_DECREF(fast); return -1; }
-    if (b.len != (Py_ssize_t)sizeof(ps_snapshot)) { PyBuffer_Release(&b); Py_DECREF(fast); PyErr_SetString(PyExc_TypeError, "snaps must hold Snapshot structures"); return -1; }
-    out[i] = *(const ps_snapshot*)b.buf;
-    PyBuffer_Release(&b);
+  Py_buffer b;
+  Py_ssize_t i = 0;
+  if ((PyList_CheckExact(seq) || PyTuple_CheckExact(seq)) && PySequence_Fast_GET_SIZE(seq) == n) {
+    for (; i < n; ++i) {
+      PyObject* o = PySequence_Fast_GET_ITEM(seq, i);
+      if ((PyObject*)Py_TYPE(o) != snapshot_type) break;
+      if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE)) return -1;
+      out[i] = *(const ps_snapshot*)b.buf;
+      PyBuffer_Release(&b);
+    }
+    if (i == n) return 0;
   }
-  Py_DECREF(fast);
+  PyObject* c = PyObject_CallFunction(as_snapshots, "On", seq, n);
+  if (!c) return -1;
+  const int rc = PyObject_GetBuffer(c, &b, PyBUF_SIMPLE);
+  Py_DECREF(c);
+  if (rc) return -1;
+  memcpy(out, b.buf, (size_t)n * sizeof(ps_snapshot));
+  PyBuffer_Release(&b);
   return 0;
 }
 
@@ -127,7 +139,7 @@ static PyObject* result(const ps_apply_result* r) {
 #define WANT(n) if (nargs != (n)) { PyErr_SetString(PyExc_TypeError, "wrong number of arguments"); return NULL; }
 
 static PyObject* bind(PyObject* m, PyObject* const* a, Py_ssize_t nargs) {
-  WANT(4)
+  WANT(5)
   static const struct { const char* name; void** f; } table[] = {
       {"ps_pull_snapshot", (void**)&f_pull}, {"ps_queue_reserve", (void**)&f_reserve}, {"workers_grad_step", (void**)&f_grad},
       {"workers_grad_step_summed", (void**)&f_summed}, {"workers_eval", (void**)&f_eval}, {"ps_enqueue", (void**)&f_enqueue},
@@ -144,6 +156,8 @@ static PyObject* bind(PyObject* m, PyObject* const* a, Py_ssize_t nargs) {
   Py_XSETREF(error_type, a[2]);
   Py_INCREF(a[3]);
   Py_XSETREF(as_array, a[3]);
+  Py_INCREF(a[4]);
+  Py_XSETREF(as_snapshots, a[4]);
   Py_RETURN_NONE;
 }
 

@@ -116,7 +116,8 @@ def load(path=None):
         m.bind({n: C.cast(getattr(L, n), C.c_void_p).value for n in
                 ("ps_pull_snapshot", "ps_queue_reserve", "workers_grad_step", "workers_grad_step_summed", "workers_eval",
                  "ps_enqueue", "ps_apply", "ps_apply_stale", "ps_apply_summed", "ps_last_error")}, Snapshot, PSError,
-               lambda o, kind: np.ascontiguousarray(o, dtype=(np.int32, np.int64, np.uint64)[kind]))
+               lambda o, kind: np.ascontiguousarray(o, dtype=(np.int32, np.int64, np.uint64)[kind]),
+               lambda snaps, n: (Snapshot * n)(*snaps))
         _lib, _marshal = L, m
     return L
 

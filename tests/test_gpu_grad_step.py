@@ -382,6 +382,26 @@ def test_more_workers_than_any_server_takes_are_refused_by_the_library(W):
     srv.close()
 
 
+def test_snapshots_of_a_call_in_every_form():
+    """A generator, an array of structures and plain pairs are snapshots; too few of them leave workers without weights, which
+    the library refuses; too many, and what is no snapshot although it has a snapshot's size, are refused by ctypes."""
+    torch, ps, srv, _ = _setup(2, 1)
+    x, y = torch.rand((2, 1, 28, 28), device="cuda"), torch.zeros((2, 1), dtype=torch.int32, device="cuda")
+    s = srv.ps_pull_snapshot(0)
+    want = srv.workers_eval([s, s], x, y)[0]
+    for form in ((s, s), iter([s, s]), (ps.Snapshot * 2)(s, s), [(s.version, s.dev_ptr)] * 2):
+        assert torch.equal(srv.workers_eval(form, x, y)[0], want)
+    with pytest.raises(ps.PSError) as e:
+        srv.workers_eval([s], x, y)
+    assert e.value.name == "PS_ERR_BAD_ARG" and "no weights" in str(e.value)
+    with pytest.raises(IndexError):
+        srv.workers_eval([s] * 3, x, y)
+    for other in (np.array([s.version, s.dev_ptr], dtype=np.uint64), bytes(s)):
+        with pytest.raises(TypeError):
+            srv.workers_eval([other, other], x, y)
+    srv.close()
+
+
 # 1,026 rows: two chunks on the FP32 path; 12,480 rows: four, the last of one worker
 @pytest.mark.parametrize("precision,W,b", [(0, 3, 4), (0, 9, 5), (2, 9, 5), (2, 8, 16), (0, 9, 114), (2, 13, 960)])
 def test_tick_from_host_buffers_matches_the_oracle(precision, W, b):

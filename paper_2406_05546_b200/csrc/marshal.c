@@ -34,35 +34,30 @@ static PyObject* raise(int32_t rc) {
   return NULL;
 }
 
-/* Integer arguments: anything int() takes. */
-static int as_i64(PyObject* o, int64_t* v) {
-  PyObject* i = PyNumber_Long(o);
-  if (!i) return -1;
-  *v = PyLong_AsLongLong(i);
-  Py_DECREF(i);
-  return *v == -1 && PyErr_Occurred() ? -1 : 0;
-}
-static int as_u64(PyObject* o, uint64_t* v) {      /* wraps like a C conversion */
+/* Integer arguments: anything int() takes, wrapped like a C conversion, as ctypes does it. */
+static int as_u64(PyObject* o, uint64_t* v) {
   PyObject* i = PyNumber_Long(o);
   if (!i) return -1;
   *v = PyLong_AsUnsignedLongLongMask(i);
   Py_DECREF(i);
   return PyErr_Occurred() ? -1 : 0;
 }
+static int i32(PyObject* o, int32_t* v) {
+  uint64_t w;
+  if (as_u64(o, &w)) return -1;
+  *v = (int32_t)(uint32_t)w;
+  return 0;
+}
 static int as_ptr(PyObject* o, void** p) {         /* None or an address */
   if (o == Py_None) { *p = NULL; return 0; }
   *p = PyLong_AsVoidPtr(o);
   return !*p && PyErr_Occurred() ? -1 : 0;
 }
-static int as_float(PyObject* o, float* v) {
-  *v = (float)PyFloat_AsDouble(o);
-  return PyErr_Occurred() ? -1 : 0;
-}
-static int i32(PyObject* o, int32_t* v) {
-  int64_t w;
-  if (as_i64(o, &w)) return -1;
-  if (w < INT32_MIN || w > INT32_MAX) { PyErr_SetString(PyExc_OverflowError, "value does not fit 32 bits"); return -1; }
-  *v = (int32_t)w;
+static int as_float(PyObject* o, float* v) {       /* anything float() takes */
+  PyObject* f = PyNumber_Float(o);
+  if (!f) return -1;
+  *v = (float)PyFloat_AS_DOUBLE(f);
+  Py_DECREF(f);
   return 0;
 }
 
@@ -177,13 +172,14 @@ static PyObject* pull(PyObject* m, PyObject* const* a, Py_ssize_t nargs) {
   return s;
 }
 
-/* (ctx, ids int64[n]) */
+/* (ctx, n, ids int64[n]) */
 static PyObject* reserve(PyObject* m, PyObject* const* a, Py_ssize_t nargs) {
-  WANT(2)
+  WANT(3)
   void* ctx;
+  int32_t n;
   Py_buffer b;
-  if (as_ptr(a[0], &ctx) || PyObject_GetBuffer(a[1], &b, PyBUF_WRITABLE)) return NULL;
-  const int32_t rc = f_reserve((ps_ctx*)ctx, (int32_t)(b.len / 8), (int64_t*)b.buf);
+  if (as_ptr(a[0], &ctx) || i32(a[1], &n) || PyObject_GetBuffer(a[2], &b, PyBUF_WRITABLE)) return NULL;
+  const int32_t rc = f_reserve((ps_ctx*)ctx, n, (int64_t*)b.buf);
   PyBuffer_Release(&b);
   if (rc) return raise(rc);
   Py_RETURN_NONE;

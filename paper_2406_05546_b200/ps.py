@@ -199,7 +199,7 @@ class ParameterServer:
 
     def ps_queue_reserve(self, n):
         ids = np.empty(n, dtype=np.int64)
-        _marshal.reserve(self._addr, ids)
+        _marshal.reserve(self._addr, n, ids)
         return ids
 
     def ps_slot_ptr(self, slot):
@@ -263,7 +263,8 @@ class ParameterServer:
 
     def ps_enqueue(self, worker_ids, base_versions, step, slot_ids=None, grads_dev=None):
         if grads_dev is not None:
-            n = len(worker_ids)
+            worker_ids = np.ascontiguousarray(worker_ids, dtype=np.int32)
+            n = worker_ids.shape[0]
             assert grads_dev.is_cuda and grads_dev.dtype == self._torch.float32 and grads_dev.shape == (n, P_PAD) and grads_dev.is_contiguous()
         _marshal.enqueue(self._addr, slot_ids, grads_dev.data_ptr() if grads_dev is not None else None, worker_ids, base_versions, step)
 

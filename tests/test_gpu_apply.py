@@ -583,6 +583,26 @@ def test_the_binding_reads_integers_in_every_form(form):
     assert (got[0] == got[1]).all() and (got[0] != theta).any()
 
 
+def test_the_binding_takes_numbers_as_int_and_float_do():
+    """One worker's id and version need no list; numbers may be text or arrays without a dimension; a count that int() refuses is refused."""
+    _, ps, _, _ = _pair(queue_slots=8)
+    theta, grad, got = synth.init_params(seed=1), _pad(synth.random_gradients(1, seed=3)), []
+    for worker, base, lr, mode in ((0, 0, "0.01", str(ps.SYNC)), (np.int64(0), np.array(0), np.float32(0.01), np.array(ps.SYNC)), ([0], [0], 0.01, ps.SYNC)):
+        srv = ps.ParameterServer(theta, max_batch=1, max_workers=8, queue_slots=8)
+        srv.ps_enqueue(worker, base, 0, grads_dev=grad)
+        assert srv.ps_apply(mode, lr)["applied"] == 1
+        got.append(srv.ps_export_params()[0])
+        for n in ((2, 3), [3], 2.0):
+            with pytest.raises(TypeError):
+                srv.ps_queue_reserve(n)
+        assert len(srv.ps_queue_reserve(np.int16(3))) == 3
+        with pytest.raises(ps.PSError) as e:
+            srv.ps_pull_snapshot(2 ** 31)      # wraps to a negative worker
+        assert e.value.name == "PS_ERR_BAD_ARG"
+        srv.close()
+    assert (got[0] == got[2]).all() and (got[1] == got[2]).all() and (got[0] != theta).any()
+
+
 def test_the_binding_refuses_what_is_no_integer_array():
     _, ps, _, srv = _pair(queue_slots=8)
     g = _pad(synth.random_gradients(2, seed=3))

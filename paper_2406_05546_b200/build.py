@@ -1,5 +1,5 @@
 """Compile the CUDA library in-tree: paper_2406_05546_b200/libps_b200.so (sm_100a only), and the binding's argument
-marshalling, _marshal.so."""
+marshalling, _marshal, an extension of the running Python (with its headers and the C compiler that nvcc calls as well)."""
 import glob
 import os
 import subprocess
@@ -9,7 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libps_b200.so")
-MARSHAL = os.path.join(HERE, "_marshal.so")
+MARSHAL = os.path.join(HERE, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))      # the suffix names the Python it was built for
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 
@@ -41,7 +41,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
 def build_marshal(force: bool = False) -> str:
     src, header = os.path.join(CSRC, "marshal.c"), os.path.join(ROOT, "include", "ps.h")
     if force or not os.path.exists(MARSHAL) or any(os.path.getmtime(d) > os.path.getmtime(MARSHAL) for d in (src, header)):
-        subprocess.run(["gcc", "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"),
+        subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"),
                         "-o", MARSHAL, src], check=True)
     return MARSHAL
 

@@ -45,6 +45,14 @@ def test_struct_sizes_match_header_layout():
     assert ps.P_PAD % 64 == 0 and ps.P_PAD >= ps.P
 
 
+def test_the_marshalling_extension_is_the_running_pythons():
+    import importlib.machinery
+    from paper_2406_05546_b200 import _marshal, build
+    assert _marshal.__file__ == build.MARSHAL
+    # the suffix this Python looks for first, which names its version: another one builds its own file
+    assert build.MARSHAL.endswith(importlib.machinery.EXTENSION_SUFFIXES[0]) and len(importlib.machinery.EXTENSION_SUFFIXES[0]) > len(".so")
+
+
 def test_one_pass_clipping_is_chosen_where_it_fits_only():
     """A CTA of the one-pass kernel covers up to 1,408 of the 203,328 float4 columns: 145 SMs cover them all, 144 do not."""
     fits = ps.load()["_ZN3psk13clip_sum_fitsEi"]

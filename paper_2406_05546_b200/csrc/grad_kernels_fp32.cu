@@ -357,7 +357,7 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
     if (n < 0) return -1;
     launches += 2 + n;
   } else {
-      launch_conv1_fwd(a, wt, gt, ws, st, prof);
+    launch_conv1_fwd(a, wt, gt, ws, st, prof);
     launch_conv2_direct(true, a, gt, ws, st, prof);
     launch_fc1_fwd_fp32(a, wt, gt, ws, st, prof);
     launches += 3;

@@ -22,12 +22,6 @@ namespace psk {
 
 namespace {
 
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
 // ------------------------------------------------------------------------------------------------
 // Forward (FWD) and input gradient.  A block takes up to SPB samples that share a weight snapshot and NC of the output
 // channels (blockIdx.y).  The input of CH channels at a time lies in zero-bordered planes (position (y, x) at row
@@ -79,15 +73,16 @@ __global__ void __launch_bounds__(conv_threads<SPB>(), SPB > 1 ? 2 : 1) conv2_di
     if (FWD) cp_async_commit();
   };
   auto place = [&](int buf) {      // input gradient: the fetched elements' windows, losers cleared
-    if (FWD) return;
+    if constexpr (!FWD) {
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int e = tid + k * THREADS;
-      const int sp = e / (CH * 49), rem = e - sp * (CH * 49), ch = rem / 49, p = rem - ch * 49, py = p / 7, px = p - py * 7;
-      if (e < ITEMS) {
-        float* d = planes + buf * BUF + (sp * CH + ch) * CV_PLANE + (2 * py + 1) * CV_PITCH + 2 * px + 2;
-        *reinterpret_cast<float2*>(d) = make_float2(gc[k] == 0u ? gv[k] : 0.f, gc[k] == 1u ? gv[k] : 0.f);
-        *reinterpret_cast<float2*>(d + CV_PITCH) = make_float2(gc[k] == 2u ? gv[k] : 0.f, gc[k] == 3u ? gv[k] : 0.f);
+      for (int k = 0; k < PER; ++k) {
+        const int e = tid + k * THREADS;
+        const int sp = e / (CH * 49), rem = e - sp * (CH * 49), ch = rem / 49, p = rem - ch * 49, py = p / 7, px = p - py * 7;
+        if (e < ITEMS) {
+          float* d = planes + buf * BUF + (sp * CH + ch) * CV_PLANE + (2 * py + 1) * CV_PITCH + 2 * px + 2;
+          *reinterpret_cast<float2*>(d) = make_float2(gc[k] == 0u ? gv[k] : 0.f, gc[k] == 1u ? gv[k] : 0.f);
+          *reinterpret_cast<float2*>(d + CV_PITCH) = make_float2(gc[k] == 2u ? gv[k] : 0.f, gc[k] == 3u ? gv[k] : 0.f);
+        }
       }
     }
   };
@@ -114,7 +109,7 @@ __global__ void __launch_bounds__(conv_threads<SPB>(), SPB > 1 ? 2 : 1) conv2_di
   }
   for (int c = 0; c < N_CHUNKS; ++c) {
     const int buf = c & 1;
-    if (FWD) cp_async_wait0();
+    if (FWD) cp_async_wait<0>();
     __syncthreads();                               // chunk c is complete; the other buffer is no longer read
     if (c + 1 < N_CHUNKS) fetch(c + 1, buf ^ 1);
     if (active) {
@@ -242,7 +237,7 @@ __global__ void __launch_bounds__(DW_THREADS, 2) conv2_dw_direct(GradStepArgs a,
   int s = r0 / a.b, wend = (s + 1) * a.b, seg = blockIdx.x * segs, send = r0 + seg_len;
   for (int row = r0; row < r1; ++row) {
     const int buf = (row - r0) & 1;
-    cp_async_wait0();
+    cp_async_wait<0>();
     __syncthreads();
     const bool more = row + 1 < r1;
     const bool flush = !more || row + 1 == wend || row + 1 == send;

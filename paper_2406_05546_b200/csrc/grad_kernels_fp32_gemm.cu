@@ -26,13 +26,6 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-// 16 bytes global -> shared; zeros if !valid
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(valid ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 enum { G_FWD = 0, G_DX = 1, G_DW = 2 };
 template <int OP> struct GemmShape {
   static constexpr int N = OP == G_FWD ? HID : FLAT;
@@ -198,7 +191,7 @@ __global__ void __launch_bounds__(256, 2) sgemm_tile(GradStepArgs a, WorkerTable
     if (OP == G_FWD) v = fc1_activation(v, m, n, io.theta, a, wt);
     *reinterpret_cast<float4*>(io.C + (int64_t)m * S::LDC + n) = v;
   };
-  if (SPLIT) {
+  if constexpr (SPLIT) {
     // partial tiles through distributed shared memory: rank r adds its share of the tile over all ranks in order
     cg::cluster_group cl = cg::this_cluster();
     __syncthreads();
@@ -223,20 +216,20 @@ __global__ void __launch_bounds__(256, 2) sgemm_tile(GradStepArgs a, WorkerTable
       if (m < io.m_end && n < S::N) store(m, n, v);
     }
     cl.sync();                                              // a CTA's shared memory outlives its readers
-    return;
-  }
+  } else {
 #pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    const int m = io.m0 + row_of(i);
-    if (m >= io.m_end) continue;
+    for (int i = 0; i < TM; ++i) {
+      const int m = io.m0 + row_of(i);
+      if (m >= io.m_end) continue;
 #pragma unroll
-    for (int q = 0; q < TN / 4; ++q) {
-      const int n = n0 + tx * 4 + 64 * q;
-      if (n >= S::N) continue;
-      float4 v;
-      unpack2(acc[i][2 * q], v.x, v.y);
-      unpack2(acc[i][2 * q + 1], v.z, v.w);
-      store(m, n, v);
+      for (int q = 0; q < TN / 4; ++q) {
+        const int n = n0 + tx * 4 + 64 * q;
+        if (n >= S::N) continue;
+        float4 v;
+        unpack2(acc[i][2 * q], v.x, v.y);
+        unpack2(acc[i][2 * q + 1], v.z, v.w);
+        store(m, n, v);
+      }
     }
   }
 }
@@ -244,7 +237,7 @@ __global__ void __launch_bounds__(256, 2) sgemm_tile(GradStepArgs a, WorkerTable
 // Forward product, few rows: tiles of TM x TN with RM x RN sums per thread of 128, every sum taken over k in order (a split
 // of k would change its last bits, and with them the sign of a unit whose sum lies within rounding distance of zero).  Both
 // operands stay as they lie, k contiguous; a thread takes four k of each with 16-byte loads, and steps of 32 k arrive in a
-// four-stage ring of asynchronous copies.
+// three-stage ring of asynchronous copies.
 constexpr int SQ_K = 32, SQ_PITCH = SQ_K + 4, SQ_STAGES = 3;
 template <int TM, int TN, int RM, int RN>
 __global__ void __launch_bounds__(128) sgemm_fwd_seq(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws) {
@@ -320,9 +313,6 @@ __global__ void __launch_bounds__(128) sgemm_fwd_seq(GradStepArgs a, WorkerTable
   }
 }
 
-// The same for very few rows: a tile of 16 x 16 whose operands (16 rows of each, all of k) fit into shared memory at once.
-// They arrive by asynchronous copies in seven chunks of k, all asked for at the start, so that little but the chain of a
-// sum's 1,568 multiply-adds takes time once the first chunk has landed.
 // A load the compiler leaves where it stands: it would otherwise sink every operand to its use, and the chain of
 // multiply-adds would wait for shared memory at every step.
 __device__ __forceinline__ float4 lds4(uint32_t addr) {
@@ -330,6 +320,10 @@ __device__ __forceinline__ float4 lds4(uint32_t addr) {
   asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
   return v;
 }
+
+// The same for very few rows: a tile of 16 x 16 whose operands (16 rows of each, all of k) fit into shared memory at once.
+// They arrive by asynchronous copies in seven chunks of k, all asked for at the start, so that little but the chain of a
+// sum's 1,568 multiply-adds takes time once the first chunk has landed.
 constexpr int RW_CHUNKS = 7, RW_K = FLAT / RW_CHUNKS, RW_PITCH = FLAT + 4;     // 1,572 words: rows four banks apart
 constexpr int RW_SMEM = 32 * RW_PITCH * 4;
 static_assert(RW_CHUNKS == 7 && 32 * RW_K / 4 % 128 == 0, "the waits below; whole rounds of copies");
@@ -457,7 +451,6 @@ __global__ void __launch_bounds__(256) sgemm_dx_skinny(GradStepArgs a, WorkerTab
 //   forward       16 x 16    18   19    29    52
 //                 32 x 16    22   21    22    30    40    52    74     85    105
 //                 64 x 16              29    29    48    48    56     72     89    119
-//                 64 x 32              44    44    45    46    68     68     85    103
 //                 128 x 64                                                   99     99    179     590
 //                 112 x 128                                                        162    163     562
 //                 (64 x 64 with k split over a cluster, other bits: 17 at 64 rows, 25 at 256, 37 at 512, 64 at 1024)
@@ -465,7 +458,7 @@ __global__ void __launch_bounds__(256) sgemm_dx_skinny(GradStepArgs a, WorkerTab
 //                 64 x 64    17   13    17    23          35           58           103
 //                 128 x 64                                                   61     87    162     567
 //                 112 x 128                                                         92    173     540
-// (64 x 64: k split over a cluster, about 400 CTAs, at least eight steps of k each.)
+// (64 x 64: k split over a cluster of up to four CTAs, about 400 in all, at least eight steps of k each.)
 // Beyond that the time is the number of tiles per SM times a tile's time, which for tiles taken two at a time is
 // 0.86 of a single one's: 112 x 128 tiles cost 1 alone and 1.73 as a pair, 128 x 64 tiles 0.605 and 1.1.
 template <int OP>
@@ -487,7 +480,7 @@ void run_grouped(const GradStepArgs& a, const WorkerTable& wt, const GroupTable&
     if (rows <= 1024) {
       const dim3 grid((N + 63) / 64, group_tiles(gt, a.b, 64));
       unsigned split = 1;
-      while (split < 8 && grid.x * grid.y * split * 2 <= 400u && HID / GK / (2 * split) >= 8) split *= 2;
+      while (split < 4 && grid.x * grid.y * split * 2 <= 400u) split *= 2;
       launch_cluster(sgemm_tile<OP, 4, 4, true>, dim3(grid.x, grid.y, split), 256, Tile<OP, 4, 4>::SMEM, (int)split, st, a, wt, gt, ws);
       return;
     }

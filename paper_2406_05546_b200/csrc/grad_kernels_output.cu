@@ -200,16 +200,17 @@ __global__ void __launch_bounds__(FC2_THREADS, 1) output_layer(GradStepArgs a, W
     for (int w = 0; w < FC2_THREADS / 32; ++w) t += warp_loss[w];
     part[NCLS * HID + HID + NCLS] = t;
   }
-  if (EVAL) return;
+  if constexpr (!EVAL) {
 #pragma unroll
-  for (int k = 0; k < NCLS / 2; ++k) {
-    float lo, hi;
-    unpack2(gwk[k], lo, hi);
-    part[2 * k * HID + tid] = lo;
-    part[(2 * k + 1) * HID + tid] = hi;
+    for (int k = 0; k < NCLS / 2; ++k) {
+      float lo, hi;
+      unpack2(gwk[k], lo, hi);
+      part[2 * k * HID + tid] = lo;
+      part[(2 * k + 1) * HID + tid] = hi;
+    }
+    part[NCLS * HID + tid] = gb1;
+    if (tid < NCLS) part[NCLS * HID + HID + tid] = gb2;
   }
-  part[NCLS * HID + tid] = gb1;
-  if (tid < NCLS) part[NCLS * HID + HID + tid] = gb2;
 }
 
 }  // namespace

@@ -37,8 +37,8 @@ REPLAY_TRAFFIC_PER_GRADIENT = 2.654663e9 / 816
 # dram bytes (read + written) per sample of the grad-step kernels, from one ncu capture of a reduced case
 # (W=128, b=64: 8,192 samples; traffic grows in proportion to the samples, except for fc1_dw, whose 3.2 MB of output per
 # worker do not depend on the batch: its figure holds at b = 64 only); None = not captured since the kernel changed
-KERNEL_TRAFFIC_PER_SAMPLE = {"conv2_dw": 13011, "conv1_fwd": 6939, "conv2_bwd": 5167, "fc1_dw": 51258, "conv2_fwd": 9152,
-                             "fc1_dx": 2445, "fc1_fwd": 6671, "fc2_fwd_bwd": 2060, "conv1_bwd": 12564}
+KERNEL_TRAFFIC_PER_SAMPLE = {"conv2_dw": 12990, "conv1_fwd": 6878, "conv2_bwd": 5189, "fc1_dw": 51223, "conv2_fwd": 9143,
+                             "fc1_dx": 2445, "fc1_fwd": 6684, "fc2_fwd_bwd": 2060, "conv1_bwd": 12566}
 
 
 # Algorithmic HBM bytes of the tensor-core path's grad-step kernels at (W, b): what each must read and write once

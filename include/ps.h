@@ -297,10 +297,10 @@ int32_t ps_tick_host_wait(ps_ctx* ctx, ps_apply_result* out);
 /* Exercises the give-up path of the library's bounded waits without disturbing anything (no counterpart in the
  * paper's method; it serves failure detection).  Every wait of the tensor-core kernels on a barrier has a cycle
  * limit; when it runs out the kernel sets bit 1 of the status word, releases what it holds and returns, and
- * ps_stats() then reports PS_ERR_DEVICE_STATUS.  This call launches, on the context's stream, one warp that waits on
- * a barrier of its own at which nobody arrives, for at most limit_cycles SM clock cycles (1..2e9; 20,000 is about
- * 10 microseconds), and then does exactly that.  Nothing else is touched; the context stays usable, but its status
- * word keeps the bit until the context is destroyed. */
+ * ps_stats() then reports PS_ERR_DEVICE_STATUS.  This call launches, on the context's stream, four warps, three of which
+ * wait on a complete barrier of their own and one on a barrier at which nobody arrives, for at most limit_cycles SM clock
+ * cycles (1..2e9; 20,000 is about 10 microseconds); they settle that all of them stop, and then do exactly that.  Nothing
+ * else is touched; the context stays usable, but its status word keeps the bit until the context is destroyed. */
 int32_t ps_selftest_wait_timeout(ps_ctx* ctx, int64_t limit_cycles);
 
 /* Per-kernel timing for measurement (no counterpart in the paper's method; it serves the roofline

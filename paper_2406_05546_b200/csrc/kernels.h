@@ -256,7 +256,8 @@ int launch_clip_factors(const float* queue, int64_t K, float clip, float* coef_k
 int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, int32_t* correct,
                 cudaStream_t st, Profiler* prof);
 
-// One warp waits on a barrier nobody arrives at, for at most limit_cycles, then sets STATUS_WAIT_TIMEOUT in *status.
+// One warp of four waits on a barrier nobody arrives at, for at most limit_cycles; all four then stop, and STATUS_WAIT_TIMEOUT
+// is set in *status.
 int launch_wait_timeout_probe(uint32_t* status, long long limit_cycles, cudaStream_t st);
 
 }  // namespace psk

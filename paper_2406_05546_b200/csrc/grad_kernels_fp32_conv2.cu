@@ -11,9 +11,9 @@
 // The multiply-adds are packed pairs over output channels (half the instructions; the pipe's rate is the same).
 //
 // Measured (B200, 128 workers x 128 samples, 29.6 GFLOP per product, 0.40 ms at the pipe's rate): forward 1.25 -> 0.70 ms;
-// input and filter gradient together 8.40 -> 0.64 + 0.64 ms (the former kernel did both with one multiply-add per word
+// input and filter gradient together 8.40 -> 0.64 + 0.65 ms (the former kernel did both with one multiply-add per word
 // read and skipped zero gradients with a branch that the lanes of a warp took differently).  At 2 x 8: 57 -> 13 us and
-// 402 -> 15 + 15 us.  The packed pipe is busy 62-66 % of the time (ncu); scalar multiply-adds instead: 0.78 / 0.72 /
+// 402 -> 15 + 15 us.  The FP32 pipe is busy 66 - 69 % of the time (ncu, half the samples); scalar multiply-adds instead: 0.78 / 0.72 /
 // 0.67 ms; three blocks of 8-channel threads per SM: 0.77 / 0.66 ms.
 #include "device_common.cuh"
 #include "kernels.h"

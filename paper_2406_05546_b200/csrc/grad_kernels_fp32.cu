@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(256) conv1_bwd(GradStepArgs a, WorkerTable wt,
   }
 }
 
-// ---- sums the per-block partial gradients in block order, finishes the loss and zeroes the padding.
+// ---- sums the per-block partial gradients in a fixed order, finishes the loss and zeroes the padding.
 // part1 and part2 hold n_chunks / n_chunks2 slots per worker; all of them are summed when seg_len == 0, otherwise one
 // for every range of seg_len rows that meets the worker's b rows.
 // A worker's outputs are numbered conv2 (4640), conv1 (160), output layer (5642), loss, padding; a block takes

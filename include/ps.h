@@ -65,7 +65,8 @@ enum {
   PS_ERR_DEVICE_STATUS = -9     /* a kernel's own input check tripped (e.g. a label outside 0..9) */
 };
 
-/* Arithmetic of the dense contractions of part A.  PS_FP32: everything on the FP32 pipes.  PS_BF16: the
+/* Arithmetic of the dense contractions of part A.  PS_FP32: single precision
+ * throughout; the dense layer's products run on the tensor cores with every operand as three BF16 pieces.  PS_BF16: the
  * tensor-core path: BF16 operands (fp32 accumulation) in the products of the second convolution and in the
  * first convolution's filter gradient, TF32 operands in the 512-unit layer; the first convolution's forward
  * pass and the output layer stay FP32.  PS_TF32 is reserved and not built (ps_create refuses it). */

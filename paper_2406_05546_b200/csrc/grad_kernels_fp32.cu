@@ -1,4 +1,4 @@
-// Worker-side gradient step on the FP32 CUDA cores: the paper's small CNN (model endnote),
+// Worker-side gradient step, FP32 path (the dense layer's products are in grad_kernels_x3_gemm.cu): the paper's small CNN (model endnote),
 // forward and backward, for W workers that may hold different weight snapshots.
 //
 // Rows of every activation buffer are (sorted worker s, sample i) -> s*b + i, where the sorted
@@ -357,10 +357,11 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
     if (n < 0) return -1;
     launches += 2 + n;
   } else {
+    launch_prep_w1_x3(gt, ws, st, prof);
     launch_conv1_fwd(a, wt, gt, ws, st, prof);
     launch_conv2_direct(true, a, gt, ws, st, prof);
-    launch_fc1_fwd_fp32(a, wt, gt, ws, st, prof);
-    launches += 3;
+    if (launch_fc1_fwd_x3(a, wt, gt, ws, st, prof, false) < 0) return -1;
+    launches += 4;
   }
   launch_output_layer(true, a, wt, gt, ws, st, prof);
   TIMED(K_EVAL_FINISH, launch_pdl(eval_finish, dim3(a.W), 128, 0, st, a, wt, ws, correct));
@@ -437,14 +438,19 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     launches += 4;
   } else {
     cudaStream_t s1 = side.s1 ? side.s1 : st, s2 = side.s2 ? side.s2 : st;
+    // the pieces of W1 are made next to the convolutions
+    if (side.s1) { cudaEventRecord(side.fork1, st); cudaStreamWaitEvent(s1, side.fork1, 0); }
+    launch_prep_w1_x3(gt, ws, s1, prof);
+    if (side.s1) cudaEventRecord(side.join1, s1);
     launch_conv1_fwd(a, wt, gt, ws, st, prof);
     launch_conv2_direct(true, a, gt, ws, st, prof);
-    launch_fc1_fwd_fp32(a, wt, gt, ws, st, prof);
+    if (side.s1) cudaStreamWaitEvent(st, side.join1, 0);
+    if (launch_fc1_fwd_x3(a, wt, gt, ws, st, prof, side.s1 != nullptr) < 0) return -1;
     launch_output_layer(false, a, wt, gt, ws, st, prof);
     if (side.s1) { cudaEventRecord(side.fork1, st); cudaStreamWaitEvent(s1, side.fork1, 0); }
-    launch_fc1_dw_fp32(sum ? a_dw : a, sum ? wt_dw : wt, gt, ws, s1, prof);
+    if (launch_fc1_dw_x3(sum ? a_dw : a, sum ? wt_dw : wt, gt, ws, s1, prof) < 0) return -1;
     if (side.s1) cudaEventRecord(side.join1, s1);
-    launch_fc1_dx_fp32(a, wt, gt, ws, st, prof);
+    if (launch_fc1_dx_x3(a, wt, gt, ws, st, prof) < 0) return -1;
     if (side.s2) { cudaEventRecord(side.fork2, st); cudaStreamWaitEvent(s2, side.fork2, 0); }
     n_chunks2 = launch_conv2_dw_direct(a, ws, s2, prof, &seg_len);
     if (side.s2) cudaEventRecord(side.join2, s2);
@@ -454,7 +460,7 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     if (side.s2) cudaStreamWaitEvent(st, side.join2, 0);
     if (sum) TIMED(K_CONV_GRAD_REDUCE, (fused_finish<<<dim3(FUSED_W1_BLOCKS + FUSED_SMALL_BLOCKS), 256, 0, st>>>(a, wt, ws, sum->super_part, sum->n_super, sum->grad_sum, n_chunks1b, 0, n_chunks2, seg_len)));
     else TIMED(K_CONV_GRAD_REDUCE, (conv_grad_reduce<<<dim3(a.W, (RED_OUTPUTS + red_per_block - 1) / red_per_block), 256, 0, st>>>(a, wt, ws, red_per_block, n_chunks1b, 0, n_chunks2, seg_len)));
-    launches = 10;
+    launches = 11;
   }
   return cudaGetLastError() == cudaSuccess ? launches : -1;
 }

@@ -15,6 +15,7 @@
 // read and skipped zero gradients with a branch that the lanes of a warp took differently).  At 2 x 8: 57 -> 13 us and
 // 402 -> 15 + 15 us.  The FP32 pipe is busy 66 - 69 % of the time (ncu, half the samples); scalar multiply-adds instead: 0.78 / 0.72 /
 // 0.67 ms; three blocks of 8-channel threads per SM: 0.77 / 0.66 ms.
+#include "bf16x3.cuh"
 #include "device_common.cuh"
 #include "kernels.h"
 
@@ -161,7 +162,9 @@ __global__ void __launch_bounds__(conv_threads<SPB>(), SPB > 1 ? 2 : 1) conv2_di
           const float r = fmaxf(v[h][j], 0.f);
           if (r > best) { best = r; bi = j; }
         }
-        ws.p2[row * FLAT + n * 49 + pos] = best;
+        const Bf16x3 s = split3(best, 0.f);        // its readers are the dense layer's products
+#pragma unroll
+        for (int p = 0; p < PIECES; ++p) ws.p2x[((int64_t)p * a.W * a.b + row) * FLAT + n * 49 + pos] = (uint16_t)s.p[p];
         ws.code2[row * FLAT + n * 49 + pos] = best > 0.f ? (uint8_t)bi : (uint8_t)4;
       } else {
         float* d = ws.dp1 + row * P1_ELEMS + n * 196 + 2 * py * 14 + 2 * px;

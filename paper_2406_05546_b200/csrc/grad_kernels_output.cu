@@ -12,6 +12,7 @@
 // Measured (B200, ~6 us of event overhead included; before: one block per worker, pre-activation gradients written by the
 // first part and read back by the second): 14.5 -> 9 us at 2 x 8, 21.5 -> 10.7 at 8 x 64, 37 -> 33 at 128 x 128 (two blocks
 // per worker).  One and two samples per warp instead of four, at twice the blocks per SM: 10.5 / 10.7 / 41 and 10.7 / 11.8 / 35.
+#include "bf16x3.cuh"
 #include "device_common.cuh"
 #include "kernels.h"
 
@@ -25,7 +26,7 @@ constexpr int DZ_CHUNK = 128;      // samples whose logits gradients are held in
 constexpr int W2T_PITCH = 12;      // 48-byte rows: 16-byte loads of consecutive rows fall on distinct banks
 static_assert(FC2_THREADS == HID, "thread = hidden unit");
 
-template <bool EVAL>
+template <bool EVAL, bool FP32>
 __global__ void __launch_bounds__(FC2_THREADS, 1) output_layer(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws) {
   __shared__ __align__(16) float w2t[HID][W2T_PITCH];     // w2t[j][c] = W2[c][j]; the two pad columns are zero
   __shared__ __align__(16) float dzs[DZ_CHUNK][W2T_PITCH];   // logits gradients of a chunk of samples
@@ -158,6 +159,8 @@ __global__ void __launch_bounds__(FC2_THREADS, 1) output_layer(GradStepArgs a, W
     }
     const float* dp = ws.d + ((int64_t)s * a.b + c0) * HID + tid;
     float* da1p = ws.da1 + ((int64_t)s * a.b + c0) * HID + tid;
+    uint16_t* da1x = ws.da1x + ((int64_t)s * a.b + c0) * HID + tid;
+    const int64_t piece = (int64_t)a.W * a.b * HID;
     constexpr int U = 8;                                  // activations in flight per thread
     for (int i0 = 0; i0 < n; i0 += U) {
       float dval[U];
@@ -179,8 +182,15 @@ __global__ void __launch_bounds__(FC2_THREADS, 1) output_layer(GradStepArgs a, W
         float lo, hi;
         unpack2(e, lo, hi);
         float o = dval[u] > 0.f ? (lo + hi) * scale : 0.f;   // the unit passed ReLU and dropout
-        if (a.precision != 0) o = round_tf32(o);             // it feeds tensor-core products only
-        da1p[(int64_t)(i0 + u) * HID] = o;
+        // it feeds tensor-core products only: as TF32, or (FP32 path) as three BF16 pieces
+        if (!FP32) {
+          o = round_tf32(o);
+          da1p[(int64_t)(i0 + u) * HID] = o;
+        } else {
+          const Bf16x3 sp = split3(o, 0.f);
+#pragma unroll
+          for (int p = 0; p < PIECES; ++p) da1x[p * piece + (int64_t)(i0 + u) * HID] = (uint16_t)sp.p[p];
+        }
         gb1 += o;
       }
     }
@@ -219,8 +229,9 @@ __global__ void __launch_bounds__(FC2_THREADS, 1) output_layer(GradStepArgs a, W
 
 void launch_output_layer(bool eval, const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof) {
   const dim3 grid(a.W, fc2_split(a.W, a.b));
-  if (eval) TIMED(K_FC2_FWD_BWD, launch_pdl(output_layer<true>, dim3(grid), FC2_THREADS, 0, st, a, wt, gt, ws));
-  else TIMED(K_FC2_FWD_BWD, launch_pdl(output_layer<false>, dim3(grid), FC2_THREADS, 0, st, a, wt, gt, ws));
+  if (eval) TIMED(K_FC2_FWD_BWD, launch_pdl(output_layer<true, false>, dim3(grid), FC2_THREADS, 0, st, a, wt, gt, ws));
+  else if (a.precision == 0) TIMED(K_FC2_FWD_BWD, launch_pdl(output_layer<false, true>, dim3(grid), FC2_THREADS, 0, st, a, wt, gt, ws));
+  else TIMED(K_FC2_FWD_BWD, launch_pdl(output_layer<false, false>, dim3(grid), FC2_THREADS, 0, st, a, wt, gt, ws));
 }
 
 }  // namespace psk

@@ -580,16 +580,24 @@ bool make_map_mn(CUtensorMap* m, const float* base, uint64_t F, uint64_t b, uint
 
 }  // namespace
 
-bool encode_tensor_map_f32(CUtensorMap* m, const float* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
-                           const uint32_t* box) {
+static bool encode_tensor_map(CUtensorMap* m, CUtensorMapDataType type, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
+                              const uint32_t* box, CUtensorMapSwizzle swizzle, CUtensorMapL2promotion promotion) {
   if (!g_encode || rank < 1 || rank > 5) return false;
   cuuint64_t d[5], sb[4];
   cuuint32_t bx[5], es[5];
   for (int i = 0; i < rank; ++i) { d[i] = dims[i]; bx[i] = box[i]; es[i] = 1; }
   for (int i = 0; i + 1 < rank; ++i) sb[i] = strides_bytes[i];
-  return g_encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)rank, const_cast<float*>(base), d, sb, bx, es,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+  return g_encode(m, type, (cuuint32_t)rank, const_cast<void*>(base), d, sb, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, promotion,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+bool encode_tensor_map_f32(CUtensorMap* m, const float* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
+                           const uint32_t* box) {
+  return encode_tensor_map(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, base, rank, dims, strides_bytes, box, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+}
+bool encode_tensor_map_bf16(CUtensorMap* m, const uint16_t* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
+                            const uint32_t* box, int swizzle) {
+  return encode_tensor_map(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, base, rank, dims, strides_bytes, box,
+                           swizzle == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
 }
 
 #define TIMED(id, launch) do { if (prof) prof->begin(id, st); launch; if (prof) prof->end(st); } while (0)

@@ -114,10 +114,10 @@ struct Workspace {
   float* p1;       // conv1 -> ReLU -> pool: [rows][16][14][14] fp32 (FP32 path) or [rows][2 planes][256][8] BF16 (tensor-core path)
   uint8_t* code1;  // [rows][3136]        pool-1 decisions. FP32 path: [16][196], argmax 0..3, 4 = no gradient (max <= 0); tensor-core path:
                    //                     [4 channel quads][196][4], the byte 1 << argmax, 0 = no gradient
-  float* p2;       // [rows][1568]        conv2 -> ReLU -> pool, channel-major flatten
+  float* p2;       // [rows][1568]        conv2 -> ReLU -> pool, channel-major flatten (tensor-core path)
   uint8_t* code2;  // [rows][1568]
   float* d;        // [rows][512]         fc1 -> ReLU -> dropout (scaled)
-  float* da1;      // [rows][512]         gradient w.r.t. fc1 pre-activation
+  float* da1;      // [rows][512]         gradient w.r.t. fc1 pre-activation (tensor-core path)
   float* dp2;      // [rows][1568]        gradient w.r.t. p2 (tensor-core path: BF16 in the first half of each row)
   float* dp1;      // [rows][3136]        gradient w.r.t. p1; [16][196] fp32 (FP32 path) or [4 channel quads][196][4] BF16 in the first half of the row (tensor-core path)
   float* part2;    // [W][chunks][4640]   per-block partial conv2 weight/bias gradients
@@ -125,6 +125,8 @@ struct Workspace {
   float* partf;    // [W][fc2_split][FC_PART] per-block partial output-layer gradients and loss sums
   float* w1r;      // [groups][512][1568] TF32-rounded fc1 weights of each weight group of the call
   float* w1tr;     // [groups][1568][512] and their transpose
+  uint16_t *p2x, *da1x;   // FP32 path: p2 and da1 as BF16 pieces, [3][rows of the call][1568] and [3][rows of the call][512]
+  uint16_t* w1x;   // FP32 path: [groups][3][512][1568] W1 as BF16 pieces
   uint8_t* bank2;  // [groups][BANK2_BYTES] conv2's filters as its kernels' tensor-core operands (forward, then input gradient)
   uint32_t* status;
 };
@@ -138,7 +140,7 @@ struct GradStepArgs {
   uint64_t seed, step;
   float drop_p;
   uint32_t drop_thresh;   // keep iff word >= thresh
-  int precision;          // 0 = FP32 CUDA cores; otherwise tensor cores (BF16 convolution products, TF32 dense layer)
+  int precision;          // 0 = FP32 (dense layer on the tensor cores, operands in BF16 pieces); otherwise tensor cores (BF16 convolution products, TF32 dense layer)
   int skip_prep_w1;       // the rounded copies of the dense-layer weights of these very snapshots are still valid
   int after_wait = 0;     // the caller has just made the stream wait for another one
 };
@@ -174,11 +176,12 @@ int launch_dropout_mask(uint64_t seed, uint32_t worker, uint64_t step, int b, ui
                         uint8_t* keep, cudaStream_t st, Profiler* prof);
 int configure_fp32_conv2_kernels();
 void launch_conv2_direct(bool fwd, const GradStepArgs& a, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
-int configure_fp32_gemm_kernels();
-void launch_fc1_fwd_fp32(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
-void launch_fc1_dx_fp32(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
-void launch_fc1_dw_fp32(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
 int launch_conv2_dw_direct(const GradStepArgs& a, const Workspace& ws, cudaStream_t st, Profiler* prof, int* seg_len);
+int configure_x3_gemm_kernels();
+void launch_prep_w1_x3(const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
+int launch_fc1_fwd_x3(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof, bool after_join);
+int launch_fc1_dx_x3(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
+int launch_fc1_dw_x3(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
 extern int g_sm_count;   // SMs of the current device, set by configure_tc5_kernels
 int configure_tc5_kernels();
 int configure_conv5_kernels();

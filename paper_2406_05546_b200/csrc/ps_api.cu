@@ -148,10 +148,18 @@ void layout(ps_ctx* x, const ps_config& c, void* arena, void* pinned, uint64_t* 
   const uint64_t p1_elems = c.precision != PS_FP32 ? psk::P1_PLANE_ELEMS : psk::P1_ELEMS;
   ws.p1 = a.take<float>(rows * p1_elems * 4);
   ws.code1 = a.take<uint8_t>(rows * psk::P1_ELEMS);
-  ws.p2 = a.take<float>(rows * psk::FLAT * 4);
+  ws.p2 = ws.da1 = nullptr;
+  ws.p2x = ws.da1x = ws.w1x = nullptr;
+  if (c.precision != PS_FP32) {
+    ws.p2 = a.take<float>(rows * psk::FLAT * 4);
+    ws.da1 = a.take<float>(rows * psk::HID * 4);
+  } else {
+    ws.p2x = a.take<uint16_t>(3 * rows * psk::FLAT * 2);
+    ws.da1x = a.take<uint16_t>(3 * rows * psk::HID * 2);
+    ws.w1x = a.take<uint16_t>(3 * std::min<uint64_t>(psk::MAX_GROUPS, c.max_workers) * psk::HID * psk::FLAT * 2);      // as many groups as a call can have
+  }
   ws.code2 = a.take<uint8_t>(rows * psk::FLAT);
   ws.d = a.take<float>(rows * psk::HID * 4);
-  ws.da1 = a.take<float>(rows * psk::HID * 4);
   ws.dp2 = a.take<float>(rows * psk::FLAT * 4);
   ws.dp1 = a.take<float>(rows * psk::P1_ELEMS * 4);
   ws.part2 = a.take<float>((uint64_t)c.max_workers * chunks * psk::C2_GRAD * 4);
@@ -270,7 +278,7 @@ int32_t ps_create(const ps_config* cfg, const float* init_params_host, ps_ctx** 
   x->ckpt_version.assign(x->ckpt_buf.size(), 0);
   double t = std::floor((double)cfg->dropout_p * 4294967296.0);
   x->drop_thresh = t <= 0.0 ? 0u : (t >= 4294967295.0 ? 0xFFFFFFFFu : (uint32_t)t);
-  if (psk::configure_apply_kernels() != 0 || psk::configure_fp32_conv2_kernels() != 0 || psk::configure_fp32_gemm_kernels() != 0 || psk::configure_tc5_kernels() != 0 || psk::configure_conv5_kernels() != 0 || psk::configure_conv1_kernels() != 0 || psk::configure_dw5_kernels() != 0 || psk::configure_c1d5_kernels() != 0) { delete x; return fail(PS_ERR_CUDA, "kernel configuration failed: %s", cudaGetErrorString(cudaGetLastError())); }
+  if (psk::configure_apply_kernels() != 0 || psk::configure_fp32_conv2_kernels() != 0 || psk::configure_tc5_kernels() != 0 || psk::configure_x3_gemm_kernels() != 0 || psk::configure_conv5_kernels() != 0 || psk::configure_conv1_kernels() != 0 || psk::configure_dw5_kernels() != 0 || psk::configure_c1d5_kernels() != 0) { delete x; return fail(PS_ERR_CUDA, "kernel configuration failed: %s", cudaGetErrorString(cudaGetLastError())); }
   {
     // two side streams let independent branches of the backward pass overlap (they allocate no device memory)
     bool ok = cudaStreamCreateWithFlags(&x->side.s1, cudaStreamNonBlocking) == cudaSuccess &&

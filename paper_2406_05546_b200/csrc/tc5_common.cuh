@@ -173,5 +173,8 @@ __device__ __forceinline__ uint32_t plain_desc_lo(uint32_t addr, uint32_t lbo) {
 // dimension i + 1), box as given, no swizzle, out-of-range elements read as zero.  False on failure.
 bool encode_tensor_map_f32(CUtensorMap* m, const float* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
                            const uint32_t* box);
+// The same of a BF16 tensor, with a swizzle of 64 or 128 bytes.
+bool encode_tensor_map_bf16(CUtensorMap* m, const uint16_t* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
+                            const uint32_t* box, int swizzle);
 
 }  // namespace psk

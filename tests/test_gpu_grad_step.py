@@ -143,6 +143,66 @@ def test_fp32_path_at_the_edges_of_its_kernel_choices(W, b, kw):
     _run_and_compare(W, b, **kw)
 
 
+# One row; one row more than a 128-row tile; 18 / 19 and 4 / 5 tiles of rows, where fewer CTAs share a tile's k; 11 / 12 and 37 / 38
+# tiles, beyond which one CTA does; k of the weight gradient just below, at and above a stage of 32 samples and a sum of 128;
+# three weight groups whose rows end inside a tile.
+@pytest.mark.parametrize("W,b,n_versions", [(1, 1, 1), (1, 31, 1), (1, 129, 1), (2, 256, 1), (3, 171, 1), (11, 128, 1), (11, 129, 1), (18, 128, 1), (19, 127, 1),
+                                             (37, 128, 1), (38, 127, 1), (70, 33, 3)])
+def test_fp32_dense_layer_at_the_edges_of_its_tiles(W, b, n_versions):
+    """What the three products of the dense layer give, through the tensors that a pooling decision of a convolution hardly moves
+    (of the millions of windows here some lie within rounding distance of a tie, and the filters' gradients depend on it), against
+    float64, first, middle and last worker:
+      - the output layer's gradients (forward product; a unit at zero adds nothing to them) within the path's tolerance;
+      - fc1.w and fc1.b (weight gradient) within it in all units but two: of a worker's 512 b decisions whether a unit is above zero
+        a few in ten million lie within rounding distance, so that one falls the other way in one worker of thirty, and moves its
+        unit's row; a wrong tile moves 128 units, or some columns of all;
+      - conv2.b, the sum of what the input gradient passes back through the windows above zero, within 1e-3 of its 2-norm: a window at
+        zero is one of its 49 b terms (1.2e-4 of the largest element in the worst worker seen), a wrong tile a thirteenth of all."""
+    torch, ps, srv, theta0 = _setup(W, b, n_versions)
+    thetas = {0: theta0}
+    for v in range(1, n_versions):
+        g = np.zeros((1, ps.P_PAD), dtype=np.float32)
+        g[0, :ps.P] = synth.random_gradients(1, seed=50 + v, scale=2.0)[0]
+        srv.ps_enqueue([0], [v - 1], 0, grads_dev=torch.from_numpy(g).cuda())
+        srv.ps_apply(ps.ASYNC, 0.01)
+        thetas[v], _ = srv.ps_export_params(0)
+    gen = torch.Generator(device="cuda").manual_seed(W + b)
+    x = torch.rand((W, b, 28, 28), generator=gen, device="cuda")
+    y = torch.randint(0, 10, (W, b), generator=gen, device="cuda", dtype=torch.int32)
+    snaps = [srv.ps_pull_snapshot(w, w % n_versions) for w in range(W)]
+    grads = torch.full((W, ps.P_PAD), float("nan"), device="cuda")
+    srv.workers_grad_step(snaps, range(W), x, y, SEED, 2, grads_dev=grads)
+    assert srv.ps_stats()["device_status"] == 0 and torch.isfinite(grads).all()
+    for w in sorted({0, W // 2, W - 1}):
+        want = _float64_gradient(thetas[snaps[w].version], x[w], y[w], srv.ps_dropout_mask(SEED, w, 2, b))
+        for name, off, shape in synth.layout():
+            got = grads[w, off:off + int(np.prod(shape))].double()
+            ref, tol = want[name], TOL_FP32 * want[name].abs().max()
+            if name == "conv2.b":
+                assert (got - ref).norm() <= 1e-3 * ref.norm(), w
+            elif name in ("fc1.w", "fc1.b"):
+                assert int(((got - ref).abs() > tol).view(512, -1).any(dim=1).sum()) <= 2, (w, name)
+            elif name in ("fc2.w", "fc2.b"):
+                assert (got - ref).abs().max() <= tol, (w, name)
+    srv.close()
+
+
+@pytest.mark.parametrize("W,b", [(1, 3), (5, 1000)])
+def test_fp32_dense_layer_keeps_an_infinite_sum(W, b):
+    """A hidden unit whose weights are all infinite, over inputs that are all positive, is infinite (and not NaN, which ReLU
+    would turn into zero): the loss cannot be finite."""
+    from paper_2406_05546_b200 import ps
+    import torch
+    theta = np.abs(synth.init_params(1, bias_scale=0.05))
+    off = next(o for n, o, _ in synth.layout() if n == "fc1.w")
+    theta[off + 7 * 1568:off + 8 * 1568] = np.inf
+    srv = ps.ParameterServer(theta, max_workers=W, max_batch=b, queue_slots=1)
+    x = torch.rand((W, b, 28, 28), device="cuda") + 0.5
+    loss, *_ = srv.workers_eval([srv.ps_pull_snapshot(0)] * W, x, torch.zeros((W, b), dtype=torch.int32, device="cuda"))
+    assert not torch.isfinite(loss).any()
+    srv.close()
+
+
 def _float64_gradient(theta, x, y, keep, drop_p=0.25):
     """One worker's gradient in float64 on the device: {tensor name: flat gradient}."""
     import torch

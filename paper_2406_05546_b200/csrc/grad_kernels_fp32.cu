@@ -7,8 +7,9 @@
 //
 // Every reduction is taken in a fixed order (no floating-point atomics), so that two runs on the
 // same inputs give the same bits.
-#include "kernels.h"
+#include "bf16x3.cuh"
 #include "device_common.cuh"
+#include "kernels.h"
 
 namespace psk {
 
@@ -19,10 +20,43 @@ namespace {
 // evaluates all 16 channels from registers (576 multiply-adds per 8 + 48 shared-memory loads).
 // (FP32 path; the tensor-core path has its own kernel, which writes the layout its convolutions copy from.)
 constexpr int CONV1_SPB = 8;      // most samples per block
-__global__ void __launch_bounds__(224) conv1_fwd(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws, int spb) {
+
+// The second convolution's filters of a weight group as its kernels' operands, one row of eight values (in pieces) per thread.
+// Blocks of conv1_fwd beyond its workers do it, so that the next kernel finds them without a launch or a fork of their own.
+constexpr int BANK3_ROWS = 2 * BANK3_FWD_ROWS + 12 * 48, BANK3_UNITS = (BANK3_ROWS + 223) / 224;      // blocks per weight group
+__device__ __forceinline__ void build_bank3(const float* __restrict__ theta, uint8_t* __restrict__ bank, int e, const Bank3Taps& taps) {
+  if (e >= BANK3_ROWS) return;
+  float v[8];
+  uint8_t* d;
+  int piece_bytes;
+  if (e < 2 * BANK3_FWD_ROWS) {      // forward: [piece][octet of input channels][row = block, output channel]
+    const int oct = e / BANK3_FWD_ROWS, row = e - oct * BANK3_FWD_ROWS, oc = row & 31, tap = taps.tap[row >> 5];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = theta[OFF_C2W + (oc * 16 + oct * 8 + i) * 9 + tap];
+    d = bank + e * 16;
+    piece_bytes = 2 * BANK3_FWD_ROWS * 16;
+  } else {                           // input gradient: [filter row][octet of output channels][piece][column = kx, input channel]
+    const int u = e - 2 * BANK3_FWD_ROWS, ko = u / 48, col = u - ko * 48, ky = ko >> 2, o8 = ko & 3, kx = col >> 4, ic = col & 15;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = theta[OFF_C2W + ((o8 * 8 + i) * 16 + ic) * 9 + ky * 3 + kx];
+    d = bank + BANK3_FWD_BYTES + (ko * PIECES * 48 + col) * 16;
+    piece_bytes = 48 * 16;
+  }
+  const Bf16x3 s[4] = {split3(v[0], v[1]), split3(v[2], v[3]), split3(v[4], v[5]), split3(v[6], v[7])};
+#pragma unroll
+  for (int p = 0; p < PIECES; ++p) *reinterpret_cast<uint4*>(d + p * piece_bytes) = make_uint4(s[0].p[p], s[1].p[p], s[2].p[p], s[3].p[p]);
+}
+
+__global__ void __launch_bounds__(224) conv1_fwd(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws, int spb, const __grid_constant__ Bank3Taps taps) {
   __shared__ __align__(16) float xs[2][30][32];
   __shared__ __align__(16) float w[16][12];   // 9 taps + bias + padding
   const int s = blockIdx.y, tid = threadIdx.x;
+  if (s >= a.W) {
+    const int u = (s - a.W) * gridDim.x + blockIdx.x, g = u / BANK3_UNITS;
+    pdl_enter();
+    if (g < gt.n_groups) build_bank3(gt.theta[g], ws.bank2 + (int64_t)g * BANK3_BYTES, (u - g * BANK3_UNITS) * 224 + tid, taps);
+    return;
+  }
   const float* theta = group_theta(wt, gt, s);
   pdl_enter();       // the weights may come from the apply just before
   if (tid < 160) {
@@ -46,8 +80,22 @@ __global__ void __launch_bounds__(224) conv1_fwd(GradStepArgs a, WorkerTable wt,
     const int cur = (i - i0) & 1;
     __syncthreads();                       // image `cur` is complete; image `cur^1` is no longer read
     if (i + 1 < i1) stage(i + 1, cur ^ 1);
-    if (!active) continue;
     const int64_t row = (int64_t)s * a.b + i;
+    // a position's sixteen channels in pieces: six 16-byte slots; Y and X in the bordered map
+    auto store = [&](int Y, int X, const float (&v)[16]) {
+      uint8_t* d = ws.p1x + row * P1X_BYTES + Y * P1X_ROW + ((X & 1) * 8 + (X >> 1)) * 16;
+#pragma unroll
+      for (int o = 0; o < 2; ++o) {
+        const Bf16x3 q[4] = {split3(v[8 * o], v[8 * o + 1]), split3(v[8 * o + 2], v[8 * o + 3]), split3(v[8 * o + 4], v[8 * o + 5]), split3(v[8 * o + 6], v[8 * o + 7])};
+#pragma unroll
+        for (int p = 0; p < PIECES; ++p) *reinterpret_cast<uint4*>(d + (2 * p + o) * 256) = make_uint4(q[0].p[p], q[1].p[p], q[2].p[p], q[3].p[p]);
+      }
+    };
+    if (!active) {                         // 28 threads for the zeros at either end of the fourteen image rows: whole runs leave
+      const float zero[16] = {};
+      store((tid - 196) / 2 + 1, (tid & 1) * 15, zero);
+      continue;
+    }
     float patch[4][4];
 #pragma unroll
     for (int yy = 0; yy < 4; ++yy) {
@@ -83,8 +131,7 @@ __global__ void __launch_bounds__(224) conv1_fwd(GradStepArgs a, WorkerTable wt,
     const int pp = tid;
 #pragma unroll
     for (int ch = 0; ch < 16; ++ch) ws.code1[row * P1_ELEMS + ch * 196 + pp] = outc[ch];
-#pragma unroll
-    for (int ch = 0; ch < 16; ++ch) ws.p1[row * P1_ELEMS + ch * 196 + pp] = outv[ch];
+    store(py + 1, px + 1, outv);
   }
 }
 
@@ -341,7 +388,8 @@ static int samples_per_block(int rows, int least, int most) {
 }
 static void launch_conv1_fwd(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof) {
   const int spb = samples_per_block(a.W * a.b, 1, CONV1_SPB);
-  TIMED(K_CONV1_FWD, launch_pdl_if(!a.after_wait, conv1_fwd, dim3((a.b + spb - 1) / spb, a.W), 224, 0, st, a, wt, gt, ws, spb));
+  const int chunks = (a.b + spb - 1) / spb, bank = (gt.n_groups * BANK3_UNITS + chunks - 1) / chunks;
+  TIMED(K_CONV1_FWD, launch_pdl_if(!a.after_wait, conv1_fwd, dim3(chunks, a.W + bank), 224, 0, st, a, wt, gt, ws, spb, conv2_fwd_x3_taps()));
 }
 
 // Evaluation pass: the forward kernels of the grad step with the dropout switched off, then the per-worker loss and hit
@@ -359,7 +407,7 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
   } else {
     launch_prep_w1_x3(gt, ws, st, prof);
     launch_conv1_fwd(a, wt, gt, ws, st, prof);
-    launch_conv2_direct(true, a, gt, ws, st, prof);
+    launch_conv2_fwd_x3(a, gt, ws, st, prof);
     if (launch_fc1_fwd_x3(a, wt, gt, ws, st, prof, false) < 0) return -1;
     launches += 4;
   }
@@ -443,7 +491,7 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     launch_prep_w1_x3(gt, ws, s1, prof);
     if (side.s1) cudaEventRecord(side.join1, s1);
     launch_conv1_fwd(a, wt, gt, ws, st, prof);
-    launch_conv2_direct(true, a, gt, ws, st, prof);
+    launch_conv2_fwd_x3(a, gt, ws, st, prof);
     if (side.s1) cudaStreamWaitEvent(st, side.join1, 0);
     if (launch_fc1_fwd_x3(a, wt, gt, ws, st, prof, side.s1 != nullptr) < 0) return -1;
     launch_output_layer(false, a, wt, gt, ws, st, prof);
@@ -452,9 +500,9 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     if (side.s1) cudaEventRecord(side.join1, s1);
     if (launch_fc1_dx_x3(a, wt, gt, ws, st, prof) < 0) return -1;
     if (side.s2) { cudaEventRecord(side.fork2, st); cudaStreamWaitEvent(s2, side.fork2, 0); }
-    n_chunks2 = launch_conv2_dw_direct(a, ws, s2, prof, &seg_len);
+    n_chunks2 = launch_conv2_dw_x3(a, ws, s2, prof, &seg_len);
     if (side.s2) cudaEventRecord(side.join2, s2);
-    launch_conv2_direct(false, a, gt, ws, st, prof);
+    launch_conv2_dx_x3(a, gt, ws, st, prof);
     TIMED(K_CONV1_BWD, launch_pdl(conv1_bwd, dim3(n_chunks1b, a.W), 256, 0, st, a, wt, ws, spb1b, n_chunks1b));
     if (side.s1) cudaStreamWaitEvent(st, side.join1, 0);
     if (side.s2) cudaStreamWaitEvent(st, side.join2, 0);

@@ -44,6 +44,14 @@ constexpr int BANK2_DX_ROWS = 12 * 48, BANK2_DX_BYTES = BANK2_DX_ROWS * 16, BANK
 constexpr uint8_t BANK2_ZERO_BLOCK = 255;
 struct Bank2Taps { uint8_t tap[BANK2_BLOCKS]; };      // filter tap ky * 3 + kx of a block's 32 filters; BANK2_ZERO_BLOCK: zeros
 
+// FP32 path: the same filters as BF16 pieces (bf16x3.cuh) for its own kernels, [piece][octet][row] forward and
+// [filter row][octet][piece][column] for the input gradient; and the first convolution's output, [image row of the bordered
+// map][piece][octet of channels][slot (X & 1) * 8 + X / 2][8 channels] BF16.
+constexpr int BANK3_BLOCKS = 36, BANK3_FWD_ROWS = 32 * BANK3_BLOCKS, BANK3_FWD_BYTES = 3 * 2 * BANK3_FWD_ROWS * 16;
+constexpr int BANK3_DX_BYTES = 12 * 3 * 48 * 16, BANK3_BYTES = BANK3_FWD_BYTES + BANK3_DX_BYTES;
+struct Bank3Taps { uint8_t tap[BANK3_BLOCKS]; };      // filter tap ky * 3 + kx of a block's 32 filters
+constexpr int P1X_ROW = 3 * 2 * 16 * 16, P1X_BYTES = 16 * P1X_ROW;
+
 constexpr uint32_t STATUS_BAD_LABEL = 1u;
 constexpr uint32_t STATUS_WAIT_TIMEOUT = 2u;   // a bounded barrier wait in a tensor-core kernel gave up
 
@@ -111,11 +119,12 @@ struct GroupTable {
 
 // Activation workspace carved from the arena (rows = sorted worker * b + sample).
 struct Workspace {
-  float* p1;       // conv1 -> ReLU -> pool: [rows][16][14][14] fp32 (FP32 path) or [rows][2 planes][256][8] BF16 (tensor-core path)
+  float* p1;       // conv1 -> ReLU -> pool: [rows][2 planes][256][8] BF16 (tensor-core path)
+  uint8_t* p1x;    // the same in BF16 pieces: [rows][P1X_BYTES] (FP32 path)
   uint8_t* code1;  // [rows][3136]        pool-1 decisions. FP32 path: [16][196], argmax 0..3, 4 = no gradient (max <= 0); tensor-core path:
                    //                     [4 channel quads][196][4], the byte 1 << argmax, 0 = no gradient
   float* p2;       // [rows][1568]        conv2 -> ReLU -> pool, channel-major flatten (tensor-core path)
-  uint8_t* code2;  // [rows][1568]
+  uint8_t* code2;  // [rows][1568]        [8 channel quads][49][4], argmax 0..3, 4 = no gradient
   float* d;        // [rows][512]         fc1 -> ReLU -> dropout (scaled)
   float* da1;      // [rows][512]         gradient w.r.t. fc1 pre-activation (tensor-core path)
   float* dp2;      // [rows][1568]        gradient w.r.t. p2 (tensor-core path: BF16 in the first half of each row)
@@ -127,7 +136,7 @@ struct Workspace {
   float* w1tr;     // [groups][1568][512] and their transpose
   uint16_t *p2x, *da1x;   // FP32 path: p2 and da1 as BF16 pieces, [3][rows of the call][1568] and [3][rows of the call][512]
   uint16_t* w1x;   // FP32 path: [groups][3][512][1568] W1 as BF16 pieces
-  uint8_t* bank2;  // [groups][BANK2_BYTES] conv2's filters as its kernels' tensor-core operands (forward, then input gradient)
+  uint8_t* bank2;  // [groups][BANK2_BYTES] (FP32 path: BANK3_BYTES) conv2's filters as its kernels' operands (forward, then input gradient)
   uint32_t* status;
 };
 
@@ -174,9 +183,11 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
                      cudaStream_t st, const SideStreams& side, Profiler* prof, const SummedStep* sum = nullptr);
 int launch_dropout_mask(uint64_t seed, uint32_t worker, uint64_t step, int b, uint32_t thresh,
                         uint8_t* keep, cudaStream_t st, Profiler* prof);
-int configure_fp32_conv2_kernels();
-void launch_conv2_direct(bool fwd, const GradStepArgs& a, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
-int launch_conv2_dw_direct(const GradStepArgs& a, const Workspace& ws, cudaStream_t st, Profiler* prof, int* seg_len);
+int configure_x3_conv2_kernels();
+const Bank3Taps& conv2_fwd_x3_taps();
+void launch_conv2_fwd_x3(const GradStepArgs& a, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
+void launch_conv2_dx_x3(const GradStepArgs& a, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
+int launch_conv2_dw_x3(const GradStepArgs& a, const Workspace& ws, cudaStream_t st, Profiler* prof, int* seg_len);
 int configure_x3_gemm_kernels();
 void launch_prep_w1_x3(const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof);
 int launch_fc1_fwd_x3(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof, bool after_join);

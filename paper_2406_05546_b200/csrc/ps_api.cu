@@ -145,8 +145,10 @@ void layout(ps_ctx* x, const ps_config& c, void* arena, void* pinned, uint64_t* 
   float* norm_part = a.take<float>((uint64_t)c.queue_slots * psk::NORM_CHUNKS * 4);
   uint64_t* clip_words = a.take<uint64_t>(psk::CLIP_EXCHANGE_BYTES);
   psk::Workspace ws;
-  const uint64_t p1_elems = c.precision != PS_FP32 ? psk::P1_PLANE_ELEMS : psk::P1_ELEMS;
-  ws.p1 = a.take<float>(rows * p1_elems * 4);
+  ws.p1 = nullptr;
+  ws.p1x = nullptr;
+  if (c.precision != PS_FP32) ws.p1 = a.take<float>(rows * psk::P1_PLANE_ELEMS * 4);
+  else ws.p1x = a.take<uint8_t>(rows * psk::P1X_BYTES);
   ws.code1 = a.take<uint8_t>(rows * psk::P1_ELEMS);
   ws.p2 = ws.da1 = nullptr;
   ws.p2x = ws.da1x = ws.w1x = nullptr;
@@ -167,8 +169,9 @@ void layout(ps_ctx* x, const ps_config& c, void* arena, void* pinned, uint64_t* 
   ws.partf = a.take<float>((uint64_t)std::min(c.max_workers * psk::FC2_MAX_SPLIT, std::max<int>(c.max_workers, psk::FC2_BLOCKS)) * psk::FC_PART * 4);
   ws.status = a.take<uint32_t>(ALIGN);
   ws.w1r = ws.w1tr = nullptr;
-  ws.bank2 = nullptr;
-  if (c.precision != PS_FP32) {
+  if (c.precision == PS_FP32) {
+    ws.bank2 = a.take<uint8_t>(std::min<uint64_t>(psk::MAX_GROUPS, c.max_workers) * psk::BANK3_BYTES);
+  } else {
     const uint64_t groups = std::min<uint64_t>(psk::MAX_GROUPS, std::min<uint64_t>(c.max_workers, c.ring_depth));
     ws.w1r = a.take<float>(groups * psk::HID * psk::FLAT * 4);
     ws.w1tr = a.take<float>(groups * psk::HID * psk::FLAT * 4);
@@ -278,7 +281,7 @@ int32_t ps_create(const ps_config* cfg, const float* init_params_host, ps_ctx** 
   x->ckpt_version.assign(x->ckpt_buf.size(), 0);
   double t = std::floor((double)cfg->dropout_p * 4294967296.0);
   x->drop_thresh = t <= 0.0 ? 0u : (t >= 4294967295.0 ? 0xFFFFFFFFu : (uint32_t)t);
-  if (psk::configure_apply_kernels() != 0 || psk::configure_fp32_conv2_kernels() != 0 || psk::configure_tc5_kernels() != 0 || psk::configure_x3_gemm_kernels() != 0 || psk::configure_conv5_kernels() != 0 || psk::configure_conv1_kernels() != 0 || psk::configure_dw5_kernels() != 0 || psk::configure_c1d5_kernels() != 0) { delete x; return fail(PS_ERR_CUDA, "kernel configuration failed: %s", cudaGetErrorString(cudaGetLastError())); }
+  if (psk::configure_apply_kernels() != 0 || psk::configure_x3_conv2_kernels() != 0 || psk::configure_tc5_kernels() != 0 || psk::configure_x3_gemm_kernels() != 0 || psk::configure_conv5_kernels() != 0 || psk::configure_conv1_kernels() != 0 || psk::configure_dw5_kernels() != 0 || psk::configure_c1d5_kernels() != 0) { delete x; return fail(PS_ERR_CUDA, "kernel configuration failed: %s", cudaGetErrorString(cudaGetLastError())); }
   {
     // two side streams let independent branches of the backward pass overlap (they allocate no device memory)
     bool ok = cudaStreamCreateWithFlags(&x->side.s1, cudaStreamNonBlocking) == cudaSuccess &&
@@ -301,9 +304,10 @@ int32_t ps_create(const ps_config* cfg, const float* init_params_host, ps_ctx** 
   for (auto& r : x->replicas)
     if (e == cudaSuccess) e = cudaMemcpyAsync(r.buf, x->io_stage, VEC_BYTES, cudaMemcpyHostToDevice, x->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->status_dev, 0, ALIGN, x->st);
-  // tensor-core path: the zero borders of the plane-layout activations are written once, here
-  if (e == cudaSuccess && cfg->precision != PS_FP32)
-    e = cudaMemsetAsync(x->ws.p1, 0, (uint64_t)cfg->max_workers * cfg->max_batch * psk::P1_PLANE_ELEMS * 4, x->st);
+  // the zero borders of the first convolution's output are written once, here
+  const uint64_t rows = (uint64_t)cfg->max_workers * cfg->max_batch;
+  if (e == cudaSuccess)
+    e = cfg->precision != PS_FP32 ? cudaMemsetAsync(x->ws.p1, 0, rows * psk::P1_PLANE_ELEMS * 4, x->st) : cudaMemsetAsync(x->ws.p1x, 0, rows * psk::P1X_BYTES, x->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(x->st);
   if (e != cudaSuccess) { delete x; return cuda_fail(e, "ps_create upload"); }
   *out = x;

@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(F_THREADS, 2) conv2_fwd_tc5(GradStepArgs a, Gr
   uint16_t* Wk = reinterpret_cast<uint16_t*>(smem + F_NBUF * F_BUF_BYTES);
   float* bias = reinterpret_cast<float*>(smem + F_NBUF * F_BUF_BYTES + F_W_BYTES);
   Pipe* pipe = reinterpret_cast<Pipe*>(smem + F_NBUF * F_BUF_BYTES + F_W_BYTES + 128);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
   // a CTA walks over a contiguous range of rows (worker-major samples) that share one weight snapshot
   int grp, r_begin, r_end;
   if (!locate_row_range(gt, a.b, range_len, blockIdx.x, grp, r_begin, r_end)) return;
@@ -159,39 +159,36 @@ __global__ void __launch_bounds__(F_THREADS, 2) conv2_fwd_tc5(GradStepArgs a, Gr
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = pipe->tmem_base;
+  const uint32_t tmem = warp_uniform(pipe->tmem_base);
   pdl_enter();
 
   if (warp == 0) {
-    if (lane == 0) {
-      const uint32_t w_lo = plain_desc_lo(smem_u32(Wk), F_W_ROWS * 16);
-      // one pass of the outer loop takes the four tile buffers in turn (unrolled: buffer, accumulator and the parity of
-      // the accumulator's barrier are constants of each copy of the body, and the backward branch comes once per four tiles)
-      static_assert(F_NBUF == 4, "the accumulator parities below assume four tile buffers");
-      const uint32_t a_lo0 = plain_desc_lo(smem_u32(smem), F_PLANE_BYTES);
-      bool go_on = mbar_wait(&pipe->w_full, 0);
-      if (!go_on) pipe->abort_flag = 1;
-      uint32_t parity = 0;
-      for (int t = 0; go_on && t < n_tiles; parity ^= 1) {
+    const uint32_t w_lo = plain_desc_lo(smem_u32(Wk), F_W_ROWS * 16);
+    // one pass of the outer loop takes the four tile buffers in turn (unrolled: buffer, accumulator and the parity of
+    // the accumulator's barrier are constants of each copy of the body, and the backward branch comes once per four tiles)
+    static_assert(F_NBUF == 4, "the accumulator parities below assume four tile buffers");
+    const uint32_t a_lo0 = plain_desc_lo(smem_u32(smem), F_PLANE_BYTES);
+    bool go_on = warp_wait(&pipe->w_full, 0, &pipe->abort_flag);
+    if (!go_on) pipe->abort_flag = 1;
+    uint32_t parity = 0;
+    for (int t = 0; go_on && t < n_tiles; parity ^= 1) {
 #pragma unroll
-        for (int buf = 0; buf < F_NBUF; ++buf, ++t) {
-          const int ab = buf & 1;
-          if (t >= n_tiles) { go_on = false; break; }
-          if (!mbar_wait(&pipe->a_full[buf], parity)) { pipe->abort_flag = 1; go_on = false; break; }
-          // tile t = 4 k + buf is the (2 k + buf / 2)-th user of its accumulator: it waits for the phase of the user before
-          if (t >= 2 && !mbar_wait(&pipe->acc_empty[ab], ((buf >> 1) ^ 1) & 1)) { pipe->abort_flag = 1; go_on = false; break; }
-          if (pipe->abort_flag) { go_on = false; break; }
-          tc_fence_after();
-          // 16 MMAs, one per input shift (K = 16 channels); every descriptor is a per-tile base plus a table entry
-          const uint32_t a_lo = a_lo0 + buf * (F_BUF_BYTES / 16);
-          const uint32_t d_tmem = tmem + ab * 128;
+      for (int buf = 0; buf < F_NBUF; ++buf, ++t) {
+        const int ab = buf & 1;
+        if (t >= n_tiles) { go_on = false; break; }
+        if (!warp_wait(&pipe->a_full[buf], parity, &pipe->abort_flag)) { pipe->abort_flag = 1; go_on = false; break; }
+        // tile t = 4 k + buf is the (2 k + buf / 2)-th user of its accumulator: it waits for the phase of the user before
+        if (t >= 2 && !warp_wait(&pipe->acc_empty[ab], ((buf >> 1) ^ 1) & 1, &pipe->abort_flag)) { pipe->abort_flag = 1; go_on = false; break; }
+        tc_fence_after();
+        // 16 MMAs, one per input shift (K = 16 channels); every descriptor is a per-tile base plus a table entry
+        const uint32_t a_lo = a_lo0 + buf * (F_BUF_BYTES / 16);
+        const uint32_t d_tmem = tmem + ab * 128;
 #pragma unroll
-          for (int op = 0; op < F_OPS; ++op)
-            umma_f16_split(d_tmem + fold.d_col[op], a_lo + fold.a_off[op], plain_desc_hi(512), w_lo + fold.b_row[op],
-                           plain_desc_hi(128), fold.idesc[op], op ? 1u : 0u);
-          umma_commit(&pipe->a_empty[buf]);
-          umma_commit(&pipe->acc_full[ab]);
-        }
+        for (int op = 0; op < F_OPS; ++op)
+          umma_f16(d_tmem + fold.d_col[op], a_lo + fold.a_off[op], plain_desc_hi(512), w_lo + fold.b_row[op],
+                   plain_desc_hi(128), fold.idesc[op], op ? 1u : 0u);
+        umma_commit(&pipe->a_empty[buf]);
+        umma_commit(&pipe->acc_full[ab]);
       }
     }
   } else if (warp == 1) {
@@ -286,7 +283,7 @@ __global__ void __launch_bounds__(THREADS, 2) conv2_dx_tc5(GradStepArgs a, Group
   uint16_t* Wk = reinterpret_cast<uint16_t*>(smem + 2 * X_BUF_BYTES);
   uint8_t* raw = smem + 2 * X_BUF_BYTES + X_W_BYTES;        // raw slots filled by bulk copies
   Pipe* pipe = reinterpret_cast<Pipe*>(smem + 2 * X_BUF_BYTES + X_W_BYTES + X_RAW_SLOTS * X_RAW_BYTES);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
   int grp, r_begin, r_end;
   if (!locate_row_range(gt, a.b, range_len, blockIdx.x, grp, r_begin, r_end)) return;
   const int n_tiles = r_end - r_begin;
@@ -301,42 +298,39 @@ __global__ void __launch_bounds__(THREADS, 2) conv2_dx_tc5(GradStepArgs a, Group
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = pipe->tmem_base;
+  const uint32_t tmem = warp_uniform(pipe->tmem_base);
   pdl_enter();
 
   if (warp == 0) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16(128, 48);
-      const uint32_t w_lo = plain_desc_lo(smem_u32(Wk), 48 * 16);
-      // one pass of the outer loop takes the two plane buffers in turn (unrolled: the buffer's addresses are constants
-      // of its copy of the body, and the backward branch comes once per two tiles)
-      const uint32_t a_lo0 = plain_desc_lo(smem_u32(smem), X_PLANE_BYTES);
-      bool go_on = mbar_wait(&pipe->w_full, 0);
-      if (!go_on) pipe->abort_flag = 1;
-      uint32_t parity = 0;
-      for (int t = 0; go_on && t < n_tiles; parity ^= 1) {
+    constexpr uint32_t idesc = idesc_bf16(128, 48);
+    const uint32_t w_lo = plain_desc_lo(smem_u32(Wk), 48 * 16);
+    // one pass of the outer loop takes the two plane buffers in turn (unrolled: the buffer's addresses are constants
+    // of its copy of the body, and the backward branch comes once per two tiles)
+    const uint32_t a_lo0 = plain_desc_lo(smem_u32(smem), X_PLANE_BYTES);
+    bool go_on = warp_wait(&pipe->w_full, 0, &pipe->abort_flag);
+    if (!go_on) pipe->abort_flag = 1;
+    uint32_t parity = 0;
+    for (int t = 0; go_on && t < n_tiles; parity ^= 1) {
 #pragma unroll
-        for (int buf = 0; buf < 2; ++buf, ++t) {
-          if (t >= n_tiles) { go_on = false; break; }
-          if (!mbar_wait(&pipe->a_full[buf], parity)) { pipe->abort_flag = 1; go_on = false; break; }
-          if (t >= 2 && !mbar_wait(&pipe->acc_empty[buf], parity ^ 1)) { pipe->abort_flag = 1; go_on = false; break; }
-          if (pipe->abort_flag) { go_on = false; break; }
-          tc_fence_after();
-          const uint32_t a_lo = a_lo0 + buf * (X_BUF_BYTES / 16);
-          const uint32_t d_tmem = tmem + buf * 128;
-          // 12 MMAs: per block of 128 positions and filter row ky, the products with the three taps of that row sit
-          // side by side in the 48 accumulator columns (kx, ic); the rows read are shifted by the filter row only
+      for (int buf = 0; buf < 2; ++buf, ++t) {
+        if (t >= n_tiles) { go_on = false; break; }
+        if (!warp_wait(&pipe->a_full[buf], parity, &pipe->abort_flag)) { pipe->abort_flag = 1; go_on = false; break; }
+        if (t >= 2 && !warp_wait(&pipe->acc_empty[buf], parity ^ 1, &pipe->abort_flag)) { pipe->abort_flag = 1; go_on = false; break; }
+        tc_fence_after();
+        const uint32_t a_lo = a_lo0 + buf * (X_BUF_BYTES / 16);
+        const uint32_t d_tmem = tmem + buf * 128;
+        // 12 MMAs: per block of 128 positions and filter row ky, the products with the three taps of that row sit
+        // side by side in the 48 accumulator columns (kx, ic); the rows read are shifted by the filter row only
 #pragma unroll
-          for (int ky = 0; ky < 3; ++ky)
+        for (int ky = 0; ky < 3; ++ky)
 #pragma unroll
-            for (int q = 0; q < 2; ++q)                                        // 16 output channels per MMA
+          for (int q = 0; q < 2; ++q)                                        // 16 output channels per MMA
 #pragma unroll
-              for (int m = 0; m < 2; ++m)
-                umma_f16_split(d_tmem + m * 48, a_lo + (2 * q) * (X_PLANE_BYTES / 16) + m * 128 + (2 - ky) * 16 + 1, plain_desc_hi(128),
-                               w_lo + ((ky * 4 + 2 * q) * 48), plain_desc_hi(128), idesc, (ky | q) ? 1u : 0u);
-          umma_commit(&pipe->a_empty[buf]);
-          umma_commit(&pipe->acc_full[buf]);
-        }
+            for (int m = 0; m < 2; ++m)
+              umma_f16(d_tmem + m * 48, a_lo + (2 * q) * (X_PLANE_BYTES / 16) + m * 128 + (2 - ky) * 16 + 1, plain_desc_hi(128),
+                       w_lo + ((ky * 4 + 2 * q) * 48), plain_desc_hi(128), idesc, (ky | q) ? 1u : 0u);
+        umma_commit(&pipe->a_empty[buf]);
+        umma_commit(&pipe->acc_full[buf]);
       }
     }
   } else if (warp <= LOADERS / 32) {

@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(W5_THREADS, 1) conv2_dw_tc5(GradStepArgs a, Wo
   extern __shared__ __align__(1024) uint8_t sm[];
   uint8_t* raw = sm + W5_NSTAGE * W5_STAGE_BYTES;
   W5Bars* bars = reinterpret_cast<W5Bars*>(raw + W5_NRAW * W5_RAW_SLOT);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = warp_uniform(tid >> 5);
   const int total = a.W * a.b;
   const int r0 = blockIdx.x * seg_len, r1 = min(r0 + seg_len, total), n_samples = r1 - r0;
 
@@ -113,51 +113,48 @@ __global__ void __launch_bounds__(W5_THREADS, 1) conv2_dw_tc5(GradStepArgs a, Wo
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = bars->tmem_base;
+  const uint32_t tmem = warp_uniform(bars->tmem_base);
   pdl_enter();
 
   if (warp == 0) {
     // ---------------- MMA issue
-    if (lane == 0) {
-      // This loop is one thread's serial instruction stream, with nothing to hide its latencies: an integer division
-      // or modulo here costs hundreds of cycles per sample, so stage, parity, descriptors and the next write-out row are
-      // all carried along as counters.
-      constexpr uint32_t idesc = w5_idesc(64, 96);
-      constexpr uint32_t stage_step = W5_STAGE_BYTES / 16;
-      const uint32_t a_lo0 = plain_desc_lo(smem_u32(sm), 128);
-      // B at k-step ks starts at the stored row of y = ks (14 - ks rows in); its two k-chunks are the halves of a row
-      const uint32_t b_lo0 = plain_desc_lo(smem_u32(sm) + W5_A_BYTES + 14 * W5_B_ROW, W5_B_HALF);
-      const uint32_t full0 = smem_u32(&bars->op_full[0]), empty0 = smem_u32(&bars->op_empty[0]);
-      uint32_t parity = 0, writes = 0;
-      int flush_at = min(r1, (r0 / a.b + 1) * a.b) - 1 - r0;     // index in the range of the next row that ends a worker or the range
-      bool fresh = true;                       // the next MMA starts a new sum
-      bool go_on = true;
-      // One pass of the outer loop takes the stages in turn (unrolled: a stage's addresses are constants of its copy
-      // of the body, and the backward branch, after which the instruction fetch starts afresh, comes once per three samples).
-      for (int n = 0; go_on && n < n_samples; parity ^= 1) {
+    // This loop is one warp's serial instruction stream, with nothing to hide its latencies: an integer division
+    // or modulo here costs hundreds of cycles per sample, so stage, parity, descriptors and the next write-out row are
+    // all carried along as counters.
+    constexpr uint32_t idesc = w5_idesc(64, 96);
+    constexpr uint32_t stage_step = W5_STAGE_BYTES / 16;
+    const uint32_t a_lo0 = plain_desc_lo(smem_u32(sm), 128);
+    // B at k-step ks starts at the stored row of y = ks (14 - ks rows in); its two k-chunks are the halves of a row
+    const uint32_t b_lo0 = plain_desc_lo(smem_u32(sm) + W5_A_BYTES + 14 * W5_B_ROW, W5_B_HALF);
+    uint32_t parity = 0, writes = 0;
+    int flush_at = min(r1, (r0 / a.b + 1) * a.b) - 1 - r0;     // index in the range of the next row that ends a worker or the range
+    bool fresh = true;                       // the next MMA starts a new sum
+    bool go_on = true;
+    // One pass of the outer loop takes the stages in turn (unrolled: a stage's addresses are constants of its copy
+    // of the body, and the backward branch, after which the instruction fetch starts afresh, comes once per three samples).
+    for (int n = 0; go_on && n < n_samples; parity ^= 1) {
 #pragma unroll
-        for (int st = 0; st < W5_NSTAGE; ++st, ++n) {
-          if (n >= n_samples) { go_on = false; break; }
-          const uint32_t a_lo = a_lo0 + st * stage_step, b_lo = b_lo0 + st * stage_step;
-          if (!mbar_wait_addr(full0 + 8 * st, parity) || bars->abort_flag) { bars->abort_flag = 1; go_on = false; break; }
+      for (int st = 0; st < W5_NSTAGE; ++st, ++n) {
+        if (n >= n_samples) { go_on = false; break; }
+        const uint32_t a_lo = a_lo0 + st * stage_step, b_lo = b_lo0 + st * stage_step;
+        if (!warp_wait(&bars->op_full[st], parity, &bars->abort_flag)) { bars->abort_flag = 1; go_on = false; break; }
+        tc_fence_after();
+        // contraction indices 16 ks .. 16 ks + 15 (image row ks of the bordered input): two chunks of 128 bytes.
+        // Rows 0 and 15 are the input's zero border, so their products vanish and are not issued.
+#pragma unroll
+        for (int ks = 1; ks < 15; ++ks)
+          umma_f16(tmem, a_lo + ks * 16, plain_desc_hi(W5_GROUP_BYTES), b_lo - ks * (W5_B_ROW / 16), plain_desc_hi(128), idesc,
+                   (ks == 1 && fresh) ? 0u : 1u);
+        fresh = false;
+        umma_commit(&bars->op_empty[st]);
+        if (n == flush_at) {
+          // last row of the range or of a worker: hand the sum to the write-out warps and wait until they have read it
+          umma_commit(&bars->acc_full);
+          if (!warp_wait(&bars->acc_empty, writes & 1, &bars->abort_flag)) { bars->abort_flag = 1; go_on = false; break; }
           tc_fence_after();
-          // contraction indices 16 ks .. 16 ks + 15 (image row ks of the bordered input): two chunks of 128 bytes.
-          // Rows 0 and 15 are the input's zero border, so their products vanish and are not issued.
-#pragma unroll
-          for (int ks = 1; ks < 15; ++ks)
-            umma_f16_split(tmem, a_lo + ks * 16, plain_desc_hi(W5_GROUP_BYTES), b_lo - ks * (W5_B_ROW / 16), plain_desc_hi(128), idesc,
-                           (ks == 1 && fresh) ? 0u : 1u);
-          fresh = false;
-          umma_commit_addr(empty0 + 8 * st);
-          if (n == flush_at) {
-            // last row of the range or of a worker: hand the sum to the write-out warps and wait until they have read it
-            umma_commit(&bars->acc_full);
-            if (!mbar_wait(&bars->acc_empty, writes & 1)) { bars->abort_flag = 1; go_on = false; break; }
-            tc_fence_after();
-            ++writes;
-            fresh = true;
-            flush_at = min(flush_at + a.b, n_samples - 1);
-          }
+          ++writes;
+          fresh = true;
+          flush_at = min(flush_at + a.b, n_samples - 1);
         }
       }
     }

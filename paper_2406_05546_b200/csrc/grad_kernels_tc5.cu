@@ -1,5 +1,5 @@
 // The three products of the 512-unit dense layer on the fifth-generation tensor cores:
-// tcgen05.mma (kind::tf32) issued by one thread, operands brought into 128-byte-swizzled shared
+// tcgen05.mma (kind::tf32) issued by one warp, operands brought into 128-byte-swizzled shared
 // memory by TMA (cp.async.bulk.tensor, each CTA loading its own tiles), accumulators in tensor memory, read back with
 // tcgen05.ld for the epilogue.
 //
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(gemm_threads(EPI), 1) tc5_gemm(const __grid_co
   volatile uint32_t* abort_flag = tmem_slot + 1;
   float* epi_stage = reinterpret_cast<float*>(tiles + STAGES * STAGE_BYTES + 256);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int n_k = (ga.K + BK - 1) / BK;
 
   if (threadIdx.x == 0) {
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(gemm_threads(EPI), 1) tc5_gemm(const __grid_co
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_acc = *tmem_slot;
+  const uint32_t tmem_acc = warp_uniform(*tmem_slot);
   pdl_enter();
 
   if (warp == 0) {
@@ -195,37 +195,35 @@ __global__ void __launch_bounds__(gemm_threads(EPI), 1) tc5_gemm(const __grid_co
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = instr_desc_tf32(BM, BN, MN);
-      const uint32_t desc_hi = (uint32_t)((MN ? smem_desc_mn_sw128(0, 0) : smem_desc_sw128(0)) >> 32);
-      int it = 0, tile_i = 0;
-      bool ok = true;
-      TileWalk tw = tile_walk_begin(ga);
-      for (int t = blockIdx.x; t < ga.n_tiles && ok; t += gridDim.x, tile_walk_next(tw, ga)) {
-        TileCoord c;
-        if (!decode_tile<BN>(tw, ga, gt, a.b, c)) continue;
-        const int ab = tile_i & 1;
-        if (tile_i >= 2 && !mbar_wait(&acc_empty[ab], ((tile_i >> 1) - 1) & 1)) { *abort_flag = 1; break; }
+    constexpr uint32_t idesc = instr_desc_tf32(BM, BN, MN);
+    const uint32_t desc_hi = (uint32_t)((MN ? smem_desc_mn_sw128(0, 0) : smem_desc_sw128(0)) >> 32);
+    int it = 0, tile_i = 0;
+    bool ok = true;
+    TileWalk tw = tile_walk_begin(ga);
+    for (int t = blockIdx.x; t < ga.n_tiles && ok; t += gridDim.x, tile_walk_next(tw, ga)) {
+      TileCoord c;
+      if (!decode_tile<BN>(tw, ga, gt, a.b, c)) continue;
+      const int ab = tile_i & 1;
+      if (tile_i >= 2 && !warp_wait(&acc_empty[ab], ((tile_i >> 1) - 1) & 1, abort_flag)) { *abort_flag = 1; break; }
+      tc_fence_after();
+      for (int kb = 0; kb < n_k; ++kb, ++it) {
+        const int s = it % STAGES;
+        if (!warp_wait(&full[s], (it / STAGES) & 1, abort_flag)) { *abort_flag = 1; ok = false; break; }
         tc_fence_after();
-        for (int kb = 0; kb < n_k; ++kb, ++it) {
-          const int s = it % STAGES;
-          if (!mbar_wait(&full[s], (it / STAGES) & 1) || *abort_flag) { *abort_flag = 1; ok = false; break; }
-          tc_fence_after();
-          // k-contiguous operands: eight k = 32 bytes along the swizzled row; m/n-contiguous operands: eight k
-          // = eight 128-byte rows.  (Descriptor addresses count 16-byte units.)
-          const uint32_t a_lo = MN ? (uint32_t)smem_desc_mn_sw128(base + s * STAGE_BYTES, BK * 128)
-                                   : (uint32_t)smem_desc_sw128(base + s * STAGE_BYTES);
-          const uint32_t b_lo = MN ? (uint32_t)smem_desc_mn_sw128(base + s * STAGE_BYTES + A_BYTES, BK * 128)
-                                   : (uint32_t)smem_desc_sw128(base + s * STAGE_BYTES + A_BYTES);
-          constexpr uint32_t K_STEP = MN ? 1024 / 16 : 32 / 16;
+        // k-contiguous operands: eight k = 32 bytes along the swizzled row; m/n-contiguous operands: eight k
+        // = eight 128-byte rows.  (Descriptor addresses count 16-byte units.)
+        const uint32_t a_lo = MN ? (uint32_t)smem_desc_mn_sw128(base + s * STAGE_BYTES, BK * 128)
+                                 : (uint32_t)smem_desc_sw128(base + s * STAGE_BYTES);
+        const uint32_t b_lo = MN ? (uint32_t)smem_desc_mn_sw128(base + s * STAGE_BYTES + A_BYTES, BK * 128)
+                                 : (uint32_t)smem_desc_sw128(base + s * STAGE_BYTES + A_BYTES);
+        constexpr uint32_t K_STEP = MN ? 1024 / 16 : 32 / 16;
 #pragma unroll
-          for (int k = 0; k < BK / 8; ++k)
-            umma_tf32_split(tmem_acc + ab * BN, a_lo + k * K_STEP, desc_hi, b_lo + k * K_STEP, desc_hi, idesc, (kb | k) ? 1u : 0u);
-          umma_commit(&empty[s]);            // the stage may be refilled once these MMAs have read it
-        }
-        if (ok) umma_commit(&acc_full[ab]);
-        ++tile_i;
+        for (int k = 0; k < BK / 8; ++k)
+          umma_tf32(tmem_acc + ab * BN, a_lo + k * K_STEP, desc_hi, b_lo + k * K_STEP, desc_hi, idesc, (kb | k) ? 1u : 0u);
+        umma_commit(&empty[s]);            // the stage may be refilled once these MMAs have read it
       }
+      if (ok) umma_commit(&acc_full[ab]);
+      ++tile_i;
     }
   } else {
     const int quarter = warp & 3;
@@ -331,7 +329,7 @@ __global__ void __launch_bounds__(192, 2) tc5_fwd_narrow(const __grid_constant__
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
   volatile uint32_t* abort_flag = tmem_slot + 1;
   float* stage_out = reinterpret_cast<float*>(tiles + NR_STAGES * NR_STAGE + 256);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, n0 = blockIdx.x * NR_BN;
+  const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31, n0 = blockIdx.x * NR_BN;
   int grp = 0, m0 = 0, m_end = 0;
   if (!locate_group_tile<NR_BM>(gt, a.b, blockIdx.y, grp, m0, m_end)) return;
   const int n_k = (ga.K + 2 * BK - 1) / (2 * BK);      // what lies beyond K arrives as zeros
@@ -348,7 +346,7 @@ __global__ void __launch_bounds__(192, 2) tc5_fwd_narrow(const __grid_constant__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = warp_uniform(*tmem_slot);
   pdl_enter();
   if (warp == 0) {
     if (lane == 0) {
@@ -365,29 +363,26 @@ __global__ void __launch_bounds__(192, 2) tc5_fwd_narrow(const __grid_constant__
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = instr_desc_tf32(NR_BM, NR_BN);
-      const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0) >> 32);
-      const uint32_t a_lo0 = (uint32_t)smem_desc_sw128(base), b_lo0 = (uint32_t)smem_desc_sw128(base + NR_A);
-      const uint32_t full0 = smem_u32(full), empty0 = smem_u32(empty);
-      bool go_on = true;
-      uint32_t parity = 0;
-      for (int kb = 0; go_on && kb < n_k; parity ^= 1) {
+    constexpr uint32_t idesc = instr_desc_tf32(NR_BM, NR_BN);
+    const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0) >> 32);
+    const uint32_t a_lo0 = (uint32_t)smem_desc_sw128(base), b_lo0 = (uint32_t)smem_desc_sw128(base + NR_A);
+    bool go_on = true;
+    uint32_t parity = 0;
+    for (int kb = 0; go_on && kb < n_k; parity ^= 1) {
 #pragma unroll
-        for (int s = 0; s < NR_STAGES; ++s, ++kb) {
-          if (kb >= n_k) { go_on = false; break; }
-          if (!mbar_wait_addr(full0 + 8 * s, parity) || *abort_flag) { *abort_flag = 1; go_on = false; break; }
-          tc_fence_after();
+      for (int s = 0; s < NR_STAGES; ++s, ++kb) {
+        if (kb >= n_k) { go_on = false; break; }
+        if (!warp_wait(&full[s], parity, abort_flag)) { *abort_flag = 1; go_on = false; break; }
+        tc_fence_after();
 #pragma unroll
-          for (int k = 0; k < 2 * BK / 8; ++k) {
-            const uint32_t off = s * (NR_STAGE / 16) + (k / 4) * (NR_HALF / 16) + 2 * (k % 4);
-            umma_tf32_split(tmem, a_lo0 + off, desc_hi, b_lo0 + off, desc_hi, idesc, (s | k) ? 1u : (kb ? 1u : 0u));
-          }
-          umma_commit_addr(empty0 + 8 * s);
+        for (int k = 0; k < 2 * BK / 8; ++k) {
+          const uint32_t off = s * (NR_STAGE / 16) + (k / 4) * (NR_HALF / 16) + 2 * (k % 4);
+          umma_tf32(tmem, a_lo0 + off, desc_hi, b_lo0 + off, desc_hi, idesc, (s | k) ? 1u : (kb ? 1u : 0u));
         }
+        umma_commit(&empty[s]);
       }
-      umma_commit(acc_full);
     }
+    umma_commit(acc_full);
   } else {
     if (warps_agree<1, 128>(mbar_wait(acc_full, 0))) {      // the four warps meet at a barrier below: all of them or none
       tc_fence_after();
@@ -445,7 +440,7 @@ __global__ void __launch_bounds__(256, 1) tc5_dx_split(const __grid_constant__ G
   uint64_t* acc_full = full + S::KB;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
   volatile uint32_t* abort_flag = tmem_slot + 1;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rank = blockIdx.z, n0 = blockIdx.x * S::BN;
+  const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31, rank = blockIdx.z, n0 = blockIdx.x * S::BN;
   int grp = 0, m0 = 0, m_end = 0;
   if (!locate_group_tile<BM>(gt, a.b, blockIdx.y, grp, m0, m_end)) return;           // the same for all CTAs of a cluster
   if (tid == 0) {
@@ -466,21 +461,20 @@ __global__ void __launch_bounds__(256, 1) tc5_dx_split(const __grid_constant__ G
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = warp_uniform(*tmem_slot);
   pdl_enter();
-  if (warp == 1 && lane == 0) {
+  if (warp == 1) {
     constexpr uint32_t idesc = instr_desc_tf32(BM, S::BN);
     const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0) >> 32);
     for (int i = 0; i < S::KB; ++i) {
-      if (!mbar_wait(&full[i], 0)) { *abort_flag = 1; break; }
+      if (!warp_wait(&full[i], 0, abort_flag)) { *abort_flag = 1; break; }
       tc_fence_after();
       const uint32_t a_lo = (uint32_t)smem_desc_sw128(base + i * S::STAGE_BYTES), b_lo = (uint32_t)smem_desc_sw128(base + i * S::STAGE_BYTES + A_BYTES);
 #pragma unroll
-      for (int k = 0; k < BK / 8; ++k) umma_tf32_split(tmem, a_lo + 2 * k, desc_hi, b_lo + 2 * k, desc_hi, idesc, (i | k) ? 1u : 0u);
+      for (int k = 0; k < BK / 8; ++k) umma_tf32(tmem, a_lo + 2 * k, desc_hi, b_lo + 2 * k, desc_hi, idesc, (i | k) ? 1u : 0u);
     }
     umma_commit(acc_full);
   }
-  __syncwarp();
   float* part = reinterpret_cast<float*>(tiles);
   if (__syncthreads_and(mbar_wait(acc_full, 0))) {          // tensor memory is read by whole warps: all threads or none
     tc_fence_after();

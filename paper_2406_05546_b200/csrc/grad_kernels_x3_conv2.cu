@@ -172,11 +172,11 @@ __global__ void __launch_bounds__(F_THREADS, 1) conv2_fwd_x3(GradStepArgs a, Gro
         const uint32_t start = i == 0 || i == 5 ? 0u : 1u;
 #pragma unroll
         for (int op = 0; op < F_OPS; ++op)
-          umma_f16_warp(di + fold.d_col[op], ai + fold.a_off[op], plain_desc_hi(2 * P1X_ROW), bi + fold.b_row[op], plain_desc_hi(128), fold.idesc[op],
-                        op ? 1u : start);
+          umma_f16(di + fold.d_col[op], ai + fold.a_off[op], plain_desc_hi(2 * P1X_ROW), bi + fold.b_row[op], plain_desc_hi(128), fold.idesc[op],
+                   op ? 1u : start);
       }
-      umma_commit_warp(&a_empty[buf]);
-      umma_commit_warp(&acc_full[buf]);
+      umma_commit(&a_empty[buf]);
+      umma_commit(&acc_full[buf]);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -349,12 +349,12 @@ __global__ void __launch_bounds__(X_THREADS, 1) conv2_dx_x3(GradStepArgs a, Grou
           for (int q = 0; q < 2; ++q)                      // sixteen output channels
 #pragma unroll
             for (int p = 0; p < PIECES; ++p)
-              umma_f16_warp(d + p * 48, a_lo + p * (X_PIECE_BYTES / 16) + 2 * q * (X_PLANE_BYTES / 16) + (2 - ky) * 16, plain_desc_hi(128),
+              umma_f16(d + p * 48, a_lo + p * (X_PIECE_BYTES / 16) + 2 * q * (X_PLANE_BYTES / 16) + (2 - ky) * 16, plain_desc_hi(128),
                             w_lo + (ky * 4 + 2 * q) * (OCT / 16), plain_desc_hi(128), idesc_x3(48 * (PIECES - p), false), (ky | q | p) ? 1u : 0u);
-        umma_commit_warp(&acc_full[ab]);
+        umma_commit(&acc_full[ab]);
         if (++ab == X_ACC) { ab = 0; ab_parity ^= 1; }
       }
-      if (ok) umma_commit_warp(&a_empty[buf]);
+      if (ok) umma_commit(&a_empty[buf]);
     }
   } else if (warp <= 8) {
     const int grp_w = (warp - 1) >> 2, lt = (tid - 32) & 127;
@@ -517,14 +517,14 @@ __global__ void __launch_bounds__(D_THREADS, 1) conv2_dw_x3(GradStepArgs a, Work
 #pragma unroll
         for (int k = 0; k < 14; ++k) {                     // image rows 2 (k / 2) and + 1, columns of parity k & 1
           const int xp = (k & 1) + kx;                     // the first column read, 0 .. 3
-          umma_f16_warp(tmem + kx * 144, g_lo + (k >> 1) * (2 * D_G_ROW / 16) + (k & 1) * 8, plain_desc_hi(256),
+          umma_f16(tmem + kx * 144, g_lo + (k >> 1) * (2 * D_G_ROW / 16) + (k & 1) * 8, plain_desc_hi(256),
                         p_lo + (k >> 1) * (2 * P1X_ROW / 16) + (xp & 1) * 8 + (xp >> 1), plain_desc_hi(256), idesc, k ? 1u : 0u);
         }
-        umma_commit_warp(&acc_full[kx]);
+        umma_commit(&acc_full[kx]);
       }
       if (!ok) break;
-      umma_commit_warp(&p1_empty[slot]);
-      umma_commit_warp(&g_empty[st]);
+      umma_commit(&p1_empty[slot]);
+      umma_commit(&g_empty[st]);
       if (++slot == D_P1_SLOTS) { slot = 0; slot_parity ^= 1; }
     }
   } else if (warp == 1) {

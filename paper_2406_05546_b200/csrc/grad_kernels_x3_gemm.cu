@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_x3(const __grid_constant__ Ma
   uint64_t* small_empty = lead_empty + BUFS; // [BUFS] epilogue -> MMA
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(small_empty + BUFS);
   volatile uint32_t* abort_flag = tmem_slot + 1;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
   const int n_k = (ga.K + BK - 1) / BK;
   int kb0 = 0, kb1 = n_k;                    // this CTA's blocks of k
   if (S::SPLIT) {
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_x3(const __grid_constant__ Ma
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = warp_uniform(*tmem_slot);
   pdl_enter();
 
   if (warp == 0) {
@@ -157,42 +157,40 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_x3(const __grid_constant__ Ma
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = instr_desc<S>(), ha = desc_hi<S::A_MN>(), hb = desc_hi<S::B_MN>();
-      constexpr uint32_t pa = S::A_PIECE / 16, pb = S::B_PIECE / 16, ka = k_step<S::A_MN>(), kbs = k_step<S::B_MN>();
-      int s = 0, lead = 0, tile_i = 0;       // stage; chunks of leading products, and tiles, so far
-      uint32_t parity = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < ga.n_tiles && ok; t += gridDim.x) {
-        Tile c;
-        if (!decode<S>(ga, gt, a.b, t, c)) continue;
-        const uint32_t d_small = tmem + (BUFS + tile_i % BUFS) * S::ACC;
-        if (tile_i >= BUFS && !mbar_wait(&small_empty[tile_i % BUFS], ((tile_i / BUFS) - 1) & 1)) { *abort_flag = 1; break; }
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(&full[s], parity) || *abort_flag) { *abort_flag = 1; ok = false; break; }
-          tc_fence_after();
-          const uint32_t a_lo = desc_lo<S::A_MN>(base + s * S::STAGE), b_lo = desc_lo<S::B_MN>(base + s * S::STAGE + S::A_BYTES);
-          const bool first = (kb - kb0) % CHUNK == 0, last = (kb - kb0) % CHUNK == CHUNK - 1 || kb + 1 == kb1;
+    constexpr uint32_t idesc = instr_desc<S>(), ha = desc_hi<S::A_MN>(), hb = desc_hi<S::B_MN>();
+    constexpr uint32_t pa = S::A_PIECE / 16, pb = S::B_PIECE / 16, ka = k_step<S::A_MN>(), kbs = k_step<S::B_MN>();
+    int s = 0, lead = 0, tile_i = 0;       // stage; chunks of leading products, and tiles, so far
+    uint32_t parity = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < ga.n_tiles && ok; t += gridDim.x) {
+      Tile c;
+      if (!decode<S>(ga, gt, a.b, t, c)) continue;
+      const uint32_t d_small = tmem + (BUFS + tile_i % BUFS) * S::ACC;
+      if (tile_i >= BUFS && !warp_wait(&small_empty[tile_i % BUFS], ((tile_i / BUFS) - 1) & 1, abort_flag)) { *abort_flag = 1; break; }
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!warp_wait(&full[s], parity, abort_flag)) { *abort_flag = 1; ok = false; break; }
+        tc_fence_after();
+        const uint32_t a_lo = desc_lo<S::A_MN>(base + s * S::STAGE), b_lo = desc_lo<S::B_MN>(base + s * S::STAGE + S::A_BYTES);
+        const bool first = (kb - kb0) % CHUNK == 0, last = (kb - kb0) % CHUNK == CHUNK - 1 || kb + 1 == kb1;
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k)
+        for (int k = 0; k < BK / 16; ++k)
 #pragma unroll
-            for (int i = 0; i < 5; ++i) {    // l h, m m, h l, m h, h m
-              const int i_a = i == 0 ? 2 : (i == 1 || i == 3 ? 1 : 0), i_b = i == 2 ? 2 : (i == 1 || i == 4 ? 1 : 0);
-              umma_f16_split(d_small, a_lo + i_a * pa + k * ka, ha, b_lo + i_b * pb + k * kbs, hb, idesc, (k | i) ? 1u : (kb > kb0 ? 1u : 0u));
-            }
-          if (first && lead >= BUFS) {
-            if (!mbar_wait(&lead_empty[lead % BUFS], ((lead / BUFS) - 1) & 1)) { *abort_flag = 1; ok = false; break; }
-            tc_fence_after();
+          for (int i = 0; i < 5; ++i) {    // l h, m m, h l, m h, h m
+            const int i_a = i == 0 ? 2 : (i == 1 || i == 3 ? 1 : 0), i_b = i == 2 ? 2 : (i == 1 || i == 4 ? 1 : 0);
+            umma_f16(d_small, a_lo + i_a * pa + k * ka, ha, b_lo + i_b * pb + k * kbs, hb, idesc, (k | i) ? 1u : (kb > kb0 ? 1u : 0u));
           }
-          const uint32_t d_lead = tmem + (lead % BUFS) * S::ACC;
-#pragma unroll
-          for (int k = 0; k < BK / 16; ++k) umma_f16_split(d_lead, a_lo + k * ka, ha, b_lo + k * kbs, hb, idesc, k ? 1u : (first ? 0u : 1u));
-          umma_commit(&empty[s]);
-          if (last) { umma_commit(&lead_full[lead % BUFS]); ++lead; }
-          if (++s == STAGES) { s = 0; parity ^= 1; }
+        if (first && lead >= BUFS) {
+          if (!warp_wait(&lead_empty[lead % BUFS], ((lead / BUFS) - 1) & 1, abort_flag)) { *abort_flag = 1; ok = false; break; }
+          tc_fence_after();
         }
-        ++tile_i;
+        const uint32_t d_lead = tmem + (lead % BUFS) * S::ACC;
+#pragma unroll
+        for (int k = 0; k < BK / 16; ++k) umma_f16(d_lead, a_lo + k * ka, ha, b_lo + k * kbs, hb, idesc, k ? 1u : (first ? 0u : 1u));
+        umma_commit(&empty[s]);
+        if (last) { umma_commit(&lead_full[lead % BUFS]); ++lead; }
+        if (++s == STAGES) { s = 0; parity ^= 1; }
       }
+      ++tile_i;
     }
   } else {
     const int quarter = warp & 3, half = (warp - 2) >> 2, col0 = half * COLS;

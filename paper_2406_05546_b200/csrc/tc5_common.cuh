@@ -72,54 +72,33 @@ __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* m
       ::"r"(smem_u32(smem_dst)), "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
 
-__device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// Same, with each descriptor given as its two 32-bit halves: the high half (strides, version, layout) is
-// a constant of the kernel and the low half is "start address / 16 + a compile-time offset", so a fully
-// unrolled issue loop costs one integer add per operand and MMA.
-__device__ __forceinline__ void umma_tf32_split(uint32_t tmem_d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
-                                                uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-      "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
-      "setp.ne.b32 p, %6, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %5, p;\n\t}"
-      ::"r"(tmem_d), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
-}
+// MMAs, issued by a whole warp that has stayed together: one lane of it, always the same, issues.  Where a single lane's branch computes
+// the operands' addresses, each of them goes from a vector register to a uniform one for every instruction; where the warp's lanes agree
+// they are computed in uniform registers to begin with.  Clocks per instruction of the second convolution's products on the FP32
+// path (M = 128, N = 32 .. 144, K = 16), one lane's branch -> whole warp: forward 86 -> 56, input gradient 96 -> 72.  us of kernels whose one
+// issuing thread was behind: conv2_dw_tc5 85.4 -> 71.8 at 128 x 128 and 14.6 -> 12.8 at 4 x 16, tc5_fwd_narrow 17.9 -> 15.2 at 2 x 8, gemm_x3's
+// weight gradient 171 -> 164 at 128 x 128, tc5_gemm's input gradient 53.7 -> 51.5; where two CTAs of an SM issue in turn (conv2_fwd_tc5,
+// conv2_dx_tc5) nothing changes.
+// Each descriptor is given as its two 32-bit halves: the high half (strides, version, layout) is a constant of the kernel and the low half
+// is "start address / 16 + a compile-time offset", so that an unrolled issue loop costs one integer add per operand and MMA.
+// BF16 / FP16 inputs: K = 16 per instruction; TF32: K = 8.  fp32 accumulation.
+#define PSK_UMMA(NAME, KIND)                                                                                                       \
+  __device__ __forceinline__ void NAME(uint32_t tmem_d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc, \
+                                       uint32_t accumulate) {                                                                      \
+    asm volatile(                                                                                                                  \
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"                                                                           \
+        "elect.sync _|q, 0xffffffff;\n\t"                                                                                          \
+        "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"                                                                       \
+        "setp.ne.b32 p, %6, 0;\n\t"                                                                                                \
+        "@q tcgen05.mma.cta_group::1.kind::" KIND " [%0], da, db, %5, p;\n\t}"                                                     \
+        ::"r"(tmem_d), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");                        \
+  }
+PSK_UMMA(umma_f16, "f16")
+PSK_UMMA(umma_tf32, "tf32")
+#undef PSK_UMMA
 
-// BF16 / FP16 inputs (K = 16 per instruction), fp32 accumulation; descriptors as above.
-__device__ __forceinline__ void umma_f16_split(uint32_t tmem_d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
-                                               uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-      "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
-      "setp.ne.b32 p, %6, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
-      ::"r"(tmem_d), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
-}
-
-__device__ __forceinline__ void umma_commit_addr(uint32_t bar_addr) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar_addr) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint64_t* bar) { umma_commit_addr(smem_u32(bar)); }
-// The same for a whole warp that has stayed together: one lane of it, always the same, issues.  An address that a single lane's branch
-// computes goes from a vector register to a uniform one for every operand of every instruction; where the warp's lanes agree
-// it is computed in uniform registers to begin with.  Clocks per instruction of the second convolution's products on the
-// FP32 path (M = 128, N = 32 .. 144, K = 16), before -> after: forward 86 -> 56, input gradient 96 -> 72.
-__device__ __forceinline__ void umma_f16_warp(uint32_t tmem_d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
-      "elect.sync _|q, 0xffffffff;\n\t"
-      "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
-      "setp.ne.b32 p, %6, 0;\n\t"
-      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
-      ::"r"(tmem_d), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void umma_commit_warp(uint64_t* bar) {
+// Arrives on the barrier when the warp's MMAs so far are done.
+__device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile(
       "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
       "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)) : "memory");

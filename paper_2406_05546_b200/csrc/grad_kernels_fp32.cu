@@ -15,15 +15,47 @@ namespace psk {
 
 namespace {
 
-// ---- conv1 (1->16, 3x3, pad 1) + ReLU + 2x2 max pool.  A block handles up to CONV1_SPB samples of one
-// worker.  Thread = pooled position: it reads the 4x4 input patch under its 2x2 window once and
-// evaluates all 16 channels from registers (576 multiply-adds per 8 + 48 shared-memory loads).
-// (FP32 path; the tensor-core path has its own kernel, which writes the layout its convolutions copy from.)
-constexpr int CONV1_SPB = 8;      // most samples per block
+// ---- conv1 (1->16, 3x3, pad 1) + ReLU + 2x2 max pool, and its filter gradient.  (FP32 path; the tensor-core path has its own kernels.)
+// A thread owns a quad of four output channels, packed multiply-adds over channel pairs, and takes seven of a sample's 784 items
+// (pooled position, quad) in turn: per item it reads the 4x4 input patch under its pooling window once.  The next sample's
+// image is fetched into registers meanwhile.
+// Measured (~6 us of event overhead included) at 128 x 128 (3.7 GFLOP, 58 us at the packed multiply-add's rate) / 16 x 64: forward 193 / 20.1 us
+// with scalar multiply-adds and all sixteen channels of a position in one thread, 162 / 17 now, 187 with six blocks per SM (80 registers);
+// filter gradient 171 / 19.0 with one multiply-add per pixel read, 146 / 19.0 now (170 / 24 with an item's gradients fetched one item
+// ahead).  The FMA pipe is busy for half of the cycles, the issue slots likewise: four blocks of four warps leave latencies open.
+constexpr int CONV1_SPB = 8;            // most samples per block, forward
+constexpr int CONV1_ITEMS = 112;        // items taken at a time: 28 positions (two rows of 14) x 4 quads
+constexpr int CONV1_THREADS = 128;      // the last sixteen have none
+constexpr int CONV1_PITCH = 32, CONV1_IMAGE = 30 * CONV1_PITCH;      // zero-bordered image, column x at x + 1
+
+// The thread's seven pixels of an image; where they go.
+struct ImagePart {
+  float v[7];
+  __device__ __forceinline__ void load(const float* x, int tid) {
+#pragma unroll
+    for (int k = 0; k < 7; ++k) v[k] = tid < CONV1_ITEMS ? x[tid + CONV1_ITEMS * k] : 0.f;
+  }
+  __device__ __forceinline__ void store(float* image, int tid) const {      // 112 pixels = four rows
+    float* d = image + (tid / IMG + 1) * CONV1_PITCH + tid % IMG + 1;
+    if (tid < CONV1_ITEMS) {
+#pragma unroll
+      for (int k = 0; k < 7; ++k) d[4 * k * CONV1_PITCH] = v[k];
+    }
+  }
+};
+// The 4x4 patch under the pooling window at (py, px), every value in both halves.
+__device__ __forceinline__ void load_patch(const float* image, int py, int px, u64 (&dup)[4][4]) {
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const float2 lo = *reinterpret_cast<const float2*>(image + (2 * py + r) * CONV1_PITCH + 2 * px);
+    const float2 hi = *reinterpret_cast<const float2*>(image + (2 * py + r) * CONV1_PITCH + 2 * px + 2);
+    dup[r][0] = pack2(lo.x, lo.x); dup[r][1] = pack2(lo.y, lo.y); dup[r][2] = pack2(hi.x, hi.x); dup[r][3] = pack2(hi.y, hi.y);
+  }
+}
 
 // The second convolution's filters of a weight group as its kernels' operands, one row of eight values (in pieces) per thread.
 // Blocks of conv1_fwd beyond its workers do it, so that the next kernel finds them without a launch or a fork of their own.
-constexpr int BANK3_ROWS = 2 * BANK3_FWD_ROWS + 12 * 48, BANK3_UNITS = (BANK3_ROWS + 223) / 224;      // blocks per weight group
+constexpr int BANK3_ROWS = 2 * BANK3_FWD_ROWS + 12 * 48, BANK3_UNITS = (BANK3_ROWS + CONV1_THREADS - 1) / CONV1_THREADS;      // blocks per weight group
 __device__ __forceinline__ void build_bank3(const float* __restrict__ theta, uint8_t* __restrict__ bank, int e, const Bank3Taps& taps) {
   if (e >= BANK3_ROWS) return;
   float v[8];
@@ -47,166 +79,199 @@ __device__ __forceinline__ void build_bank3(const float* __restrict__ theta, uin
   for (int p = 0; p < PIECES; ++p) *reinterpret_cast<uint4*>(d + p * piece_bytes) = make_uint4(s[0].p[p], s[1].p[p], s[2].p[p], s[3].p[p]);
 }
 
-__global__ void __launch_bounds__(224) conv1_fwd(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws, int spb, const __grid_constant__ Bank3Taps taps) {
-  __shared__ __align__(16) float xs[2][30][32];
-  __shared__ __align__(16) float w[16][12];   // 9 taps + bias + padding
+__global__ void __launch_bounds__(CONV1_THREADS, 4) conv1_fwd(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws, int spb, const __grid_constant__ Bank3Taps taps) {
+  __shared__ __align__(16) float xs[2][CONV1_IMAGE];
   const int s = blockIdx.y, tid = threadIdx.x;
   if (s >= a.W) {
     const int u = (s - a.W) * gridDim.x + blockIdx.x, g = u / BANK3_UNITS;
     pdl_enter();
-    if (g < gt.n_groups) build_bank3(gt.theta[g], ws.bank2 + (int64_t)g * BANK3_BYTES, (u - g * BANK3_UNITS) * 224 + tid, taps);
+    if (g < gt.n_groups) build_bank3(gt.theta[g], ws.bank2 + (int64_t)g * BANK3_BYTES, (u - g * BANK3_UNITS) * CONV1_THREADS + tid, taps);
     return;
   }
   const float* theta = group_theta(wt, gt, s);
-  pdl_enter();       // the weights may come from the apply just before
-  if (tid < 160) {
-    if (tid < 144) w[tid / 9][tid % 9] = theta[OFF_C1W + tid];
-    else w[tid - 144][9] = theta[OFF_C1B + tid - 144];
-  }
-  for (int t = tid; t < 2 * 30 * 32; t += 224) (&xs[0][0][0])[t] = 0.f;
+  for (int t = tid; t < 2 * CONV1_IMAGE; t += CONV1_THREADS) (&xs[0][0])[t] = 0.f;
+  const int cg = tid & 3, px = (tid >> 2) % 14, py0 = (tid >> 2) / 14;
   const int i0 = blockIdx.x * spb, i1 = min(i0 + spb, a.b);
-  const int py = tid / 14, px = tid - py * 14;
-  const bool active = tid < 196;
+  const float* x = a.x + (int64_t)wt.src[s] * a.b * (IMG * IMG);
+  pdl_enter();       // the weights may come from the apply just before
+  ImagePart next;
+  next.load(x + (int64_t)i0 * (IMG * IMG), tid);
+  u64 wp[2][10];     // wp[cp][k] = tap k of channels 4 cg + 2 cp and + 1; k = 9 is the bias
+#pragma unroll
+  for (int cp = 0; cp < 2; ++cp) {
+    const int c0 = 4 * cg + 2 * cp;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) wp[cp][k] = pack2(theta[OFF_C1W + c0 * 9 + k], theta[OFF_C1W + (c0 + 1) * 9 + k]);
+    wp[cp][9] = pack2(theta[OFF_C1B + c0], theta[OFF_C1B + c0 + 1]);
+  }
   __syncthreads();
-  auto stage = [&](int i, int bufi) {
-    const float* x = a.x + ((int64_t)wt.src[s] * a.b + i) * (IMG * IMG);
-    for (int t = tid; t < IMG * IMG; t += 224) {
-      int yy = t / IMG, xx = t - yy * IMG;
-      xs[bufi][yy + 1][xx + 1] = x[t];
-    }
-  };
-  stage(i0, 0);
+  next.store(xs[0], tid);
   for (int i = i0; i < i1; ++i) {
     const int cur = (i - i0) & 1;
     __syncthreads();                       // image `cur` is complete; image `cur^1` is no longer read
-    if (i + 1 < i1) stage(i + 1, cur ^ 1);
-    const int64_t row = (int64_t)s * a.b + i;
-    // a position's sixteen channels in pieces: six 16-byte slots; Y and X in the bordered map
-    auto store = [&](int Y, int X, const float (&v)[16]) {
-      uint8_t* d = ws.p1x + row * P1X_BYTES + Y * P1X_ROW + ((X & 1) * 8 + (X >> 1)) * 16;
+    if (i + 1 < i1) next.load(x + (int64_t)(i + 1) * (IMG * IMG), tid);
+    if (tid < CONV1_ITEMS) {
+      const int64_t row = (int64_t)s * a.b + i;
+      // a position's channel quad in pieces, half of a 16-byte slot each; Y and X in the bordered map
+      uint8_t* out = ws.p1x + row * P1X_BYTES + (cg >> 1) * 256 + (cg & 1) * 8;
+      auto slot = [&](int Y, int X) { return out + Y * P1X_ROW + ((X & 1) * 8 + (X >> 1)) * 16; };
+      {                                    // the zeros at either end of the fourteen image rows: whole runs leave
+        uint8_t* d = slot((tid >> 3) + 1, ((tid >> 2) & 1) * 15);
 #pragma unroll
-      for (int o = 0; o < 2; ++o) {
-        const Bf16x3 q[4] = {split3(v[8 * o], v[8 * o + 1]), split3(v[8 * o + 2], v[8 * o + 3]), split3(v[8 * o + 4], v[8 * o + 5]), split3(v[8 * o + 6], v[8 * o + 7])};
-#pragma unroll
-        for (int p = 0; p < PIECES; ++p) *reinterpret_cast<uint4*>(d + (2 * p + o) * 256) = make_uint4(q[0].p[p], q[1].p[p], q[2].p[p], q[3].p[p]);
+        for (int p = 0; p < PIECES; ++p) *reinterpret_cast<uint2*>(d + p * 512) = make_uint2(0u, 0u);
       }
-    };
-    if (!active) {                         // 28 threads for the zeros at either end of the fourteen image rows: whole runs leave
-      const float zero[16] = {};
-      store((tid - 196) / 2 + 1, (tid & 1) * 15, zero);
-      continue;
-    }
-    float patch[4][4];
+#pragma unroll 1
+      for (int k = 0; k < 7; ++k) {
+        const int py = py0 + 2 * k;
+        u64 dup[4][4], acc[2][4];
+        load_patch(xs[cur], py, px, dup);
 #pragma unroll
-    for (int yy = 0; yy < 4; ++yy) {
-      float2 lo = *reinterpret_cast<const float2*>(&xs[cur][2 * py + yy][2 * px]);
-      float2 hi = *reinterpret_cast<const float2*>(&xs[cur][2 * py + yy][2 * px + 2]);
-      patch[yy][0] = lo.x; patch[yy][1] = lo.y; patch[yy][2] = hi.x; patch[yy][3] = hi.y;
-    }
-    float outv[16];
-    uint8_t outc[16];
+        for (int cp = 0; cp < 2; ++cp)
 #pragma unroll
-    for (int ch = 0; ch < 16; ++ch) {
-      const float4 w0 = *reinterpret_cast<const float4*>(&w[ch][0]);
-      const float4 w1 = *reinterpret_cast<const float4*>(&w[ch][4]);
-      const float4 w2 = *reinterpret_cast<const float4*>(&w[ch][8]);
-      const float wv[9] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w, w2.x};
-      const float bias = w2.y;
-      float best = 0.f;
-      int bi = 0;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int jy = j >> 1, jx = j & 1;
-        float v = bias;
+          for (int j = 0; j < 4; ++j) acc[cp][j] = wp[cp][9];
 #pragma unroll
         for (int ky = 0; ky < 3; ++ky)
 #pragma unroll
-          for (int kx = 0; kx < 3; ++kx) v = fmaf(wv[ky * 3 + kx], patch[jy + ky][jx + kx], v);
-        float r = fmaxf(v, 0.f);
-        if (j == 0 || r > best) { best = r; bi = j; }
-      }
-      outv[ch] = best;
-      outc[ch] = best > 0.f ? (uint8_t)bi : (uint8_t)4;
-    }
-    const int pp = tid;
+          for (int kx = 0; kx < 3; ++kx)
 #pragma unroll
-    for (int ch = 0; ch < 16; ++ch) ws.code1[row * P1_ELEMS + ch * 196 + pp] = outc[ch];
-    store(py + 1, px + 1, outv);
+            for (int cp = 0; cp < 2; ++cp)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) acc[cp][j] = ffma2(wp[cp][ky * 3 + kx], dup[(j >> 1) + ky][(j & 1) + kx], acc[cp][j]);
+        float v[4][4];     // [channel][window element]
+#pragma unroll
+        for (int cp = 0; cp < 2; ++cp)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) unpack2(acc[cp][j], v[2 * cp][j], v[2 * cp + 1][j]);
+        // ReLU then max = max then ReLU; the winner is the first window element that reaches the maximum.  The maximum is taken
+        // against the smallest positive number: no element of a dead window equals it, and its pieces are zeros.
+        float best[4];
+        uint32_t codes = 0u;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float m = fmaxf(fmaxf(fmaxf(v[c][0], v[c][1]), fmaxf(v[c][2], v[c][3])), __int_as_float(1));
+          best[c] = m;
+          uint32_t e = v[c][3] == m ? 3u << (8 * c) : 4u << (8 * c);
+          e = v[c][2] == m ? 2u << (8 * c) : e;
+          e = v[c][1] == m ? 1u << (8 * c) : e;
+          codes |= v[c][0] == m ? 0u : e;
+        }
+        const Bf16x3 q0 = split3(best[0], best[1]), q1 = split3(best[2], best[3]);
+        uint8_t* d = slot(py + 1, px + 1);
+#pragma unroll
+        for (int p = 0; p < PIECES; ++p) *reinterpret_cast<uint2*>(d + p * 512) = make_uint2(q0.p[p], q1.p[p]);
+        reinterpret_cast<uint32_t*>(ws.code1 + row * P1_ELEMS)[cg * 196 + py * 14 + px] = codes;
+      }
+    }
+    next.store(xs[cur ^ 1], tid);
   }
 }
 
-// ---- backward through pool1, ReLU and conv1 (filter / bias gradients only: the input needs none).
-// Thread (channel, lane of 16) owns 13 pooled positions of its channel.  The image, the pooling decisions
-// and the pooled gradients of the NEXT sample are fetched into registers while the current one is
-// accumulated, so that no global-memory latency sits between the multiply-adds.
+// ---- backward through pool1, ReLU and conv1 (filter / bias gradients only: the input needs none): per window element the pooled
+// gradients of the channels that it won, all others cleared, times the patch.  A sample's gradients and decisions arrive by
+// asynchronous copies while the sample before is added up.
 constexpr int CONV1B_SPB = 16;            // most samples per block
-__global__ void __launch_bounds__(256) conv1_bwd(GradStepArgs a, WorkerTable wt, Workspace ws, int spb, int n_chunks) {
-  __shared__ float xs[30][31];
-  constexpr int PER = 13;                   // ceil(196 / 16)
-  const int s = blockIdx.y, tid = threadIdx.x;
-  const int oc = tid >> 4, l = tid & 15;
-  float gw[9], gb = 0.f;
+__global__ void __launch_bounds__(CONV1_THREADS, 4) conv1_bwd(GradStepArgs a, WorkerTable wt, Workspace ws, int spb, int n_chunks) {
+  __shared__ __align__(16) float xs[2][CONV1_IMAGE];
+  __shared__ __align__(16) float4 gs[2][7][CONV1_ITEMS];
+  __shared__ uint32_t cs[2][7][CONV1_ITEMS];
+  float (*red)[C1_GRAD] = reinterpret_cast<float (*)[C1_GRAD]>(&gs[0][0][0]);      // the warps' sums take their place
+  const int s = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int cg = tid & 3, pos0 = tid >> 2, px = pos0 % 14, py0 = pos0 / 14;
+  const bool active = tid < CONV1_ITEMS;
+  for (int t = tid; t < 2 * CONV1_IMAGE; t += CONV1_THREADS) (&xs[0][0])[t] = 0.f;
+  const int i0 = blockIdx.x * spb, i1 = min(i0 + spb, a.b);
+  const float* x = a.x + (int64_t)wt.src[s] * a.b * (IMG * IMG);
+  const int64_t row0 = (int64_t)s * a.b;
+  u64 gw[2][9];                             // channel pair x tap
+  float gb[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-  for (int k = 0; k < 9; ++k) gw[k] = 0.f;
-  for (int t = tid; t < 30 * 31; t += 256) (&xs[0][0])[t] = 0.f;
-  const int i0 = blockIdx.x * spb;
-  const int i1 = min(i0 + spb, a.b);
-  float xr[4], gr[PER];
-  int cr[PER];
-  auto prefetch = [&](int i) {
-    const int64_t row = (int64_t)s * a.b + i;
-    const float* x = a.x + ((int64_t)wt.src[s] * a.b + i) * (IMG * IMG);
+  for (int cp = 0; cp < 2; ++cp)
 #pragma unroll
-    for (int k = 0; k < 4; ++k) xr[k] = tid + 256 * k < IMG * IMG ? x[tid + 256 * k] : 0.f;
+    for (int k = 0; k < 9; ++k) gw[cp][k] = 0ull;
+  // a thread's items of a sample, in its own places: dp1 and the decisions are [quad][position][4 channels]
+  auto fetch = [&](int i) {
+    if (active) {
+      const int buf = (i - i0) & 1;
+      const float4* g = reinterpret_cast<const float4*>(ws.dp1 + (row0 + i) * P1_ELEMS) + cg * 196 + pos0;
+      const uint32_t* c = reinterpret_cast<const uint32_t*>(ws.code1 + (row0 + i) * P1_ELEMS) + cg * 196 + pos0;
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int pp = l + 16 * k;
-      cr[k] = pp < 196 ? (int)ws.code1[row * P1_ELEMS + oc * 196 + pp] : 4;
-      gr[k] = pp < 196 ? ws.dp1[row * P1_ELEMS + oc * 196 + pp] : 0.f;
-    }
-  };
-  pdl_enter();
-  prefetch(i0);
-  for (int i = i0; i < i1; ++i) {
-    __syncthreads();                        // the previous sample's image is no longer read
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int t = tid + 256 * k;
-      if (t < IMG * IMG) xs[t / IMG + 1][t % IMG + 1] = xr[k];
-    }
-    float g_cur[PER];
-    int c_cur[PER];
-#pragma unroll
-    for (int k = 0; k < PER; ++k) { g_cur[k] = gr[k]; c_cur[k] = cr[k]; }
-    __syncthreads();
-    if (i + 1 < i1) prefetch(i + 1);
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      if (c_cur[k] < 4) {
-        const int pp = l + 16 * k;
-        const float g = g_cur[k];
-        const int y = 2 * (pp / 14) + (c_cur[k] >> 1), xq = 2 * (pp % 14) + (c_cur[k] & 1);
-        gb += g;
-#pragma unroll
-        for (int ky = 0; ky < 3; ++ky)
-#pragma unroll
-          for (int kx = 0; kx < 3; ++kx) gw[ky * 3 + kx] = fmaf(g, xs[y + ky][xq + kx], gw[ky * 3 + kx]);
+      for (int k = 0; k < 7; ++k) {
+        cp_async16(&gs[buf][k][tid], g + 28 * k, true);
+        cp_async4(&cs[buf][k][tid], c + 28 * k);
       }
     }
-  }
-  // fixed-order reduction over the 16 lanes that share an output channel
+    cp_async_commit();
+  };
+  ImagePart next;
+  next.load(x + (int64_t)i0 * (IMG * IMG), tid);
+  __syncthreads();
+  next.store(xs[0], tid);
+  pdl_enter();
+  fetch(i0);
+  for (int i = i0; i < i1; ++i) {
+    const int cur = (i - i0) & 1;
+    __syncthreads();                        // image `cur` is complete; image `cur^1` is no longer read
+    if (i + 1 < i1) {
+      next.load(x + (int64_t)(i + 1) * (IMG * IMG), tid);
+      fetch(i + 1);
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
+    }
+#pragma unroll 1
+    for (int k = 0; k < 7; ++k) {
+      const float4 g4 = active ? gs[cur][k][tid] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const uint32_t code = active ? cs[cur][k][tid] : 0x04040404u;
+      const float g[4] = {g4.x, g4.y, g4.z, g4.w};
+      u64 dup[4][4];
+      load_patch(xs[cur], active ? py0 + 2 * k : 0, px, dup);
+      uint32_t c[4];
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) {
-    gb += __shfl_xor_sync(0xffffffffu, gb, o);
+      for (int ch = 0; ch < 4; ++ch) {
+        c[ch] = (code >> (8 * ch)) & 255u;
+        gb[ch] += c[ch] < 4u ? g[ch] : 0.f;
+      }
 #pragma unroll
-    for (int k = 0; k < 9; ++k) gw[k] += __shfl_xor_sync(0xffffffffu, gw[k], o);
-  }
-  if (l == 0) {
-    float* part = ws.part1 + ((int64_t)s * n_chunks + blockIdx.x) * C1_GRAD;
+      for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int k = 0; k < 9; ++k) part[oc * 9 + k] = gw[k];
-    part[144 + oc] = gb;
+        for (int cp = 0; cp < 2; ++cp) {
+          const u64 gj = pack2(c[2 * cp] == j ? g[2 * cp] : 0.f, c[2 * cp + 1] == j ? g[2 * cp + 1] : 0.f);
+#pragma unroll
+          for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+            for (int kx = 0; kx < 3; ++kx) gw[cp][ky * 3 + kx] = ffma2(gj, dup[(j >> 1) + ky][(j & 1) + kx], gw[cp][ky * 3 + kx]);
+        }
+    }
+    next.store(xs[cur ^ 1], tid);
   }
+  __syncthreads();
+  // fixed-order sums: the eight lanes of a quad, then the four warps
+  auto over_lanes = [](float v) {
+#pragma unroll
+    for (int o = 16; o >= 4; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+#pragma unroll
+  for (int cp = 0; cp < 2; ++cp)
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      float lo, hi;
+      unpack2(gw[cp][k], lo, hi);
+      lo = over_lanes(lo);
+      hi = over_lanes(hi);
+      if (lane < 4) {
+        red[warp][(4 * cg + 2 * cp) * 9 + k] = lo;
+        red[warp][(4 * cg + 2 * cp + 1) * 9 + k] = hi;
+      }
+    }
+#pragma unroll
+  for (int ch = 0; ch < 4; ++ch) {
+    const float t = over_lanes(gb[ch]);
+    if (lane < 4) red[warp][144 + 4 * cg + ch] = t;
+  }
+  __syncthreads();
+  float* part = ws.part1 + ((int64_t)s * n_chunks + blockIdx.x) * C1_GRAD;
+  for (int o = tid; o < C1_GRAD; o += CONV1_THREADS) part[o] = (red[0][o] + red[1][o]) + (red[2][o] + red[3][o]);
 }
 
 // ---- sums the per-block partial gradients in a fixed order, finishes the loss and zeroes the padding.
@@ -389,7 +454,7 @@ static int samples_per_block(int rows, int least, int most) {
 static void launch_conv1_fwd(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof) {
   const int spb = samples_per_block(a.W * a.b, 1, CONV1_SPB);
   const int chunks = (a.b + spb - 1) / spb, bank = (gt.n_groups * BANK3_UNITS + chunks - 1) / chunks;
-  TIMED(K_CONV1_FWD, launch_pdl_if(!a.after_wait, conv1_fwd, dim3(chunks, a.W + bank), 224, 0, st, a, wt, gt, ws, spb, conv2_fwd_x3_taps()));
+  TIMED(K_CONV1_FWD, launch_pdl_if(!a.after_wait, conv1_fwd, dim3(chunks, a.W + bank), CONV1_THREADS, 0, st, a, wt, gt, ws, spb, conv2_fwd_x3_taps()));
 }
 
 // Evaluation pass: the forward kernels of the grad step with the dropout switched off, then the per-worker loss and hit
@@ -503,7 +568,7 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     n_chunks2 = launch_conv2_dw_x3(a, ws, s2, prof, &seg_len);
     if (side.s2) cudaEventRecord(side.join2, s2);
     launch_conv2_dx_x3(a, gt, ws, st, prof);
-    TIMED(K_CONV1_BWD, launch_pdl(conv1_bwd, dim3(n_chunks1b, a.W), 256, 0, st, a, wt, ws, spb1b, n_chunks1b));
+    TIMED(K_CONV1_BWD, launch_pdl(conv1_bwd, dim3(n_chunks1b, a.W), CONV1_THREADS, 0, st, a, wt, ws, spb1b, n_chunks1b));
     if (side.s1) cudaStreamWaitEvent(st, side.join1, 0);
     if (side.s2) cudaStreamWaitEvent(st, side.join2, 0);
     if (sum) TIMED(K_CONV_GRAD_REDUCE, (fused_finish<<<dim3(FUSED_W1_BLOCKS + FUSED_SMALL_BLOCKS), 256, 0, st>>>(a, wt, ws, sum->super_part, sum->n_super, sum->grad_sum, n_chunks1b, 0, n_chunks2, seg_len)));

@@ -417,12 +417,15 @@ __global__ void __launch_bounds__(X_THREADS, 1) conv2_dx_x3(GradStepArgs a, Grou
         if (lane == 0) mbar_arrive(&acc_empty[ab]);
         if (++ab == X_ACC) { ab = 0; ab_parity ^= 1; }
         const int r = m * 128 + quarter * 32 + lane, y = r >> 4, x = r & 15;
-        float* out = ws.dp1 + (int64_t)(r_begin + t) * P1_ELEMS + y * 14 + x;
 #pragma unroll
         for (int ic = 0; ic < 16; ++ic) {
           const float right = __shfl_down_sync(0xffffffffu, e[0][ic], 1), left = __shfl_up_sync(0xffffffffu, e[2][ic], 1);
-          const float v = (e[1][ic] + right) + (x == 0 ? 0.f : left);
-          if (y < 14 && x < 14) out[ic * 196] = v;
+          e[1][ic] = (e[1][ic] + right) + (x == 0 ? 0.f : left);
+        }
+        if (y < 14 && x < 14) {              // [channel quad][position][4 channels]
+          float4* out = reinterpret_cast<float4*>(ws.dp1 + (int64_t)(r_begin + t) * P1_ELEMS) + y * 14 + x;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) out[q * 196] = make_float4(e[1][4 * q], e[1][4 * q + 1], e[1][4 * q + 2], e[1][4 * q + 3]);
         }
       }
     }

@@ -121,14 +121,14 @@ struct GroupTable {
 struct Workspace {
   float* p1;       // conv1 -> ReLU -> pool: [rows][2 planes][256][8] BF16 (tensor-core path)
   uint8_t* p1x;    // the same in BF16 pieces: [rows][P1X_BYTES] (FP32 path)
-  uint8_t* code1;  // [rows][3136]        pool-1 decisions. FP32 path: [16][196], argmax 0..3, 4 = no gradient (max <= 0); tensor-core path:
-                   //                     [4 channel quads][196][4], the byte 1 << argmax, 0 = no gradient
+  uint8_t* code1;  // [rows][3136]        pool-1 decisions. [4 channel quads][196][4]; FP32 path: argmax 0..3, 4 = no gradient (max <= 0); tensor-core path:
+                   //                     the byte 1 << argmax, 0 = no gradient
   float* p2;       // [rows][1568]        conv2 -> ReLU -> pool, channel-major flatten (tensor-core path)
   uint8_t* code2;  // [rows][1568]        [8 channel quads][49][4], argmax 0..3, 4 = no gradient
   float* d;        // [rows][512]         fc1 -> ReLU -> dropout (scaled)
   float* da1;      // [rows][512]         gradient w.r.t. fc1 pre-activation (tensor-core path)
   float* dp2;      // [rows][1568]        gradient w.r.t. p2 (tensor-core path: BF16 in the first half of each row)
-  float* dp1;      // [rows][3136]        gradient w.r.t. p1; [16][196] fp32 (FP32 path) or [4 channel quads][196][4] BF16 in the first half of the row (tensor-core path)
+  float* dp1;      // [rows][3136]        gradient w.r.t. p1, [4 channel quads][196][4]: fp32 (FP32 path) or BF16 in the first half of the row (tensor-core path)
   float* part2;    // [W][chunks][4640]   per-block partial conv2 weight/bias gradients
   float* part1;    // [W][chunks][160]    per-block partial conv1 weight/bias gradients
   float* partf;    // [W][fc2_split][FC_PART] per-block partial output-layer gradients and loss sums

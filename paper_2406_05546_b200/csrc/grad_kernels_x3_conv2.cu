@@ -21,8 +21,8 @@
 //
 // Measured (B200; 29.6 GFLOP per product at 128 workers x 128 samples, six times that on the tensor cores: 112 us at the measured
 // BF16 rate; ~6 us of event overhead included; before: packed FP32 multiply-adds at two thirds of their pipe's rate): forward 696 ->
-// 202, input gradient 636 -> 181, filter gradient 651 -> 302 us; at 16 x 64: 56 -> 25, 57 -> 22, 56 -> 35; at 2 x 8: 12 -> 13, 15 -> 11,
-// 15 -> 15.  Forward and input gradient are bound by the instructions' own time; the filter gradient takes 1.5 times as many products as
+// 200, input gradient 636 -> 178, filter gradient 651 -> 266 us; at 16 x 64: 56 -> 25, 57 -> 21, 56 -> 31; at 2 x 8: 12 -> 13, 15 -> 11,
+// 15 -> 14.  Forward and input gradient are bound by the instructions' own time; the filter gradient takes 1.5 times as many products as
 // it needs, rounded up to 128 rows.  Relative error against float64, median over workers, 128 x 128: conv2.w 1.6e-7 -> 1.0e-7, conv1.w
 // 1.2e-7 -> 0.9e-7; 2 x 8: 3.2e-7 -> 1.7e-7, 3.6e-7 -> 2.1e-7.
 //
@@ -50,10 +50,6 @@ __device__ __forceinline__ void tmem_alloc_all(uint32_t* slot) {
 }
 __device__ __forceinline__ void tmem_free_all(uint32_t tmem) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_ALL) : "memory");
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr));
 }
 __device__ __forceinline__ void report_abort(uint32_t* status) {
   atomicOr(status, STATUS_WAIT_TIMEOUT);
@@ -443,12 +439,12 @@ __global__ void __launch_bounds__(X_THREADS, 1) conv2_dx_x3(GradStepArgs a, Grou
 // for a filter row's three taps, 42 a sample (14 per filter column kx, which has an accumulator of its own), with nothing to
 // stage but g2: p1x is used as it arrives.  A sample's sums (14 instructions' worth) are added up in registers, the leading ones with
 // the products of h and the others' pieces; the warps of the three pieces of g2 meet only when a sum is written out.
-// Warps: 0 = MMA, 1 = copies of p1x, 2 = copies of dp2 and decisions, then staging, then twelve for the read-out (tensor-memory
-// quarter = piece, filter column = group of four); the fourth quarter's three warps sum the bias gradient.  A CTA walks over a
-// contiguous range of rows and writes a partial sum every seg_len rows and where the range leaves a worker.
+// Warps: 0 = MMA, 1 = copies of p1x, 2 = copies of dp2 and decisions, 3, 7, 11, 15 = staging (3 also sums the bias gradient), the others =
+// read-out (tensor-memory quarter = piece, group of four warps = filter column).  A read-out takes a round trip of 425 clk to tensor memory
+// per load, so it has as many registers as sixteen warps leave: three trips instead of six.  A CTA walks over a contiguous range of
+// rows and writes a partial sum every seg_len rows and where the range leaves a worker.
 // ------------------------------------------------------------------------------------------------
-constexpr int D_STAGE_GROUPS = 1;                            // of four staging warps, on samples in turn (two: 310 instead of 302 us at 128 x 128, registers run short)
-constexpr int D_READ_WARP = 4 + 4 * D_STAGE_GROUPS, D_THREADS = 32 * (D_READ_WARP + 12), D_P1_SLOTS = 3, D_RAW_SLOTS = 4;
+constexpr int D_THREADS = 512, D_READERS = 288, D_P1_SLOTS = 3, D_RAW_SLOTS = 4;
 constexpr int D_G_ROW = PIECES * 4 * 256;                    // image row of g2: [piece][octet][slot (x & 1) * 8 + x / 2][8 channels]
 constexpr int D_G_BYTES = 14 * D_G_ROW + 1024;               // the dropped rows of the last image row read a kilobyte behind it
 constexpr int D_GAP = 128;
@@ -456,7 +452,7 @@ constexpr int D_XCHG_BYTES = 3 * 2 * 48 * 32 * 4;            // read-out: [kx][p
 constexpr int D_OUT_PITCH = 145;                             // write-out: an output channel's 144 filter taps, one word of padding
 static_assert(32 * D_OUT_PITCH * 4 <= D_XCHG_BYTES, "the taps take the exchange area's place");
 constexpr int D_BARS = 2 * D_P1_SLOTS + 2 * D_RAW_SLOTS + 2 * 2 + 2 * 3;
-constexpr int D_SMEM = 2 * D_G_BYTES + D_P1_SLOTS * P1X_BYTES + D_GAP + D_XCHG_BYTES + D_RAW_SLOTS * RAW_BYTES + 3 * 32 * 4 + D_BARS * 8 + 16;
+constexpr int D_SMEM = 2 * D_G_BYTES + D_P1_SLOTS * P1X_BYTES + D_GAP + D_XCHG_BYTES + D_RAW_SLOTS * RAW_BYTES + D_BARS * 8 + 16;
 static_assert(D_SMEM <= 227 * 1024 && D_G_BYTES % 16 == 0, "shared memory");
 
 __global__ void __launch_bounds__(D_THREADS, 1) conv2_dw_x3(GradStepArgs a, Workspace ws, int segs, int seg_len, int slots) {
@@ -464,8 +460,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) conv2_dw_x3(GradStepArgs a, Work
   uint8_t* p1s = smem + 2 * D_G_BYTES;
   float* xchg = reinterpret_cast<float*>(p1s + D_P1_SLOTS * P1X_BYTES + D_GAP);
   uint8_t* raw = reinterpret_cast<uint8_t*>(xchg) + D_XCHG_BYTES;
-  float* bias_x = reinterpret_cast<float*>(raw + D_RAW_SLOTS * RAW_BYTES);
-  uint64_t* p1_full = reinterpret_cast<uint64_t*>(bias_x + 96);
+  uint64_t* p1_full = reinterpret_cast<uint64_t*>(raw + D_RAW_SLOTS * RAW_BYTES);
   uint64_t* p1_empty = p1_full + D_P1_SLOTS;
   uint64_t* raw_full = p1_empty + D_P1_SLOTS;
   uint64_t* raw_empty = raw_full + D_RAW_SLOTS;
@@ -487,7 +482,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) conv2_dw_x3(GradStepArgs a, Work
   if (tid <= D_P1_SLOTS) *reinterpret_cast<uint4*>(p1s + tid * P1X_BYTES) = make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) {
     for (int i = 0; i < D_P1_SLOTS; ++i) { mbar_init(&p1_full[i], 1); mbar_init(&p1_empty[i], 1); }
-    for (int i = 0; i < D_RAW_SLOTS; ++i) { mbar_init(&raw_full[i], 1); mbar_init(&raw_empty[i], 4 + 3); }
+    for (int i = 0; i < D_RAW_SLOTS; ++i) { mbar_init(&raw_full[i], 1); mbar_init(&raw_empty[i], 4); }
     for (int i = 0; i < 2; ++i) { mbar_init(&g_full[i], 4); mbar_init(&g_empty[i], 1); }
     for (int i = 0; i < 3; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 3); }
     *abort_flag = 0;
@@ -551,10 +546,12 @@ __global__ void __launch_bounds__(D_THREADS, 1) conv2_dw_x3(GradStepArgs a, Work
         bulk_load(raw + slot * RAW_BYTES + FLAT * 4, ws.code2 + row * FLAT, FLAT, &raw_full[slot]);
       }
     }
-  } else if (warp >= 4 && warp < D_READ_WARP) {
-    const int lt = tid & 127;
-    for (int n = (warp - 4) >> 2; n < n_samples; n += D_STAGE_GROUPS) {
-      const int st = n & 1, slot = n % D_RAW_SLOTS;
+  } else if ((warp & 3) == 3) {
+    const int lt = (warp >> 2) * 32 + lane;
+    int s = r0 / a.b, wend = (s + 1) * a.b, seg = blockIdx.x * segs, send = r0 + seg_len;
+    float gb = 0.f;                          // bias gradient; lane = output channel
+    for (int n = 0; n < n_samples; ++n) {
+      const int st = n & 1, slot = n % D_RAW_SLOTS, row = r0 + n;
       bool ok = mbar_wait(&raw_full[slot], (n / D_RAW_SLOTS) & 1);
       if (ok && n >= 2) ok = mbar_wait(&g_empty[st], ((n >> 1) - 1) & 1);
       if (!__all_sync(0xffffffffu, ok && !*abort_flag)) { *abort_flag = 1; break; }
@@ -567,92 +564,83 @@ __global__ void __launch_bounds__(D_THREADS, 1) conv2_dw_x3(GradStepArgs a, Work
       }
       fence_proxy_async_smem();
       __syncwarp();
-      if (lane == 0) { mbar_arrive(&g_full[st]); mbar_arrive(&raw_empty[slot]); }
+      if (lane == 0) mbar_arrive(&g_full[st]);
+      if (warp == 3) {
+        const float* g = reinterpret_cast<const float*>(rp) + lane * 49;
+        const uint8_t* code = rp + FLAT * 4 + (lane >> 2) * 196 + (lane & 3);
+        float t[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int p = 0; p < 49; ++p) t[p % 7] += code[p * 4] < 4 ? g[p] : 0.f;
+        gb += ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + t[6]);
+        if (row + 1 == r1 || row + 1 == wend || row + 1 == send) {
+          ws.part2[((int64_t)s * slots + (seg - (s * a.b) / seg_len)) * C2_GRAD + 4608 + lane] = gb;
+          gb = 0.f;
+          if (row + 1 == wend) { ++s; wend += a.b; }
+          if (row + 1 == send) { ++seg; send += seg_len; }
+        }
+        __syncwarp();
+      }
+      if (lane == 0) mbar_arrive(&raw_empty[slot]);
     }
-  } else if (warp >= D_READ_WARP) {
-    const int piece = warp & 3, kx = (warp - D_READ_WARP) >> 2;
+  } else {
+    const int piece = warp & 3, kx = (warp >> 2) - 1;
     int s = r0 / a.b, wend = (s + 1) * a.b, seg = blockIdx.x * segs, send = r0 + seg_len;
     float sum[48];                           // (ky, input channel); lane = output channel
-    float gb = 0.f;
 #pragma unroll
     for (int i = 0; i < 48; ++i) sum[i] = 0.f;
     bool ok = true;
     for (int n = 0; n < n_samples; ++n) {
       const int row = r0 + n;
-      if (piece < PIECES) {
-        ok = ok && warp_wait(&acc_full[kx], n & 1, abort_flag);
-        if (ok) {
-          tc_fence_after();
-          const uint32_t at = tmem + ((uint32_t)(piece * 32) << 16) + (uint32_t)(kx * 144);
+      ok = ok && warp_wait(&acc_full[kx], n & 1, abort_flag);
+      if (ok) {
+        tc_fence_after();
+        const uint32_t at = tmem + ((uint32_t)(piece * 32) << 16) + (uint32_t)(kx * 144);
 #pragma unroll
-          for (int c = 0; c < 6; ++c) {      // eight input channels of filter row c / 2
-            uint32_t h[8], m[8], l[8];
-            const uint32_t ac = at + (c >> 1) * 48 + (c & 1) * 8;
-            tmem_ld8(ac, h);
-            if (piece < 2) tmem_ld8(ac + 16, m);
-            if (piece < 1) tmem_ld8(ac + 32, l);
-            tmem_ld_wait();
+        for (int ky = 0; ky < 3; ++ky) {
+          uint32_t h[16], m[16], l[16];
+          tmem_ld16(at + ky * 48, h);
+          if (piece < 2) tmem_ld16(at + ky * 48 + 16, m);
+          if (piece < 1) tmem_ld16(at + ky * 48 + 32, l);
+          tmem_ld_wait();
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const float v = piece == 0 ? join3(__uint_as_float(h[i]), __uint_as_float(m[i]) + __uint_as_float(l[i]))
-                                         : (piece == 1 ? __uint_as_float(h[i]) + __uint_as_float(m[i]) : __uint_as_float(h[i]));
-              sum[c * 8 + i] += v;
-            }
+          for (int i = 0; i < 16; ++i) {
+            const float v = piece == 0 ? join3(__uint_as_float(h[i]), __uint_as_float(m[i]) + __uint_as_float(l[i]))
+                                       : (piece == 1 ? __uint_as_float(h[i]) + __uint_as_float(m[i]) : __uint_as_float(h[i]));
+            sum[ky * 16 + i] += v;
           }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&acc_empty[kx]);
         }
-      } else {                               // bias: lane = output channel, positions kx, kx + 3, ...
-        const int slot = n % D_RAW_SLOTS;
-        ok = ok && warp_wait(&raw_full[slot], (n / D_RAW_SLOTS) & 1, abort_flag);
-        if (ok) {
-          const float* g = reinterpret_cast<const float*>(raw + slot * RAW_BYTES) + lane * 49;
-          const uint8_t* code = raw + slot * RAW_BYTES + FLAT * 4 + (lane >> 2) * 196 + (lane & 3);
-          float t[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-          for (int k = 0; k < 17; ++k) {
-            const int p = kx + 3 * k;
-            if (p < 49 && code[p * 4] < 4) t[k & 3] += g[p];
-          }
-          gb += (t[0] + t[1]) + (t[2] + t[3]);
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&raw_empty[slot]);
-        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acc_empty[kx]);
       }
-      if (!ok) *abort_flag = 1;              // and on to the write-out, where all twelve warps stop
+      if (!ok) *abort_flag = 1;              // and on to the write-out, where all nine warps stop
       if (row + 1 == r1 || row + 1 == wend || row + 1 == send) {
-        // the twelve warps meet: the pieces' sums of a filter column, then the three thirds of the bias gradient
+        // the nine warps meet: the pieces' sums of a filter column, then all columns' taps in the order of the output
         float* x = xchg + kx * (2 * 48 * 32);
-        if (piece == 1 || piece == 2) {
+        if (piece > 0) {
 #pragma unroll
           for (int i = 0; i < 48; ++i) x[((piece - 1) * 48 + i) * 32 + lane] = sum[i];
-        } else if (piece == 3) {
-          bias_x[kx * 32 + lane] = gb;
         }
-        if (!warps_agree<1, 384>(ok)) break;
-        float* part = ws.part2 + ((int64_t)s * slots + (seg - (s * a.b) / seg_len)) * C2_GRAD;
+        if (!warps_agree<1, D_READERS>(ok)) break;
         if (piece == 0) {
 #pragma unroll
           for (int i = 0; i < 48; ++i) sum[i] = join3(sum[i], x[i * 32 + lane] + x[(48 + i) * 32 + lane]);
-        } else if (piece == 3 && kx == 0) {
-          part[4608 + lane] = (bias_x[lane] + bias_x[32 + lane]) + bias_x[64 + lane];
         }
-        asm volatile("bar.sync 1, 384;" ::: "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(D_READERS) : "memory");
         if (piece == 0) {
 #pragma unroll
           for (int i = 0; i < 48; ++i) xchg[lane * D_OUT_PITCH + (i & 15) * 9 + (i >> 4) * 3 + kx] = sum[i];
         }
-        asm volatile("bar.sync 1, 384;" ::: "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(D_READERS) : "memory");
+        float* part = ws.part2 + ((int64_t)s * slots + (seg - (s * a.b) / seg_len)) * C2_GRAD;
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
-          const int i = k * 384 + (tid - 32 * D_READ_WARP);
+        for (int k = 0; k < 4608 / D_READERS; ++k) {
+          const int i = k * D_READERS + (kx * 3 + piece) * 32 + lane;
           part[i] = xchg[i + i / 144];                       // D_OUT_PITCH = 144 + 1
         }
-        asm volatile("bar.sync 1, 384;" ::: "memory");       // and has been read before the next write-out
+        asm volatile("bar.sync 1, %0;" ::"n"(D_READERS) : "memory");       // and has been read before the next write-out
 #pragma unroll
         for (int i = 0; i < 48; ++i) sum[i] = 0.f;
-        gb = 0.f;
         if (row + 1 == wend) { ++s; wend += a.b; }
         if (row + 1 == send) { ++seg; send += seg_len; }
       }

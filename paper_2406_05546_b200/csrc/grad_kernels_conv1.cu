@@ -25,12 +25,6 @@ namespace psk {
 
 namespace {
 
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float r;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-
 constexpr int C1_SPS = 1;                                // samples per step
 constexpr int C1_THREADS = 112 * C1_SPS;
 constexpr int C1_BLOCKS_PER_SM = 6 / C1_SPS;
@@ -69,6 +63,9 @@ __device__ __forceinline__ void build_bank2(const float* __restrict__ theta, uin
 // (one sample per step, six blocks per SM) keep the blocks' phases apart: the barrier of a step lines up the
 // multiply-add phases of all warps of a block, and with few large blocks the FMA pipe idles while all of them
 // pool and store.
+// EVAL: an evaluation, where nobody reads the pooling decisions; without finding and writing them in the two convolutions a pass over 80 x
+// 125 samples takes 140 instead of 160 us.
+template <bool EVAL>
 __global__ void __launch_bounds__(C1_THREADS, C1_BLOCKS_PER_SM) conv1_fwd_planes(const __grid_constant__ CUtensorMap xmap, GradStepArgs a,
                                                                   WorkerTable wt, GroupTable gt, Workspace ws, int spb, const __grid_constant__ Bank2Taps taps) {
   extern __shared__ __align__(128) uint8_t sm[];
@@ -169,7 +166,7 @@ __global__ void __launch_bounds__(C1_THREADS, C1_BLOCKS_PER_SM) conv1_fwd_planes
       const int row = (py + 1) * 16 + col_row, pos = py * 14 + px;
       *reinterpret_cast<uint2*>(ob + sp * C1_PLANES_BYTES + (cg >> 1) * (C1_PLANES_BYTES / 2) + row * 16 + (cg & 1) * 8) =
           make_uint2(bf16_pair(best[0], best[1]), bf16_pair(best[2], best[3]));
-      *reinterpret_cast<uint32_t*>(ob + C1_SPS * C1_PLANES_BYTES + sp * P1_ELEMS + cg * 784 + pos * 4) = codes;
+      if (!EVAL) *reinterpret_cast<uint32_t*>(ob + C1_SPS * C1_PLANES_BYTES + sp * P1_ELEMS + cg * 784 + pos * 4) = codes;
     }
     fence_proxy_async_smem();
     if (tid == 0) bulk_wait_read0();      // the previous step's copies have read their buffer, which the next step overwrites
@@ -177,7 +174,7 @@ __global__ void __launch_bounds__(C1_THREADS, C1_BLOCKS_PER_SM) conv1_fwd_planes
     if (tid == 0) {
       const int64_t row0 = (int64_t)s * a.b + i0 + C1_SPS * st;
       bulk_store(reinterpret_cast<uint8_t*>(ws.p1) + row0 * C1_PLANES_BYTES, ob, n_s * C1_PLANES_BYTES);
-      bulk_store(ws.code1 + row0 * P1_ELEMS, ob + C1_SPS * C1_PLANES_BYTES, n_s * P1_ELEMS);
+      if (!EVAL) bulk_store(ws.code1 + row0 * P1_ELEMS, ob + C1_SPS * C1_PLANES_BYTES, n_s * P1_ELEMS);
       bulk_commit();
       if (st + C1_STAGES < n_steps) issue(st + C1_STAGES);
     }
@@ -191,11 +188,11 @@ __global__ void __launch_bounds__(C1_THREADS, C1_BLOCKS_PER_SM) conv1_fwd_planes
 #define TIMED(id, launch) do { if (prof) prof->begin(id, st); launch; if (prof) prof->end(st); } while (0)
 
 int configure_conv1_kernels() {
-  return allow_smem((const void*)(conv1_fwd_planes), C1_SMEM) == cudaSuccess ? 0 : -1;
+  return allow_smem((const void*)(conv1_fwd_planes<false>), C1_SMEM) == cudaSuccess && allow_smem((const void*)(conv1_fwd_planes<true>), C1_SMEM) == cudaSuccess ? 0 : -1;
 }
 
 // The caller's images [W*b][28][28] as a 3-d tensor; a.x must be 16-byte aligned.  Returns 1 (kernels launched) or -1.
-int launch_conv1_fwd_planes(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
+int launch_conv1_fwd_planes(bool eval, const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                             cudaStream_t st, Profiler* prof) {
   CUtensorMap xmap;
   const uint64_t dims[3] = {IMG, IMG, (uint64_t)a.W * a.b};
@@ -208,7 +205,7 @@ int launch_conv1_fwd_planes(const GradStepArgs& a, const WorkerTable& wt, const 
   const int slots = C1_BLOCKS_PER_SM * g_sm_count, rows = a.W * a.b;
   const int spb = rows <= slots ? 1 : (rows <= 2 * slots ? 2 : C1_SPB);
   const int chunks = (a.b + spb - 1) / spb;
-  TIMED(K_CONV1_FWD, launch_pdl_if(!a.after_wait, conv1_fwd_planes, dim3(chunks, a.W + (gt.n_groups * BANK2_UNITS + chunks - 1) / chunks), C1_THREADS, C1_SMEM, st, xmap, a, wt, gt, ws, spb, conv2_fwd_taps()));
+  TIMED(K_CONV1_FWD, launch_pdl_if(!a.after_wait, eval ? conv1_fwd_planes<true> : conv1_fwd_planes<false>, dim3(chunks, a.W + (gt.n_groups * BANK2_UNITS + chunks - 1) / chunks), C1_THREADS, C1_SMEM, st, xmap, a, wt, gt, ws, spb, conv2_fwd_taps()));
   return 1;
 }
 

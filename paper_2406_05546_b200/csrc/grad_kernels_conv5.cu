@@ -134,6 +134,7 @@ const FoldTables& fold_tables() {
   return t;
 }
 
+template <bool EVAL>      // an evaluation: nobody reads the pooling decisions
 __global__ void __launch_bounds__(F_THREADS, 2) conv2_fwd_tc5(GradStepArgs a, GroupTable gt, Workspace ws, int range_len, const __grid_constant__ FoldTable fold) {
   extern __shared__ __align__(128) uint8_t smem[];
   uint16_t* Wk = reinterpret_cast<uint16_t*>(smem + F_NBUF * F_BUF_BYTES);
@@ -236,16 +237,23 @@ __global__ void __launch_bounds__(F_THREADS, 2) conv2_fwd_tc5(GradStepArgs a, Gr
         for (int o = 0; o < 16; ++o) {
           const int oc = ch * 16 + o;
           const float v0 = __uint_as_float(v[0][o]), v1 = __uint_as_float(v[1][o]), v2 = __uint_as_float(v[2][o]), v3 = __uint_as_float(v[3][o]);
-          const float m = fmaxf(fmaxf(v0, v1), fmaxf(v2, v3));
-          const uint32_t bi = v0 == m ? 0u : (v1 == m ? 1u : (v2 == m ? 2u : 3u));
+          const float m = fmaxf(max3(v0, v1, v2), v3);
           const float best = fmaxf(m + bias[oc], 0.f);
           ws.p2[row * FLAT + oc * 49 + pp] = round_tf32(best);   // its only readers are TF32 products
-          codes[o >> 2] |= (best > 0.f ? bi : 4u) << (8 * (o & 3));
+          if (!EVAL) {
+            const int at = 8 * (o & 3);
+            uint32_t e = v2 == m ? 2u << at : 3u << at;
+            e = v1 == m ? 1u << at : e;
+            e = v0 == m ? 0u : e;
+            codes[o >> 2] |= best > 0.f ? e : 4u << at;
+          }
         }
         // decisions as [channel quad][position][4 channels] bytes
-        uint32_t* c2 = reinterpret_cast<uint32_t*>(ws.code2 + row * FLAT);
+        if (!EVAL) {
+          uint32_t* c2 = reinterpret_cast<uint32_t*>(ws.code2 + row * FLAT);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) c2[(ch * 4 + q) * 49 + pp] = codes[q];
+          for (int q = 0; q < 4; ++q) c2[(ch * 4 + q) * 49 + pp] = codes[q];
+        }
       }
     }
   }
@@ -450,19 +458,20 @@ __global__ void __launch_bounds__(THREADS, 2) conv2_dx_tc5(GradStepArgs a, Group
 #define TIMED(id, launch) do { if (prof) prof->begin(id, st); launch; if (prof) prof->end(st); } while (0)
 
 int configure_conv5_kernels() {
-  cudaError_t e = allow_smem((const void*)(conv2_fwd_tc5), F_SMEM);
+  cudaError_t e = allow_smem((const void*)(conv2_fwd_tc5<false>), F_SMEM);
+  if (e == cudaSuccess) e = allow_smem((const void*)(conv2_fwd_tc5<true>), F_SMEM);
   if (e == cudaSuccess) e = allow_smem((const void*)(conv2_dx_tc5), X_SMEM);
   return e == cudaSuccess ? 0 : -1;
 }
 
 const Bank2Taps& conv2_fwd_taps() { return fold_tables().taps; }
 
-void launch_conv2_fwd_tc5(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
+void launch_conv2_fwd_tc5(bool eval, const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                           cudaStream_t st, Profiler* prof) {
   const FoldTable& fold = fold_tables().fold;
   int len;
   const int n = plan_row_ranges(gt, a.b, 2 * g_sm_count, 2, &len);      // two CTAs per SM, tiles of two samples
-  TIMED(K_CONV2_FWD, launch_pdl(conv2_fwd_tc5, dim3(n), F_THREADS, F_SMEM, st, a, gt, ws, len, fold));
+  TIMED(K_CONV2_FWD, launch_pdl(eval ? conv2_fwd_tc5<true> : conv2_fwd_tc5<false>, dim3(n), F_THREADS, F_SMEM, st, a, gt, ws, len, fold));
 }
 
 void launch_conv2_dx_tc5(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,

@@ -464,8 +464,8 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
   int launches = 0;
   if (a.precision != 0) {
     if (!a.skip_prep_w1) launches += launch_prep_w1(gt, ws, st, prof);
-    if (launch_conv1_fwd_planes(a, wt, gt, ws, st, prof) < 0) return -1;
-    launch_conv2_fwd_tc5(a, wt, gt, ws, st, prof);
+    if (launch_conv1_fwd_planes(true, a, wt, gt, ws, st, prof) < 0) return -1;
+    launch_conv2_fwd_tc5(true, a, wt, gt, ws, st, prof);
     const int n = launch_fc1_fwd_tc5(a, wt, gt, ws, st, prof);
     if (n < 0) return -1;
     launches += 2 + n;
@@ -521,8 +521,8 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
       launches += launch_prep_w1(gt, ws, s1, prof);
       if (side.s1) cudaEventRecord(side.join1, s1);
     }
-    if (launch_conv1_fwd_planes(a, wt, gt, ws, st, prof) < 0) return -1;
-    launch_conv2_fwd_tc5(a, wt, gt, ws, st, prof);
+    if (launch_conv1_fwd_planes(false, a, wt, gt, ws, st, prof) < 0) return -1;
+    launch_conv2_fwd_tc5(false, a, wt, gt, ws, st, prof);
     if (!a.skip_prep_w1 && side.s1) cudaStreamWaitEvent(st, side.join1, 0);
     int n = launch_fc1_fwd_tc5(a, wt, gt, ws, st, prof, side.s1 && !a.skip_prep_w1);
     if (n < 0) return -1;

@@ -204,10 +204,10 @@ int launch_conv1_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const Work
                         int* seg_len);
 int launch_conv2_dw_tc5(const GradStepArgs& a, const WorkerTable& wt, const Workspace& ws, cudaStream_t st, Profiler* prof,
                         int* seg_len, bool in_line);
-int launch_conv1_fwd_planes(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
+int launch_conv1_fwd_planes(bool eval, const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                             cudaStream_t st, Profiler* prof);
 const Bank2Taps& conv2_fwd_taps();
-void launch_conv2_fwd_tc5(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
+void launch_conv2_fwd_tc5(bool eval, const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                           cudaStream_t st, Profiler* prof);
 void launch_conv2_dx_tc5(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws,
                          cudaStream_t st, Profiler* prof);

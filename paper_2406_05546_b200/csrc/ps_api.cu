@@ -304,10 +304,16 @@ int32_t ps_create(const ps_config* cfg, const float* init_params_host, ps_ctx** 
   for (auto& r : x->replicas)
     if (e == cudaSuccess) e = cudaMemcpyAsync(r.buf, x->io_stage, VEC_BYTES, cudaMemcpyHostToDevice, x->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->status_dev, 0, ALIGN, x->st);
-  // the zero borders of the first convolution's output are written once, here
+  // the zero borders of the first convolution's output are written once, here; on the FP32 path the first and the last image row (a
+  // sample's last and the next one's first lie together), the others' ends are written with them
   const uint64_t rows = (uint64_t)cfg->max_workers * cfg->max_batch;
-  if (e == cudaSuccess)
-    e = cfg->precision != PS_FP32 ? cudaMemsetAsync(x->ws.p1, 0, rows * psk::P1_PLANE_ELEMS * 4, x->st) : cudaMemsetAsync(x->ws.p1x, 0, rows * psk::P1X_BYTES, x->st);
+  if (e == cudaSuccess && cfg->precision != PS_FP32) e = cudaMemsetAsync(x->ws.p1, 0, rows * psk::P1_PLANE_ELEMS * 4, x->st);
+  if (e == cudaSuccess && cfg->precision == PS_FP32) {
+    uint8_t* last = x->ws.p1x + 15 * psk::P1X_ROW;
+    e = cudaMemsetAsync(x->ws.p1x, 0, psk::P1X_ROW, x->st);
+    if (e == cudaSuccess && rows > 1) e = cudaMemset2DAsync(last, psk::P1X_BYTES, 0, 2 * psk::P1X_ROW, rows - 1, x->st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(last + (rows - 1) * psk::P1X_BYTES, 0, psk::P1X_ROW, x->st);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(x->st);
   if (e != cudaSuccess) { delete x; return cuda_fail(e, "ps_create upload"); }
   *out = x;

@@ -21,7 +21,7 @@
 //
 // Measured (B200; 29.6 GFLOP per product at 128 workers x 128 samples, six times that on the tensor cores: 112 us at the measured
 // BF16 rate; ~6 us of event overhead included; before: packed FP32 multiply-adds at two thirds of their pipe's rate): forward 696 ->
-// 200, input gradient 636 -> 178, filter gradient 651 -> 266 us; at 16 x 64: 56 -> 25, 57 -> 21, 56 -> 31; at 2 x 8: 12 -> 13, 15 -> 11,
+// 200, input gradient 636 -> 176, filter gradient 651 -> 266 us; at 16 x 64: 56 -> 25, 57 -> 21, 56 -> 31; at 2 x 8: 12 -> 13, 15 -> 11,
 // 15 -> 14.  Forward and input gradient are bound by the instructions' own time; the filter gradient takes 1.5 times as many products as
 // it needs, rounded up to 128 rows.  Relative error against float64, median over workers, 128 x 128: conv2.w 1.6e-7 -> 1.0e-7, conv1.w
 // 1.2e-7 -> 0.9e-7; 2 x 8: 3.2e-7 -> 1.7e-7, 3.6e-7 -> 2.1e-7.
@@ -278,10 +278,11 @@ __device__ __forceinline__ void place_g2(const uint8_t* raw, int o8, int p, Stor
 // 48 accumulator columns, and the pieces of the filters next to one another: g's h takes the filters' h, m, l (N = 144), its m h
 // and m (N = 96, one range to the right), its l h (N = 48, two to the right): the first range holds the leading products, the
 // other two the small ones.  36 MMAs a sample instead of 72; an MMA of M = 128, K = 16 takes 40 clk or N / 2, whichever is more.
-// The epilogue adds a filter row's columns with lane shifts.
-// Warps: 0 = MMA, 1..8 = staging (two groups on alternate samples), 9..12 = epilogue, 13 = copies.
+// The epilogue adds a filter row's columns with lane shifts; with one group of four warps for both blocks it takes 178 instead of 176 us at
+// 128 x 128.
+// Warps: 0 = MMA, 1..8 = staging (two groups on alternate samples), 9..16 = epilogue (a group of four for either block of rows), 17 = copies.
 // ------------------------------------------------------------------------------------------------
-constexpr int X_THREADS = 448, X_RAW_SLOTS = 8, X_ACC = 3;
+constexpr int X_THREADS = 576, X_RAW_SLOTS = 8, X_ACC = 3;
 constexpr int X_PLANE_BYTES = (256 + 51) * 16;             // 34 rows of tap overrun; a pitch of 3 rows mod 8 spreads the staging stores over the banks
 constexpr int X_PIECE_BYTES = 4 * X_PLANE_BYTES, X_BUF_BYTES = PIECES * X_PIECE_BYTES;
 constexpr int X_BARS = 2 * 2 + 2 * X_ACC + 2 * X_RAW_SLOTS + 1;
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__(X_THREADS, 1) conv2_dx_x3(GradStepArgs a, Grou
       __syncwarp();
       if (lane == 0) { mbar_arrive(&a_full[buf]); mbar_arrive(&raw_empty[slot]); }
     }
-  } else if (warp == 13) {
+  } else if (warp == 17) {
     if (lane == 0) {
       mbar_expect_tx(w_full, BANK3_DX_BYTES);
       bulk_load(Wk, ws.bank2 + (int64_t)grp * BANK3_BYTES + BANK3_FWD_BYTES, BANK3_DX_BYTES, w_full);
@@ -384,45 +385,42 @@ __global__ void __launch_bounds__(X_THREADS, 1) conv2_dx_x3(GradStepArgs a, Grou
       }
     }
   } else {
-    const int quarter = warp & 3;
-    int ab = 0;
+    const int quarter = warp & 3, m = (warp - 9) >> 2;
+    int ab = m;
     uint32_t ab_parity = 0;
-    bool ok = true;
-    for (int t = 0; ok && t < n_tiles; ++t) {
-#pragma unroll 1
-      for (int m = 0; m < 2; ++m) {
-        if (!warp_wait(&acc_full[ab], ab_parity, abort_flag)) { *abort_flag = 1; ok = false; break; }
-        tc_fence_after();
-        // the thread's position holds, per filter column kx, what the gradient AT this position sends through the taps of that
-        // column; the input gradient here collects kx = 0 from the position to the right, kx = 1 from itself and kx = 2 from
-        // the position to the left (zero borders make the rows' ends right)
-        float e[3][16];
+    for (int t = 0; t < n_tiles; ++t) {
+      if (!warp_wait(&acc_full[ab], ab_parity, abort_flag)) { *abort_flag = 1; break; }
+      tc_fence_after();
+      // the thread's position holds, per filter column kx, what the gradient AT this position sends through the taps of that
+      // column; the input gradient here collects kx = 0 from the position to the right, kx = 1 from itself and kx = 2 from
+      // the position to the left (zero borders make the rows' ends right)
+      float e[3][16];
 #pragma unroll
-        for (int kx = 0; kx < 3; ++kx) {
-          uint32_t lead[16], s1[16], s2[16];
-          const uint32_t at = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ab * 144 + kx * 16);
-          tmem_ld16(at, lead);
-          tmem_ld16(at + 48, s1);
-          tmem_ld16(at + 96, s2);
-          tmem_ld_wait();
+      for (int kx = 0; kx < 3; ++kx) {
+        uint32_t lead[16], s1[16], s2[16];
+        const uint32_t at = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ab * 144 + kx * 16);
+        tmem_ld16(at, lead);
+        tmem_ld16(at + 48, s1);
+        tmem_ld16(at + 96, s2);
+        tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 16; ++i) e[kx][i] = join3(__uint_as_float(lead[i]), __uint_as_float(s1[i]) + __uint_as_float(s2[i]));
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[ab]);
-        if (++ab == X_ACC) { ab = 0; ab_parity ^= 1; }
-        const int r = m * 128 + quarter * 32 + lane, y = r >> 4, x = r & 15;
+        for (int i = 0; i < 16; ++i) e[kx][i] = join3(__uint_as_float(lead[i]), __uint_as_float(s1[i]) + __uint_as_float(s2[i]));
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acc_empty[ab]);
+      ab += 2;                             // every second use of the accumulators is this group's
+      if (ab >= X_ACC) { ab -= X_ACC; ab_parity ^= 1; }
+      const int r = m * 128 + quarter * 32 + lane, y = r >> 4, x = r & 15;
 #pragma unroll
-        for (int ic = 0; ic < 16; ++ic) {
-          const float right = __shfl_down_sync(0xffffffffu, e[0][ic], 1), left = __shfl_up_sync(0xffffffffu, e[2][ic], 1);
-          e[1][ic] = (e[1][ic] + right) + (x == 0 ? 0.f : left);
-        }
-        if (y < 14 && x < 14) {              // [channel quad][position][4 channels]
-          float4* out = reinterpret_cast<float4*>(ws.dp1 + (int64_t)(r_begin + t) * P1_ELEMS) + y * 14 + x;
+      for (int ic = 0; ic < 16; ++ic) {
+        const float right = __shfl_down_sync(0xffffffffu, e[0][ic], 1), left = __shfl_up_sync(0xffffffffu, e[2][ic], 1);
+        e[1][ic] = (e[1][ic] + right) + (x == 0 ? 0.f : left);
+      }
+      if (y < 14 && x < 14) {              // [channel quad][position][4 channels]
+        float4* out = reinterpret_cast<float4*>(ws.dp1 + (int64_t)(r_begin + t) * P1_ELEMS) + y * 14 + x;
 #pragma unroll
-          for (int q = 0; q < 4; ++q) out[q * 196] = make_float4(e[1][4 * q], e[1][4 * q + 1], e[1][4 * q + 2], e[1][4 * q + 3]);
-        }
+        for (int q = 0; q < 4; ++q) out[q * 196] = make_float4(e[1][4 * q], e[1][4 * q + 1], e[1][4 * q + 2], e[1][4 * q + 3]);
       }
     }
   }

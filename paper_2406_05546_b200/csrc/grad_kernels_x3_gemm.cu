@@ -15,8 +15,8 @@
 // Every wait on an mbarrier is bounded, as in the other tensor-core kernels.
 //
 // Measured (B200; 26.3 GFLOP per product at 128 workers x 128 samples, six times that on the tensor cores: 95 us at the measured BF16
-// rate; ~6 us of event overhead included; before: packed FP32 multiply-adds): forward 560 -> 124, input gradient 539 -> 151, weight
-// gradient 515 -> 172 us (its 411 MiB of writes take 66 us at the copy rate); at 16 x 64: 72 -> 22, 58 -> 23, 42 -> 21; at 2 x 8: 17 -> 15,
+// rate; ~6 us of event overhead included; before: packed FP32 multiply-adds): forward 560 -> 119, input gradient 539 -> 144, weight
+// gradient 515 -> 163 us (its 411 MiB of writes take 66 us at the copy rate); at 16 x 64: 72 -> 22, 58 -> 23, 42 -> 21; at 2 x 8: 17 -> 15,
 // 11 -> 13, 9 -> 11.  Ticks, before -> now: 2 x 8 62.8 -> 59.3 us, 4 x 16 82 -> 81 .. 86, 8 x 16 127 -> 103, 8 x 64 251 -> 175, 32 x 64 659 -> 431: the
 // former kernels are better at no size.
 #include <cooperative_groups.h>
@@ -48,6 +48,7 @@ template <int OP_, int BN_, int BUFS_, int STAGES_, bool SPLIT_> struct Shape {
   static constexpr int A_PIECE = A_MN ? 64 * BK * 2 : BM * BK * 2, B_PIECE = B_MN ? 64 * BK * 2 : BN * BK * 2;
   static constexpr int SMEM = 1024 /* alignment slack */ + STAGES * STAGE + 256 /* barriers */ + (OP == X_DW ? EPI_WARPS * OUT_WARP_BYTES : 0);
   static constexpr int COLS = BN / 2, PART_PITCH = BN + 4;      // columns of an epilogue thread; partial tile in shared memory
+  static constexpr int TRIP = COLS > 112 ? 32 : 64;             // columns of a read of the accumulator (three warps share 16,384 registers)
   static_assert(2 * BUFS * ACC <= 512 && STAGE % 1024 == 0 && SMEM <= 227 * 1024 && COLS % 16 == 0, "tile shape");
   static_assert(!SPLIT || BM * PART_PITCH * 4 <= STAGES * STAGE, "the partial tile takes the operands' place");
 };
@@ -207,31 +208,31 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_x3(const __grid_constant__ Ma
         const int lb = lead % BUFS, sb = tile_i % BUFS;
         if (!warp_wait(&lead_full[lb], (lead / BUFS) & 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        if (kb + CHUNK < kb1) {
+        // as many columns per round trip to tensor memory as there are registers for: input gradient 145.9 -> 143.8 us at 128 x 128, the others
+        // as with sixteen
+        auto drain = [&](uint32_t at, auto add) {
 #pragma unroll
-          for (int j0 = 0; j0 < COLS; j0 += 16) {
-            uint32_t r[16];
-            tmem_ld16(t_lane + lb * S::ACC + j0, r);
+          for (int j0 = 0; j0 < COLS; j0 += S::TRIP) {
+            uint32_t r[S::TRIP / 16][16];
+#pragma unroll
+            for (int i = 0; i < S::TRIP / 16; ++i)
+              if (j0 + 16 * i < COLS) tmem_ld16(at + j0 + 16 * i, r[i]);
             tmem_ld_wait();
 #pragma unroll
-            for (int j = 0; j < 16; ++j) sum[j0 + j] += __uint_as_float(r[j]);
-          }
-        } else {
+            for (int i = 0; i < S::TRIP / 16; ++i)
 #pragma unroll
-          for (int j0 = 0; j0 < COLS; j0 += 16) {
-            uint32_t r[16], u[16];
-            tmem_ld16(t_lane + (BUFS + sb) * S::ACC + j0, u);
-            tmem_ld16(t_lane + lb * S::ACC + j0, r);
-            tmem_ld_wait();
-#pragma unroll
-            for (int j = 0; j < 16; ++j) sum[j0 + j] = join3(sum[j0 + j] + __uint_as_float(r[j]), __uint_as_float(u[j]));
+              for (int j = 0; j < 16; ++j)
+                if (j0 + 16 * i < COLS) sum[j0 + 16 * i + j] = add(sum[j0 + 16 * i + j], __uint_as_float(r[i][j]));
           }
-        }
+        };
+        drain(t_lane + lb * S::ACC, [](float a, float v) { return a + v; });
+        const bool last = kb + CHUNK >= kb1;
+        if (last) drain(t_lane + (BUFS + sb) * S::ACC, [](float a, float v) { return join3(a, v); });
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
           mbar_arrive(&lead_empty[lb]);
-          if (kb + CHUNK >= kb1) mbar_arrive(&small_empty[sb]);
+          if (last) mbar_arrive(&small_empty[sb]);
         }
         ++lead;
       }

@@ -283,7 +283,7 @@ def main():
     ap.add_argument("--warmup", type=int, default=5)
     ap.add_argument("--impl", default="b200", choices=["b200", "reference"])
     ap.add_argument("--precision", default="bf16", choices=["fp32", "bf16"],
-                    help="arithmetic of the dense contractions of the grad step: fp32 = CUDA cores; bf16 = tensor "
+                    help="arithmetic of the dense contractions of the grad step: fp32 = tensor cores, operands in three BF16 pieces; bf16 = tensor "
                          "cores (BF16 operands in the convolution products, TF32 in the 512-unit layer)")
     ap.add_argument("--case", default="bench", choices=["bench", "small"],
                     help="small: a reduced run for profiler captures (see --workers/--batch/--ticks/--down-ticks)")
@@ -440,7 +440,9 @@ def main():
         configs = {f"config{n}": measure_config(n, args.precision, pool_x, pool_y) for n in (1, 2, 3, 4)}
         if args.precision != "fp32":
             fp32_path = measure_config(5, "fp32", pool_x, pool_y)
-            fp32_path["frac_of_fp32_pipe"] = fp32_path["tflops"] / (148 * 128 * 2 * peaks["sm_max_mhz"] / 1e6)
+            roofs = [kernel_roofline(k, 1.0, W, b, peaks, "fp32") for k in ("conv1_fwd", "conv2_fwd", "fc1_fwd", "fc2_fwd_bwd", "fc1_dw", "fc1_dx",
+                                                                            "conv2_bwd", "conv2_dw", "conv1_bwd")]
+            fp32_path["frac_of_composite_roofline"] = sum(r["flops"] / (r["peak"] * 1e9) for r in roofs) / fp32_path["grad_step_ms"]
     barrier()
 
     # ---- deferred replay of a DOWN_TICKS outage (83 GB of buffered gradients)
@@ -615,6 +617,10 @@ def kernel_roofline(name, ms_per_launch, W, b, peaks, precision, sustained=False
             return {"kernel": name, "bound": "tensor", "achieved": ach, "peak": bf16_peak_tflops, "unit": "TFLOP/s",
                     "frac": ach / bf16_peak_tflops, "traffic": None, "flops": flops[name],
                     "peak_source": f"{peaks['source']} {which} bf16 GEMM"}
+        if precision == "fp32" and name != "conv1_bwd" and name in tf32_kernels | bf16_kernels:      # FP32 as three BF16 pieces: six products each
+            return {"kernel": name, "bound": "tensor", "achieved": ach, "peak": bf16_peak_tflops / 6, "unit": "TFLOP/s",
+                    "frac": ach / (bf16_peak_tflops / 6), "traffic": None, "flops": flops[name],
+                    "peak_source": f"a sixth of the {peaks['source']} {which} bf16 GEMM"}
         return {"kernel": name, "bound": "alu", "achieved": ach, "peak": fp32_peak_tflops, "unit": "TFLOP/s",
                 "frac": ach / fp32_peak_tflops, "traffic": None, "flops": flops[name],
                 "peak_source": "148 SMs x 128 FP32 lanes x 2 x max SM clock"}

@@ -1,4 +1,4 @@
-// Worker-side gradient step, FP32 path (the dense layer's products are in grad_kernels_x3_gemm.cu): the paper's small CNN (model endnote),
+// Worker-side gradient step, FP32 path (the second convolution is in grad_kernels_x3_conv2.cu, the dense layer in grad_kernels_x3_gemm.cu): the paper's small CNN (model endnote),
 // forward and backward, for W workers that may hold different weight snapshots.
 //
 // Rows of every activation buffer are (sorted worker s, sample i) -> s*b + i, where the sorted

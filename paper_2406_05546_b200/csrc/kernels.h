@@ -149,7 +149,7 @@ struct GradStepArgs {
   uint64_t seed, step;
   float drop_p;
   uint32_t drop_thresh;   // keep iff word >= thresh
-  int precision;          // 0 = FP32 (dense layer on the tensor cores, operands in BF16 pieces); otherwise tensor cores (BF16 convolution products, TF32 dense layer)
+  int precision;          // 0 = FP32 (second convolution and dense layer on the tensor cores, operands in BF16 pieces); otherwise tensor cores (BF16 convolution products, TF32 dense layer)
   int skip_prep_w1;       // the rounded copies of the dense-layer weights of these very snapshots are still valid
   int after_wait = 0;     // the caller has just made the stream wait for another one
 };

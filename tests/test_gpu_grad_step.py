@@ -125,8 +125,7 @@ def test_stale_snapshots_grouped_over_three_versions():
     _run_and_compare(5, 6, lags=[2, 0, 1, 2, 0], n_versions=3)
 
 
-# 128 / 129 and 1,536 / 1,547 rows: the last and first sizes of the FP32 path's three forms of the second convolution;
-# batches that leave one sample over in blocks of five, ranges of rows that cross workers, two weight versions.  At the
+# 128 / 129 and 1,536 / 1,547 rows, batches that leave one sample over, ranges of rows that cross workers, two weight versions.  At the
 # larger sizes two or three workers spread over the blocks are compared, and the first convolution's gradient is allowed
 # what pooling decisions within single-precision rounding of a tie can move it by (there are millions of them).
 @pytest.mark.parametrize("W,b,kw", [(2, 64, {}), (3, 43, {"lags": [1, 0, 1], "n_versions": 2}), (16, 96, {"check": (0, 8, 15)}),

@@ -42,6 +42,13 @@ struct ImagePart {
       for (int k = 0; k < 7; ++k) d[4 * k * CONV1_PITCH] = v[k];
     }
   }
+  // Is one of them infinite or NaN?
+  __device__ __forceinline__ bool odd() const {
+    float t = 0.f;
+#pragma unroll
+    for (int k = 0; k < 7; ++k) t = fmaf(v[k], 0.f, t);
+    return t != t;
+  }
 };
 // The 4x4 patch under the pooling window at (py, px), every value in both halves.
 __device__ __forceinline__ void load_patch(const float* image, int py, int px, u64 (&dup)[4][4]) {
@@ -168,7 +175,8 @@ __global__ void __launch_bounds__(CONV1_THREADS, 4) conv1_fwd(GradStepArgs a, Wo
 
 // ---- backward through pool1, ReLU and conv1 (filter / bias gradients only: the input needs none): per window element the pooled
 // gradients of the channels that it won, all others cleared, times the patch.  A sample's gradients and decisions arrive by
-// asynchronous copies while the sample before is added up.
+// asynchronous copies while the sample before is added up.  A cleared gradient times a pixel that is not finite is NaN, and no part of the
+// gradient, which is a sum over the winners' patches: an image with such a pixel takes its products one by one.
 constexpr int CONV1B_SPB = 16;            // most samples per block
 __global__ void __launch_bounds__(CONV1_THREADS, 4) conv1_bwd(GradStepArgs a, WorkerTable wt, Workspace ws, int spb, int n_chunks) {
   __shared__ __align__(16) float xs[2][CONV1_IMAGE];
@@ -210,7 +218,7 @@ __global__ void __launch_bounds__(CONV1_THREADS, 4) conv1_bwd(GradStepArgs a, Wo
   fetch(i0);
   for (int i = i0; i < i1; ++i) {
     const int cur = (i - i0) & 1;
-    __syncthreads();                        // image `cur` is complete; image `cur^1` is no longer read
+    const bool odd = __syncthreads_or(next.odd());      // image `cur`, which `next` still holds, is complete; image `cur^1` is no longer read
     if (i + 1 < i1) {
       next.load(x + (int64_t)(i + 1) * (IMG * IMG), tid);
       fetch(i + 1);
@@ -218,8 +226,31 @@ __global__ void __launch_bounds__(CONV1_THREADS, 4) conv1_bwd(GradStepArgs a, Wo
     } else {
       cp_async_wait<0>();
     }
+    if (odd) {
 #pragma unroll 1
-    for (int k = 0; k < 7; ++k) {
+      for (int k = 0; k < 7 && active; ++k) {
+        const float4 g4 = gs[cur][k][tid];
+        const uint32_t code = cs[cur][k][tid];
+        const float g[4] = {g4.x, g4.y, g4.z, g4.w};
+        const float* window = xs[cur] + 2 * (py0 + 2 * k) * CONV1_PITCH + 2 * px;
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) {
+          const uint32_t c = (code >> (8 * ch)) & 255u;
+          if (c > 3u) continue;
+          gb[ch] += g[ch];
+          const float* patch = window + (c >> 1) * CONV1_PITCH + (c & 1);
+#pragma unroll
+          for (int t = 0; t < 9; ++t) {
+            float v[2];
+            unpack2(gw[ch >> 1][t], v[0], v[1]);
+            v[ch & 1] = fmaf(g[ch], patch[t / 3 * CONV1_PITCH + t % 3], v[ch & 1]);
+            gw[ch >> 1][t] = pack2(v[0], v[1]);
+          }
+        }
+      }
+    }
+#pragma unroll 1
+    for (int k = odd ? 7 : 0; k < 7; ++k) {
       const float4 g4 = active ? gs[cur][k][tid] : make_float4(0.f, 0.f, 0.f, 0.f);
       const uint32_t code = active ? cs[cur][k][tid] : 0x04040404u;
       const float g[4] = {g4.x, g4.y, g4.z, g4.w};

@@ -255,6 +255,49 @@ def test_fp32_second_convolution_keeps_an_infinite_sum():
     srv.close()
 
 
+# Pixels that are not finite, in the first, a middle and the last sample of a worker and beside samples without any; (8, 130) has several samples
+# per block of the first convolution's filter gradient.
+@pytest.mark.parametrize("value", [float("nan"), float("-inf")])
+@pytest.mark.parametrize("W,b", [(1, 1), (2, 7), (8, 130)])
+def test_fp32_pixel_that_no_winner_reads_leaves_the_gradient_finite(W, b, value):
+    """A window element that reads a NaN loses against ReLU's zero, and so does one that reads minus infinity through positive filters:
+    such a pixel is in no winner's patch, and the filter gradient of the first convolution, a sum over the winners' patches, does not
+    see it.  Against float64 with the elements that read the pixel taken out, within the path's tolerance (and, at 8 x 130, what its own
+    open decisions allow)."""
+    import torch.nn.functional as F
+    from oracle import cnn
+    from paper_2406_05546_b200 import ps
+    import torch
+    theta = synth.init_params(seed=1, bias_scale=0.05)
+    theta[:144] = np.abs(theta[:144])
+    theta[144:160] = -0.1
+    srv = ps.ParameterServer(theta, max_workers=W, max_batch=b, queue_slots=W)
+    gen = torch.Generator(device="cuda").manual_seed(W + b)
+    x = torch.rand((W, b, 28, 28), generator=gen, device="cuda")
+    y = torch.randint(0, 10, (W, b), generator=gen, device="cuda", dtype=torch.int32)
+    odd = torch.zeros((W, b, 28, 28), dtype=torch.bool, device="cuda")
+    for i, (r, c) in zip((0, b // 2, b - 1), ((0, 0), (13, 6), (27, 27))):
+        odd[0, i, r, c] = odd[W - 1, i, c, r] = True
+    grads = torch.full((W, ps.P_PAD), float("nan"), device="cuda")
+    srv.workers_grad_step([srv.ps_pull_snapshot(w) for w in range(W)], range(W), torch.where(odd, value, x), y, SEED, 2, grads_dev=grads)
+    assert torch.isfinite(grads).all()
+    for w in sorted({0, W - 1}):
+        keep = srv.ps_dropout_mask(SEED, w, 2, b)
+        p = {n: torch.from_numpy(theta[o:o + int(np.prod(s))].astype(np.float64).reshape(s)).cuda().requires_grad_(True) for n, o, s in synth.layout()}
+        reads = F.max_pool2d(odd[w].double()[:, None], 3, 1, 1) > 0
+        a1 = F.conv2d(torch.where(odd[w], 0.0, x[w].double())[:, None], p["conv1.w"], p["conv1.b"], padding=1).masked_fill(reads, -1.0)
+        h = F.max_pool2d(F.relu(a1), 2)
+        h = F.max_pool2d(F.relu(F.conv2d(h, p["conv2.w"], p["conv2.b"], padding=1)), 2).flatten(1)
+        h = F.relu(F.linear(h, p["fc1.w"], p["fc1.b"])) * keep.double() / 0.75
+        F.cross_entropy(F.linear(h, p["fc2.w"], p["fc2.b"]), y[w].long()).backward()
+        allowed = _conv1_allowance(theta, x[w].cpu().numpy(), y[w].cpu().numpy(), cnn.dropout_keep(SEED, w, 2, b, 0.25), 0.25) if b > 7 else np.zeros(16)
+        for name, off, shape in synth.layout()[:2]:
+            want = p[name].grad.flatten()
+            off_by = (grads[w, off:off + want.numel()].double() - want).abs().view(16, -1).amax(1).cpu().numpy()
+            assert (off_by <= TOL_FP32 * float(want.abs().max()) + allowed).all(), (w, name)
+    srv.close()
+
+
 def _float64_gradient(theta, x, y, keep, drop_p=0.25):
     """One worker's gradient in float64 on the device: {tensor name: flat gradient}."""
     import torch

@@ -16,8 +16,9 @@
 //
 // Products that share an operand piece share an instruction where their columns can be neighbours (input and filter gradient).
 //
-// Zero padding and window losers are multiplied like other values, as the packed multiply-adds before did; a filter gradient
-// may get a NaN from an infinite activation of the map's last column one filter column further than FP32 would give one.
+// Zero padding and window losers are multiplied like other values: where an infinite activation meets a zero gradient, the taps
+// concerned are NaN, as in any FP32 sum over the map.  What is no position of the map is no part of a sum: the filter gradient's columns of
+// padding never meet an infinity (see there).
 //
 // Measured (B200; 29.6 GFLOP per product at 128 workers x 128 samples, six times that on the tensor cores: 112 us at the measured
 // BF16 rate; ~6 us of event overhead included; before: packed FP32 multiply-adds at two thirds of their pipe's rate): forward 696 ->
@@ -441,6 +442,12 @@ __global__ void __launch_bounds__(X_THREADS, 1) conv2_dx_x3(GradStepArgs a, Grou
 // read-out (tensor-memory quarter = piece, group of four warps = filter column).  A read-out takes a round trip of 425 clk to tensor memory
 // per load, so it has as many registers as sixteen warps leave: three trips instead of six.  A CTA walks over a contiguous range of
 // rows and writes a partial sum every seg_len rows and where the range leaves a worker.
+//
+// The zeros in g2's columns 14 and 15 meet column 13 of the map (slot 7) in the products of filter column 0 with even columns, and column 0 (slot
+// 8) in those of filter column 1 with odd and of filter column 2 with even columns, which take nothing else from there.  In a sample with an
+// infinity in one of the two slots (p1x is never NaN) the products are therefore taken in another order, and either slot is cleared once
+// only they are left of those that read it.  (The staging warp that has least to stage looks for one.  A sum of such a sample with plain multiply-adds by the
+// read-out warps costs the others 5 us at 128 x 128, by their registers.)
 // ------------------------------------------------------------------------------------------------
 constexpr int D_THREADS = 512, D_READERS = 288, D_P1_SLOTS = 3, D_RAW_SLOTS = 4;
 constexpr int D_G_ROW = PIECES * 4 * 256;                    // image row of g2: [piece][octet][slot (x & 1) * 8 + x / 2][8 channels]
@@ -449,7 +456,7 @@ constexpr int D_GAP = 128;
 constexpr int D_XCHG_BYTES = 3 * 2 * 48 * 32 * 4;            // read-out: [kx][piece m, l][column][lane]
 constexpr int D_OUT_PITCH = 145;                             // write-out: an output channel's 144 filter taps, one word of padding
 static_assert(32 * D_OUT_PITCH * 4 <= D_XCHG_BYTES, "the taps take the exchange area's place");
-constexpr int D_BARS = 2 * D_P1_SLOTS + 2 * D_RAW_SLOTS + 2 * 2 + 2 * 3;
+constexpr int D_BARS = 2 * D_P1_SLOTS + 2 * D_RAW_SLOTS + 2 * 2 + 2 * 3 + 1;
 constexpr int D_SMEM = 2 * D_G_BYTES + D_P1_SLOTS * P1X_BYTES + D_GAP + D_XCHG_BYTES + D_RAW_SLOTS * RAW_BYTES + D_BARS * 8 + 16;
 static_assert(D_SMEM <= 227 * 1024 && D_G_BYTES % 16 == 0, "shared memory");
 
@@ -466,8 +473,10 @@ __global__ void __launch_bounds__(D_THREADS, 1) conv2_dw_x3(GradStepArgs a, Work
   uint64_t* g_empty = g_full + 2;
   uint64_t* acc_full = g_empty + 2;
   uint64_t* acc_empty = acc_full + 3;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 3);
+  uint64_t* read = acc_empty + 3;                // the products so far have read their operands
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(read + 1);
   volatile uint32_t* abort_flag = tmem_slot + 1;
+  volatile uint32_t* infinite = tmem_slot + 2;   // [2] has the staged sample an infinity in columns 0 or 13?
   const int tid = threadIdx.x, lane = tid & 31, warp = warp_uniform(tid >> 5);
   const int total = a.W * a.b, r0 = blockIdx.x * segs * seg_len, r1 = min(r0 + segs * seg_len, total), n_samples = r1 - r0;
 
@@ -483,6 +492,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) conv2_dw_x3(GradStepArgs a, Work
     for (int i = 0; i < D_RAW_SLOTS; ++i) { mbar_init(&raw_full[i], 1); mbar_init(&raw_empty[i], 4); }
     for (int i = 0; i < 2; ++i) { mbar_init(&g_full[i], 4); mbar_init(&g_empty[i], 1); }
     for (int i = 0; i < 3; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 3); }
+    mbar_init(read, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -499,24 +509,60 @@ __global__ void __launch_bounds__(D_THREADS, 1) conv2_dw_x3(GradStepArgs a, Work
     // to the next eight k, here the next image row
     const uint32_t g_lo0 = plain_desc_lo(smem_u32(smem), D_G_ROW), p_lo0 = plain_desc_lo(smem_u32(p1s), P1X_ROW);
     int slot = 0;
-    uint32_t slot_parity = 0;
+    uint32_t slot_parity = 0, read_parity = 0;
     bool ok = true;
     for (int n = 0; ok && n < n_samples; ++n) {
       const int st = n & 1;
       if (!warp_wait(&p1_full[slot], slot_parity, abort_flag) || !warp_wait(&g_full[st], (n >> 1) & 1, abort_flag)) { *abort_flag = 1; break; }
       tc_fence_after();
       const uint32_t g_lo = g_lo0 + st * (D_G_BYTES / 16), p_lo = p_lo0 + slot * (P1X_BYTES / 16);
-#pragma unroll 1
-      for (int kx = 0; kx < 3; ++kx) {
-        if (n > 0 && !warp_wait(&acc_empty[kx], (n - 1) & 1, abort_flag)) { *abort_flag = 1; ok = false; break; }
+      auto issue = [&](int kx, int k, uint32_t add) {                    // image rows 2 (k / 2) and + 1, columns of parity k & 1
+        const int xp = (k & 1) + kx;                       // the first column read, 0 .. 3
+        umma_f16(tmem + kx * 144, g_lo + (k >> 1) * (2 * D_G_ROW / 16) + (k & 1) * 8, plain_desc_hi(256),
+                 p_lo + (k >> 1) * (2 * P1X_ROW / 16) + (xp & 1) * 8 + (xp >> 1), plain_desc_hi(256), idesc, add);
+      };
+      if (warp_uniform(infinite[st])) {
+        for (int kx = 0; ok && kx < 3 && n > 0; ++kx) ok = warp_wait(&acc_empty[kx], (n - 1) & 1, abort_flag);
         tc_fence_after();
-#pragma unroll
-        for (int k = 0; k < 14; ++k) {                     // image rows 2 (k / 2) and + 1, columns of parity k & 1
-          const int xp = (k & 1) + kx;                     // the first column read, 0 .. 3
-          umma_f16(tmem + kx * 144, g_lo + (k >> 1) * (2 * D_G_ROW / 16) + (k & 1) * 8, plain_desc_hi(256),
-                        p_lo + (k >> 1) * (2 * P1X_ROW / 16) + (xp & 1) * 8 + (xp >> 1), plain_desc_hi(256), idesc, k ? 1u : 0u);
+        auto clear = [&](int x_slot) {                     // of all rows and octets, in the leading piece
+          umma_commit(read);
+          if (!warp_wait(read, read_parity, abort_flag)) { ok = false; return; }
+          read_parity ^= 1;
+          *reinterpret_cast<uint4*>(p1s + slot * P1X_BYTES + (lane >> 1) * P1X_ROW + (lane & 1) * 256 + x_slot * 16) = make_uint4(0u, 0u, 0u, 0u);
+          fence_proxy_async_smem();
+          __syncwarp();
+          tc_fence_after();
+        };
+        if (ok) {
+#pragma unroll 1
+          for (int k = 1; k < 14; k += 2) issue(0, k, k > 1);
+#pragma unroll 1
+          for (int k = 0; k < 14; k += 2) issue(1, k, k > 0);
+          clear(8);
         }
-        umma_commit(&acc_full[kx]);
+        if (ok) {
+#pragma unroll 1
+          for (int k = 1; k < 14; k += 2) issue(1, k, 1);
+#pragma unroll 1
+          for (int k = 0; k < 14; ++k) issue(2, k, k > 0);
+          clear(7);
+        }
+        if (ok) {
+#pragma unroll 1
+          for (int k = 0; k < 14; k += 2) issue(0, k, 1);
+          for (int kx = 0; kx < 3; ++kx) umma_commit(&acc_full[kx]);
+        } else {
+          *abort_flag = 1;
+        }
+      } else {
+#pragma unroll 1
+        for (int kx = 0; kx < 3; ++kx) {
+          if (n > 0 && !warp_wait(&acc_empty[kx], (n - 1) & 1, abort_flag)) { *abort_flag = 1; ok = false; break; }
+          tc_fence_after();
+#pragma unroll
+          for (int k = 0; k < 14; ++k) issue(kx, k, k > 0);
+          umma_commit(&acc_full[kx]);
+        }
       }
       if (!ok) break;
       umma_commit(&p1_empty[slot]);
@@ -554,6 +600,19 @@ __global__ void __launch_bounds__(D_THREADS, 1) conv2_dw_x3(GradStepArgs a, Work
       if (ok && n >= 2) ok = mbar_wait(&g_empty[st], ((n >> 1) - 1) & 1);
       if (!__all_sync(0xffffffffu, ok && !*abort_flag)) { *abort_flag = 1; break; }
       const uint8_t* rp = raw + slot * RAW_BYTES;
+      if (warp == 15) {                      // (it stages one item a thread, the others two)
+        const int p1_slot = n % D_P1_SLOTS;
+        ok = mbar_wait(&p1_full[p1_slot], (n / D_P1_SLOTS) & 1);
+        if (!__all_sync(0xffffffffu, ok && !*abort_flag)) { *abort_flag = 1; break; }
+        uint32_t top = 0;
+        if (lane < 28) {                     // slots 7 and 8 of a row of the map and an octet of channels: leading pieces, which are never negative
+          const uint4* v = reinterpret_cast<const uint4*>(p1s + p1_slot * P1X_BYTES + ((lane >> 1) + 1) * P1X_ROW + (lane & 1) * 256 + 7 * 16);
+#pragma unroll
+          for (int i = 0; i < 2; ++i) top |= (v[i].x + 0x00800080u) | (v[i].y + 0x00800080u) | (v[i].z + 0x00800080u) | (v[i].w + 0x00800080u);
+        }
+        const bool any = __any_sync(0xffffffffu, (top & 0x80008000u) != 0);
+        if (lane == 0) infinite[st] = any;
+      }
 #pragma unroll 1
       for (int e = lt; e < 4 * 49; e += 128) {
         const int o8 = e / 49, p = e - o8 * 49, py = p / 7, px = p - py * 7;

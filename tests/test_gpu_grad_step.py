@@ -298,6 +298,60 @@ def test_fp32_pixel_that_no_winner_reads_leaves_the_gradient_finite(W, b, value)
     srv.close()
 
 
+# The first and the last column of the map, in one, some and all samples of a range of rows
+@pytest.mark.parametrize("W,b,samples", [(1, 1, (0,)), (1, 3, (1,)), (2, 300, (0, 1, 2, 3, 4, 150, 299)), (3, 20, tuple(range(20)))])
+@pytest.mark.parametrize("col", [0, 13])
+def test_fp32_infinite_activation_reaches_only_the_filter_taps_that_read_it(W, b, samples, col):
+    """An infinite activation at an end of a row of the second convolution's input, under filters that make every window above it lose:
+    the gradients passed back there are zeros, and zero times infinity is NaN, in the taps (of that input channel) that take the activation from
+    some position of the map.  The other taps, those that would take it from a column outside of it among them, are finite and, like
+    the bias, within 1e-3 of float64 in 2-norm (the bound of the tiles' edges)."""
+    import torch.nn.functional as F
+    from paper_2406_05546_b200 import ps
+    import torch
+    theta = synth.init_params(seed=1, bias_scale=0.05)
+    rng = np.random.default_rng(3)
+    theta[:144] = -0.1 * rng.random(144)        # channels 1 .. 15: minus infinity where they read the pixel
+    theta[:9] = 0.1                             # channel 0: infinite there
+    theta[144:160] = 0.2
+    off = next(o for n, o, _ in synth.layout() if n == "conv2.w")
+    taps = theta[off:off + 4608].reshape(32, 16, 9)
+    taps[:, 0] = -np.abs(taps[:, 0])
+    srv = ps.ParameterServer(theta, max_workers=W, max_batch=b, queue_slots=W)
+    gen = torch.Generator(device="cuda").manual_seed(b)
+    x = torch.rand((W, b, 28, 28), generator=gen, device="cuda")
+    y = torch.randint(0, 10, (W, b), generator=gen, device="cuda", dtype=torch.int32)
+    x[0, list(samples), 0, 0 if col == 0 else 27] = float("inf")
+    grads = torch.zeros((W, ps.P_PAD), device="cuda")
+    loss, _ = srv.workers_grad_step([srv.ps_pull_snapshot(w) for w in range(W)], range(W), x, y, SEED, 2, grads_dev=grads)
+    assert torch.isfinite(loss).all() and srv.ps_stats()["device_status"] == 0
+    for w in sorted({0, W - 1}):
+        p = {n: torch.from_numpy(theta[o:o + int(np.prod(s))].astype(np.float64).reshape(s)).cuda().requires_grad_(not n.startswith("conv1")) for n, o, s in synth.layout()}
+        # the pixel stands for 1e30, which decides every window alike and reaches nothing above
+        p1 = F.max_pool2d(F.relu(F.conv2d(x[w].double().clamp(max=1e30)[:, None], p["conv1.w"], p["conv1.b"], padding=1)), 2)
+        a2 = F.conv2d(p1, p["conv2.w"], p["conv2.b"], padding=1)
+        a2.retain_grad()
+        h = F.max_pool2d(F.relu(a2), 2).flatten(1)
+        h = F.relu(F.linear(h, p["fc1.w"], p["fc1.b"])) * srv.ps_dropout_mask(SEED, w, 2, b).double() / 0.75
+        F.cross_entropy(F.linear(h, p["fc2.w"], p["fc2.b"]), y[w].long()).backward()
+        # a tap's sum over the positions of the map that it reads a position of the map from
+        p1 = torch.where(p1 > 1e20, float("inf"), p1)
+        want = torch.zeros((32, 16, 3, 3), dtype=torch.float64, device="cuda")
+        for ky in range(3):
+            for kx in range(3):
+                ys, xs = slice(max(0, 1 - ky), min(14, 15 - ky)), slice(max(0, 1 - kx), min(14, 15 - kx))
+                yi, xi = slice(ys.start + ky - 1, ys.stop + ky - 1), slice(xs.start + kx - 1, xs.stop + kx - 1)
+                for ic in range(16):
+                    want[:, ic, ky, kx] = (a2.grad[:, :, ys, xs] * p1[:, ic:ic + 1, yi, xi]).sum((0, 2, 3))
+        got, want = grads[w, off:off + 4608].double(), want.flatten()
+        assert int(want.isnan().sum()) == (32 * 4 if w == 0 else 0) and torch.equal(got.isnan(), want.isnan())
+        fine = ~want.isnan()
+        assert (got - want)[fine].norm() <= 1e-3 * want[fine].norm()
+        db = a2.grad.sum((0, 2, 3))
+        assert (grads[w, off + 4608:off + 4640].double() - db).norm() <= 1e-3 * db.norm()
+    srv.close()
+
+
 def _float64_gradient(theta, x, y, keep, drop_p=0.25):
     """One worker's gradient in float64 on the device: {tensor name: flat gradient}."""
     import torch

@@ -20,6 +20,7 @@
 #include <stdint.h>
 
 #include "device_common.cuh"
+#include "kernels.h"
 
 namespace psk {
 
@@ -52,6 +53,17 @@ __device__ __forceinline__ Bf16x3 split3(float a, float b) {
   if (!(fabsf(a) <= MOST)) split3_huge(a, 0, o);
   if (!(fabsf(b) <= MOST)) split3_huge(b, 16, o);
   return o;
+}
+
+// Eight values of the dense layer's weights, i onwards, of weight group g: [group][piece][512][1568].
+constexpr int W1_ELEMS = HID * FLAT;
+__device__ __forceinline__ void split_w1(const float* __restrict__ theta, uint16_t* __restrict__ w1x, int g, int i) {
+  const float4* src = reinterpret_cast<const float4*>(theta + OFF_F1W + i);
+  const float4 v0 = src[0], v1 = src[1];
+  const Bf16x3 s0 = split3(v0.x, v0.y), s1 = split3(v0.z, v0.w), s2 = split3(v1.x, v1.y), s3 = split3(v1.z, v1.w);
+#pragma unroll
+  for (int p = 0; p < PIECES; ++p)
+    *reinterpret_cast<uint4*>(w1x + ((int64_t)g * PIECES + p) * W1_ELEMS + i) = make_uint4(s0.p[p], s1.p[p], s2.p[p], s3.p[p]);
 }
 
 // The sum of the leading products with that of the small ones.

@@ -62,7 +62,10 @@ __device__ __forceinline__ void load_patch(const float* image, int py, int px, u
 
 // The second convolution's filters of a weight group as its kernels' operands, one row of eight values (in pieces) per thread.
 // Blocks of conv1_fwd beyond its workers do it, so that the next kernel finds them without a launch or a fork of their own.
+// Behind them come, in an evaluation, W1_UNITS blocks per weight group for the dense layer's.
 constexpr int BANK3_ROWS = 2 * BANK3_FWD_ROWS + 12 * 48, BANK3_UNITS = (BANK3_ROWS + CONV1_THREADS - 1) / CONV1_THREADS;      // blocks per weight group
+constexpr int W1_UNITS = W1_ELEMS / (8 * CONV1_THREADS);
+static_assert(W1_ELEMS % (8 * CONV1_THREADS) == 0, "whole blocks");
 __device__ __forceinline__ void build_bank3(const float* __restrict__ theta, uint8_t* __restrict__ bank, int e, const Bank3Taps& taps) {
   if (e >= BANK3_ROWS) return;
   float v[8];
@@ -86,13 +89,19 @@ __device__ __forceinline__ void build_bank3(const float* __restrict__ theta, uin
   for (int p = 0; p < PIECES; ++p) *reinterpret_cast<uint4*>(d + p * piece_bytes) = make_uint4(s[0].p[p], s[1].p[p], s[2].p[p], s[3].p[p]);
 }
 
-__global__ void __launch_bounds__(CONV1_THREADS, 4) conv1_fwd(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws, int spb, const __grid_constant__ Bank3Taps taps) {
+__global__ void __launch_bounds__(CONV1_THREADS, 4) conv1_fwd(GradStepArgs a, WorkerTable wt, GroupTable gt, Workspace ws, int spb, int w1_units, const __grid_constant__ Bank3Taps taps) {
   __shared__ __align__(16) float xs[2][CONV1_IMAGE];
   const int s = blockIdx.y, tid = threadIdx.x;
   if (s >= a.W) {
-    const int u = (s - a.W) * gridDim.x + blockIdx.x, g = u / BANK3_UNITS;
+    const int u = (s - a.W) * gridDim.x + blockIdx.x, u1 = u - gt.n_groups * BANK3_UNITS;
     pdl_enter();
-    if (g < gt.n_groups) build_bank3(gt.theta[g], ws.bank2 + (int64_t)g * BANK3_BYTES, (u - g * BANK3_UNITS) * CONV1_THREADS + tid, taps);
+    if (u1 < 0) {
+      const int g = u / BANK3_UNITS;
+      build_bank3(gt.theta[g], ws.bank2 + (int64_t)g * BANK3_BYTES, (u - g * BANK3_UNITS) * CONV1_THREADS + tid, taps);
+    } else if (u1 < gt.n_groups * w1_units) {
+      const int g = u1 / W1_UNITS;
+      split_w1(gt.theta[g], ws.w1x, g, ((u1 - g * W1_UNITS) * CONV1_THREADS + tid) * 8);
+    }
     return;
   }
   const float* theta = group_theta(wt, gt, s);
@@ -482,14 +491,15 @@ static int samples_per_block(int rows, int least, int most) {
   while (spb < most && (rows + spb - 1) / spb > 8 * g_sm_count) spb *= 2;
   return spb;
 }
-static void launch_conv1_fwd(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof) {
+static void launch_conv1_fwd(bool with_w1, const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, cudaStream_t st, Profiler* prof) {
   const int spb = samples_per_block(a.W * a.b, 1, CONV1_SPB);
-  const int chunks = (a.b + spb - 1) / spb, bank = (gt.n_groups * BANK3_UNITS + chunks - 1) / chunks;
-  TIMED(K_CONV1_FWD, launch_pdl_if(!a.after_wait, conv1_fwd, dim3(chunks, a.W + bank), CONV1_THREADS, 0, st, a, wt, gt, ws, spb, conv2_fwd_x3_taps()));
+  const int w1_units = with_w1 ? W1_UNITS : 0, chunks = (a.b + spb - 1) / spb, more = (gt.n_groups * (BANK3_UNITS + w1_units) + chunks - 1) / chunks;
+  TIMED(K_CONV1_FWD, launch_pdl_if(!a.after_wait, conv1_fwd, dim3(chunks, a.W + more), CONV1_THREADS, 0, st, a, wt, gt, ws, spb, w1_units, conv2_fwd_x3_taps()));
 }
 
 // Evaluation pass: the forward kernels of the grad step with the dropout switched off, then the per-worker loss and hit
-// count.
+// count.  FP32 path: there is no side stream here for the pieces of W1, and a launch of their own costs more than spare blocks of conv1_fwd
+// (us per pass, own launch / spare blocks: 1 x 1 27.9 / 25.0, 2 x 8 29.8 / 25.5, 16 x 8 32.0 / 28.6, 80 x 125 354 / 349).
 int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& gt, const Workspace& ws, int32_t* correct,
                 cudaStream_t st, Profiler* prof) {
   int launches = 0;
@@ -501,11 +511,10 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
     if (n < 0) return -1;
     launches += 2 + n;
   } else {
-    launch_prep_w1_x3(gt, ws, st, prof);
-    launch_conv1_fwd(a, wt, gt, ws, st, prof);
+    launch_conv1_fwd(true, a, wt, gt, ws, st, prof);
     launch_conv2_fwd_x3(a, gt, ws, st, prof);
     if (launch_fc1_fwd_x3(a, wt, gt, ws, st, prof, false) < 0) return -1;
-    launches += 4;
+    launches += 3;
   }
   launch_output_layer(true, a, wt, gt, ws, st, prof);
   TIMED(K_EVAL_FINISH, launch_pdl(eval_finish, dim3(a.W), 128, 0, st, a, wt, ws, correct));
@@ -586,7 +595,7 @@ int launch_grad_step(const GradStepArgs& a, const WorkerTable& wt, const GroupTa
     if (side.s1) { cudaEventRecord(side.fork1, st); cudaStreamWaitEvent(s1, side.fork1, 0); }
     launch_prep_w1_x3(gt, ws, s1, prof);
     if (side.s1) cudaEventRecord(side.join1, s1);
-    launch_conv1_fwd(a, wt, gt, ws, st, prof);
+    launch_conv1_fwd(false, a, wt, gt, ws, st, prof);
     launch_conv2_fwd_x3(a, gt, ws, st, prof);
     if (side.s1) cudaStreamWaitEvent(st, side.join1, 0);
     if (launch_fc1_fwd_x3(a, wt, gt, ws, st, prof, side.s1 != nullptr) < 0) return -1;

@@ -311,17 +311,10 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_x3(const __grid_constant__ Ma
   }
 }
 
-// The pieces of every weight group's W1: [group][piece][512][1568] BF16.
-constexpr int W1_ELEMS = HID * FLAT;
+// The pieces of every weight group's W1.
 __global__ void __launch_bounds__(256) prep_w1_x3(GroupTable gt, uint16_t* __restrict__ w1x) {
-  const int i = (blockIdx.x * 256 + threadIdx.x) * 8, g = blockIdx.y;
-  if (i >= W1_ELEMS) return;
-  const float4* src = reinterpret_cast<const float4*>(gt.theta[g] + OFF_F1W + i);
-  const float4 v0 = src[0], v1 = src[1];
-  const Bf16x3 s0 = split3(v0.x, v0.y), s1 = split3(v0.z, v0.w), s2 = split3(v1.x, v1.y), s3 = split3(v1.z, v1.w);
-#pragma unroll
-  for (int p = 0; p < PIECES; ++p)
-    *reinterpret_cast<uint4*>(w1x + ((int64_t)g * PIECES + p) * W1_ELEMS + i) = make_uint4(s0.p[p], s1.p[p], s2.p[p], s3.p[p]);
+  const int i = (blockIdx.x * 256 + threadIdx.x) * 8;
+  if (i < W1_ELEMS) split_w1(gt.theta[blockIdx.y], w1x, blockIdx.y, i);
 }
 
 // BF16 tensor of `rank` dimensions (dims[0] contiguous; pitch[i] elements between neighbours of dimension i + 1).

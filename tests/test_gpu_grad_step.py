@@ -241,6 +241,35 @@ def test_fp32_second_convolution_at_the_edges_of_its_tiles(W, b, n_versions):
     srv.close()
 
 
+@pytest.mark.parametrize("W,b,n_versions", [(1, 1, 1), (2, 8, 1), (3, 1, 3), (5, 37, 2)])
+def test_fp32_evaluation_lays_out_the_weights_of_every_version_in_its_first_kernel(W, b, n_versions):
+    """Five launches, and the losses of float64 for workers on different versions (one sample per worker: all spare blocks in one column of
+    the first kernel's grid)."""
+    import torch.nn.functional as F
+    torch, ps, srv, theta0 = _setup(W, b, n_versions, drop_p=0.0)
+    thetas = {0: theta0}
+    for v in range(1, n_versions):
+        g = np.zeros((1, ps.P_PAD), dtype=np.float32)
+        g[0, :ps.P] = synth.random_gradients(1, seed=50 + v, scale=2.0)[0]
+        srv.ps_enqueue([0], [v - 1], 0, grads_dev=torch.from_numpy(g).cuda())
+        srv.ps_apply(ps.ASYNC, 0.01)
+        thetas[v], _ = srv.ps_export_params(0)
+    gen = torch.Generator(device="cuda").manual_seed(b)
+    x = torch.rand((W, b, 28, 28), generator=gen, device="cuda")
+    y = torch.randint(0, 10, (W, b), generator=gen, device="cuda", dtype=torch.int32)
+    snaps = [srv.ps_pull_snapshot(w, w % n_versions) for w in range(W)]
+    before = srv.ps_stats()["kernel_launches"]
+    loss, *_ = srv.workers_eval(snaps, x, y)
+    assert srv.ps_stats()["kernel_launches"] - before == 5
+    for w in range(W):
+        p = {n: torch.from_numpy(thetas[snaps[w].version][o:o + int(np.prod(s))].astype(np.float64).reshape(s)).cuda() for n, o, s in synth.layout()}
+        h = F.max_pool2d(F.relu(F.conv2d(x[w].double()[:, None], p["conv1.w"], p["conv1.b"], padding=1)), 2)
+        h = F.max_pool2d(F.relu(F.conv2d(h, p["conv2.w"], p["conv2.b"], padding=1)), 2).flatten(1)
+        want = F.cross_entropy(F.linear(F.relu(F.linear(h, p["fc1.w"], p["fc1.b"])), p["fc2.w"], p["fc2.b"]), y[w].long())
+        assert abs(float(loss[w]) - float(want)) <= 1e-5 * float(want), w
+    srv.close()
+
+
 def test_fp32_second_convolution_keeps_an_infinite_sum():
     """An output channel whose filters are all infinite, over inputs that are all positive, is infinite inside the map."""
     from paper_2406_05546_b200 import ps

@@ -8,7 +8,9 @@
 // What limits the precision is its accumulator, which drops the low bits of every sum (it does not round to nearest), so that
 // the error grows with the number of instructions added up, always towards zero.  Hence
 //   - the five small products have an accumulator of their own, where the same loss is 2^-8 as large, and
-//   - the leading products are added up over at most 128 values of k, then added to a sum in registers, which rounds.
+//   - the leading products are added up over a bounded number of values of k, then added to a sum in registers, which rounds: 64 in the
+//     dense layer's forward product, 128 in its gradients, 144 and 96 in the second convolution forward and its input gradient, 224 in its
+//     filter gradient.  (The small products over all of k: their loss is 2^-8 of it.)
 // Error relative to float64, 2-norm, of 512 x 128 sums over K = 1,600 of N(0, 1) x N(0, 0.05^2), rectified: one chain of fused
 // multiply-adds 4.9e-7; all six products in one accumulator 1.0e-5; two accumulators 1.1e-6; leading products over 512,
 // 256, 128 and 64 values of k at a time 2.9e-7, 1.5e-7, 1.1e-7 and 1.1e-7.  K = 512: chain 2.6e-7, 128 at a time 0.8e-7;
@@ -26,6 +28,14 @@ namespace psk {
 
 constexpr int PIECES = 3;
 
+// The part of a leading sum that truncation takes from it on average: (n - 1) / 2 times 1.3e-8 to 1.6e-8 for n instructions, whatever the
+// operands' signs (partial sums grow towards the whole in the mean).  It is the same for every sample, so that it does not average out in a
+// sum over samples as rounding does.  In the forward products, on which every gradient depends, the weights' last pieces are taken larger
+// by as much: second convolution (9 instructions), dense layer (4; the input gradient has the same operand and 8).
+// Mean relative error of the sums before / with it: -6.4e-8 / 0.03e-8 and, dense layer with 8 instructions before, -4.7e-8 / -0.3e-8; input
+// gradient -4.3e-8 / -2.3e-8.
+constexpr float LOST_CONV2 = 6.4e-8f, LOST_FC1 = 2.0e-8f;
+
 struct Bf16x3 { uint32_t p[PIECES]; };      // two values: BF16 pairs, the first value in the low halves
 
 // One value that rounds past the largest BF16, or none: the piece is cut off instead.
@@ -41,7 +51,8 @@ __device__ __forceinline__ void split3_huge(float x, uint32_t shift, Bf16x3& o) 
   o.p[2] = (o.p[2] & keep) | (l << shift);
 }
 
-__device__ __forceinline__ Bf16x3 split3(float a, float b) {
+// more: the part of a value that is added to its last piece
+__device__ __forceinline__ Bf16x3 split3(float a, float b, float more = 0.f) {
   constexpr float MOST = 3.3895313892515355e38f;      // the largest BF16
   Bf16x3 o;
   o.p[0] = bf16_pair(a, b);
@@ -49,6 +60,10 @@ __device__ __forceinline__ Bf16x3 split3(float a, float b) {
   o.p[1] = bf16_pair(ra, rb);
   ra -= __uint_as_float(o.p[1] << 16);
   rb -= __uint_as_float(o.p[1] & 0xFFFF0000u);
+  if (more != 0.f) {
+    ra = fmaf(a, more, ra);
+    rb = fmaf(b, more, rb);
+  }
   o.p[2] = bf16_pair(ra, rb);
   if (!(fabsf(a) <= MOST)) split3_huge(a, 0, o);
   if (!(fabsf(b) <= MOST)) split3_huge(b, 16, o);
@@ -60,7 +75,7 @@ constexpr int W1_ELEMS = HID * FLAT;
 __device__ __forceinline__ void split_w1(const float* __restrict__ theta, uint16_t* __restrict__ w1x, int g, int i) {
   const float4* src = reinterpret_cast<const float4*>(theta + OFF_F1W + i);
   const float4 v0 = src[0], v1 = src[1];
-  const Bf16x3 s0 = split3(v0.x, v0.y), s1 = split3(v0.z, v0.w), s2 = split3(v1.x, v1.y), s3 = split3(v1.z, v1.w);
+  const Bf16x3 s0 = split3(v0.x, v0.y, LOST_FC1), s1 = split3(v0.z, v0.w, LOST_FC1), s2 = split3(v1.x, v1.y, LOST_FC1), s3 = split3(v1.z, v1.w, LOST_FC1);
 #pragma unroll
   for (int p = 0; p < PIECES; ++p)
     *reinterpret_cast<uint4*>(w1x + ((int64_t)g * PIECES + p) * W1_ELEMS + i) = make_uint4(s0.p[p], s1.p[p], s2.p[p], s3.p[p]);

@@ -84,7 +84,8 @@ __device__ __forceinline__ void build_bank3(const float* __restrict__ theta, uin
     d = bank + BANK3_FWD_BYTES + (ko * PIECES * 48 + col) * 16;
     piece_bytes = 48 * 16;
   }
-  const Bf16x3 s[4] = {split3(v[0], v[1]), split3(v[2], v[3]), split3(v[4], v[5]), split3(v[6], v[7])};
+  const float more = e < 2 * BANK3_FWD_ROWS ? LOST_CONV2 : 0.f;
+  const Bf16x3 s[4] = {split3(v[0], v[1], more), split3(v[2], v[3], more), split3(v[4], v[5], more), split3(v[6], v[7], more)};
 #pragma unroll
   for (int p = 0; p < PIECES; ++p) *reinterpret_cast<uint4*>(d + p * piece_bytes) = make_uint4(s[0].p[p], s[1].p[p], s[2].p[p], s[3].p[p]);
 }

@@ -9,8 +9,8 @@
 // the error grows with the number of instructions added up, always towards zero.  Hence
 //   - the five small products have an accumulator of their own, where the same loss is 2^-8 as large, and
 //   - the leading products are added up over a bounded number of values of k, then added to a sum in registers, which rounds: 64 in the
-//     dense layer's forward product, 128 in its gradients, 144 and 96 in the second convolution forward and its input gradient, 224 in its
-//     filter gradient.  (The small products over all of k: their loss is 2^-8 of it.)
+//     dense layer's forward product, 128 in its gradients, 80 and 64 in the second convolution forward (in two accumulators), 96 in its input
+//     gradient, 224 in its filter gradient.  (The small products over all of k: their loss is 2^-8 of it.)
 // Error relative to float64, 2-norm, of 512 x 128 sums over K = 1,600 of N(0, 1) x N(0, 0.05^2), rectified: one chain of fused
 // multiply-adds 4.9e-7; all six products in one accumulator 1.0e-5; two accumulators 1.1e-6; leading products over 512,
 // 256, 128 and 64 values of k at a time 2.9e-7, 1.5e-7, 1.1e-7 and 1.1e-7.  K = 512: chain 2.6e-7, 128 at a time 0.8e-7;
@@ -30,11 +30,11 @@ constexpr int PIECES = 3;
 
 // The part of a leading sum that truncation takes from it on average: (n - 1) / 2 times 1.3e-8 to 1.6e-8 for n instructions, whatever the
 // operands' signs (partial sums grow towards the whole in the mean).  It is the same for every sample, so that it does not average out in a
-// sum over samples as rounding does.  In the forward products, on which every gradient depends, the weights' last pieces are taken larger
-// by as much: second convolution (9 instructions), dense layer (4; the input gradient has the same operand and 8).
-// Mean relative error of the sums before / with it: -6.4e-8 / 0.03e-8 and, dense layer with 8 instructions before, -4.7e-8 / -0.3e-8; input
-// gradient -4.3e-8 / -2.3e-8.
-constexpr float LOST_CONV2 = 6.4e-8f, LOST_FC1 = 2.0e-8f;
+// sum over samples as rounding does.  In the forward products, on which every gradient depends, sums are short (4 or 5 instructions) and the
+// weights' last pieces are larger by as much (the dense layer's input gradient, of 8 instructions, has the same operand).  Mean relative
+// error without / with both: second convolution -6.4e-8 (one sum of 9 instructions) / -0.04e-8, dense layer -4.7e-8 (8) / -0.01e-8, its input
+// gradient -4.3e-8 / -2.1e-8.  fc2.w of a summed step of 128 x 128 against float64, 2-norm: 2.1e-7 / 0.8e-7, as multiply-adds that round give it.
+constexpr float LOST_CONV2 = 2.35e-8f, LOST_FC1 = 2.3e-8f;
 
 struct Bf16x3 { uint32_t p[PIECES]; };      // two values: BF16 pairs, the first value in the low halves
 

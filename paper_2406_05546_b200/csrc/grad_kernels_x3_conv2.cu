@@ -22,10 +22,10 @@
 //
 // Measured (B200; 29.6 GFLOP per product at 128 workers x 128 samples, six times that on the tensor cores: 112 us at the measured
 // BF16 rate; ~6 us of event overhead included; before: packed FP32 multiply-adds at two thirds of their pipe's rate): forward 696 ->
-// 200, input gradient 636 -> 176, filter gradient 651 -> 266 us; at 16 x 64: 56 -> 25, 57 -> 21, 56 -> 31; at 2 x 8: 12 -> 13, 15 -> 11,
+// 210, input gradient 636 -> 176, filter gradient 651 -> 271 us; at 16 x 64: 56 -> 25, 57 -> 21, 56 -> 31; at 2 x 8: 12 -> 13, 15 -> 11,
 // 15 -> 14.  Forward and input gradient are bound by the instructions' own time; the filter gradient takes 1.5 times as many products as
-// it needs, rounded up to 128 rows.  Relative error against float64, median over workers, 128 x 128: conv2.w 1.6e-7 -> 1.0e-7, conv1.w
-// 1.2e-7 -> 0.9e-7; 2 x 8: 3.2e-7 -> 1.7e-7, 3.6e-7 -> 2.1e-7.
+// it needs, rounded up to 128 rows.  Relative error against float64, median over workers, 128 x 128: conv2.w 1.7e-7 -> 0.8e-7, conv1.w
+// 1.7e-7 -> 1.0e-7; 2 x 8: 2.9e-7 -> 1.3e-7, 3.3e-7 -> 1.6e-7.
 //
 // Each kernel's stages (copies, staging, MMA issue, read-out) run in different warps and overlap through mbarriers; every wait
 // is bounded.
@@ -63,13 +63,15 @@ __device__ __forceinline__ void report_abort(uint32_t* status) {
 // accumulator columns, so that a thread holds whole windows.  One MMA per input SHIFT: window element (jy, jx) and tap (ky, kx)
 // read the input shifted by (jy + ky, jx + kx); the filters of the pairs that add up to a shift are stacked in column order.
 // The ranges are ordered (0,0) (0,1) (1,1) (1,0): a shift's window elements are neighbours but for two shifts, which take
-// two MMAs: 18 per product, 108 a tile.
+// two MMAs: 18 per product, 108 a tile.  The leading products of shifts with an even and with an odd sum of coordinates have an accumulator each
+// (a sum of nine taps in one loses more to truncation than one of five and one of four; 200 -> 210 us at 128 x 128), so that a tile takes three of the four that there is room
+// for, in turn: its small products, five sixths of its time, run while the tile before is read out.
 // Warps: 0 = MMA issue and tensor memory, 1 = copies, 2..9 = epilogue.
 // ------------------------------------------------------------------------------------------------
 constexpr int F_THREADS = 320, F_STAGES = 2, F_OPS = 18;
 constexpr int F_STAGE_BYTES = 2 * P1X_BYTES + 2 * P1X_ROW + 256;       // the padding rows' overrun
 constexpr int F_W_PIECE = 2 * BANK3_FWD_ROWS * 16;                      // [octet][row][8 channels]
-constexpr int F_BARS = 2 * F_STAGES + 2 + 2 + 1;
+constexpr int F_BARS = 2 * F_STAGES + 1 + 1 + 1;
 constexpr int F_SMEM = F_STAGES * F_STAGE_BYTES + BANK3_FWD_BYTES + 32 * 4 + F_BARS * 8 + 16;
 static_assert(F_SMEM <= 227 * 1024 && F_STAGE_BYTES % 128 == 0, "shared memory");
 
@@ -94,10 +96,11 @@ struct FoldTables {
       }
       ++n_ops;
     };
-    for (int pass = 0; pass < 2; ++pass)                 // an op that covers all columns comes first: it starts the sums
+    for (int pass = 0; pass < 4; ++pass)                 // either half begins with an op that covers all columns: it starts the sums
       for (int sy = 0; sy < 4; ++sy)
         for (int sx = 0; sx < 4; ++sx) {
-          if ((pass == 0) != (sy == 1 && sx == 1)) continue;
+          const bool starts = sy == 1 && (sx == 1 || sx == 2);
+          if (((sy + sx) & 1) != pass >> 1 || starts != ((pass & 1) == 0)) continue;
           bool used[4] = {false, false, false, false};
           for (int jy = 0; jy < 2; ++jy)
             for (int jx = 0; jx < 2; ++jx)
@@ -123,9 +126,9 @@ __global__ void __launch_bounds__(F_THREADS, 1) conv2_fwd_x3(GradStepArgs a, Gro
   float* bias = reinterpret_cast<float*>(Wk + BANK3_FWD_BYTES);
   uint64_t* a_full = reinterpret_cast<uint64_t*>(bias + 32);      // [F_STAGES] copies -> MMA
   uint64_t* a_empty = a_full + F_STAGES;                          // [F_STAGES] MMA -> copies
-  uint64_t* acc_full = a_empty + F_STAGES;                        // [2] MMA -> epilogue
-  uint64_t* acc_empty = acc_full + 2;                             // [2] epilogue -> MMA
-  uint64_t* w_full = acc_empty + 2;
+  uint64_t* acc_full = a_empty + F_STAGES;                        // MMA -> epilogue
+  uint64_t* acc_empty = acc_full + 1;                             // epilogue -> MMA
+  uint64_t* w_full = acc_empty + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(w_full + 1);
   volatile uint32_t* abort_flag = tmem_slot + 1;
   const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
@@ -137,7 +140,8 @@ __global__ void __launch_bounds__(F_THREADS, 1) conv2_fwd_x3(GradStepArgs a, Gro
   // bytes never written by a copy (the overrun of the padding rows, a missing second sample) only feed rows that are dropped
   if (tid == 0) {
     for (int i = 0; i < F_STAGES; ++i) { mbar_init(&a_full[i], 1); mbar_init(&a_empty[i], 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 8); }
+    mbar_init(acc_full, 1);
+    mbar_init(acc_empty, 8);
     mbar_init(w_full, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -157,23 +161,30 @@ __global__ void __launch_bounds__(F_THREADS, 1) conv2_fwd_x3(GradStepArgs a, Gro
     if (!ok) *abort_flag = 1;
     for (int t = 0; ok && t < n_tiles; ++t) {
       const int buf = t & 1;
-      const uint32_t parity = (t >> 1) & 1;
-      if (!warp_wait(&a_full[buf], parity, abort_flag) || (t >= 2 && !warp_wait(&acc_empty[buf], parity ^ 1, abort_flag))) { *abort_flag = 1; break; }
+      if (!warp_wait(&a_full[buf], (t >> 1) & 1, abort_flag)) { *abort_flag = 1; break; }
       tc_fence_after();
-      const uint32_t a_lo = a_lo0 + buf * (F_STAGE_BYTES / 16), d = tmem + buf * 256;
-      // l h, m m, h l, m h, h m into the second half of the columns, then h h into the first
+      const uint32_t a_lo = a_lo0 + buf * (F_STAGE_BYTES / 16);
+      // l h, m m, h l, m h, h m into accumulator 3 t, which the tile before the last has left, then h h into 3 t + 1 and 3 t + 2, once the last
+      // tile has been read out
 #pragma unroll 1
       for (int i = 0; i < 6; ++i) {
+        if (i == 5 && t > 0) {
+          ok = warp_wait(acc_empty, (t - 1) & 1, abort_flag);
+          if (!ok) { *abort_flag = 1; break; }
+          tc_fence_after();
+        }
         const int i_a = (0x001012 >> (4 * i)) & 15, i_b = (0x010210 >> (4 * i)) & 15;
-        const uint32_t ai = a_lo + i_a * (512 / 16), bi = w_lo + i_b * (F_W_PIECE / 16), di = d + (i < 5 ? 128 : 0);
-        const uint32_t start = i == 0 || i == 5 ? 0u : 1u;
+        const uint32_t ai = a_lo + i_a * (512 / 16), bi = w_lo + i_b * (F_W_PIECE / 16);
+        const uint32_t d0 = tmem + ((3 * t + (i < 5 ? 0 : 1)) & 3) * 128, d1 = tmem + ((3 * t + (i < 5 ? 0 : 2)) & 3) * 128;
+        const uint32_t start0 = i == 0 || i == 5 ? 0u : 1u, start1 = i == 5 ? 0u : 1u;
 #pragma unroll
         for (int op = 0; op < F_OPS; ++op)
-          umma_f16(di + fold.d_col[op], ai + fold.a_off[op], plain_desc_hi(2 * P1X_ROW), bi + fold.b_row[op], plain_desc_hi(128), fold.idesc[op],
-                   op ? 1u : start);
+          umma_f16((op < F_OPS / 2 ? d0 : d1) + fold.d_col[op], ai + fold.a_off[op], plain_desc_hi(2 * P1X_ROW), bi + fold.b_row[op], plain_desc_hi(128),
+                   fold.idesc[op], op == 0 ? start0 : (op == F_OPS / 2 ? start1 : 1u));
       }
+      if (!ok) break;
       umma_commit(&a_empty[buf]);
-      umma_commit(&acc_full[buf]);
+      umma_commit(acc_full);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -192,24 +203,24 @@ __global__ void __launch_bounds__(F_THREADS, 1) conv2_fwd_x3(GradStepArgs a, Gro
     const int r = quarter * 32 + lane, g = r >> 3, px = r & 7, sp = g >> 3, py = g & 7, pp = py * 7 + px;
     const int64_t rows = (int64_t)a.W * a.b;
     for (int t = 0; t < n_tiles; ++t) {
-      const int buf = t & 1;
-      if (!warp_wait(&acc_full[buf], (t >> 1) & 1, abort_flag)) { *abort_flag = 1; break; }
+      if (!warp_wait(acc_full, t & 1, abort_flag)) { *abort_flag = 1; break; }
       tc_fence_after();
       const int64_t row = r_begin + 2 * t + sp;
       float v[4][16];                        // [column range][channel]
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        uint32_t lead[16], small[16];
-        const uint32_t at = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 256 + j * 32 + ch * 16);
-        tmem_ld16(at, lead);
-        tmem_ld16(at + 128, small);
+        uint32_t small[16], even[16], odd[16];
+        const uint32_t at = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(j * 32 + ch * 16);
+        tmem_ld16(at + (3 * t & 3) * 128, small);
+        tmem_ld16(at + ((3 * t + 1) & 3) * 128, even);
+        tmem_ld16(at + ((3 * t + 2) & 3) * 128, odd);
         tmem_ld_wait();
 #pragma unroll
-        for (int o = 0; o < 16; ++o) v[j][o] = join3(__uint_as_float(lead[o]), __uint_as_float(small[o]));
+        for (int o = 0; o < 16; ++o) v[j][o] = join3(__uint_as_float(even[o]) + __uint_as_float(odd[o]), __uint_as_float(small[o]));
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[buf]);
+      if (lane == 0) mbar_arrive(acc_empty);
       if (py < 7 && px < 7 && row < r_end) {
         uint32_t codes[4] = {0u, 0u, 0u, 0u};
 #pragma unroll

@@ -393,6 +393,61 @@ def _float64_gradient(theta, x, y, keep, drop_p=0.25):
     return {n: v.grad.flatten() for n, v in p.items()}
 
 
+# One sample; a few; the dense layer's products with k split over eight and fewer CTAs; its input gradient without; all without
+@pytest.mark.parametrize("W,b,seeds", [(1, 1, (5, 6, 7, 8, 9, 10, 11)), (2, 8, (5, 6, 7)), (3, 37, (5, 6)), (12, 128, (5,)), (38, 128, (5,))])
+def test_fp32_gradients_are_as_near_to_float64_as_single_precision(W, b, seeds):
+    """Relative 2-norm error of every gradient tensor, median over workers and inputs (a worker in which a pooling or ReLU decision
+    within rounding distance of a tie falls the other way counts no more than another).  Any one of the six products of pieces
+    left out or taken with another's operand is four times the bound or more off (test_bf16_pieces.py)."""
+    from tests.test_bf16_pieces import PRECISION_FP32
+    from paper_2406_05546_b200 import ps
+    import torch
+    errs = {}
+    for seed in seeds:
+        theta = synth.init_params(seed=seed, bias_scale=0.05)
+        srv = ps.ParameterServer(theta, max_workers=W, max_batch=b, queue_slots=W)
+        gen = torch.Generator(device="cuda").manual_seed(seed)
+        x = torch.rand((W, b, 28, 28), generator=gen, device="cuda")
+        y = torch.randint(0, 10, (W, b), generator=gen, device="cuda", dtype=torch.int32)
+        grads = torch.zeros((W, ps.P_PAD), device="cuda")
+        srv.workers_grad_step([srv.ps_pull_snapshot(w) for w in range(W)], range(W), x, y, SEED, 1, grads_dev=grads)
+        for w in range(0, W, max(1, W // 7)):
+            want = _float64_gradient(theta, x[w], y[w], srv.ps_dropout_mask(SEED, w, 1, b))
+            for name, off, shape in synth.layout():
+                got = grads[w, off:off + int(np.prod(shape))].double()
+                errs.setdefault(name, []).append(float((got - want[name]).norm() / want[name].norm()))
+        srv.close()
+    median = {name: float(np.median(e)) for name, e in errs.items()}
+    assert max(median.values()) <= PRECISION_FP32, median
+
+
+@pytest.mark.parametrize("W,b", [(1, 3), (5, 1000)])
+def test_fp32_weights_above_the_largest_bf16_stay_finite(W, b):
+    """3.4e38 is a float and rounds to no BF16: its first piece is cut off instead.  One weight of a hidden unit that the output layer does not
+    listen to (0 x infinity would be NaN there); the unit shows in the gradient of its output weights."""
+    from paper_2406_05546_b200 import ps
+    import torch
+    import torch.nn.functional as F
+    theta = synth.init_params(seed=1, bias_scale=0.05)
+    at = {n: o for n, o, _ in synth.layout()}
+    theta[160:4768] = 0.05 * np.abs(theta[160:4768])       # activations above zero and well below one
+    theta[at["fc1.w"] + 7 * 1568:at["fc1.w"] + 8 * 1568] = 0
+    theta[at["fc1.w"] + 7 * 1568 + 700] = 3.4e38
+    theta[at["fc2.w"]:at["fc2.w"] + 5120].reshape(10, 512)[:, 7] = 0
+    srv = ps.ParameterServer(theta, max_workers=W, max_batch=b, queue_slots=W, dropout_p=0.0)
+    gen = torch.Generator(device="cuda").manual_seed(b)
+    x = 0.1 * torch.rand((W, b, 28, 28), generator=gen, device="cuda")
+    y = torch.randint(0, 10, (W, b), generator=gen, device="cuda", dtype=torch.int32)
+    grads = torch.zeros((W, ps.P_PAD), device="cuda")
+    loss, _ = srv.workers_grad_step([srv.ps_pull_snapshot(w) for w in range(W)], range(W), x, y, SEED, 1, grads_dev=grads)
+    assert torch.isfinite(loss).all() and torch.isfinite(grads).all()
+    for w in sorted({0, W - 1}):
+        want = _float64_gradient(theta, x[w], y[w], torch.ones((b, 512), device="cuda"), drop_p=0.0)["fc2.w"].view(10, 512)[:, 7]
+        got = grads[w, at["fc2.w"]:at["fc2.w"] + 5120].double().view(10, 512)[:, 7]
+        assert float(want.abs().max()) > 1e35 and (got - want).norm() <= 1e-5 * want.norm()
+    srv.close()
+
+
 def test_fp32_forward_pass_loses_nothing_that_adds_up_over_samples():
     """The tensor cores' accumulators truncate.  What that takes from a forward sum is alike in every sample, so that it stays in a sum over
     samples in which rounding averages out, first of all in the output layer's gradient, which is proportional to the hidden units:

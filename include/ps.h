@@ -66,7 +66,10 @@ enum {
 };
 
 /* Arithmetic of the dense contractions of part A.  PS_FP32: single precision
- * throughout; the dense layer's products run on the tensor cores with every operand as three BF16 pieces.  PS_BF16: the
+ * throughout.  The products of the second convolution and of the dense layer run on the tensor cores with every operand as the sum of
+ * three BF16 pieces (all 24 bits; fewer below 2^-110 in magnitude) and FP32 accumulation; a worker's gradient is within about 2e-7
+ * (2-norm) of float64 where no pooling or ReLU decision lies within rounding distance of a tie.  The order of a sum depends on the
+ * call's number of rows.  Infinities and NaN propagate as in FP32 sums over the positions of the maps.  PS_BF16: the
  * tensor-core path: BF16 operands (fp32 accumulation) in the products of the second convolution and in the
  * first convolution's filter gradient, TF32 operands in the 512-unit layer; the first convolution's forward
  * pass and the output layer stay FP32.  PS_TF32 is reserved and not built (ps_create refuses it). */

@@ -524,8 +524,9 @@ int launch_eval(const GradStepArgs& a, const WorkerTable& wt, const GroupTable& 
 }
 
 // Launch order of one grad step.  On the tensor-core path the copies of the dense layer's weights are made on a
-// side stream while the convolutions run; on both paths the backward pass forks (FP32 path: 402 -> 350 us at 16 x 64,
-// 109 -> 85 at 2 x 8, most of it from the branches filling each other's last waves): once the output
+// side stream while the convolutions run; on both paths the backward pass forks (FP32 path, us per tick with no side stream / the second
+// only / both: 2 x 8 75 / 66 / 67, 8 x 16 94 / 79 / 82, 8 x 64 135 / 122 / 116, 16 x 64 171 / 166 / 160, 32 x 64 263 / 259 / 252, 128 x 128 1,546 / 1,544 /
+// 1,551: the branches fill each other's last waves): once the output
 // layer's backward has produced da1, the dense layer's per-worker weight gradient (bound by its 3.2 MB
 // per worker of writes) runs on a side stream next to the input-gradient chain, and once dp2 exists the
 // second convolution's filter gradient runs on another side stream next to its input gradient and the

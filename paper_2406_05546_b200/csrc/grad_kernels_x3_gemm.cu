@@ -15,10 +15,10 @@
 // Every wait on an mbarrier is bounded, as in the other tensor-core kernels.
 //
 // Measured (B200; 26.3 GFLOP per product at 128 workers x 128 samples, six times that on the tensor cores: 95 us at the measured BF16
-// rate; ~6 us of event overhead included; before: packed FP32 multiply-adds): forward 560 -> 119, input gradient 539 -> 144, weight
+// rate; ~6 us of event overhead included; before: packed FP32 multiply-adds): forward 560 -> 121, input gradient 539 -> 144, weight
 // gradient 515 -> 163 us (its 411 MiB of writes take 66 us at the copy rate); at 16 x 64: 72 -> 22, 58 -> 23, 42 -> 21; at 2 x 8: 17 -> 15,
-// 11 -> 13, 9 -> 11.  Ticks, before -> now: 2 x 8 62.8 -> 59.3 us, 4 x 16 82 -> 81 .. 86, 8 x 16 127 -> 103, 8 x 64 251 -> 175, 32 x 64 659 -> 431: the
-// former kernels are better at no size.
+// 11 -> 13, 9 -> 11.  Ticks, with the second convolution's products there as well: 8 x 8 75 -> 67 us, 8 x 16 125 -> 82, 8 x 64 246 -> 115, 32 x 64 649
+// -> 250: multiply-adds are better at no size.
 #include <cooperative_groups.h>
 #include <cuda.h>
 
@@ -40,7 +40,7 @@ constexpr int OUT_PITCH = 36, OUT_WARP_BYTES = 32 * OUT_PITCH * 4;      // a 32 
 
 // BUFS: accumulators of either kind that are used in turn.
 template <int OP_, int BN_, int BUFS_, int STAGES_, bool SPLIT_> struct Shape {
-  static constexpr int OP = OP_, BN = BN_, BUFS = BUFS_, STAGES = STAGES_, N = OP == X_FWD ? HID : FLAT;
+  static constexpr int OP = OP_, BN = BN_, BUFS = BUFS_, STAGES = STAGES_;
   static constexpr bool SPLIT = SPLIT_, A_MN = OP == X_DW, B_MN = OP != X_FWD;      // is the operand's row index contiguous?
   static constexpr int ACC = BN <= 128 ? 128 : 256;                               // tensor-memory columns of an accumulator
   static constexpr int B_COLS = B_MN ? (BN + 63) / 64 * 64 : BN;
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_x3(const __grid_constant__ Ma
     if (decode<S>(ga, gt, a.b, blockIdx.x, c)) {             // the same for all CTAs of a cluster
       cg::cluster_group cl = cg::this_cluster();
       cl.sync();
-      const int ranks = gridDim.z, rank = blockIdx.z, rows = min(BM, c.m_end - c.m0), cols = min(S::BN, S::N - c.n0);
+      const int ranks = gridDim.z, rank = blockIdx.z, rows = min(BM, c.m_end - c.m0), cols = min(S::BN, (S::OP == X_FWD ? HID : FLAT) - c.n0);
       float* part = reinterpret_cast<float*>(tiles);
       for (int e = rank * THREADS + tid; e < rows * (S::BN / 4); e += ranks * THREADS) {
         const int r = e / (S::BN / 4), q = e - r * (S::BN / 4), m = c.m0 + r, n = c.n0 + 4 * q;

@@ -910,10 +910,11 @@ int32_t ps_tick_host_submit(ps_ctx* x, int32_t W, int32_t b, const int32_t* lags
   if (x->ticks_submitted >= 2) CUDA_TRY(cudaStreamWaitEvent(x->copy_st, x->stage_free[set], 0));
   // A chunk has to be worth a grad step of its own: it costs the host a dozen launches and the device a chain of short
   // kernels.  us for a tick in 1 / 2 / 4 chunks, tensor-core path: 512 rows 216 / 268 / 394, 2,048 351 / 395 / 596,
-  // 4,096 562 / 584 / 702, 8,192 914 / 796 / 891, 16,384 1,694 / 1,417 / 1,312; FP32 path: 512 354 / 405 / 508,
-  // 1,024 607 / 591 / 704, 2,048 885 / 812 / 916, 8,192 2,548 / 2,410 / 2,459, all on the FP32 pipes; with its products on the tensor
-  // cores, 1 / 2 chunks on a host with a slow copy: 2,048 407 / 443, 3,072 756 / 557, 4,096 1,336 / 630, 6,144 1,008 / 919, 8,192
-  // 1,296 / 1,360.
+  // 4,096 562 / 584 / 702, 8,192 914 / 796 / 891, 16,384 1,694 / 1,417 / 1,312; FP32 path: 512 197 / 236 / 343, 1,024 270 / 329 / 406,
+  // 1,536 369 / 392 / 475, 2,048 424 / 441 / 556, 3,072 605 / 589 / 662, 4,096 707 / 651 / 740, 6,144 1,039 / 942 / 983, 8,192
+  // 1,314 / 1,133 / 1,133, 12,288 1,927 / 1,648 / 1,655, 16,384 2,506 / 2,090 / 1,972 (medians of five runs, the three in turn).
+  // The FP32 path's line at 1,024 rows is that of kernels on the FP32 pipes (607 / 591 / 704 there, 885 / 812 / 916 at 2,048); by the present times
+  // it would lie between 2,048 and 3,072.
   const bool two = rows >= (x->cfg.precision != PS_FP32 ? 6144u : 1024u);
   const int n_chunks = std::min(W, rows >= 12288 ? 4 : (two ? 2 : 1)), per = (W + n_chunks - 1) / n_chunks;
   for (int c = 0; c < n_chunks; ++c) {

@@ -151,19 +151,10 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Shared-memory matrix descriptor without swizzle, k-contiguous operand: a core matrix is 8 rows of
-// 16 bytes, stored contiguously (row pitch 16 bytes); `sbo` = byte distance between successive groups
-// of 8 rows, `lbo` = byte distance between the two 16-byte k-chunks of one MMA (K = 8 TF32 values).
-__device__ __forceinline__ uint64_t smem_desc_plain(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFF) >> 4);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
-  d |= (uint64_t)1 << 46;    // descriptor version
-  return d;                  // layout type 0: no swizzle
-}
-// The two halves of that descriptor: low = start address and leading byte offset, high = stride byte
-// offset, version and layout type.  Adding n to the low half moves the start address by 16*n bytes.
+// The two halves of a shared-memory matrix descriptor without swizzle.  k contiguous: a core matrix is 8 rows of 16 bytes, stored
+// contiguously (row pitch 16 bytes); `sbo` = byte distance between successive groups of 8 rows, `lbo` = byte distance between the two
+// 16-byte k-chunks of one MMA.  Low = start address and leading byte offset, high = stride byte offset, version and layout type (0: no
+// swizzle).  Adding n to the low half moves the start address by 16*n bytes.
 __host__ __device__ constexpr uint32_t plain_desc_hi(uint32_t sbo) { return ((sbo >> 4) & 0x3FFF) | (1u << 14); }
 __device__ __forceinline__ uint32_t plain_desc_lo(uint32_t addr, uint32_t lbo) {
   return ((addr & 0x3FFFF) >> 4) | (((lbo >> 4) & 0x3FFF) << 16);

@@ -25,7 +25,7 @@
 // 210, input gradient 636 -> 176, filter gradient 651 -> 271 us; at 16 x 64: 56 -> 25, 57 -> 21, 56 -> 31; at 2 x 8: 12 -> 13, 15 -> 11,
 // 15 -> 14.  Forward and input gradient are bound by the instructions' own time; the filter gradient takes 1.5 times as many products as
 // it needs, rounded up to 128 rows.  Relative error against float64, median over workers, 128 x 128: conv2.w 1.7e-7 -> 0.8e-7, conv1.w
-// 1.7e-7 -> 1.0e-7; 2 x 8: 2.9e-7 -> 1.3e-7, 3.3e-7 -> 1.6e-7.
+// 1.7e-7 -> 1.0e-7; 2 x 8: 2.9e-7 -> 1.2e-7, 3.3e-7 -> 1.5e-7.
 //
 // Each kernel's stages (copies, staging, MMA issue, read-out) run in different warps and overlap through mbarriers; every wait
 // is bounded.
